@@ -302,3 +302,85 @@ def run(s):
         return {"out": s.out, "lse": s.lse}
     s.ctx.seer_kcomp_append(s.shape, s.gate, s.lens, s.k_nope, first_block=0, num_blocks=s.n)
     return {"kcomp": s.kcomp}
+
+
+# ---- the same results in 64 bits, in plain torch ------------------------------------------------------------------
+
+def _rope(y, pos):
+    """Rotate-half pairing (c, c + d_gate/2); y [..., d_gate] float64, pos: one position per row of y's last but one axis."""
+    half = y.shape[-1] // 2
+    freq = THETA ** (-2.0 * torch.arange(half, device="cuda", dtype=torch.float64) / y.shape[-1])
+    ang = pos.to(torch.float64)[:, None] * freq
+    a, d = y[..., :half], y[..., half:]
+    return torch.cat([a * ang.cos() - d * ang.sin(), d * ang.cos() + a * ang.sin()], -1)
+
+
+def _pooled(rows, w, first, b):
+    """Compressed keys of the complete blocks of `rows` [n * b, d], the first of which is block `first`."""
+    x = rows.double().view(-1, b, D)
+    feat = torch.cat([x.amax(1), x.amin(1), x.mean(1)], -1)
+    return _rope(feat @ w.double().T, (first + torch.arange(len(x), device="cuda")) * b)
+
+
+def _list64(c, s, i, h, L, max_sel):
+    """The blocks that the gate selects for sequence i, KV head h, in ascending order."""
+    b, ql, g = c["block"], c["q_len"], c["hq"] // c["hkv"]
+    n, j_f = _blocks(c, L), max(0, L - ql) // b
+    n_forced = min(n - j_f, max_sel)
+    x = s.q_nope.view(c["batch"], ql, c["hq"], D)[i, :, h * g:(h + 1) * g].reshape(ql, g * D).double()
+    qg = _rope(x @ s.w_q[h].double().T, (L - ql + torch.arange(ql, device="cuda")).clamp(min=0))
+    score = (s.kcomp[i, h, :j_f].double() @ qg.T).amax(1) / math.sqrt(c["d_gate"])
+    if c["kind"] == "threshold":
+        need = int((score.softmax(0) > c["threshold"]).sum()) if j_f else 0
+        need = min(need, max_sel - n_forced)
+    else:
+        need = min(max(1, c["budget"] // b), n, max_sel) - n_forced
+    best = score.sort(descending=True, stable=True).indices[:max(0, min(need, j_f))]
+    return torch.cat([best.sort().values, torch.arange(n - n_forced, n, device="cuda")])
+
+
+def exact(case, seed):
+    """What ``run`` returns for these inputs, in 64 bits; no value is given for the lists."""
+    c, s = case, prepare(case, seed)
+    hkv, b, ql, g, lens = c["hkv"], c["block"], c["q_len"], c["hq"] // c["hkv"], _lengths(c)
+    if c["kind"] == "build":
+        kcomp = torch.zeros(s.kcomp.shape, dtype=torch.float64, device="cuda")
+        for i, L in enumerate(lens):
+            for h in range(hkv):
+                n = L // b
+                kcomp[i, h, :n] = _pooled(s.k_nope[i, h, :n * b], s.w_k[h], 0, b)
+        return {"kcomp": kcomp}
+    out = torch.zeros((c["batch"], ql, c["hq"], D), dtype=torch.float64, device="cuda")
+    lse = torch.full(out.shape[:-1], -math.inf, dtype=torch.float64, device="cuda")
+    q = s.q.view(out.shape)
+    for i, L in enumerate(lens):
+        for h in range(hkv):
+            if c["kind"] == "dense":
+                blocks = torch.arange(_blocks(c, L), device="cuda")
+            elif c["kind"] == "sparse":
+                blocks = s.idx[i, h, :int(s.cnt[i, h])].long()
+            else:
+                blocks = _list64(c, s, i, h, L, s.max_sel)
+            t = (blocks[:, None] * b + torch.arange(b, device="cuda")).view(-1)
+            t = t[t < L]
+            if s.table is None:
+                k, v = s.k[i, h, t].double(), s.v[i, h, t].double()
+            else:
+                page, row = s.table[i].long()[t // c["page"]], t % c["page"]
+                k, v = s.k[page, h, row].double(), s.v[page, h, row].double()
+            for x in range(ql):
+                z = q[i, x, h * g:(h + 1) * g].double() @ k.T * SCALE
+                z = z.masked_fill(t > L - ql + x, -math.inf)
+                lse[i, x, h * g:(h + 1) * g] = z.logsumexp(1)
+                out[i, x, h * g:(h + 1) * g] = z.softmax(1) @ v
+    res = {"out": out.view(s.q.shape), "lse": lse.view(s.lse.shape)}
+    if c["kind"] not in ("dense", "sparse"):
+        res["idx"] = res["cnt"] = None
+    if c["kind"] in ("step", "multi"):
+        kcomp = s.kcomp.double()
+        for i, L in enumerate(lens):
+            if L >= b and L % b < ql:
+                for h in range(hkv):
+                    kcomp[i, h, L // b - 1] = _pooled(s.window[i, h], s.w_k[h], L // b - 1, b)[0]
+        res["kcomp"] = kcomp
+    return res

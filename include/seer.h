@@ -114,8 +114,10 @@ typedef struct {
 /* Creates a context on CUDA device `device` and allocates its workspace
  * (workspace_bytes, 0 = a default of 64 MiB; partial results of split
  * sequences, gate scratch, status words).  *out is NULL on failure.
- * Read from the environment at creation: SEER_DECODE_WIDE_VARIANT and
- * SEER_STEP_LIST_FLAGS (the latter under seer_decode_step); read at the
+ * Read from the environment at creation: SEER_DECODE_WIDE_VARIANT,
+ * SEER_STEP_LIST_FLAGS (under seer_decode_step) and SEER_STEP_CLUSTERS (0:
+ * single-token calls never take the one-launch form for short lists, below);
+ * read at the
  * process's first gate call: SEER_GATE_WIDEN (0: the gate's clusters keep one
  * CTA per 512 compressed keys also when there are few sequences; n: they may be
  * widened while all of them fit the SMs at n CTAs each, default 2).  Also at
@@ -195,7 +197,9 @@ seer_status seer_dense_decode(seer_ctx* ctx, const seer_shape* shape, const seer
  *            list (NULL = all max_sel entries, relying on negative padding).
  * The selected blocks of all (sequence, KV head) pairs are cut into 64-token
  * tiles and dealt out evenly over the CTAs; pieces of one pair meet in a
- * log-sum-exp combine done by the last CTA to finish (no second launch).
+ * log-sum-exp combine done by the last CTA to finish (no second launch).  With
+ * few tiles per pair -- max_sel decides, at most 64 per CTA -- every pair has a
+ * thread-block cluster of its own instead, which combines in shared memory.
  * A list with no valid entry gives out = 0, lse = -inf.
  * block_idx, block_cnt and seq_lens may be written by the kernel launched just
  * before this call on the stream: they are read only once that kernel has completed.
@@ -332,8 +336,9 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
  * and token-budget selection (Eq. 1a/1c, Sec. 3.1), block-sparse decode over the selected
  * blocks (Sec. 3.3).  The results are those of the three calls
  *     seer_kcomp_append(.., first_block = -1) ; seer_gate_select(.., scores_in = NULL) ; seer_sparse_decode
- * on `stream`, with one host round trip instead of three.  (The launches go out as gate, attention,
- * append: the block that has just filled is the sequence's last block, which the gate takes without
+ * on `stream`, with one host round trip instead of three.  (With few tiles per list, as in
+ * seer_sparse_decode, and at most 16384 compressed keys per sequence, gate and attention are one launch;
+ * the append follows.  Otherwise the launches go out as gate, attention, append: the block that has just filled is the sequence's last block, which the gate takes without
  * scoring it, so the entry the append writes is first read in the next step.  When gate->max_blocks
  * blocks cover kv->max_seq_len, the attention kernel knows every list's length from the sequence
  * lengths and the budget; the gate kernel then marks each list as it finishes it and the attention

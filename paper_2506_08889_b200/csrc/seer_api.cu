@@ -52,6 +52,7 @@ struct seer_ctx {
     int list_gen;               // != 0 inside seer_decode_step: the gate marks finished lists with it, the attention kernel waits per unit
     int list_gen_last;          // the last such number handed out
     int use_list_flags;         // 0: the attention kernel of a step waits for the whole gate kernel instead (SEER_STEP_LIST_FLAGS=0)
+    int use_clusters;           // 0: short calls, too, go through the kernels of long ones (SEER_STEP_CLUSTERS=0)
     int wide_variant;           // kernel variant code for more than 16 rows per unit: 16 (tcgen05), 8 (mma.sync), 0 (by size)
     char err[512];
 };
@@ -173,7 +174,8 @@ seer_status get_map(seer_ctx* ctx, const void* base, const uint64_t dims[4], con
 
 seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const void* q, int q_len,
                           const int32_t* block_idx, const int32_t* block_cnt, int max_sel, bool sparse,
-                          void* out, float* lse, void* stream) {
+                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, int cluster = 0) {
+    // (gate: the whole step in one launch, clusters of `cluster` CTAs)
     if (!ctx) return SEER_ERR_INVALID_ARG;
     seer_status st = check_shape(ctx, shape);
     if (st != SEER_OK) return st;
@@ -307,6 +309,15 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
 #ifdef SEER_DECODE_TRACE
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
+    if (!gate && q_len == 1 && ctx->use_clusters && ctx->list_gen == 0 && ctx->sel_from_lens == 0) cluster = step_cluster_size(U, max_tiles / U, 0, 0);
+    if (cluster > 0) {
+        p.t_cnt = 1;
+        p.rows = group;
+        ce = launch_step_cluster(mk_copy, *mv, p, gate, cluster, static_cast<cudaStream_t>(stream));
+        if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "decode launch: %s", cudaGetErrorString(ce));
+        ctx->launches += 1;
+        return SEER_OK;
+    }
     for (int t0 = 0; t0 < q_len; t0 += tok_per_launch) {
         p.t_base = t0;
         p.t_cnt = q_len - t0 < tok_per_launch ? q_len - t0 : tok_per_launch;
@@ -351,6 +362,8 @@ seer_status seer_create(seer_ctx** out, int device, size_t workspace_bytes) {
     if (const char* e = getenv("SEER_DECODE_MIN_TILES")) ctx->min_tiles = atoi(e);
     ctx->use_list_flags = 1;
     if (const char* e = getenv("SEER_STEP_LIST_FLAGS")) ctx->use_list_flags = atoi(e) != 0;
+    ctx->use_clusters = 1;
+    if (const char* e = getenv("SEER_STEP_CLUSTERS")) ctx->use_clusters = atoi(e) != 0;
     ctx->wide_variant = 0;      // chosen by the number of rows
     if (const char* e = getenv("SEER_DECODE_WIDE_VARIANT")) ctx->wide_variant = atoi(e) == 16 ? 16 : atoi(e) == 8 ? 8 : 0;
     ctx->ws_bytes = workspace_bytes ? workspace_bytes : (size_t)64 << 20;
@@ -538,11 +551,10 @@ seer_status seer_dense_decode_multi(seer_ctx* ctx, const seer_shape* shape, cons
     return decode_common(ctx, shape, kv, q, q_len, nullptr, nullptr, 0, false, out, lse, stream);
 }
 
-static seer_status gate_select_common(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate,
-                                      const int32_t* seq_lens, const void* q_nope, const float* scores_in,
-                                      int token_budget, int threshold_mode, float threshold, int32_t* block_idx,
-                                      int32_t* block_cnt, int max_sel, float* scores_out, void* stream,
-                                      int q_len = 1) {
+static seer_status gate_prepare(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate,
+                                const int32_t* seq_lens, const void* q_nope, const float* scores_in,
+                                int token_budget, int threshold_mode, float threshold, int32_t* block_idx,
+                                int32_t* block_cnt, int max_sel, float* scores_out, int q_len, GateParams* out) {
     if (!ctx) return SEER_ERR_INVALID_ARG;
     seer_status st = check_shape(ctx, shape);
     if (st != SEER_OK) return st;
@@ -567,7 +579,7 @@ static seer_status gate_select_common(seer_ctx* ctx, const seer_shape* shape, co
     cudaError_t ce = cudaSetDevice(ctx->device);
     if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "cudaSetDevice: %s", cudaGetErrorString(ce));
 
-    GateParams p;
+    GateParams& p = *out;
     memset(&p, 0, sizeof p);
     p.q_nope = static_cast<const __nv_bfloat16*>(q_nope);
     p.w_q = static_cast<const __nv_bfloat16*>(gate->w_q);
@@ -601,11 +613,26 @@ static seer_status gate_select_common(seer_ctx* ctx, const seer_shape* shape, co
     p.status = reinterpret_cast<unsigned int*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 19)));
 #endif
     if (!scores_in) fill_inv_freq(p.inv_freq, gate->d_gate, gate->rope_theta);
+    return SEER_OK;
+}
+
+static seer_status gate_launch(seer_ctx* ctx, const GateParams& p, void* stream) {
     int launched = 0;
-    ce = launch_gate_select(p, static_cast<cudaStream_t>(stream), &launched);
+    const cudaError_t ce = launch_gate_select(p, static_cast<cudaStream_t>(stream), &launched);
     ctx->launches += launched;
     if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "gate launch: %s", cudaGetErrorString(ce));
     return SEER_OK;
+}
+
+static seer_status gate_select_common(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate,
+                                      const int32_t* seq_lens, const void* q_nope, const float* scores_in,
+                                      int token_budget, int threshold_mode, float threshold, int32_t* block_idx,
+                                      int32_t* block_cnt, int max_sel, float* scores_out, void* stream,
+                                      int q_len = 1) {
+    GateParams p;
+    const seer_status st = gate_prepare(ctx, shape, gate, seq_lens, q_nope, scores_in, token_budget, threshold_mode, threshold,
+                                        block_idx, block_cnt, max_sel, scores_out, q_len, &p);
+    return st != SEER_OK ? st : gate_launch(ctx, p, stream);
 }
 
 seer_status seer_gate_select(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate, const int32_t* seq_lens,
@@ -735,15 +762,31 @@ seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_
         ctx->list_gen_last = ctx->list_gen_last >= 0x7ffffff0 ? 1 : ctx->list_gen_last + 1;
         ctx->list_gen = ctx->list_gen_last;
     }
-    seer_status st = seer_gate_select(ctx, shape, gate, kv->seq_lens, q_nope, nullptr, token_budget, block_idx, block_cnt,
-                                      max_sel, nullptr, stream);
-    if (st != SEER_OK) {
-        ctx->list_gen = 0;
-        return st;
+    GateParams gp;
+    seer_status st = gate_prepare(ctx, shape, gate, kv->seq_lens, q_nope, nullptr, token_budget, 0, 0.f, block_idx, block_cnt, max_sel,
+                                  nullptr, 1, &gp);
+    // Short steps are one launch: every (sequence, KV head) unit has a cluster of its own.
+    int cluster = 0;
+    if (st == SEER_OK && ctx->use_clusters && gate->max_blocks <= kStepMaxBlocks) {
+        const long long bs = shape->block_size, cap = kv->max_seq_len > 0 ? (kv->max_seq_len + bs - 1) / bs : 1;
+        long long blocks = k_blocks < max_sel ? k_blocks : max_sel;
+        if (blocks > cap) blocks = cap;
+        const long long tiles = (blocks * bs + kTileTokens - 1) / kTileTokens;
+        cluster = step_cluster_size(shape->batch * shape->num_kv_heads, tiles, bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles,
+                                    gate->max_blocks);
     }
-    ctx->sel_from_lens = covered ? (k_blocks < max_sel ? k_blocks : max_sel) : 0;
-    st = seer_sparse_decode(ctx, shape, kv, q, block_idx, block_cnt, max_sel, out, lse, stream);
-    ctx->sel_from_lens = 0;
+    if (cluster > 0) {
+        st = decode_common(ctx, shape, kv, q, 1, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, cluster);
+    } else {
+        if (st == SEER_OK) st = gate_launch(ctx, gp, stream);
+        if (st != SEER_OK) {
+            ctx->list_gen = 0;
+            return st;
+        }
+        ctx->sel_from_lens = covered ? (k_blocks < max_sel ? k_blocks : max_sel) : 0;
+        st = seer_sparse_decode(ctx, shape, kv, q, block_idx, block_cnt, max_sel, out, lse, stream);
+        ctx->sel_from_lens = 0;
+    }
     ctx->list_gen = 0;
     if (st != SEER_OK || !k_nope) return st;
     return kcomp_append_common(ctx, shape, gate, kv->seq_lens, k_nope, k_nope_stride_batch, k_nope_stride_head,

@@ -1,0 +1,854 @@
+// Short decode calls: one thread-block cluster per (sequence, KV head) unit does everything, in one launch.
+//
+// The chain of kernels that serves long calls (seer_gate.cu, seer_decode.cu) spends, on a short one, most of its
+// time between its parts: lists through global memory, a schedule over all units, partial results published with
+// a fence and a ticket and read back by the last CTA.  Here the S CTAs (S = 1 .. 16) of a unit's cluster share
+// the unit from its first byte to its output:
+//   1. gate (GATE): the unit's gate query, spread over the cluster's warps, into every CTA's shared memory; the
+//      scores of the CTA's keys into the first CTA's; selection there; every listed tile's number into the
+//      shared memory of the CTA that will read it (tile t belongs to CTA t mod S);
+//      list (!GATE): the CTA reads its tiles' numbers from the caller's list, or counts them off (dense);
+//   2. tiles: one producer warp keeps a ring of three 64-token K/V stages in flight; eight consumer warps, two
+//      groups of four, take alternate tiles, a warp 16 tokens (the same tensor-core steps as decode_kernel);
+//   3. combine: the warps' partials meet in shared memory, the CTA's go, a slice of the channels each, to the
+//      cluster's CTAs, which write their slice of the output after one cluster barrier.
+// Nothing between the steps leaves the SMs, and no CTA waits for another except at the cluster's hardware barrier.
+#include <cooperative_groups.h>
+
+#include "seer_gate_device.cuh"
+#include "seer_internal.h"
+
+namespace cg = cooperative_groups;
+
+namespace seer {
+
+namespace {
+
+constexpr int kStages = 3;
+constexpr int kWorkers = 256;                              // eight warps: gate, consumers, combine
+constexpr int kWarps = kWorkers / 32;
+constexpr int kThreads = kWorkers + 32;                    // ... and the producer warp
+constexpr int kHalfTileBytes = kTileTokens * 128;          // 64 rows x 128 B (64 bf16 channels)
+constexpr int kTileBytes = 2 * kHalfTileBytes;             // one K or V tile: 16 KiB
+constexpr int kStageBytes = 2 * kTileBytes;                // K + V
+constexpr int kMaxS = 16;
+constexpr int kCodes = 256;                                // tile (or gathered block) numbers that a CTA holds
+constexpr int kArrivals = 2 * kStages;
+constexpr int kBins = 1024;                                // histogram of the selection: four bins a thread
+constexpr int kMergeStride = 132;                          // floats per row of a warp's partial (bank spread)
+constexpr int kBatch = 8;                                  // 16-byte pieces of compressed keys per thread in flight
+constexpr int kChunkKeys = 32;                             // keys are dealt to the cluster's CTAs in runs of 32
+
+struct __align__(1024) StepSmem {
+    // K/V ring.  Before the first tile is asked for, the gate's: the scores of the unit (first CTA; up to
+    // kStepMaxBlocks) in stages 0 and 1, the staged first batch of keys in stage 2.  After the last tile: the warps'
+    // partials.
+    unsigned char ring[kStages][kStageBytes];
+    float qg[kMaxDGate];                                   // gate query
+    __align__(16) float recv_o[8 * kHeadDim];                         // [source CTA][row][this CTA's slice of the channels]
+    float2 recv_ml[kMaxS][8];                              // [source CTA][row]: max, sum
+    float2 warp_ml[kWarps][8];
+    // Tile n arrives in stage n % 3 and is announced on full[n % 6]: the two consumer groups take the even and the odd
+    // tiles, each at its own pace, and every one of the six barriers belongs to one of them, which follows all of its
+    // phases.  (With a barrier per stage a group would miss the other's phases and could take one that is two back for
+    // the one that it waits for.)
+    uint64_t full[kArrivals], empty[kStages];
+    int meta[kArrivals];                                   // valid tokens of the tile (blocks of 16 or 32 tokens: per block, 8 bits each)
+    int codes[kCodes];                                     // GATE: this CTA's tiles: 64-token tile numbers, or the gathered blocks
+    // selection (first CTA)
+    __align__(16) int hist[kBins + 4];                     // (read four bins at a time; the one past the last is for nobody)
+    int warp_tot[kWarps];
+    uint32_t list_key[32];
+    int list_j[32];
+    uint32_t pre_min, pre_max;                             // smallest and largest key of a candidate
+    uint32_t prefix;
+    int rem, bin_cnt, list_n, last_eq;
+};
+static_assert(sizeof(StepSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
+static_assert(kCodes * kMaxS <= kStageBytes / 4, "the list in stage 2");
+static_assert(kStepMaxBlocks * 4 <= 2 * kStageBytes && kBatch * kWorkers * 16 <= kStageBytes, "the gate's use of the ring");
+static_assert(kWarps * 8 * kMergeStride * 4 <= kStages * kStageBytes, "the partials' use of the ring");
+
+__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
+
+template <bool GATE>
+struct GateArg { GateParams g; };
+template <>
+struct GateArg<false> {};
+
+// The selection of the token budget's `need` best of the candidates [0, n_cand), by the first CTA's worker warps.
+// Leaves (thr, j_eq): candidate j is taken if its key is above thr, or equal to it and j <= j_eq.  Comparisons only:
+// the lower block number wins a tie, NaN is below every number.  A histogram over a monotone linear map of
+// [min, max] leaves a few candidates in the boundary bin, which every warp ranks for itself; crowded bins and ranges
+// that are not finite take radix passes over key - min instead.
+__device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, int n_cand, int need, int words, int warp, int lane,
+                                                 uint32_t& thr, int& j_eq) {
+    const int tid = 32 * warp + lane;
+    if (need >= n_cand) { thr = 0u; j_eq = 0x7fffffff; return; }
+    if (need <= 0) { thr = 0xffffffffu; j_eq = -1; return; }
+    const uint32_t kmin = sm.pre_min, kmax = sm.pre_max;
+    const float smin = key_score(kmin), smax = key_score(kmax);
+    const float range = smax - smin, scale = (kBins - 1.f) / range;
+    const int j0 = warp * words * 32 + lane;               // this lane's candidates: j0, j0 + 32, ...
+    // (four at a time, without branches: their loads go out together)
+    auto each = [&](auto&& fn) {
+#pragma unroll 1
+        for (int e = 0; e < words; e += 4) {
+            float v[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) v[x] = sc[min(j0 + 32 * (e + x), n_cand - 1)];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) fn((e + x < words) & (j0 + 32 * (e + x) < n_cand), score_key(v[x]), j0 + 32 * (e + x));
+        }
+    };
+    // The same for passes in any order, on the scores themselves: neighbouring blocks have similar scores, so the lanes of
+    // a warp take candidates that are far apart (lane l has run l of `run` blocks, from its own place in it on: no bank
+    // conflicts); side by side, their additions to the histogram would queue for a few bins.
+    const int run = (n_cand + 31) / 32, rot = (run & 1) ? 0 : lane % run;
+    auto each_spread = [&](auto&& fn) {
+#pragma unroll 1
+        for (int q = warp; q < run; q += 4 * kWarps) {
+            float v[4];
+            int jj[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                int at = q + x * kWarps + rot;
+                at -= at >= run ? run : 0;
+                jj[x] = q + x * kWarps < run ? min(lane * run + at, n_cand) : n_cand;      // (n_cand: none)
+                v[x] = sc[min(jj[x], n_cand - 1)];
+            }
+            fn(v, jj);
+        }
+    };
+    // thread t owns bins kBins-1-4t downwards: finds the bin that straddles the rem-th best key
+    auto find_bin = [&](int rem) {
+        worker_sync();
+        const int4 c4 = *reinterpret_cast<const int4*>(&sm.hist[kBins - 4 - 4 * tid]);
+        const int c[4] = {c4.w, c4.z, c4.y, c4.x};
+        const int mine = c[0] + c[1] + c[2] + c[3];
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) sm.warp_tot[warp] = incl;
+        worker_sync();
+        int above = incl - mine;
+#pragma unroll
+        for (int w2 = 0; w2 < kWarps; ++w2) above += w2 < warp ? sm.warp_tot[w2] : 0;
+        if (above < rem && rem <= above + mine) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                if (above < rem && rem <= above + c[x]) {
+                    sm.prefix = (uint32_t)(kBins - 1 - 4 * tid - x);
+                    sm.rem = rem - above;
+                    sm.bin_cnt = c[x];
+                }
+                above += c[x];
+            }
+        }
+        worker_sync();
+    };
+    if (smin > -INFINITY && range > 0.f && range < INFINITY && scale < INFINITY) {
+        // (every score is finite here; -0 and +0 have the same bin)
+        auto bin_of = [&](float s, int j) -> int { return j < n_cand ? min(kBins - 1, (int)((s - smin) * scale)) : kBins; };
+        each_spread([&](const float (&v)[4], const int (&j)[4]) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x) atomicAdd(&sm.hist[bin_of(v[x], j[x])], 1);
+        });
+        find_bin(need);
+        const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
+        if (cnt <= 32) {
+            each_spread([&](const float (&v)[4], const int (&j)[4]) {
+                bool in[4], any = false;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) any |= in[x] = bin_of(v[x], j[x]) == bin;
+                if (any) {
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        if (in[x]) {
+                            const int slot = atomicAdd(&sm.list_n, 1);
+                            sm.list_key[slot] = score_key(v[x]);
+                            sm.list_j[slot] = j[x];
+                        }
+                    }
+                }
+            });
+            worker_sync();
+            const uint32_t key = lane < cnt ? sm.list_key[lane] : 0u;
+            const int j = lane < cnt ? sm.list_j[lane] : 0x7fffffff;
+            int rank = 0;
+            for (int m = 0; m < cnt; ++m) {
+                const uint32_t km = __shfl_sync(0xffffffffu, key, m);
+                const int jm = __shfl_sync(0xffffffffu, j, m);
+                rank += km > key || (km == key && jm < j);
+            }
+            const int src = __ffs(__ballot_sync(0xffffffffu, lane < cnt && rank == rem - 1)) - 1;
+            thr = __shfl_sync(0xffffffffu, key, src);
+            j_eq = __shfl_sync(0xffffffffu, j, src);
+            return;
+        }
+    }
+    // radix passes of ten bits over key - kmin
+    int bits_left = 32 - __clz(max(kmax - kmin, 1u)), rem = need;
+    uint32_t prefix = 0u;
+    while (bits_left > 0) {
+        const int wbits = min(10, bits_left), shift = bits_left - wbits;
+        *reinterpret_cast<int4*>(&sm.hist[4 * tid]) = make_int4(0, 0, 0, 0);
+        worker_sync();
+        each([&](bool ok, uint32_t key, int) {
+            const uint32_t rel = key - kmin;
+            if (ok && (uint32_t)((unsigned long long)rel >> (shift + wbits)) == prefix)        // (shift + wbits can be 32)
+                atomicAdd(&sm.hist[(rel >> shift) & ((1u << wbits) - 1u)], 1);
+        });
+        find_bin(rem);
+        prefix = (prefix << wbits) | sm.prefix;
+        rem = sm.rem;
+        bits_left = shift;
+    }
+    thr = kmin + prefix;
+    // the rem-th candidate whose key equals thr, in block order (a warp's candidates are one run of blocks)
+    int n_eq = 0;
+    each([&](bool ok, uint32_t key, int) { n_eq += __popc(__ballot_sync(0xffffffffu, ok && key == thr)); });
+    worker_sync();                                         // (everybody has read the last pass's totals)
+    if (lane == 0) sm.warp_tot[warp] = n_eq;
+    worker_sync();
+    int before = 0;
+#pragma unroll
+    for (int w2 = 0; w2 < kWarps; ++w2) before += w2 < warp ? sm.warp_tot[w2] : 0;
+    if (before < rem && rem <= before + n_eq) {
+        each([&](bool ok, uint32_t key, int j) {
+            const bool eq = ok && key == thr;
+            const unsigned m = __ballot_sync(0xffffffffu, eq);
+            if (eq && before + __popc(m & ((1u << lane) - 1u)) == rem - 1) sm.last_eq = j;
+            before += __popc(m);
+        });
+    }
+    worker_sync();
+    j_eq = sm.last_eq;
+}
+
+// grid (S, units), cluster (S, 1, 1).  Short calls are bound by latency: 8 units x 64 blocks (16.8 MB, 2.6 us at memory
+// speed) take 13 us from the first read to the last write, of which the gate query 1.5, the scores 1.0, the selection
+// and the lists 3.3, the tiles 2.5, the combine 2.2 and four cluster barriers 0.5 to 1.0 each.  Longer ones by memory: 64
+// units x 205 blocks (430 MB) 70 us, 6.2 TB/s; CTAs that share a unit read neighbouring blocks at the same time.
+template <bool GATE>
+__global__ void __launch_bounds__(kThreads, 2)
+step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                    const __grid_constant__ DecodeParams p, const __grid_constant__ GateArg<GATE> ga) {
+    extern __shared__ unsigned char smem_raw[];
+    StepSmem& sm = *reinterpret_cast<StepSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), s_shift = 31 - __clz(S);
+    const int u = blockIdx.y, i = u / p.num_kv_heads, h = u - i * p.num_kv_heads;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool producer = warp == kWarps;
+    // (another CTA's shared memory is written only after the barrier this opens: it is then known to be running)
+    cluster_arrive();
+    if (tid < kArrivals) {
+        mbar_init(&sm.full[tid], 1);
+        if (tid < kStages) mbar_init(&sm.empty[tid], kWarps / 2);
+        mbar_fence_init();
+    }
+    if (producer && lane == 0) {
+        tma_prefetch_desc(&map_k);
+        tma_prefetch_desc(&map_v);
+    }
+
+    int n_blocks = 0, L = 0;                               // listed blocks of the unit, cached tokens
+    if constexpr (GATE) {
+        const GateParams& g = ga.g;
+        const int n = g.group * kHeadDim, chunks = n / 8, half = g.d_gate / 2;
+        const int nit = (chunks + 31) / 32;                // 16-byte pieces of a W_q row per lane (1..4)
+        const int gw = rank * kWarps + warp, n_gw = S * kWarps;
+        const int lpk_shift = g.d_gate == 64 ? 3 : g.d_gate == 128 ? 4 : 5, lpk = 1 << lpk_shift;   // lanes per key
+        const int csub = tid & (lpk - 1);
+        const uint4* kc = reinterpret_cast<const uint4*>(g.kcomp + (size_t)u * g.max_blocks * g.d_gate);
+        // this CTA's key number lk (runs of kChunkKeys, dealt round robin) is block
+        auto block_of = [&](int lk) { return (((lk / kChunkKeys) << s_shift) + rank) * kChunkKeys + (lk & (kChunkKeys - 1)); };
+        // W_q rows of this warp's first rotary pair: constants, requested before the wait
+        uint4 wv[2][4];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint4* wrow = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + gw % half + k * half) * n);
+#pragma unroll
+            for (int it = 0; it < 4; ++it) {
+                const int ch = lane + 32 * it;
+                wv[k][it] = (!producer && it < nit && gw < half && ch < chunks) ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+        if (rank == 0) {
+            for (int x = tid; x < kBins; x += kThreads) sm.hist[x] = 0;
+            if (tid == 0) { sm.pre_min = 0xffffffffu; sm.pre_max = 0u; sm.list_n = 0; }
+        }
+        pdl_wait();                                        // queries, lengths and compressed keys are final
+        L = p.seq_lens[i];
+        const uint4* xsrc = reinterpret_cast<const uint4*>(g.q_nope + ((size_t)i * g.num_q_heads + (size_t)h * g.group) * kHeadDim);
+        uint4 xv[4];
+        const int all_chunks = (g.max_blocks + kChunkKeys - 1) / kChunkKeys;
+        const int total_cap = ((max(0, all_chunks - rank) + S - 1) >> s_shift) << (lpk_shift + 5);    // pieces, block numbers past the cache among them
+        uint4* staged = reinterpret_cast<uint4*>(sm.ring[2]);
+        float* sc_all = reinterpret_cast<float*>(sm.ring[0]);
+        if (!producer) {
+#pragma unroll
+            for (int it = 0; it < 4; ++it) {
+                const int ch = lane + 32 * it;
+                xv[it] = it < nit && ch < chunks ? __ldg(xsrc + ch) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            // the first batch of keys travels during the projection (entries past n_i - 1 exist in memory: harmless)
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) {
+                const int pc = k * kWorkers + tid, j = block_of(pc >> lpk_shift);
+                if (pc < total_cap && j < g.max_blocks) cp_async16(staged + pc, kc + ((size_t)j << lpk_shift) + csub);
+            }
+        }
+        const int n_i = L > 0 ? (L + g.block_size - 1) / g.block_size : 0;
+        const int j_f = L > 0 ? n_i - 1 : 0;               // the last block is always taken; the candidates are those before it
+        const int n_cand = min(j_f, g.max_blocks);
+        int need = 0;
+        if (n_i > 0) {
+            const int k = min(max(g.token_budget / g.block_size, 1), min(n_i, g.max_sel));
+            need = max(0, min(k - 1, n_cand));
+            n_blocks = need + 1;
+        }
+        // pieces that matter: up to the last run of keys with a candidate
+        const int cand_chunks = (n_cand + kChunkKeys - 1) / kChunkKeys;
+        const int total = ((max(0, cand_chunks - rank) + S - 1) >> s_shift) << (lpk_shift + 5);
+        cluster_wait();                                    // every CTA of the cluster has started
+        // ---- gate query: rotary pairs (c, c + d_gate/2) dealt to the cluster's warps --------------------------
+        if (!producer) {
+            for (int c = gw; c < half; c += n_gw) {
+                if (c != gw) {
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const uint4* wrow = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + c + k * half) * n);
+#pragma unroll
+                        for (int it = 0; it < 4; ++it) {
+                            const int ch = lane + 32 * it;
+                            wv[k][it] = it < nit && ch < chunks ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
+                }
+                float a = 0.f, b = 0.f;
+#pragma unroll
+                for (int it = 0; it < 4; ++it) {
+                    if (it < nit) { a += dot8(wv[0][it], xv[it]); b += dot8(wv[1][it], xv[it]); }
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    a += __shfl_xor_sync(0xffffffffu, a, off);
+                    b += __shfl_xor_sync(0xffffffffu, b, off);
+                }
+                float sn, cs;
+                rope_sincos((double)max(L - 1, 0), g.inv_freq[c], &sn, &cs);
+                if (lane < S) {                            // lane r stores into CTA r of the cluster
+                    float* dst = cluster.map_shared_rank(sm.qg, lane);
+                    dst[c] = a * cs - b * sn;
+                    dst[c + half] = b * cs + a * sn;
+                }
+            }
+        }
+        uint4 kv[kBatch];
+        auto request = [&](int cb) {
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) {
+                const int pc = cb + k * kWorkers + tid, j = block_of(pc >> lpk_shift);
+                kv[k] = pc < total && j < g.max_blocks ? __ldg(kc + ((size_t)j << lpk_shift) + csub) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        };
+        constexpr int kPieces = kWorkers * kBatch;
+        if (!producer) request(kPieces);                   // the second batch, into registers
+        cluster.sync();
+        // ---- scores, into the first CTA's shared memory --------------------------------------------------------
+        // A thread holds one piece of each of eight keys; reduce8 leaves every lane with the sum of one of the keys
+        // (that of its piece number krev).
+        if (!producer) {
+            float* sc0 = cluster.map_shared_rank(sc_all, 0);
+            const float inv = rsqrtf((float)g.d_gate);
+            const int krev = ((lane & 1) << 2) | (lane & 2) | ((lane >> 2) & 1);
+            const bool storer = (csub & ~7) == 0;
+            uint32_t kmn = 0xffffffffu, kmx = 0u;
+            float qsub[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) qsub[c] = sm.qg[8 * csub + c];
+            auto score_batch = [&](auto&& piece, int cb) {
+                float acc[kBatch];
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) acc[k] = dot8(piece(k), qsub);
+                const float v = reduce8(acc, lane, lpk) * inv;
+                const int pc = cb + krev * kWorkers + tid, j = block_of(pc >> lpk_shift);
+                if (storer && pc < total && j < n_cand) {
+                    sc0[j] = v;
+                    const uint32_t key = score_key(v);
+                    kmn = min(kmn, key);
+                    kmx = max(kmx, key);
+                }
+            };
+            for (int cb = 0; cb < total;) {
+                cp_async_wait_all();
+                score_batch([&](int k) {
+                    const int pc = k * kWorkers + tid;
+                    return cb + pc < total && block_of((cb + pc) >> lpk_shift) < g.max_blocks ? staged[pc] : make_uint4(0u, 0u, 0u, 0u);
+                }, cb);
+                cb += kPieces;
+                if (cb >= total) break;
+                // (batches alternate between the staged area and the registers; the one after the next is on its way)
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    const int pc = cb + kPieces + k * kWorkers + tid, j = block_of(pc >> lpk_shift);
+                    if (pc < total && j < g.max_blocks) cp_async16(staged + k * kWorkers + tid, kc + ((size_t)j << lpk_shift) + csub);
+                }
+                score_batch([&](int k) { return kv[k]; }, cb);
+                cb += kPieces;
+                request(cb + kPieces);
+            }
+            cp_async_wait_all();
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                kmn = min(kmn, __shfl_xor_sync(0xffffffffu, kmn, off));
+                kmx = max(kmx, __shfl_xor_sync(0xffffffffu, kmx, off));
+            }
+            if (lane == 0 && kmn <= kmx) {
+                atomicMin(cluster.map_shared_rank(&sm.pre_min, 0), kmn);
+                atomicMax(cluster.map_shared_rank(&sm.pre_max, 0), kmx);
+            }
+        }
+        cluster.sync();
+        // ---- selection, by the first CTA ----------------------------------------------------------------------------
+        if (rank == 0 && !producer) {
+            int32_t* dst = g.block_idx + (size_t)u * g.max_sel;
+            int* list = reinterpret_cast<int*>(sm.ring[2]);      // the listed blocks, ascending (the host's rule bounds their number)
+            const int words = ((n_cand + 31) / 32 + kWarps - 1) / kWarps;      // 32 candidates each, per warp
+            uint32_t thr;
+            int j_eq;
+            select_threshold(sm, sc_all, n_cand, need, words, warp, lane, thr, j_eq);
+            // which of the warp's candidates are taken: lane x keeps the words x and x + 32 (words <= 64)
+            const int jw = warp * words * 32 + lane;
+            unsigned taken[2] = {0u, 0u};
+#pragma unroll 1
+            for (int e = 0; e < words; e += 4) {
+                float v[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) v[x] = sc_all[min(jw + 32 * (e + x), n_cand - 1)];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int j = jw + 32 * (e + x);
+                    const uint32_t key = score_key(v[x]);
+                    const unsigned m = __ballot_sync(0xffffffffu, (e + x < words) & (j < n_cand) & ((key > thr) | ((key == thr) & (j <= j_eq))));
+                    if (lane == ((e + x) & 31)) { if (e + x < 32) taken[0] = m; else taken[1] = m; }
+                }
+            }
+            const int in_low = __popc(taken[0]), in_both = in_low + __popc(taken[1]);
+            int incl_low = in_low, incl_high = in_both - in_low;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int lo = __shfl_up_sync(0xffffffffu, incl_low, o), hi = __shfl_up_sync(0xffffffffu, incl_high, o);
+                if (lane >= o) { incl_low += lo; incl_high += hi; }
+            }
+            const int all_low = __shfl_sync(0xffffffffu, incl_low, 31);
+            worker_sync();
+            if (lane == 31) sm.warp_tot[warp] = incl_low + incl_high;
+            worker_sync();
+            int pos = 0;
+#pragma unroll
+            for (int w2 = 0; w2 < kWarps; ++w2) pos += w2 < warp ? sm.warp_tot[w2] : 0;
+            // every lane lists its own words' blocks
+            {
+                int at = pos + incl_low - in_low;
+                const int j_low = warp * words * 32 + 32 * lane;
+                for (unsigned m = taken[0]; m; m &= m - 1) list[at++] = j_low + __ffs(m) - 1;
+                at = pos + all_low + incl_high - (in_both - in_low);
+                for (unsigned m = taken[1]; m; m &= m - 1) list[at++] = j_low + 1024 + __ffs(m) - 1;
+            }
+            if (tid == 0) {
+                if (n_i > 0) list[need] = n_i - 1;
+                g.block_cnt[u] = n_blocks;
+            }
+            worker_sync();
+            // entry e of the list is block j: into the caller's list, and to the CTA that reads its tile(s)
+            for (int e = tid; e < g.max_sel; e += kWorkers) {
+                const int j = e < n_blocks ? list[e] : -1;
+                dst[e] = j;
+                if (e >= n_blocks) continue;
+                if (p.blocks_per_tile == 1) {
+                    for (int x = 0; x < p.tiles_per_block; ++x) {
+                        const int t = (e << p.tpb_shift) + x;
+                        if ((t >> s_shift) < kCodes) cluster.map_shared_rank(sm.codes, t & (S - 1))[t >> s_shift] = (j << p.tpb_shift) + x;
+                    }
+                } else {
+                    const int t = e >> p.bpt_shift, sub = e & (p.blocks_per_tile - 1);
+                    const int at = ((t >> s_shift) << p.bpt_shift) + sub;
+                    if (at < kCodes) cluster.map_shared_rank(sm.codes, t & (S - 1))[at] = j;
+                }
+            }
+        }
+        fence_proxy_async_smem();                          // the ring's memory goes over to the copy engine
+        __syncwarp();
+        cluster_arrive();
+    } else {
+        pdl_wait();
+        L = p.seq_lens[i];
+        if (p.block_idx) {
+            const int cnt = p.block_cnt ? p.block_cnt[u] : p.max_sel;      // (not behind the test on L: both loads in flight)
+            n_blocks = L > 0 ? max(0, min(cnt, p.max_sel)) : 0;
+        }
+        __syncthreads();                                   // barriers initialised
+    }
+
+    // ---- tiles ------------------------------------------------------------------------------------------------------
+    const bool dense = !GATE && !p.block_idx;
+    const bool small = !dense && p.blocks_per_tile > 1;
+    const int T = dense ? (L > 0 ? min((L + kTileTokens - 1) / kTileTokens, p.max_blocks_cap) : 0)
+                        : small ? (n_blocks + p.blocks_per_tile - 1) >> p.bpt_shift : n_blocks << p.tpb_shift;
+    const int n_mine = (max(0, T - rank) + S - 1) >> s_shift;
+    const int n_local = GATE ? min(n_mine, small ? kCodes >> p.bpt_shift : kCodes) : n_mine;     // (the host's rule keeps within kCodes)
+    const int row_u = i * p.num_q_heads + h * p.group;     // first of the unit's query rows
+    const int qd = lane & 3, rw = lane >> 2;
+    bool dead = false;                                     // a wait ran out: go through the motions, the results are invalid
+    if (producer) {
+        if (GATE) cluster_wait();                          // the tiles' numbers are in place
+        pdl_launch_dependents();
+        const int n_i = (L + p.block_size - 1) >> p.bs_shift;
+        for (int base = 0; base < n_local; base += 32) {
+            const int it = base + lane;
+            int row[4] = {0, 0, 0, 0}, outer[4] = {0, 0, 0, 0}, nv_all = 0, n_sub = 0;
+            if (it < n_local) {
+                const int t = (it << s_shift) + rank;
+                const int n_try = small ? p.blocks_per_tile : 1;
+                const int span = small ? p.block_size : kTileTokens;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    if (x < n_try) {
+                        int tok0 = -1;
+                        if (dense) {
+                            tok0 = t * kTileTokens;
+                        } else if (small) {
+                            const int e = (t << p.bpt_shift) + x;
+                            if (e < n_blocks) {
+                                const int blk = GATE ? sm.codes[(it << p.bpt_shift) + x] : p.block_idx[(size_t)u * p.max_sel + e];
+                                if (!GATE && blk >= n_i) raise_status(p.status, DEV_BAD_INDEX);
+                                if (blk >= 0 && blk < n_i) tok0 = blk << p.bs_shift;
+                            }
+                        } else if (GATE) {
+                            tok0 = sm.codes[it] * kTileTokens;
+                        } else {
+                            const int blk = p.block_idx[(size_t)u * p.max_sel + (t >> p.tpb_shift)];
+                            if (blk >= n_i) raise_status(p.status, DEV_BAD_INDEX);
+                            if (blk >= 0 && blk < n_i) tok0 = (blk << p.bs_shift) + (t & (p.tiles_per_block - 1)) * kTileTokens;
+                        }
+                        int nv = tok0 >= 0 ? max(0, min(span, L - tok0)) : 0;
+                        if (nv > 0) {
+                            outer[x] = i;
+                            row[x] = tok0;
+                            if (p.page_table) {
+                                const int pg = p.page_table[(size_t)i * p.page_table_stride + tok0 / p.page_size];
+                                outer[x] = pg;
+                                row[x] = tok0 % p.page_size;
+                                if (pg < 0 || pg >= p.num_pages) { raise_status(p.status, DEV_BAD_INDEX); nv = 0; }
+                            }
+                        }
+                        nv_all |= nv << (8 * x);
+                        n_sub += nv > 0;
+                    }
+                }
+            }
+            __syncwarp();
+            // lane s asks for tile s of the batch
+            const int m = min(32, n_local - base);
+            for (int s = 0; s < m; ++s) {
+                if (lane == s) {
+                    const int st = it % kStages;
+                    if (!dead && !mbar_wait(&sm.empty[st], ((it / kStages) & 1) ^ 1, p.status)) dead = true;
+                    unsigned char* dst = sm.ring[st];
+                    uint64_t* full = &sm.full[it % kArrivals];
+                    sm.meta[it % kArrivals] = nv_all;      // (the tile six back has been read: three back is, which came after it)
+                    if (dead || n_sub == 0) {
+                        mbar_arrive(full);
+                    } else if (small) {
+                        const int sub_bytes = p.block_size * 128;      // one half (64 channels) of one block
+                        mbar_arrive_expect_tx(full, (uint32_t)(n_sub * 4 * sub_bytes));
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            if ((nv_all >> (8 * x)) & 0xff) {
+                                unsigned char* d2 = dst + x * sub_bytes;
+                                tma_load_4d(d2, &map_k, full, 0, row[x], h, outer[x]);
+                                tma_load_4d(d2 + kHalfTileBytes, &map_k, full, 64, row[x], h, outer[x]);
+                                tma_load_4d(d2 + kTileBytes, &map_v, full, 0, row[x], h, outer[x]);
+                                tma_load_4d(d2 + kTileBytes + kHalfTileBytes, &map_v, full, 64, row[x], h, outer[x]);
+                            }
+                        }
+                    } else {
+                        mbar_arrive_expect_tx(full, kStageBytes);
+                        tma_load_4d(dst, &map_k, full, 0, row[0], h, outer[0]);
+                        tma_load_4d(dst + kHalfTileBytes, &map_k, full, 64, row[0], h, outer[0]);
+                        tma_load_4d(dst + kTileBytes, &map_v, full, 0, row[0], h, outer[0]);
+                        tma_load_4d(dst + kTileBytes + kHalfTileBytes, &map_v, full, 64, row[0], h, outer[0]);
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        if (!GATE) cluster_wait();                         // (the barrier opened at the top)
+    } else {
+        // Q^T B-fragments: this thread supplies row rw of the unit's queries
+        uint32_t bq[8][2];
+        {
+            const uint32_t* qrow = reinterpret_cast<const uint32_t*>(p.q + (size_t)(row_u + (rw < p.group ? rw : 0)) * kHeadDim);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                bq[ks][0] = rw < p.group ? __ldg(qrow + 8 * ks + qd) : 0u;
+                bq[ks][1] = rw < p.group ? __ldg(qrow + 8 * ks + 4 + qd) : 0u;
+            }
+        }
+        if (GATE) cluster_wait();
+        pdl_launch_dependents();
+        const int w4 = warp & 3;                           // which 16 of a tile's tokens
+        float o[8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+#pragma unroll
+        for (int a = 0; a < 8; ++a) o[a][0] = o[a][1] = o[a][2] = o[a][3] = 0.f;
+        // lane-constant parts of the ldmatrix addresses (swizzle: 16-B chunk ^= row & 7)
+        const int k_row = 16 * w4 + ((lane >> 3) & 1) * 8 + (lane & 7), k_csel = lane >> 4;
+        const int v_row = 16 * w4 + ((lane >> 4) & 1) * 8 + (lane & 7), v_csel = (lane >> 3) & 1;
+        const int sw = lane & 7;
+        // blocks of 16 or 32 tokens: which of the gathered blocks this warp's rows belong to, and where in it
+        const int sub_w = !small ? 0 : p.block_size == 16 ? w4 : w4 >> 1;
+        const int off_w = !small ? 16 * w4 : p.block_size == 16 ? 0 : (w4 & 1) * 16;
+        for (int it = warp >> 2; it < n_local; it += 2) {
+            const int st = it % kStages;
+            if (!dead && !mbar_wait(&sm.full[it % kArrivals], (it / kArrivals) & 1, p.status)) dead = true;
+            const int nvw = (small ? (sm.meta[it % kArrivals] >> (8 * sub_w)) & 0xff : sm.meta[it % kArrivals]) - off_w;   // valid tokens from this warp's first row on
+            if (nvw > 0 && !dead) {
+                const uint32_t kbase = smem_u32(sm.ring[st]), vbase = kbase + kTileBytes;
+                if (nvw < 16) {
+                    // ragged tail: rows past the sequence end may hold anything; this warp's are cleared in V, so that
+                    // a zero probability times garbage cannot produce NaN
+                    unsigned char* vt = sm.ring[st] + kTileBytes;
+                    for (int x = lane; x < (16 - nvw) * 16; x += 32) {
+                        const int r = 16 * w4 + nvw + (x >> 4), part = x & 15;
+                        *reinterpret_cast<uint4*>(vt + (part >> 3) * kHalfTileBytes + r * 128 + ((part & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                }
+                // ---- S^T = K . Q^T (four short accumulator chains) ----
+                float sa[4][4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) sa[x][0] = sa[x][1] = sa[x][2] = sa[x][3] = 0.f;
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks) {
+                    uint32_t a[4];
+                    const int c8 = ((2 * ks) & 7) + k_csel;
+                    ldmatrix_x4(a, kbase + (ks >> 2) * kHalfTileBytes + k_row * 128 + ((c8 ^ sw) << 4));
+                    mma_bf16_16816(sa[ks & 3], a, bq[ks][0], bq[ks][1]);
+                }
+                float s[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) s[x] = ((sa[0][x] + sa[1][x]) + (sa[2][x] + sa[3][x])) * p.scale_log2;
+                if (rw >= nvw) s[0] = s[1] = -INFINITY;
+                if (rw + 8 >= nvw) s[2] = s[3] = -INFINITY;
+                // ---- online softmax over this warp's 16 tokens, per row (column of S^T) ----
+                float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
+#pragma unroll
+                for (int off = 4; off < 32; off <<= 1) {
+                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, off));
+                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, off));
+                }
+                const float mn0 = fmaxf(m_run[0], mx0), mn1 = fmaxf(m_run[1], mx1);
+                // a row that has seen nothing so far keeps max = -inf; exponents are then taken against 0
+                const float mb0 = mn0 == -INFINITY ? 0.f : mn0, mb1 = mn1 == -INFINITY ? 0.f : mn1;
+                const float al0 = fast_exp2(m_run[0] - mb0), al1 = fast_exp2(m_run[1] - mb1);
+                const bool same_max = __all_sync(0xffffffffu, m_run[0] == mn0 && m_run[1] == mn1);
+                m_run[0] = mn0;
+                m_run[1] = mn1;
+                const float p0 = fast_exp2(s[0] - mb0), p1 = fast_exp2(s[1] - mb1);
+                const float p2 = fast_exp2(s[2] - mb0), p3 = fast_exp2(s[3] - mb1);
+                l_run[0] = l_run[0] * al0 + (p0 + p2);
+                l_run[1] = l_run[1] * al1 + (p1 + p3);
+                if (!same_max) {
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) { o[a][0] *= al0; o[a][1] *= al1; o[a][2] *= al0; o[a][3] *= al1; }
+                }
+                const uint32_t b0 = movmatrix_trans(pack_bf16x2(p0, p1));      // tokens 0-7 of the slice
+                const uint32_t b1 = movmatrix_trans(pack_bf16x2(p2, p3));      // tokens 8-15
+                // ---- O^T += V^T . P^T ----
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    uint32_t f[4];
+                    const int c8 = ((2 * a) & 7) + v_csel;
+                    ldmatrix_x4_trans(f, vbase + (a >> 2) * kHalfTileBytes + v_row * 128 + ((c8 ^ sw) << 4));
+                    mma_bf16_16816(o[a], f, b0, b1);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.empty[st]);
+        }
+        // ---- combine: warps, then CTAs ------------------------------------------------------------------------------
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) {
+            l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], off);
+            l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], off);
+        }
+        worker_sync();                                     // every tile has been read: the ring is free
+        float* part = reinterpret_cast<float*>(sm.ring[0]) + warp * 8 * kMergeStride;
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+            const int d0 = 16 * a + rw;
+            part[2 * qd * kMergeStride + d0] = o[a][0];
+            part[(2 * qd + 1) * kMergeStride + d0] = o[a][1];
+            part[2 * qd * kMergeStride + d0 + 8] = o[a][2];
+            part[(2 * qd + 1) * kMergeStride + d0 + 8] = o[a][3];
+        }
+        if (rw == 0) {
+            sm.warp_ml[warp][2 * qd] = make_float2(m_run[0], l_run[0]);
+            sm.warp_ml[warp][2 * qd + 1] = make_float2(m_run[1], l_run[1]);
+        }
+        __syncwarp();
+        if (!GATE) cluster_wait();                         // every CTA of the cluster has started (the barrier opened at the top)
+        worker_sync();
+        const int c_shift = 7 - s_shift;                   // log2 of the channels of a CTA's slice
+        {
+            // warp w: row w; lane: four channels
+            const int r = warp, c = 4 * lane;
+            float M = -INFINITY, l = 0.f;
+            float2 ml[kWarps];
+#pragma unroll
+            for (int x = 0; x < kWarps; ++x) {
+                ml[x] = sm.warp_ml[x][r];
+                M = fmaxf(M, ml[x].x);
+            }
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float* src = reinterpret_cast<const float*>(sm.ring[0]) + r * kMergeStride + c;
+#pragma unroll
+            for (int x = 0; x < kWarps; ++x) {
+                const float f = ml[x].x == -INFINITY ? 0.f : fast_exp2(ml[x].x - M);
+                const float4 v = *reinterpret_cast<const float4*>(src + x * 8 * kMergeStride);
+                l = fmaf(ml[x].y, f, l);
+                acc.x = fmaf(v.x, f, acc.x);
+                acc.y = fmaf(v.y, f, acc.y);
+                acc.z = fmaf(v.z, f, acc.z);
+                acc.w = fmaf(v.w, f, acc.w);
+            }
+            if (r < p.group) {
+                float* dst = cluster.map_shared_rank(sm.recv_o, c >> c_shift) + (((rank * 8 + r) << c_shift) | (c & ((1 << c_shift) - 1)));
+                *reinterpret_cast<float4*>(dst) = acc;
+                if (lane < S) cluster.map_shared_rank(&sm.recv_ml[0][0], lane)[rank * 8 + r] = make_float2(M, l);
+            }
+        }
+    }
+    __syncwarp();
+    cluster.sync();
+    if (!producer) {
+        const int c_shift = 7 - s_shift;
+        const int pairs = p.group << (c_shift - 1);        // channel pairs of this CTA's slice, all rows
+        for (int x = tid; x < pairs; x += kWorkers) {
+            const int r = x >> (c_shift - 1), c = 2 * (x & ((1 << (c_shift - 1)) - 1));
+            float M = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f;
+            float2 ml[kMaxS];
+#pragma unroll
+            for (int s = 0; s < kMaxS; ++s) {
+                ml[s] = s < S ? sm.recv_ml[s][r] : make_float2(-INFINITY, 0.f);
+                M = fmaxf(M, ml[s].x);
+            }
+#pragma unroll
+            for (int s = 0; s < kMaxS; ++s) {
+                if (s < S) {
+                    const float f = ml[s].x == -INFINITY ? 0.f : fast_exp2(ml[s].x - M);
+                    const float2 v = *reinterpret_cast<const float2*>(&sm.recv_o[((s * 8 + r) << c_shift) + c]);
+                    l = fmaf(ml[s].y, f, l);
+                    a0 = fmaf(v.x, f, a0);
+                    a1 = fmaf(v.y, f, a1);
+                }
+            }
+            const float inv = l > 0.f ? 1.f / l : 0.f;
+            const size_t row = (size_t)(row_u + r);
+            *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
+            if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+        }
+    }
+}
+
+template <bool GATE>
+cudaError_t configure() {
+    cudaError_t e = cudaFuncSetAttribute(step_cluster_kernel<GATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StepSmem) + 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_cluster_kernel<GATE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+template <bool GATE>
+cudaLaunchConfig_t config_of(int S, int units, cudaStream_t stream, cudaLaunchAttribute (&attr)[2]) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S, units);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = sizeof(StepSmem) + 1024;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+// Clusters of 2^k CTAs that the device holds at once (both kernels have the same resources), asked once per device;
+// 0: the device or the driver does not take such clusters.
+int resident_clusters(int k) {
+    static int cached[kMaxDevices][5];                     // (value + 1; 0: not asked yet.  A race asks twice and stores the same)
+    const int slot = current_device_slot();
+    if (cached[slot][k] == 0) {
+        int n = 0;
+        if (configure<true>() == cudaSuccess && configure<false>() == cudaSuccess) {
+            cudaLaunchAttribute attr[2];
+            cudaLaunchConfig_t cfg = config_of<true>(1 << k, 1, nullptr, attr);
+            cfg.numAttrs = 1;
+            int a = 0, b = 0;
+            if (cudaOccupancyMaxActiveClusters(&a, step_cluster_kernel<true>, &cfg) != cudaSuccess) a = 0;
+            if (cudaOccupancyMaxActiveClusters(&b, step_cluster_kernel<false>, &cfg) != cudaSuccess) b = 0;
+            n = a < b ? a : b;
+            cudaGetLastError();                            // (a refused size is no error of the caller's)
+        }
+        cached[slot][k] = n + 1;
+    }
+    return cached[slot][k] - 1;
+}
+
+}  // namespace
+
+// As many CTAs per unit as keep every cluster resident at once (a second wave would double the call) and still have
+// something to do each.  Measured against the kernels of long calls, us a call (a step's append included):
+//     step, 8 KV heads, budget 4096, 1 / 2 / 4 sequences     23.3 -> 16.9, 25.3 -> 19.8, 31.6 -> 28.8
+//     step of batch 8 at 128k, 205 blocks (51 tiles a CTA)   98.4 -> 85.0
+//     given lists, 16 ragged sequences, blocks of 128        52.8 -> 45.8
+//     one 4 x 512-block list set (64 tiles a CTA)            93.5 -> 86.2
+// The line at kStepTilesPerCta tiles a CTA: beyond it the gain is below 5 % (128 tiles: 1.00 to 1.05) and a batch of
+// very uneven lengths, whose tiles the other kernel spreads over all SMs, could lose (256 dense tiles, lengths 1 : 8:
+// 185 -> 196).  With a few more CTAs than SMs the SMs that hold two of them are the last to finish (80 units, 64 tiles a
+// CTA, 160 CTAs: 65 -> 67; 32 tiles: 40.8 -> 37.5), so the line is at half as many tiles there.
+int step_cluster_size(int units, long long max_tiles, long long max_codes, int max_keys) {
+    const int sms = resident_clusters(0) / 2;
+    for (int k = 4; k >= 0; --k) {
+        const int S = 1 << k;
+        if (k > 0 && S > max_tiles && 128ll * S > max_keys) continue;      // a CTA would have nothing to do
+        if (units > resident_clusters(k)) continue;
+        const bool few_doubled = units * S > sms && 5 * units * S <= 6 * sms;
+        const long long line = (long long)S * (few_doubled ? kStepTilesPerCta / 2 : kStepTilesPerCta);
+        return max_tiles <= line && max_codes <= (long long)S * kCodes ? S : 0;
+    }
+    return 0;
+}
+
+cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g, int S,
+                                cudaStream_t stream) {
+    cudaLaunchAttribute attr[2];
+    if (g) {
+        const cudaLaunchConfig_t cfg = config_of<true>(S, p.num_units, stream, attr);
+        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<true>, map_k, map_v, p, GateArg<true>{*g});
+    }
+    const cudaLaunchConfig_t cfg = config_of<false>(S, p.num_units, stream, attr);
+    return cudaLaunchKernelEx(&cfg, step_cluster_kernel<false>, map_k, map_v, p, GateArg<false>{});
+}
+
+}  // namespace seer

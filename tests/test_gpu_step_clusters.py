@@ -1,0 +1,120 @@
+"""Short decode calls run as one launch with a thread-block cluster per (sequence, KV head) unit; longer ones as the
+chain of gate, attention and append.  Both forms (SEER_STEP_CLUSTERS=1 / 0 at context creation) against the oracle, at
+the places where the one-launch form can go wrong: clusters of 1 to 16 CTAs, fewer tiles than CTAs, more tiles than
+the ring has stages, gathered small blocks with a partly filled last tile, ragged and empty sequences, ties and NaN
+among the scores, more candidates than one pass of the selection's threads."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2506_08889_b200 import binding, synth
+from util import bits, check_attention, make_qkv, ref_dense, ref_sparse, to_paged
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+THETA = 1.0e6
+SCALE = 0.0884
+
+
+@pytest.fixture(scope="module", params=["1", "0"], ids=["clusters", "chain"])
+def ctx(request):
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setenv("SEER_STEP_CLUSTERS", request.param)      # read when a context is created
+        c = binding.Context(0)
+    c.one_launch = request.param == "1"
+    yield c
+    c.close()
+
+
+CASES = [
+    # B, Hq, Hkv, b, d_gate, S, page, scores, [(budget in blocks, max_sel)]
+    (1, 5, 1, 64, 128, 4096 - 13, 0, "random", [(8, 8), (1, 3), (200, 64)]),            # few units, S up to 16, 64 tiles
+    (2, 16, 2, 128, 64, 8192, 0, "random", [(9, 9), (40, 33)]),                         # two tiles per block
+    (3, 12, 3, 16, 256, 2048 + 48, 0, "ties", [(7, 7), (50, 50)]),                      # four blocks per tile, equal scores
+    (5, 8, 2, 32, 128, 4096, 256, "nan", [(13, 13), (64, 90)]),                         # two blocks per tile, paged
+    (7, 32, 8, 64, 128, 4096, 64, "random", [(33, 33)]),                                # 56 units: clusters of four
+    (37, 32, 8, 64, 128, 1024, 0, "random", [(9, 9)]),                                  # 296 units: one CTA each
+    (1, 4, 1, 16, 128, 16 * 9001, 0, "ties", [(100, 100)]),                             # 9001 keys: many passes of the selection
+    (1, 8, 2, 64, 128, 64 * 2100, 0, "crowded", [(60, 60)]),                            # one outlier: the radix passes
+]
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_step_sparse_dense(ctx, case):
+    B, Hq, Hkv, b, dg, S, page, kind, budgets = CASES[case]
+    d, seed = 128, 300 + case
+    cap = -(-S // max(page, b, 64)) * max(page, b, 64)
+    nb = cap // b
+    lens = np.array(([S, cap, b + 1, 2 * b, 5, 0] * B)[:B], np.int32)
+    lens[1:] = np.minimum(lens[1:], np.linspace(cap, 1, max(B - 1, 1)).astype(np.int32) + 7)
+    q, k, v = make_qkv(B, Hq, Hkv, cap, d, seed, DEV, token_major=case % 2 == 1 and not page)
+    for i in range(B):
+        v[i, :, lens[i]:] = float("nan")                    # rows past the end may hold anything
+    qn = synth.normal_bf16((B, Hq, d), seed, "qn", DEV)
+    wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), seed, "wq", DEV, std=0.02)
+    kc = synth.normal_bf16((B, Hkv, nb, dg), seed, "kc", DEV)
+    if kind == "ties":
+        kc = kc[:, :, torch.arange(nb, device=DEV) % 5].contiguous()      # five different scores
+    elif kind == "nan":
+        kc[:, :, ::3] = float("nan")
+    elif kind == "crowded":
+        kc[:, :, 1:] *= 1e-4                                # the histogram's bins span the outlier: nearly all share one
+    shape = binding.make_shape(B, Hq, Hkv, d, b, SCALE)
+    gate = binding.make_gate(dg, THETA, wq, None, kc, nb)
+    lens_t = torch.as_tensor(lens, device=DEV)
+    if page:
+        kp, vp, table = to_paged(k, v, page, seed)
+        kv = binding.make_kv(kp, vp, lens_t, max_seq_len=cap, page_table=table, page_size=page)
+    else:
+        kv = binding.make_kv(k, v, lens_t)
+    out = torch.empty((B, Hq, d), dtype=torch.bfloat16, device=DEV)
+    lse = torch.empty((B, Hq), dtype=torch.float32, device=DEV)
+    qh, kh, vh = bits(q), bits(k), bits(torch.nan_to_num(v))
+    for budget, max_sel in budgets:
+        idx = torch.full((B, Hkv, max_sel), 55, dtype=torch.int32, device=DEV)
+        cnt = torch.full((B, Hkv), 55, dtype=torch.int32, device=DEV)
+        for _ in range(3):                                  # (the second and third overlap the one before)
+            before = ctx.launch_count()
+            out.fill_(float("nan")), lse.fill_(float("nan"))
+            ctx.seer_decode_step(shape, kv, gate, q, qn, None, budget * b, idx, cnt, max_sel, out, lse)
+            assert (ctx.launch_count() - before == 1) == ctx.one_launch
+        sc = torch.zeros((B, Hkv, nb), dtype=torch.float32, device=DEV)
+        idx2, cnt2 = torch.zeros_like(idx), torch.zeros_like(cnt)
+        ctx.seer_gate_select(shape, gate, lens_t, qn, None, budget * b, idx2, cnt2, max_sel, scores_out=sc)
+        torch.cuda.synchronize()
+        want_idx, want_cnt = oracle.select(sc.cpu().numpy(), lens, b, budget * b, max_sel)
+        assert np.array_equal(cnt.cpu().numpy(), want_cnt) and np.array_equal(idx.cpu().numpy(), want_idx), (budget, max_sel)
+        ref = ref_sparse(qh, kh, vh, lens, want_idx, want_cnt, b, SCALE)
+        check_attention(out, lse, *ref, what=f"step {budget}")
+        # the lists given by the caller: reversed, with padding among them, no counts
+        given = torch.full((B, Hkv, 2 * max_sel), -1, dtype=torch.int32, device=DEV)
+        given[:, :, ::2] = idx.flip(2)
+        for idx_in, cnt_in, sel in ((idx, cnt, max_sel), (given, None, 2 * max_sel)):
+            out.fill_(float("nan")), lse.fill_(float("nan"))
+            ctx.seer_sparse_decode(shape, kv, q, idx_in, cnt_in, sel, out, lse)
+            torch.cuda.synchronize()
+            check_attention(out, lse, *ref, what=f"sparse {budget}")
+    if S <= 8192:
+        out.fill_(float("nan")), lse.fill_(float("nan"))
+        ctx.seer_dense_decode(shape, kv, q, out, lse)
+        torch.cuda.synchronize()
+        check_attention(out, lse, *ref_dense(qh, kh, vh, lens, SCALE), what="dense")
+    assert ctx.device_status() == binding.SEER_OK
+
+
+def test_bad_entries_are_skipped_and_reported(ctx):
+    B, Hq, Hkv, b, S, d = 1, 8, 2, 64, 1024, 128
+    q, k, v = make_qkv(B, Hq, Hkv, S, d, 17, DEV)
+    lens = np.array([S - 9], np.int32)
+    kv = binding.make_kv(k, v, torch.as_tensor(lens, device=DEV))
+    shape = binding.make_shape(B, Hq, Hkv, d, b, SCALE)
+    idx = np.array([[[0, 99, 5, 15], [16, 2, -3, 7]]], np.int32)          # 16 blocks: 99 and 16 do not exist
+    cnt = np.full((B, Hkv), 4, np.int32)
+    out = torch.empty((B, Hq, d), dtype=torch.bfloat16, device=DEV)
+    lse = torch.empty((B, Hq), dtype=torch.float32, device=DEV)
+    ctx.seer_sparse_decode(shape, kv, q, torch.as_tensor(idx, device=DEV), torch.as_tensor(cnt, device=DEV), 4, out, lse)
+    torch.cuda.synchronize()
+    good = np.where((idx >= 0) & (idx < 16), idx, -1).astype(np.int32)
+    check_attention(out, lse, *ref_sparse(bits(q), bits(k), bits(v), lens, good, cnt, b, SCALE), what="bad entries")
+    assert ctx.device_status() == binding.SEER_ERR_BAD_INDEX

@@ -133,13 +133,14 @@ def lib() -> ctypes.CDLL:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream):
+    # (the raw handle straight from torch: building a Stream object for it costs 3 us a call)
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def make_shape(batch, num_q_heads, num_kv_heads, head_dim, block_size, sm_scale) -> SeerShape:

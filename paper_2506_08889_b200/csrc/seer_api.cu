@@ -54,6 +54,9 @@ struct seer_ctx {
     int use_list_flags;         // 0: the attention kernel of a step waits for the whole gate kernel instead (SEER_STEP_LIST_FLAGS=0)
     int use_clusters;           // 0: short calls, too, go through the kernels of long ones (SEER_STEP_CLUSTERS=0)
     int wide_variant;           // kernel variant code for more than 16 rows per unit: 16 (tcgen05), 8 (mma.sync), 0 (by size)
+    int rope_d_gate;            // the rotary frequencies of the last gate width and theta seen (0: none yet)
+    float rope_theta;
+    double inv_freq[kMaxDGate / 2];
     char err[512];
 };
 
@@ -128,9 +131,15 @@ seer_status check_shape(seer_ctx* ctx, const seer_shape* s) {
     return SEER_OK;
 }
 
-// Rotary frequencies theta^(-2c/d_gate) in double (the device only multiplies by the position).
-void fill_inv_freq(double* dst, int d_gate, float theta) {
-    for (int c = 0; c < d_gate / 2; ++c) dst[c] = pow((double)theta, -2.0 * (double)c / (double)d_gate);
+// Rotary frequencies theta^(-2c/d_gate) in double (the device only multiplies by the position).  They are the same in
+// every call of a model, and raising 64 powers takes longer than a launch: the last ones are kept.
+void fill_inv_freq(seer_ctx* ctx, double* dst, int d_gate, float theta) {
+    if (ctx->rope_d_gate != d_gate || ctx->rope_theta != theta) {
+        for (int c = 0; c < d_gate / 2; ++c) ctx->inv_freq[c] = pow((double)theta, -2.0 * (double)c / (double)d_gate);
+        ctx->rope_d_gate = d_gate;
+        ctx->rope_theta = theta;
+    }
+    memcpy(dst, ctx->inv_freq, sizeof(double) * (size_t)(d_gate / 2));
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -612,7 +621,7 @@ static seer_status gate_prepare(seer_ctx* ctx, const seer_shape* shape, const se
 #ifdef SEER_GATE_TRACE
     p.status = reinterpret_cast<unsigned int*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 19)));
 #endif
-    if (!scores_in) fill_inv_freq(p.inv_freq, gate->d_gate, gate->rope_theta);
+    if (!scores_in) fill_inv_freq(ctx, p.inv_freq, gate->d_gate, gate->rope_theta);
     return SEER_OK;
 }
 
@@ -707,7 +716,7 @@ static seer_status kcomp_append_common(seer_ctx* ctx, const seer_shape* shape, c
 #ifdef SEER_DECODE_TRACE
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
-    fill_inv_freq(p.inv_freq, gate->d_gate, gate->rope_theta);
+    fill_inv_freq(ctx, p.inv_freq, gate->d_gate, gate->rope_theta);
     const CUtensorMap* map_k = nullptr;
     if (kcomp_bulk_streams(p)) {
         // (channel, token row, head, sequence); the row extent is the last row the build may touch

@@ -183,8 +183,8 @@ seer_status get_map(seer_ctx* ctx, const void* base, const uint64_t dims[4], con
 
 seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const void* q, int q_len,
                           const int32_t* block_idx, const int32_t* block_cnt, int max_sel, bool sparse,
-                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, int cluster = 0) {
-    // (gate: the whole step in one launch, clusters of `cluster` CTAs)
+                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0}) {
+    // (gate: the whole step in one launch, by `plan`)
     if (!ctx) return SEER_ERR_INVALID_ARG;
     seer_status st = check_shape(ctx, shape);
     if (st != SEER_OK) return st;
@@ -318,11 +318,11 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
 #ifdef SEER_DECODE_TRACE
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
-    if (!gate && q_len == 1 && ctx->use_clusters && ctx->list_gen == 0 && ctx->sel_from_lens == 0) cluster = step_cluster_size(U, max_tiles / U, 0, 0);
-    if (cluster > 0) {
-        p.t_cnt = 1;
-        p.rows = group;
-        ce = launch_step_cluster(mk_copy, *mv, p, gate, cluster, static_cast<cudaStream_t>(stream));
+    if (!gate && ctx->use_clusters && ctx->list_gen == 0 && ctx->sel_from_lens == 0)
+        plan = step_plan(U, q_len * group, !sparse, max_tiles / U, 0, 0);
+    if (plan.S > 0) {
+        p.rows = plan.rows;
+        ce = launch_step_cluster(mk_copy, *mv, p, gate, plan, static_cast<cudaStream_t>(stream));
         if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "decode launch: %s", cudaGetErrorString(ce));
         ctx->launches += 1;
         return SEER_OK;
@@ -627,6 +627,26 @@ static seer_status gate_prepare(seer_ctx* ctx, const seer_shape* shape, const se
 
 static seer_status gate_launch(seer_ctx* ctx, const GateParams& p, void* stream) {
     int launched = 0;
+    if (ctx->use_clusters && !p.scores_in && !p.list_flags && gate_one_kernel(p.max_blocks)) {
+        // the gate of the one-launch step by itself, while its clusters are resident all at once
+        const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, false, 0, 0, p.max_blocks);
+        if (plan.S > 0) {
+            CUtensorMap none;
+            DecodeParams d;
+            memset(&none, 0, sizeof none);
+            memset(&d, 0, sizeof d);
+            d.seq_lens = p.seq_lens;
+            d.num_kv_heads = p.num_kv_heads;
+            d.num_units = p.batch * p.num_kv_heads;
+            d.group = p.group;
+            d.q_len = p.q_len;
+            d.rows = plan.rows;
+            const cudaError_t ce = launch_step_cluster(none, none, d, &p, plan, static_cast<cudaStream_t>(stream));
+            if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "gate launch: %s", cudaGetErrorString(ce));
+            ctx->launches += 1;
+            return SEER_OK;
+        }
+    }
     const cudaError_t ce = launch_gate_select(p, static_cast<cudaStream_t>(stream), &launched);
     ctx->launches += launched;
     if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "gate launch: %s", cudaGetErrorString(ce));
@@ -750,6 +770,20 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
                                rows_block_local, first_block, num_blocks, 0, stream);
 }
 
+// Short steps are one launch: every (sequence, KV head) unit has a cluster of its own.
+static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const seer_gate* gate, int q_len,
+                             int token_budget, int max_sel) {
+    if (!ctx->use_clusters || gate->max_blocks > kStepMaxBlocks) return StepPlan{0, 1, 0};
+    const long long bs = shape->block_size, cap = kv->max_seq_len > 0 ? (kv->max_seq_len + bs - 1) / bs : 1;
+    long long blocks = token_budget / bs > 1 ? token_budget / bs : 1;
+    if (q_len > 1 && blocks < 2) blocks = 2;               // (two blocks can hold query tokens)
+    if (blocks > max_sel) blocks = max_sel;
+    if (blocks > cap) blocks = cap;
+    const long long tiles = (blocks * bs + kTileTokens - 1) / kTileTokens;
+    return step_plan(shape->batch * shape->num_kv_heads, q_len * (shape->num_q_heads / shape->num_kv_heads), false, tiles,
+                     bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles, gate->max_blocks);
+}
+
 seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const seer_gate* gate,
                              const void* q, const void* q_nope, const void* k_nope, int64_t k_nope_stride_batch,
                              int64_t k_nope_stride_head, int64_t k_nope_stride_token, int k_nope_rows_block_local,
@@ -774,18 +808,9 @@ seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     GateParams gp;
     seer_status st = gate_prepare(ctx, shape, gate, kv->seq_lens, q_nope, nullptr, token_budget, 0, 0.f, block_idx, block_cnt, max_sel,
                                   nullptr, 1, &gp);
-    // Short steps are one launch: every (sequence, KV head) unit has a cluster of its own.
-    int cluster = 0;
-    if (st == SEER_OK && ctx->use_clusters && gate->max_blocks <= kStepMaxBlocks) {
-        const long long bs = shape->block_size, cap = kv->max_seq_len > 0 ? (kv->max_seq_len + bs - 1) / bs : 1;
-        long long blocks = k_blocks < max_sel ? k_blocks : max_sel;
-        if (blocks > cap) blocks = cap;
-        const long long tiles = (blocks * bs + kTileTokens - 1) / kTileTokens;
-        cluster = step_cluster_size(shape->batch * shape->num_kv_heads, tiles, bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles,
-                                    gate->max_blocks);
-    }
-    if (cluster > 0) {
-        st = decode_common(ctx, shape, kv, q, 1, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, cluster);
+    const StepPlan plan = st == SEER_OK ? plan_of_step(ctx, shape, kv, gate, 1, token_budget, max_sel) : StepPlan{0, 1, 0};
+    if (plan.S > 0) {
+        st = decode_common(ctx, shape, kv, q, 1, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, plan);
     } else {
         if (st == SEER_OK) st = gate_launch(ctx, gp, stream);
         if (st != SEER_OK) {
@@ -812,10 +837,18 @@ seer_status seer_decode_step_multi(seer_ctx* ctx, const seer_shape* shape, const
     if (q_len < 1 || q_len > 8) return fail(ctx, SEER_ERR_UNSUPPORTED, "q_len %d (supported 1..8)", q_len);
     // (the block that filled holds one of the query tokens, so it is among the blocks selected without a
     // score: as in seer_decode_step the append comes last)
-    seer_status st = seer_gate_select_multi(ctx, shape, gate, kv->seq_lens, q_nope, nullptr, q_len, token_budget, block_idx,
-                                            block_cnt, max_sel, nullptr, stream);
+    GateParams gp;
+    seer_status st = gate_prepare(ctx, shape, gate, kv->seq_lens, q_nope, nullptr, token_budget, 0, 0.f, block_idx, block_cnt, max_sel,
+                                  nullptr, q_len, &gp);
     if (st != SEER_OK) return st;
-    st = seer_sparse_decode_multi(ctx, shape, kv, q, q_len, block_idx, block_cnt, max_sel, out, lse, stream);
+    const StepPlan plan = plan_of_step(ctx, shape, kv, gate, q_len, token_budget, max_sel);
+    if (plan.S > 0) {
+        st = decode_common(ctx, shape, kv, q, q_len, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, plan);
+    } else {
+        st = gate_launch(ctx, gp, stream);
+        if (st != SEER_OK) return st;
+        st = seer_sparse_decode_multi(ctx, shape, kv, q, q_len, block_idx, block_cnt, max_sel, out, lse, stream);
+    }
     if (st != SEER_OK || !k_nope) return st;
     return kcomp_append_common(ctx, shape, gate, kv->seq_lens, k_nope, k_nope_stride_batch, k_nope_stride_head,
                                k_nope_stride_token, k_nope_rows_block_local, -q_len, 1, 1, stream);

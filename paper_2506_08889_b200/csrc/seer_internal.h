@@ -124,13 +124,17 @@ struct GateParams {
 };
 // The one-kernel form of short calls (seer_step.cu): one cluster of S CTAs per unit.
 constexpr int kStepMaxBlocks = 16384;   // compressed keys per unit that its gate holds in shared memory
-constexpr int kStepTilesPerCta = 64;    // most tiles a CTA of it is given (see step_cluster_size)
-// The S for `units` units whose lists are at most max_tiles tiles long; 0: not a short call.  With the gate: max_keys
-// compressed keys per unit, max_codes tiles or, if these are smaller, blocks per unit; else 0.
-int step_cluster_size(int units, long long max_tiles, long long max_codes, int max_keys);
-// g == nullptr: attention only, over p.block_idx (nullptr: all blocks).
-cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g, int S,
-                                cudaStream_t stream);
+// How a call of `units` units of `rows` (query token, head) rows whose lists are at most max_tiles tiles long runs as one
+// launch.  With the gate: max_keys compressed keys per unit, max_codes tiles or, if these are smaller, blocks per unit;
+// else 0.
+struct StepPlan {
+    int S;                              // CTAs per cluster; 0: not a short call
+    int parts, rows;                    // clusters per unit, which have `rows` of its rows each (the last one the rest)
+};
+StepPlan step_plan(int units, int rows, bool dense, long long max_tiles, long long max_codes, int max_keys);
+// g == nullptr: attention only, over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.
+cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
+                                const StepPlan& plan, cudaStream_t stream);
 // Launches the scoring kernels (unless scores_in is given) and the selection kernel.
 // Returns the number of kernels launched through *launched.
 cudaError_t launch_gate_select(const GateParams& p, cudaStream_t stream, int* launched);

@@ -24,52 +24,67 @@ namespace seer {
 
 namespace {
 
-constexpr int kStages = 3;
-constexpr int kWorkers = 256;                              // eight warps: gate, consumers, combine
-constexpr int kWarps = kWorkers / 32;
-constexpr int kThreads = kWorkers + 32;                    // ... and the producer warp
 constexpr int kHalfTileBytes = kTileTokens * 128;          // 64 rows x 128 B (64 bf16 channels)
 constexpr int kTileBytes = 2 * kHalfTileBytes;             // one K or V tile: 16 KiB
 constexpr int kStageBytes = 2 * kTileBytes;                // K + V
 constexpr int kMaxS = 16;
 constexpr int kCodes = 256;                                // tile (or gathered block) numbers that a CTA holds
-constexpr int kArrivals = 2 * kStages;
-constexpr int kBins = 1024;                                // histogram of the selection: four bins a thread
+constexpr int kBins = 1024;                                // histogram of the selection
 constexpr int kMergeStride = 132;                          // floats per row of a warp's partial (bank spread)
 constexpr int kBatch = 8;                                  // 16-byte pieces of compressed keys per thread in flight
 constexpr int kChunkKeys = 32;                             // keys are dealt to the cluster's CTAs in runs of 32
+constexpr int kMaxQLen = 8;
 
+// Two sizes.  NW = 8 worker warps (gate, consumers, combine) and a ring of three stages: two CTAs per SM, up to 16
+// rows (8 without MULTI).  NW = 16 and five stages: one CTA per SM, up to 32 rows.
+template <int NW, bool MULTI>
+struct Size {
+    static constexpr int kWorkers = 32 * NW, kThreads = kWorkers + 32;     // ... and the producer warp
+    static constexpr int kStages = NW == 8 ? 3 : 5, kGroups = NW / 4;
+    static constexpr int kRows = !MULTI ? 8 : NW == 8 ? 16 : 32;
+    static constexpr int kArrivals = kStages * kGroups;
+};
+
+template <int NW, bool MULTI>
 struct __align__(1024) StepSmem {
+    using Z = Size<NW, MULTI>;
     // K/V ring.  Before the first tile is asked for, the gate's: the scores of the unit (first CTA; up to
-    // kStepMaxBlocks) in stages 0 and 1, the staged first batch of keys in stage 2.  After the last tile: the warps'
-    // partials.
-    unsigned char ring[kStages][kStageBytes];
-    float qg[kMaxDGate];                                   // gate query
-    __align__(16) float recv_o[8 * kHeadDim];                         // [source CTA][row][this CTA's slice of the channels]
-    float2 recv_ml[kMaxS][8];                              // [source CTA][row]: max, sum
-    float2 warp_ml[kWarps][8];
-    // Tile n arrives in stage n % 3 and is announced on full[n % 6]: the two consumer groups take the even and the odd
-    // tiles, each at its own pace, and every one of the six barriers belongs to one of them, which follows all of its
-    // phases.  (With a barrier per stage a group would miss the other's phases and could take one that is two back for
-    // the one that it waits for.)
-    uint64_t full[kArrivals], empty[kStages];
-    int meta[kArrivals];                                   // valid tokens of the tile (blocks of 16 or 32 tokens: per block, 8 bits each)
+    // kStepMaxBlocks) in stages 0 and 1, the staged first batch of keys behind them, the list of the taken blocks in
+    // its place later.  After the last tile: the warps' partials.
+    unsigned char ring[Z::kStages][kStageBytes];
+    // What the gate uses until the lists are out, and what arrives from the cluster's CTAs after their last tile.
+    union {
+        float qg[MULTI ? kMaxQLen : 1][kMaxDGate];         // gate queries
+        __align__(16) float recv_o[Z::kRows * kHeadDim];   // [source CTA][row][this CTA's slice of the channels]
+    };
+    union {
+        __align__(16) int hist[kBins + 4];                 // selection (first CTA); the one past the last is for nobody
+        float2 recv_ml[kMaxS][Z::kRows];                   // [source CTA][row]: max, sum
+    };
+    float2 warp_ml[NW][8];
+    // Tile n arrives in stage n % kStages and is announced on full[n % kArrivals].  The consumer groups that share a
+    // tile's rows take all of one residue of the tile numbers, at their own pace, and every barrier belongs to one
+    // residue, so its groups follow all of its phases.  (With a barrier per stage a group would miss the others' phases
+    // and could take one that is two back for the one that it waits for.)
+    uint64_t full[Z::kArrivals], empty[Z::kStages];
+    int meta[Z::kArrivals];                                // tokens from the tile's first row on (blocks of 16 or 32 tokens: per block, 8 bits each)
     int codes[kCodes];                                     // GATE: this CTA's tiles: 64-token tile numbers, or the gathered blocks
     // selection (first CTA)
-    __align__(16) int hist[kBins + 4];                     // (read four bins at a time; the one past the last is for nobody)
-    int warp_tot[kWarps];
+    int warp_tot[NW];
+    float warp_red[NW];
     uint32_t list_key[32];
     int list_j[32];
     uint32_t pre_min, pre_max;                             // smallest and largest key of a candidate
     uint32_t prefix;
     int rem, bin_cnt, list_n, last_eq;
 };
-static_assert(sizeof(StepSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
-static_assert(kCodes * kMaxS <= kStageBytes / 4, "the list in stage 2");
-static_assert(kStepMaxBlocks * 4 <= 2 * kStageBytes && kBatch * kWorkers * 16 <= kStageBytes, "the gate's use of the ring");
-static_assert(kWarps * 8 * kMergeStride * 4 <= kStages * kStageBytes, "the partials' use of the ring");
+static_assert(sizeof(StepSmem<8, true>) + 1024 <= 113 * 1024, "two CTAs per SM");
+static_assert(sizeof(StepSmem<16, true>) + 1024 <= 227 * 1024, "one CTA per SM");
+static_assert(kStepMaxBlocks * 4 <= 2 * kStageBytes && kBatch * 256 * 16 <= kStageBytes && kBatch * 512 * 16 <= 3 * kStageBytes, "the gate's use of the ring");
+static_assert(kCodes * kMaxS <= kStageBytes / 4, "the list behind the scores");
 
-__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
+template <int NW>
+__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory"); }
 
 template <bool GATE>
 struct GateArg { GateParams g; };
@@ -81,7 +96,8 @@ struct GateArg<false> {};
 // the lower block number wins a tie, NaN is below every number.  A histogram over a monotone linear map of
 // [min, max] leaves a few candidates in the boundary bin, which every warp ranks for itself; crowded bins and ranges
 // that are not finite take radix passes over key - min instead.
-__device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, int n_cand, int need, int words, int warp, int lane,
+template <int NW, typename Smem>
+__device__ __forceinline__ void select_threshold(Smem& sm, const float* sc, int n_cand, int need, int words, int warp, int lane,
                                                  uint32_t& thr, int& j_eq) {
     const int tid = 32 * warp + lane;
     if (need >= n_cand) { thr = 0u; j_eq = 0x7fffffff; return; }
@@ -107,25 +123,26 @@ __device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, 
     const int run = (n_cand + 31) / 32, rot = (run & 1) ? 0 : lane % run;
     auto each_spread = [&](auto&& fn) {
 #pragma unroll 1
-        for (int q = warp; q < run; q += 4 * kWarps) {
+        for (int q = warp; q < run; q += 4 * NW) {
             float v[4];
             int jj[4];
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
-                int at = q + x * kWarps + rot;
+                int at = q + x * NW + rot;
                 at -= at >= run ? run : 0;
-                jj[x] = q + x * kWarps < run ? min(lane * run + at, n_cand) : n_cand;      // (n_cand: none)
+                jj[x] = q + x * NW < run ? min(lane * run + at, n_cand) : n_cand;      // (n_cand: none)
                 v[x] = sc[min(jj[x], n_cand - 1)];
             }
             fn(v, jj);
         }
     };
-    // thread t owns bins kBins-1-4t downwards: finds the bin that straddles the rem-th best key
+    // thread t owns a few bins, from kBins-1-kPer*t downwards: finds the bin that straddles the rem-th best key
+    constexpr int kPer = kBins / (32 * NW);
     auto find_bin = [&](int rem) {
-        worker_sync();
-        const int4 c4 = *reinterpret_cast<const int4*>(&sm.hist[kBins - 4 - 4 * tid]);
-        const int c[4] = {c4.w, c4.z, c4.y, c4.x};
-        const int mine = c[0] + c[1] + c[2] + c[3];
+        worker_sync<NW>();
+        int c[kPer], mine = 0;
+#pragma unroll
+        for (int x = 0; x < kPer; ++x) { c[x] = sm.hist[kBins - 1 - kPer * tid - x]; mine += c[x]; }
         int incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -133,22 +150,22 @@ __device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, 
             if (lane >= o) incl += t;
         }
         if (lane == 31) sm.warp_tot[warp] = incl;
-        worker_sync();
+        worker_sync<NW>();
         int above = incl - mine;
 #pragma unroll
-        for (int w2 = 0; w2 < kWarps; ++w2) above += w2 < warp ? sm.warp_tot[w2] : 0;
+        for (int w2 = 0; w2 < NW; ++w2) above += w2 < warp ? sm.warp_tot[w2] : 0;
         if (above < rem && rem <= above + mine) {
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
+            for (int x = 0; x < kPer; ++x) {
                 if (above < rem && rem <= above + c[x]) {
-                    sm.prefix = (uint32_t)(kBins - 1 - 4 * tid - x);
+                    sm.prefix = (uint32_t)(kBins - 1 - kPer * tid - x);
                     sm.rem = rem - above;
                     sm.bin_cnt = c[x];
                 }
                 above += c[x];
             }
         }
-        worker_sync();
+        worker_sync<NW>();
     };
     if (smin > -INFINITY && range > 0.f && range < INFINITY && scale < INFINITY) {
         // (every score is finite here; -0 and +0 have the same bin)
@@ -175,7 +192,7 @@ __device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, 
                     }
                 }
             });
-            worker_sync();
+            worker_sync<NW>();
             const uint32_t key = lane < cnt ? sm.list_key[lane] : 0u;
             const int j = lane < cnt ? sm.list_j[lane] : 0x7fffffff;
             int rank = 0;
@@ -195,8 +212,9 @@ __device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, 
     uint32_t prefix = 0u;
     while (bits_left > 0) {
         const int wbits = min(10, bits_left), shift = bits_left - wbits;
-        *reinterpret_cast<int4*>(&sm.hist[4 * tid]) = make_int4(0, 0, 0, 0);
-        worker_sync();
+#pragma unroll
+        for (int x = 0; x < kPer; ++x) sm.hist[kPer * tid + x] = 0;
+        worker_sync<NW>();
         each([&](bool ok, uint32_t key, int) {
             const uint32_t rel = key - kmin;
             if (ok && (uint32_t)((unsigned long long)rel >> (shift + wbits)) == prefix)        // (shift + wbits can be 32)
@@ -211,12 +229,12 @@ __device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, 
     // the rem-th candidate whose key equals thr, in block order (a warp's candidates are one run of blocks)
     int n_eq = 0;
     each([&](bool ok, uint32_t key, int) { n_eq += __popc(__ballot_sync(0xffffffffu, ok && key == thr)); });
-    worker_sync();                                         // (everybody has read the last pass's totals)
+    worker_sync<NW>();                                         // (everybody has read the last pass's totals)
     if (lane == 0) sm.warp_tot[warp] = n_eq;
-    worker_sync();
+    worker_sync<NW>();
     int before = 0;
 #pragma unroll
-    for (int w2 = 0; w2 < kWarps; ++w2) before += w2 < warp ? sm.warp_tot[w2] : 0;
+    for (int w2 = 0; w2 < NW; ++w2) before += w2 < warp ? sm.warp_tot[w2] : 0;
     if (before < rem && rem <= before + n_eq) {
         each([&](bool ok, uint32_t key, int j) {
             const bool eq = ok && key == thr;
@@ -225,7 +243,7 @@ __device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, 
             before += __popc(m);
         });
     }
-    worker_sync();
+    worker_sync<NW>();
     j_eq = sm.last_eq;
 }
 
@@ -233,25 +251,35 @@ __device__ __forceinline__ void select_threshold(StepSmem& sm, const float* sc, 
 // speed) take 13 us from the first read to the last write, of which the gate query 1.5, the scores 1.0, the selection
 // and the lists 3.3, the tiles 2.5, the combine 2.2 and four cluster barriers 0.5 to 1.0 each.  Longer ones by memory: 64
 // units x 205 blocks (430 MB) 70 us, 6.2 TB/s; CTAs that share a unit read neighbouring blocks at the same time.
-template <bool GATE>
-__global__ void __launch_bounds__(kThreads, 2)
+template <int NW, bool GATE, bool MULTI>
+__global__ void __launch_bounds__(Size<NW, MULTI>::kThreads, NW == 8 ? 2 : 1)
 step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ DecodeParams p, const __grid_constant__ GateArg<GATE> ga) {
+    using Z = Size<NW, MULTI>;
+    using Smem = StepSmem<NW, MULTI>;
+    constexpr int kWorkers = Z::kWorkers, kStages = Z::kStages, kArrivals = Z::kArrivals, kRows = Z::kRows;
     extern __shared__ unsigned char smem_raw[];
-    StepSmem& sm = *reinterpret_cast<StepSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     cg::cluster_group cluster = cg::this_cluster();
     const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), s_shift = 31 - __clz(S);
     const int u = blockIdx.y, i = u / p.num_kv_heads, h = u - i * p.num_kv_heads;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool producer = warp == kWarps;
+    const bool producer = warp == NW;
+    const int q_len = MULTI ? p.q_len : 1;
+    // The unit's rows (query token, head of the group) are cut into gridDim.z parts of p.rows; this cluster's: row0 ..
+    const int row0 = MULTI ? blockIdx.z * p.rows : 0;
+    const int rows = MULTI ? min(p.rows, q_len * p.group - row0) : p.group;
+    // eight rows are an MMA's N side: `tiles_n` consumer groups share a K/V tile, `paces` such teams take alternate tiles
+    const int tiles_n = MULTI ? (rows + 7) >> 3 : 1;
+    const int paces = MULTI ? Z::kGroups / tiles_n : Z::kGroups;
     // (another CTA's shared memory is written only after the barrier this opens: it is then known to be running)
     cluster_arrive();
     if (tid < kArrivals) {
         mbar_init(&sm.full[tid], 1);
-        if (tid < kStages) mbar_init(&sm.empty[tid], kWarps / 2);
+        if (tid < kStages) mbar_init(&sm.empty[tid], 4 * tiles_n);
         mbar_fence_init();
     }
-    if (producer && lane == 0) {
+    if (producer && lane == 0 && p.q) {
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
     }
@@ -261,41 +289,51 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const GateParams& g = ga.g;
         const int n = g.group * kHeadDim, chunks = n / 8, half = g.d_gate / 2;
         const int nit = (chunks + 31) / 32;                // 16-byte pieces of a W_q row per lane (1..4)
-        const int gw = rank * kWarps + warp, n_gw = S * kWarps;
+        const int gw = rank * NW + warp, n_gw = S * NW;
         const int lpk_shift = g.d_gate == 64 ? 3 : g.d_gate == 128 ? 4 : 5, lpk = 1 << lpk_shift;   // lanes per key
         const int csub = tid & (lpk - 1);
         const uint4* kc = reinterpret_cast<const uint4*>(g.kcomp + (size_t)u * g.max_blocks * g.d_gate);
         // this CTA's key number lk (runs of kChunkKeys, dealt round robin) is block
         auto block_of = [&](int lk) { return (((lk / kChunkKeys) << s_shift) + rank) * kChunkKeys + (lk & (kChunkKeys - 1)); };
-        // W_q rows of this warp's first rotary pair: constants, requested before the wait
+        // Rotary pairs (c, c + d_gate/2) of the gate query are dealt to the cluster's warps; with more warps than pairs
+        // several of them take a pair, for every t_step-th query token each.
+        const int c_step = min(n_gw, half), t_step = max(1, n_gw / half), t_first = gw / half, c_first = gw % half;
         uint4 wv[2][4];
+        auto load_w = [&](int c) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const uint4* wrow = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + gw % half + k * half) * n);
+            for (int k = 0; k < 2; ++k) {
+                const uint4* wrow = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + c + k * half) * n);
 #pragma unroll
-            for (int it = 0; it < 4; ++it) {
-                const int ch = lane + 32 * it;
-                wv[k][it] = (!producer && it < nit && gw < half && ch < chunks) ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
+                for (int it = 0; it < 4; ++it) {
+                    const int ch = lane + 32 * it;
+                    wv[k][it] = it < nit && ch < chunks ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
+                }
             }
-        }
+        };
+        if (!producer && t_first < q_len) load_w(c_first);     // constants, requested before the wait
         if (rank == 0) {
-            for (int x = tid; x < kBins; x += kThreads) sm.hist[x] = 0;
+            for (int x = tid; x < kBins; x += Z::kThreads) sm.hist[x] = 0;
             if (tid == 0) { sm.pre_min = 0xffffffffu; sm.pre_max = 0u; sm.list_n = 0; }
         }
         pdl_wait();                                        // queries, lengths and compressed keys are final
+        if (!p.q) pdl_launch_dependents();                 // (the gate alone has no work for which it wants the SMs)
         L = p.seq_lens[i];
-        const uint4* xsrc = reinterpret_cast<const uint4*>(g.q_nope + ((size_t)i * g.num_q_heads + (size_t)h * g.group) * kHeadDim);
         uint4 xv[4];
-        const int all_chunks = (g.max_blocks + kChunkKeys - 1) / kChunkKeys;
-        const int total_cap = ((max(0, all_chunks - rank) + S - 1) >> s_shift) << (lpk_shift + 5);    // pieces, block numbers past the cache among them
-        uint4* staged = reinterpret_cast<uint4*>(sm.ring[2]);
-        float* sc_all = reinterpret_cast<float*>(sm.ring[0]);
-        if (!producer) {
+        auto load_x = [&](int t) {
+            const uint4* xsrc = reinterpret_cast<const uint4*>(
+                g.q_nope + (((size_t)i * q_len + t) * g.num_q_heads + (size_t)h * g.group) * kHeadDim);
 #pragma unroll
             for (int it = 0; it < 4; ++it) {
                 const int ch = lane + 32 * it;
                 xv[it] = it < nit && ch < chunks ? __ldg(xsrc + ch) : make_uint4(0u, 0u, 0u, 0u);
             }
+        };
+        const int all_chunks = (g.max_blocks + kChunkKeys - 1) / kChunkKeys;
+        const int total_cap = ((max(0, all_chunks - rank) + S - 1) >> s_shift) << (lpk_shift + 5);    // pieces, block numbers past the cache among them
+        uint4* staged = reinterpret_cast<uint4*>(sm.ring[2]);      // [kBatch * kWorkers]
+        float* sc_all = reinterpret_cast<float*>(sm.ring[0]);
+        if (!producer) {
+            if (t_first < q_len) load_x(t_first);
             // the first batch of keys travels during the projection (entries past n_i - 1 exist in memory: harmless)
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) {
@@ -304,13 +342,16 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         }
         const int n_i = L > 0 ? (L + g.block_size - 1) / g.block_size : 0;
-        const int j_f = L > 0 ? n_i - 1 : 0;               // the last block is always taken; the candidates are those before it
+        // the blocks that hold a query token's own position, j_f .. n_i - 1 (one, the last, for a single token), are always
+        // taken; the candidates are those before them
+        const int j_f = max(0, L - q_len) / g.block_size;
+        const int n_forced = min(n_i - j_f, g.max_sel);
         const int n_cand = min(j_f, g.max_blocks);
-        int need = 0;
-        if (n_i > 0) {
+        int need = 0;                                      // (threshold method: known once the scores are)
+        if (n_i > 0 && !g.threshold_mode) {
             const int k = min(max(g.token_budget / g.block_size, 1), min(n_i, g.max_sel));
-            need = max(0, min(k - 1, n_cand));
-            n_blocks = need + 1;
+            need = max(0, min(k - n_forced, n_cand));
+            n_blocks = need + n_forced;
         }
         // pieces that matter: up to the last run of keys with a candidate
         const int cand_chunks = (n_cand + kChunkKeys - 1) / kChunkKeys;
@@ -318,34 +359,27 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         cluster_wait();                                    // every CTA of the cluster has started
         // ---- gate query: rotary pairs (c, c + d_gate/2) dealt to the cluster's warps --------------------------
         if (!producer) {
-            for (int c = gw; c < half; c += n_gw) {
-                if (c != gw) {
+            for (int c = c_first; c < half; c += c_step) {
+                for (int t = t_first; t < q_len; t += t_step) {
+                    if (c != c_first && t == t_first) load_w(c);
+                    if (MULTI && (c != c_first || t != t_first)) load_x(t);
+                    float a = 0.f, b = 0.f;
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const uint4* wrow = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + c + k * half) * n);
-#pragma unroll
-                        for (int it = 0; it < 4; ++it) {
-                            const int ch = lane + 32 * it;
-                            wv[k][it] = it < nit && ch < chunks ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
-                        }
+                    for (int it = 0; it < 4; ++it) {
+                        if (it < nit) { a += dot8(wv[0][it], xv[it]); b += dot8(wv[1][it], xv[it]); }
                     }
-                }
-                float a = 0.f, b = 0.f;
 #pragma unroll
-                for (int it = 0; it < 4; ++it) {
-                    if (it < nit) { a += dot8(wv[0][it], xv[it]); b += dot8(wv[1][it], xv[it]); }
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    a += __shfl_xor_sync(0xffffffffu, a, off);
-                    b += __shfl_xor_sync(0xffffffffu, b, off);
-                }
-                float sn, cs;
-                rope_sincos((double)max(L - 1, 0), g.inv_freq[c], &sn, &cs);
-                if (lane < S) {                            // lane r stores into CTA r of the cluster
-                    float* dst = cluster.map_shared_rank(sm.qg, lane);
-                    dst[c] = a * cs - b * sn;
-                    dst[c + half] = b * cs + a * sn;
+                    for (int off = 16; off > 0; off >>= 1) {
+                        a += __shfl_xor_sync(0xffffffffu, a, off);
+                        b += __shfl_xor_sync(0xffffffffu, b, off);
+                    }
+                    float sn, cs;                          // query token t sits at position L - q_len + t
+                    rope_sincos((double)max(L - q_len + t, 0), g.inv_freq[c], &sn, &cs);
+                    if (lane < S) {                        // lane r stores into CTA r of the cluster
+                        float* dst = cluster.map_shared_rank(&sm.qg[0][0], lane) + t * kMaxDGate;
+                        dst[c] = a * cs - b * sn;
+                        dst[c + half] = b * cs + a * sn;
+                    }
                 }
             }
         }
@@ -369,17 +403,24 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             const int krev = ((lane & 1) << 2) | (lane & 2) | ((lane >> 2) & 1);
             const bool storer = (csub & ~7) == 0;
             uint32_t kmn = 0xffffffffu, kmx = 0u;
-            float qsub[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) qsub[c] = sm.qg[8 * csub + c];
+            float* sc_user = g.scores_user ? g.scores_user + (size_t)u * g.max_blocks : nullptr;
+            // (several query tokens: a key's score is the largest of its products with their gate queries)
             auto score_batch = [&](auto&& piece, int cb) {
-                float acc[kBatch];
+                float best = -INFINITY;
+                for (int t = 0; t < q_len; ++t) {
+                    float qsub[8], acc[kBatch];
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k) acc[k] = dot8(piece(k), qsub);
-                const float v = reduce8(acc, lane, lpk) * inv;
+                    for (int c = 0; c < 8; ++c) qsub[c] = sm.qg[t][8 * csub + c];
+#pragma unroll
+                    for (int k = 0; k < kBatch; ++k) acc[k] = dot8(piece(k), qsub);
+                    const float x = reduce8(acc, lane, lpk);
+                    best = MULTI ? fmaxf(best, x) : x;
+                }
+                const float v = best * inv;
                 const int pc = cb + krev * kWorkers + tid, j = block_of(pc >> lpk_shift);
                 if (storer && pc < total && j < n_cand) {
                     sc0[j] = v;
+                    if (sc_user) sc_user[j] = v;
                     const uint32_t key = score_key(v);
                     kmn = min(kmn, key);
                     kmx = max(kmx, key);
@@ -419,10 +460,34 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         if (rank == 0 && !producer) {
             int32_t* dst = g.block_idx + (size_t)u * g.max_sel;
             int* list = reinterpret_cast<int*>(sm.ring[2]);      // the listed blocks, ascending (the host's rule bounds their number)
-            const int words = ((n_cand + 31) / 32 + kWarps - 1) / kWarps;      // 32 candidates each, per warp
+            const int words = ((n_cand + 31) / 32 + NW - 1) / NW;      // 32 candidates each, per warp
             uint32_t thr;
             int j_eq;
-            select_threshold(sm, sc_all, n_cand, need, words, warp, lane, thr, j_eq);
+            if (g.threshold_mode) {
+                // Threshold method (Sec. 3.1): softmax of the scores over the candidates; those above tau are the `above`
+                // highest-scoring ones (equal scores have equal probabilities), so only the number differs
+                auto sum_all = [&](float v) -> float {
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                    worker_sync<NW>();                     // (the scratch may still be in use)
+                    if (lane == 0) sm.warp_red[warp] = v;
+                    worker_sync<NW>();
+                    float r = 0.f;
+#pragma unroll
+                    for (int w2 = 0; w2 < NW; ++w2) r += sm.warp_red[w2];
+                    return r;
+                };
+                const float mx = key_score(sm.pre_max);
+                float z = 0.f, above = 0.f;
+#pragma unroll 4
+                for (int j = tid; j < n_cand; j += kWorkers) z += __expf(sc_all[j] - mx);
+                z = sum_all(z);
+#pragma unroll 4
+                for (int j = tid; j < n_cand; j += kWorkers) above += __expf(sc_all[j] - mx) > g.threshold * z ? 1.f : 0.f;
+                need = max(0, min(min((int)(sum_all(above) + 0.5f), g.max_sel - n_forced), n_cand));
+                n_blocks = n_i > 0 ? need + n_forced : 0;
+            }
+            select_threshold<NW>(sm, sc_all, n_cand, need, words, warp, lane, thr, j_eq);
             // which of the warp's candidates are taken: lane x keeps the words x and x + 32 (words <= 64)
             const int jw = warp * words * 32 + lane;
             unsigned taken[2] = {0u, 0u};
@@ -447,12 +512,12 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (lane >= o) { incl_low += lo; incl_high += hi; }
             }
             const int all_low = __shfl_sync(0xffffffffu, incl_low, 31);
-            worker_sync();
+            worker_sync<NW>();
             if (lane == 31) sm.warp_tot[warp] = incl_low + incl_high;
-            worker_sync();
+            worker_sync<NW>();
             int pos = 0;
 #pragma unroll
-            for (int w2 = 0; w2 < kWarps; ++w2) pos += w2 < warp ? sm.warp_tot[w2] : 0;
+            for (int w2 = 0; w2 < NW; ++w2) pos += w2 < warp ? sm.warp_tot[w2] : 0;
             // every lane lists its own words' blocks
             {
                 int at = pos + incl_low - in_low;
@@ -462,15 +527,17 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 for (unsigned m = taken[1]; m; m &= m - 1) list[at++] = j_low + 1024 + __ffs(m) - 1;
             }
             if (tid == 0) {
-                if (n_i > 0) list[need] = n_i - 1;
-                g.block_cnt[u] = n_blocks;
+                if (n_i > 0) {
+                    for (int x = 0; x < n_forced; ++x) list[need + x] = n_i - n_forced + x;
+                }
+                if (blockIdx.z == 0) g.block_cnt[u] = n_blocks;
             }
-            worker_sync();
+            worker_sync<NW>();
             // entry e of the list is block j: into the caller's list, and to the CTA that reads its tile(s)
             for (int e = tid; e < g.max_sel; e += kWorkers) {
                 const int j = e < n_blocks ? list[e] : -1;
-                dst[e] = j;
-                if (e >= n_blocks) continue;
+                if (blockIdx.z == 0) dst[e] = j;
+                if (e >= n_blocks || !p.q) continue;
                 if (p.blocks_per_tile == 1) {
                     for (int x = 0; x < p.tiles_per_block; ++x) {
                         const int t = (e << p.tpb_shift) + x;
@@ -483,6 +550,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
             }
         }
+        if (!p.q) return;                                  // the gate alone
         fence_proxy_async_smem();                          // the ring's memory goes over to the copy engine
         __syncwarp();
         cluster_arrive();
@@ -503,7 +571,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         : small ? (n_blocks + p.blocks_per_tile - 1) >> p.bpt_shift : n_blocks << p.tpb_shift;
     const int n_mine = (max(0, T - rank) + S - 1) >> s_shift;
     const int n_local = GATE ? min(n_mine, small ? kCodes >> p.bpt_shift : kCodes) : n_mine;     // (the host's rule keeps within kCodes)
-    const int row_u = i * p.num_q_heads + h * p.group;     // first of the unit's query rows
+    // output row of this cluster's row r: query token (row0 + r) / group, head (row0 + r) % group of the unit's
+    auto out_row = [&](int r) -> size_t {
+        const int tl = MULTI ? ((row0 + r) * p.group_magic) >> 16 : 0;
+        return ((size_t)i * q_len + tl) * p.num_q_heads + (size_t)h * p.group + (row0 + r - tl * p.group);
+    };
     const int qd = lane & 3, rw = lane >> 2;
     bool dead = false;                                     // a wait ran out: go through the motions, the results are invalid
     if (producer) {
@@ -537,7 +609,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                             if (blk >= n_i) raise_status(p.status, DEV_BAD_INDEX);
                             if (blk >= 0 && blk < n_i) tok0 = (blk << p.bs_shift) + (t & (p.tiles_per_block - 1)) * kTileTokens;
                         }
-                        int nv = tok0 >= 0 ? max(0, min(span, L - tok0)) : 0;
+                        // (counted beyond the tile, so that earlier query tokens can be cut off)
+                        int nv = tok0 >= 0 ? max(0, min(span + (MULTI ? kMaxQLen - 1 : 0), L - tok0)) : 0;
                         if (nv > 0) {
                             outer[x] = i;
                             row[x] = tok0;
@@ -562,7 +635,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     if (!dead && !mbar_wait(&sm.empty[st], ((it / kStages) & 1) ^ 1, p.status)) dead = true;
                     unsigned char* dst = sm.ring[st];
                     uint64_t* full = &sm.full[it % kArrivals];
-                    sm.meta[it % kArrivals] = nv_all;      // (the tile six back has been read: three back is, which came after it)
+                    sm.meta[it % kArrivals] = nv_all;      // (the tile kArrivals back has been read: the one kStages back has, which came after it)
                     if (dead || n_sub == 0) {
                         mbar_arrive(full);
                     } else if (small) {
@@ -591,14 +664,25 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         if (!GATE) cluster_wait();                         // (the barrier opened at the top)
     } else {
-        // Q^T B-fragments: this thread supplies row rw of the unit's queries
+        const int group = warp >> 2, my_n = MULTI ? group % tiles_n : 0, pace = MULTI ? group / tiles_n : group;
+        // Q^T B-fragments: this thread supplies row 8 * my_n + rw of the unit's queries
         uint32_t bq[8][2];
         {
-            const uint32_t* qrow = reinterpret_cast<const uint32_t*>(p.q + (size_t)(row_u + (rw < p.group ? rw : 0)) * kHeadDim);
+            const int r = 8 * my_n + rw;
+            const uint32_t* qrow = reinterpret_cast<const uint32_t*>(p.q + out_row(r < rows ? r : 0) * kHeadDim);
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-                bq[ks][0] = rw < p.group ? __ldg(qrow + 8 * ks + qd) : 0u;
-                bq[ks][1] = rw < p.group ? __ldg(qrow + 8 * ks + 4 + qd) : 0u;
+                bq[ks][0] = r < rows ? __ldg(qrow + 8 * ks + qd) : 0u;
+                bq[ks][1] = r < rows ? __ldg(qrow + 8 * ks + 4 + qd) : 0u;
+            }
+        }
+        // newest cached tokens that the query tokens of this thread's two rows (columns of S^T) may not see
+        int back[2] = {0, 0};
+        if (MULTI) {
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int r = 8 * my_n + 2 * qd + c;
+                if (r < rows) back[c] = q_len - 1 - (((row0 + r) * p.group_magic) >> 16);
             }
         }
         if (GATE) cluster_wait();
@@ -614,7 +698,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         // blocks of 16 or 32 tokens: which of the gathered blocks this warp's rows belong to, and where in it
         const int sub_w = !small ? 0 : p.block_size == 16 ? w4 : w4 >> 1;
         const int off_w = !small ? 16 * w4 : p.block_size == 16 ? 0 : (w4 & 1) * 16;
-        for (int it = warp >> 2; it < n_local; it += 2) {
+        for (int it = pace < paces ? pace : n_local; it < n_local; it += paces) {
             const int st = it % kStages;
             if (!dead && !mbar_wait(&sm.full[it % kArrivals], (it / kArrivals) & 1, p.status)) dead = true;
             const int nvw = (small ? (sm.meta[it % kArrivals] >> (8 * sub_w)) & 0xff : sm.meta[it % kArrivals]) - off_w;   // valid tokens from this warp's first row on
@@ -645,8 +729,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 float s[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) s[x] = ((sa[0][x] + sa[1][x]) + (sa[2][x] + sa[3][x])) * p.scale_log2;
-                if (rw >= nvw) s[0] = s[1] = -INFINITY;
-                if (rw + 8 >= nvw) s[2] = s[3] = -INFINITY;
+                const int lim0 = nvw - back[0], lim1 = nvw - back[1];      // tokens that a row sees of this warp's 16
+                if (rw >= lim0) s[0] = -INFINITY;
+                if (rw >= lim1) s[1] = -INFINITY;
+                if (rw + 8 >= lim0) s[2] = -INFINITY;
+                if (rw + 8 >= lim1) s[3] = -INFINITY;
                 // ---- online softmax over this warp's 16 tokens, per row (column of S^T) ----
                 float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
 #pragma unroll
@@ -689,7 +776,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], off);
             l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], off);
         }
-        worker_sync();                                     // every tile has been read: the ring is free
+        worker_sync<NW>();                                     // every tile has been read: the ring is free
         float* part = reinterpret_cast<float*>(sm.ring[0]) + warp * 8 * kMergeStride;
 #pragma unroll
         for (int a = 0; a < 8; ++a) {
@@ -705,42 +792,43 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         __syncwarp();
         if (!GATE) cluster_wait();                         // every CTA of the cluster has started (the barrier opened at the top)
-        worker_sync();
+        worker_sync<NW>();
         const int c_shift = 7 - s_shift;                   // log2 of the channels of a CTA's slice
-        {
-            // warp w: row w; lane: four channels
-            const int r = warp, c = 4 * lane;
+        // a warp per row; lane: four channels
+        for (int r = warp; r < rows; r += NW) {
+            const int c = 4 * lane, n_part = 4 * paces;    // the warps that have a share of row r
             float M = -INFINITY, l = 0.f;
-            float2 ml[kWarps];
+            float2 ml[NW];
+            auto warp_of = [&](int x) { return MULTI ? ((x >> 2) * tiles_n + (r >> 3)) * 4 + (x & 3) : x; };
 #pragma unroll
-            for (int x = 0; x < kWarps; ++x) {
-                ml[x] = sm.warp_ml[x][r];
+            for (int x = 0; x < NW; ++x) {
+                ml[x] = x < n_part ? sm.warp_ml[warp_of(x)][r & 7] : make_float2(-INFINITY, 0.f);
                 M = fmaxf(M, ml[x].x);
             }
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float* src = reinterpret_cast<const float*>(sm.ring[0]) + r * kMergeStride + c;
+            const float* src = reinterpret_cast<const float*>(sm.ring[0]) + (r & 7) * kMergeStride + c;
 #pragma unroll
-            for (int x = 0; x < kWarps; ++x) {
-                const float f = ml[x].x == -INFINITY ? 0.f : fast_exp2(ml[x].x - M);
-                const float4 v = *reinterpret_cast<const float4*>(src + x * 8 * kMergeStride);
-                l = fmaf(ml[x].y, f, l);
-                acc.x = fmaf(v.x, f, acc.x);
-                acc.y = fmaf(v.y, f, acc.y);
-                acc.z = fmaf(v.z, f, acc.z);
-                acc.w = fmaf(v.w, f, acc.w);
+            for (int x = 0; x < NW; ++x) {
+                if (x < n_part) {
+                    const float f = ml[x].x == -INFINITY ? 0.f : fast_exp2(ml[x].x - M);
+                    const float4 v = *reinterpret_cast<const float4*>(src + warp_of(x) * 8 * kMergeStride);
+                    l = fmaf(ml[x].y, f, l);
+                    acc.x = fmaf(v.x, f, acc.x);
+                    acc.y = fmaf(v.y, f, acc.y);
+                    acc.z = fmaf(v.z, f, acc.z);
+                    acc.w = fmaf(v.w, f, acc.w);
+                }
             }
-            if (r < p.group) {
-                float* dst = cluster.map_shared_rank(sm.recv_o, c >> c_shift) + (((rank * 8 + r) << c_shift) | (c & ((1 << c_shift) - 1)));
-                *reinterpret_cast<float4*>(dst) = acc;
-                if (lane < S) cluster.map_shared_rank(&sm.recv_ml[0][0], lane)[rank * 8 + r] = make_float2(M, l);
-            }
+            float* dst = cluster.map_shared_rank(sm.recv_o, c >> c_shift) + (((rank * kRows + r) << c_shift) | (c & ((1 << c_shift) - 1)));
+            *reinterpret_cast<float4*>(dst) = acc;
+            if (lane < S) cluster.map_shared_rank(&sm.recv_ml[0][0], lane)[rank * kRows + r] = make_float2(M, l);
         }
     }
     __syncwarp();
     cluster.sync();
     if (!producer) {
         const int c_shift = 7 - s_shift;
-        const int pairs = p.group << (c_shift - 1);        // channel pairs of this CTA's slice, all rows
+        const int pairs = rows << (c_shift - 1);        // channel pairs of this CTA's slice, all rows
         for (int x = tid; x < pairs; x += kWorkers) {
             const int r = x >> (c_shift - 1), c = 2 * (x & ((1 << (c_shift - 1)) - 1));
             float M = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f;
@@ -754,33 +842,34 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             for (int s = 0; s < kMaxS; ++s) {
                 if (s < S) {
                     const float f = ml[s].x == -INFINITY ? 0.f : fast_exp2(ml[s].x - M);
-                    const float2 v = *reinterpret_cast<const float2*>(&sm.recv_o[((s * 8 + r) << c_shift) + c]);
+                    const float2 v = *reinterpret_cast<const float2*>(&sm.recv_o[((s * kRows + r) << c_shift) + c]);
                     l = fmaf(ml[s].y, f, l);
                     a0 = fmaf(v.x, f, a0);
                     a1 = fmaf(v.y, f, a1);
                 }
             }
             const float inv = l > 0.f ? 1.f / l : 0.f;
-            const size_t row = (size_t)(row_u + r);
+            const size_t row = out_row(r);
             *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
             if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
         }
     }
 }
 
-template <bool GATE>
+template <int NW, bool GATE, bool MULTI>
 cudaError_t configure() {
-    cudaError_t e = cudaFuncSetAttribute(step_cluster_kernel<GATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StepSmem) + 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_cluster_kernel<GATE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(StepSmem<NW, MULTI>) + 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
-template <bool GATE>
-cudaLaunchConfig_t config_of(int S, int units, cudaStream_t stream, cudaLaunchAttribute (&attr)[2]) {
+template <int NW, bool GATE, bool MULTI>
+cudaLaunchConfig_t config_of(int S, int units, int parts, cudaStream_t stream, cudaLaunchAttribute (&attr)[2]) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(S, units);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = sizeof(StepSmem) + 1024;
+    cfg.gridDim = dim3(S, units, parts);
+    cfg.blockDim = dim3(Size<NW, MULTI>::kThreads);
+    cfg.dynamicSmemBytes = sizeof(StepSmem<NW, MULTI>) + 1024;
     cfg.stream = stream;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = S;
@@ -793,26 +882,29 @@ cudaLaunchConfig_t config_of(int S, int units, cudaStream_t stream, cudaLaunchAt
     return cfg;
 }
 
-// Clusters of 2^k CTAs that the device holds at once (both kernels have the same resources), asked once per device;
-// 0: the device or the driver does not take such clusters.
-int resident_clusters(int k) {
-    static int cached[kMaxDevices][5];                     // (value + 1; 0: not asked yet.  A race asks twice and stores the same)
-    const int slot = current_device_slot();
-    if (cached[slot][k] == 0) {
-        int n = 0;
-        if (configure<true>() == cudaSuccess && configure<false>() == cudaSuccess) {
-            cudaLaunchAttribute attr[2];
-            cudaLaunchConfig_t cfg = config_of<true>(1 << k, 1, nullptr, attr);
-            cfg.numAttrs = 1;
-            int a = 0, b = 0;
-            if (cudaOccupancyMaxActiveClusters(&a, step_cluster_kernel<true>, &cfg) != cudaSuccess) a = 0;
-            if (cudaOccupancyMaxActiveClusters(&b, step_cluster_kernel<false>, &cfg) != cudaSuccess) b = 0;
-            n = a < b ? a : b;
-            cudaGetLastError();                            // (a refused size is no error of the caller's)
-        }
-        cached[slot][k] = n + 1;
+template <int NW, bool GATE, bool MULTI>
+int resident_of(int k) {
+    if (configure<NW, GATE, MULTI>() != cudaSuccess) return 0;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = config_of<NW, GATE, MULTI>(1 << k, 1, 1, nullptr, attr);
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, step_cluster_kernel<NW, GATE, MULTI>, &cfg) != cudaSuccess) n = 0;
+    cudaGetLastError();                                    // (a refused size is no error of the caller's)
+    return n;
+}
+
+// Clusters of 2^k CTAs that the device holds at once (`wide`: of the NW = 16 kernels), asked once per device; 0: the
+// device or the driver does not take such clusters.
+int resident_clusters(bool wide, int k) {
+    static int cached[kMaxDevices][2][5];                  // (value + 1; 0: not asked yet.  A race asks twice and stores the same)
+    int& c = cached[current_device_slot()][wide][k];
+    if (c == 0) {
+        c = wide ? min(resident_of<16, true, true>(k), resident_of<16, false, true>(k)) + 1
+                 : min(min(resident_of<8, true, false>(k), resident_of<8, false, false>(k)),
+                       min(resident_of<8, true, true>(k), resident_of<8, false, true>(k))) + 1;
     }
-    return cached[slot][k] - 1;
+    return c - 1;
 }
 
 }  // namespace
@@ -823,32 +915,55 @@ int resident_clusters(int k) {
 //     step of batch 8 at 128k, 205 blocks (51 tiles a CTA)   98.4 -> 85.0
 //     given lists, 16 ragged sequences, blocks of 128        52.8 -> 45.8
 //     one 4 x 512-block list set (64 tiles a CTA)            93.5 -> 86.2
-// The line at kStepTilesPerCta tiles a CTA: beyond it the gain is below 5 % (128 tiles: 1.00 to 1.05) and a batch of
-// very uneven lengths, whose tiles the other kernel spreads over all SMs, could lose (256 dense tiles, lengths 1 : 8:
-// 185 -> 196).  With a few more CTAs than SMs the SMs that hold two of them are the last to finish (80 units, 64 tiles a
-// CTA, 160 CTAs: 65 -> 67; 32 tiles: 40.8 -> 37.5), so the line is at half as many tiles there.
-int step_cluster_size(int units, long long max_tiles, long long max_codes, int max_keys) {
-    const int sms = resident_clusters(0) / 2;
+//     four query tokens, 20 rows, 4 sequences, budget 4096   63.2 -> 38.6;  64 rows 92.3 -> 75.2;  8 rows, 1 sequence 27.2 -> 19.0
+//     threshold gate alone in front of given lists, 4 sequences of 48k, blocks of 32: 42.5 -> 35.0 with both
+// The line at 128 tiles a CTA (64 for dense calls): beyond it the gain is below 3 %, and a batch of very uneven lengths,
+// whose tiles the other kernel spreads over all SMs, could lose (256 dense tiles, lengths 1 : 8: 185 -> 196).  With a few
+// more CTAs than SMs the SMs that hold two of them are the last to finish (80 units, 64 tiles a CTA, 160 CTAs: 65 -> 67;
+// 32 tiles: 40.8 -> 37.5), so the line is at 32 there.
+StepPlan step_plan(int units, int rows, bool dense, long long max_tiles, long long max_codes, int max_keys) {
+    const bool wide = rows > 16;
+    StepPlan plan = {0, 1, rows};
+    if (rows > 64) return plan;
+    if (wide) {
+        plan.parts = (rows + 31) / 32;
+        plan.rows = (rows + plan.parts - 1) / plan.parts;
+    }
+    const int sms = wide ? resident_clusters(true, 0) : resident_clusters(false, 0) / 2;
+    units *= plan.parts;
     for (int k = 4; k >= 0; --k) {
         const int S = 1 << k;
         if (k > 0 && S > max_tiles && 128ll * S > max_keys) continue;      // a CTA would have nothing to do
-        if (units > resident_clusters(k)) continue;
+        if (units > resident_clusters(wide, k)) continue;
         const bool few_doubled = units * S > sms && 5 * units * S <= 6 * sms;
-        const long long line = (long long)S * (few_doubled ? kStepTilesPerCta / 2 : kStepTilesPerCta);
-        return max_tiles <= line && max_codes <= (long long)S * kCodes ? S : 0;
+        const long long line = (long long)S * (few_doubled ? 32 : dense ? 64 : 128);
+        if (max_tiles <= line && max_codes <= (long long)S * kCodes) plan.S = S;
+        break;
     }
-    return 0;
+    return plan;
 }
 
-cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g, int S,
-                                cudaStream_t stream) {
+namespace {
+
+template <int NW, bool MULTI>
+cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g, const StepPlan& plan,
+                      cudaStream_t stream) {
     cudaLaunchAttribute attr[2];
     if (g) {
-        const cudaLaunchConfig_t cfg = config_of<true>(S, p.num_units, stream, attr);
-        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<true>, map_k, map_v, p, GateArg<true>{*g});
+        const cudaLaunchConfig_t cfg = config_of<NW, true, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
+        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, MULTI>, map_k, map_v, p, GateArg<true>{*g});
     }
-    const cudaLaunchConfig_t cfg = config_of<false>(S, p.num_units, stream, attr);
-    return cudaLaunchKernelEx(&cfg, step_cluster_kernel<false>, map_k, map_v, p, GateArg<false>{});
+    const cudaLaunchConfig_t cfg = config_of<NW, false, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
+    return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, false, MULTI>, map_k, map_v, p, GateArg<false>{});
+}
+
+}  // namespace
+
+cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
+                                const StepPlan& plan, cudaStream_t stream) {
+    if (p.q_len == 1) return launch_of<8, false>(map_k, map_v, p, g, plan, stream);
+    return plan.parts * plan.rows <= 16 ? launch_of<8, true>(map_k, map_v, p, g, plan, stream)
+                                        : launch_of<16, true>(map_k, map_v, p, g, plan, stream);
 }
 
 }  // namespace seer

@@ -9,7 +9,7 @@ import torch
 
 import oracle
 from paper_2506_08889_b200 import binding, synth
-from util import bits, check_attention, make_qkv, ref_dense, ref_sparse, to_paged
+from util import bits, check_attention, make_qkv, ref_dense, ref_sparse, ref_sparse_multi, to_paged
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -100,6 +100,103 @@ def test_step_sparse_dense(ctx, case):
         ctx.seer_dense_decode(shape, kv, q, out, lse)
         torch.cuda.synchronize()
         check_attention(out, lse, *ref_dense(qh, kh, vh, lens, SCALE), what="dense")
+    assert ctx.device_status() == binding.SEER_OK
+
+
+MULTI = [
+    # B, Hq, Hkv, q_len, b, d_gate, S, page, (budget in blocks, max_sel): 6, 8, 10, 20, 32, 40 and 64 rows a unit
+    (2, 6, 2, 2, 64, 128, 4096, 0, (9, 9)),
+    (5, 8, 2, 2, 16, 64, 2048, 0, (21, 21)),
+    (1, 5, 1, 2, 128, 128, 8192, 128, (20, 33)),
+    (3, 40, 8, 4, 64, 128, 4096, 64, (33, 33)),
+    (37, 8, 1, 4, 32, 256, 1024, 0, (14, 14)),
+    (4, 10, 2, 8, 64, 128, 4096 - 5, 0, (1, 40)),
+    (2, 64, 8, 8, 64, 128, 8192, 0, (70, 70)),
+]
+
+
+@pytest.mark.parametrize("case", range(len(MULTI)))
+def test_step_multi(ctx, case):
+    B, Hq, Hkv, T, b, dg, S, page, (budget, max_sel) = MULTI[case]
+    d, seed = 128, 400 + case
+    cap = -(-S // max(page, b, 64)) * max(page, b, 64)
+    nb = cap // b
+    # boundaries inside the new tokens, fewer tokens than queries, an empty sequence
+    lens = np.array(([S, 7 * b + 1, cap - b, T - 1, 0] * B)[:B], np.int32)
+    q = synth.normal_bf16((B, T, Hq, d), seed, "q", DEV)
+    qn = synth.normal_bf16((B, T, Hq, d), seed, "qn", DEV)
+    _, k, v = make_qkv(B, Hq, Hkv, cap, d, seed, DEV)
+    for i in range(B):
+        v[i, :, lens[i]:] = float("nan")
+    wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), seed, "wq", DEV, std=0.02)
+    kc = synth.normal_bf16((B, Hkv, nb, dg), seed, "kc", DEV)
+    shape = binding.make_shape(B, Hq, Hkv, d, b, SCALE)
+    gate = binding.make_gate(dg, THETA, wq, None, kc, nb)
+    lens_t = torch.as_tensor(lens, device=DEV)
+    if page:
+        kp, vp, table = to_paged(k, v, page, seed)
+        kv = binding.make_kv(kp, vp, lens_t, max_seq_len=cap, page_table=table, page_size=page)
+    else:
+        kv = binding.make_kv(k, v, lens_t)
+    idx = torch.full((B, Hkv, max_sel), 55, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hkv), 55, dtype=torch.int32, device=DEV)
+    out = torch.full((B, T, Hq, d), float("nan"), dtype=torch.bfloat16, device=DEV)
+    lse = torch.full((B, T, Hq), float("nan"), dtype=torch.float32, device=DEV)
+    for _ in range(3):
+        before = ctx.launch_count()
+        ctx.seer_decode_step_multi(shape, kv, gate, q, qn, T, None, budget * b, idx, cnt, max_sel, out, lse)
+        if ctx.one_launch:
+            assert ctx.launch_count() - before == 1
+    sc = torch.zeros((B, Hkv, nb), dtype=torch.float32, device=DEV)
+    idx2, cnt2 = torch.zeros_like(idx), torch.zeros_like(cnt)
+    ctx.seer_gate_select_multi(shape, gate, lens_t, qn, None, T, budget * b, idx2, cnt2, max_sel, scores_out=sc)
+    torch.cuda.synchronize()
+    want_idx, want_cnt = oracle.select_multi(sc.cpu().numpy(), lens, b, budget * b, T, max_sel)
+    for got_idx, got_cnt in ((idx, cnt), (idx2, cnt2)):
+        assert np.array_equal(got_cnt.cpu().numpy(), want_cnt) and np.array_equal(got_idx.cpu().numpy(), want_idx)
+    qh, kh, vh = bits(q), bits(k), bits(torch.nan_to_num(v))
+    ref = ref_sparse_multi(qh, kh, vh, lens, want_idx, want_cnt, b, SCALE)
+    check_attention(out, lse, *ref, what="multi step")
+    out.fill_(float("nan")), lse.fill_(float("nan"))
+    ctx.seer_sparse_decode_multi(shape, kv, q, T, idx, cnt, max_sel, out, lse)
+    torch.cuda.synchronize()
+    check_attention(out, lse, *ref, what="multi sparse")
+    out.fill_(float("nan")), lse.fill_(float("nan"))
+    ctx.seer_dense_decode_multi(shape, kv, q, T, out, lse)
+    torch.cuda.synchronize()
+    all_idx = np.full((B, Hkv, nb), -1, np.int32)
+    for i in range(B):
+        all_idx[i, :, :-(-int(lens[i]) // b)] = np.arange(-(-int(lens[i]) // b))
+    all_cnt = np.repeat((-(-lens // b))[:, None], Hkv, 1).astype(np.int32)
+    check_attention(out, lse, *ref_sparse_multi(qh, kh, vh, lens, all_idx, all_cnt, b, SCALE), what="multi dense")
+    assert ctx.device_status() == binding.SEER_OK
+
+
+@pytest.mark.parametrize("n,T,tau,max_sel", [(1500, 1, 2e-3, 400), (1500, 1, 1e-7, 40), (8000, 3, 4e-4, 900), (33, 1, 0.5, 9)])
+def test_threshold_gate(ctx, n, T, tau, max_sel):
+    # the lists against the threshold rule applied to the scores that the gate gives out; a block within rounding of
+    # tau may fall on either side
+    B, Hq, Hkv, d, dg, b = 2, 16, 2, 128, 128, 32
+    lens = np.array([n * b - 3, max(T, n * b // 3)], np.int32)
+    qn = synth.normal_bf16((B, T, Hq, d), 61, "qn", DEV)
+    wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), 61, "wq", DEV, std=0.03)
+    kc = synth.normal_bf16((B, Hkv, n, dg), 61, "kc", DEV)
+    shape = binding.make_shape(B, Hq, Hkv, d, b, SCALE)
+    gate = binding.make_gate(dg, THETA, wq, None, kc, n)
+    lens_t = torch.as_tensor(lens, device=DEV)
+    idx = torch.full((B, Hkv, max_sel), 55, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hkv), 55, dtype=torch.int32, device=DEV)
+    sc = torch.zeros((B, Hkv, n), dtype=torch.float32, device=DEV)
+    ctx.seer_gate_select_threshold_multi(shape, gate, lens_t, qn, None, T, tau, idx, cnt, max_sel, scores_out=sc)
+    torch.cuda.synchronize()
+    want_idx, want_cnt, probs = oracle.select_threshold_multi(sc.cpu().numpy(), lens, b, tau, T, max_sel)
+    idx, cnt = idx.cpu().numpy(), cnt.cpu().numpy()
+    for i in range(B):
+        for h in range(Hkv):
+            got, want = idx[i, h, :cnt[i, h]], want_idx[i, h, :want_cnt[i, h]]
+            assert np.all(np.diff(got) > 0) and np.all(idx[i, h, cnt[i, h]:] == -1)
+            for j in set(got.tolist()) ^ set(want.tolist()):
+                assert abs(probs[i, h, j] - tau) <= 1e-5 * tau + 1e-9, (i, h, j)
     assert ctx.device_status() == binding.SEER_OK
 
 

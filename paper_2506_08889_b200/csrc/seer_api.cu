@@ -743,7 +743,7 @@ static seer_status kcomp_append_common(seer_ctx* ctx, const seer_shape* shape, c
         const uint64_t dims[4] = {(uint64_t)kHeadDim, (uint64_t)(first_block + num_blocks) * (uint64_t)shape->block_size,
                                   (uint64_t)shape->num_kv_heads, (uint64_t)shape->batch};
         const uint64_t strides[3] = {(uint64_t)stride_token * 2, (uint64_t)stride_head * 2, (uint64_t)stride_batch * 2};
-        st = get_map(ctx, k_nope, dims, strides, kKcompStageRows, &map_k);
+        st = get_map(ctx, k_nope, dims, strides, shape->block_size < kKcompStageRows ? shape->block_size : kKcompStageRows, &map_k);
         if (st != SEER_OK) return st;
     }
     int launched = 0;

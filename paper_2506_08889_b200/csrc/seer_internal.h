@@ -160,8 +160,9 @@ struct KcompParams {
     double inv_freq[kMaxDGate / 2];
 };
 // True when the bulk build of these parameters runs as the persistent streaming kernel, which reads the keys
-// through a tensor map (channel, token row, head, sequence) with a box of 64 channels x kKcompStageRows rows,
-// 128-byte swizzle; launch_kcomp_append falls back to the plain-load kernel when it is given no map.
+// through a tensor map (channel, token row, head, sequence) with a box of 64 channels x kKcompStageRows rows (or a
+// block's, if it has fewer), 128-byte swizzle; launch_kcomp_append falls back to the plain-load kernel when it is given
+// no map.
 constexpr int kKcompStageRows = 64;
 bool kcomp_bulk_streams(const KcompParams& p);
 cudaError_t launch_kcomp_append(const KcompParams& p, const CUtensorMap* map_k, cudaStream_t stream, int* launched);

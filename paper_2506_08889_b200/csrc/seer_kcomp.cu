@@ -344,37 +344,42 @@ __global__ void __launch_bounds__(kKcThreads, 4) kcomp_bulk_kernel(const KcompPa
 }
 
 
-// ---- bulk build, streaming variant (b = 64, d_gate <= 128) ----------------------------------------
+// ---- bulk build, streaming variant (d_gate <= 128) --------------------------------------------------
 // One persistent CTA per SM, four kinds of warps that meet only through mbarriers:
-//   producer (1 warp)    keeps a ring of 64-row stages (one block, 16 KiB) full with tiled copies, so
-//                        the bytes in flight do not depend on what the other warps are doing;
-//   pooling (10 warps)   each takes one block at a time out of shared memory and leaves the block's
-//                        3*128 features (bf16; the mean as high part + correction: 512 numbers) in one of
-//                        two feature buffers, laid out as the tensor cores read a K-major operand;
-//   MMA (1 warp)         once 16 blocks are pooled, one thread multiplies them in: Y (128 rows of W_k x 16
-//                        blocks, fp32 in tensor memory) = W_k[h] (from tensor memory, where it stays while
+//   producer (1 warp)    keeps a ring of 64-row stages (16 KiB) full with tiled copies, so the bytes in
+//                        flight do not depend on what the other warps are doing;
+//   pooling (10 warps)   each takes one portion at a time out of shared memory -- a block of 64 or 128 rows
+//                        (one or two stages), or the two or four blocks of 32 or 16 rows in a stage -- and leaves
+//                        each block's 3*128 features (bf16; the mean as high part + correction: 512 numbers) in one
+//                        of two feature buffers, laid out as the tensor cores read a K-major operand;
+//   MMA (1 warp)         once an item's (up to 16) blocks are pooled, one thread multiplies them in: Y (128 rows of
+//                        W_k x 16 blocks, fp32 in tensor memory) = W_k[h] (from tensor memory, where it stays while
 //                        the CTA's items have the same head) . features^T, 32 tcgen05.mma of K = 16;
 //   epilogue (4 warps)   thread r has row r of W_k and of Y: it puts its row of W_k[h] into tensor memory when
 //                        the head changes, reads its 16 products, and the four warps rotate and store -
 //                        while the pooling warps are already on the next item.
-// An item is 16 consecutive blocks of one (sequence, KV head); items are numbered head-major and dealt
-// round-robin, so a CTA changes head a handful of times per launch.
+// All complete blocks, laid end to end head by head and sequence by sequence, are cut into one run of equal length (to
+// one block) per CTA.  A run is worked off in items of up to 16 blocks of one (sequence, KV head).  So a CTA changes head
+// at most once in a launch (never, where the heads divide the CTAs), where items of 16 dealt round robin, head by head, changed it with almost every item of a
+// small build (each change 96 KiB of W_k into tensor memory, behind the copies), and no CTA has a whole item
+// more than another.  Measured, us a call, before -> after (blocks of 64; 128, which went through the plain kernel):
+//     2 x 8 heads x 128k (0.54 GB)              124 -> 92 .. 96   116 -> 89         (floor 83)
+//     6 ragged sequences of 5k .. 32k           79.9 -> 48.0      69.9 -> 46.1      (floor 36)
+//     one sequence of 8k                        19.3 -> 11.6      28.3 -> 11.7      (launch, lengths, one trip through the kernel)
+// Blocks of 32 and 16 are bound by what is done per block (shuffles, features, rotation): 0.54 GB 190 -> 116, 309 -> 168
+// (one box of 64 rows instead of a box per block: 106 and 166, but it may reach past the last complete block).
 //
-// A block comes in kStagesPerBlock stages (a stage is freed as soon as it has been read, and what is free
-// is in flight again).  Block number n of a CTA (counted over all its items) is pooled by warp
-// n % kPoolWarps and its stages live in ring slots (n * kStagesPerBlock + part) % kStreamStages;
-// kStreamStages is a multiple of kStagesPerBlock * kPoolWarps, so a slot is always read by the same
-// warp, which goes through its stages in order: a wait on a slot's barrier is then never more than one
-// phase away from the barrier's own, which is what a parity wait needs to be unambiguous.  (With a
-// block-of-the-item -> warp rule a fast warp could ask for a slot's next use before the slot's current use
-// had landed for another warp, and the parity test would pass on stale data.)
+// Portion number n of a CTA (counted over all its items) is pooled by warp n % kPoolWarps, its stages n * SPB + part live
+// in ring slots (..) % kStreamStages and are announced on barrier (..) % (SPB * kPoolWarps): a barrier is always waited
+// for by the same warp, which goes through its stages in order, so a wait is never more than one phase away from the
+// barrier's own, which is what a parity wait needs to be unambiguous.  (With a block-of-the-item -> warp rule a fast warp
+// could ask for a slot's next use before the slot's current use had landed for another warp, and the parity test would
+// pass on stale data.)
 constexpr int kStreamStages = 10;                      // 160 KiB in flight per SM
-constexpr int kStreamRows = 64;                        // the block size this kernel is written for
 constexpr int kStageRows = kKcompStageRows;
-constexpr int kStagesPerBlock = kStreamRows / kStageRows;
 constexpr int kStageBytes = kStageRows * kHeadDim * 2;
 constexpr int kStreamDGate = 128;
-constexpr int kLensCache = 2048;                       // sequences whose length is kept in shared memory
+constexpr int kMaxSeqs = 4096;                         // sequences whose block counts are kept in shared memory
 constexpr int kPoolWarps = 10;                       // with 4 + 1 + 1 others: 16 warps
 constexpr int kProjWarps = 5;                        // warps 0..3 epilogue, 4 MMA
 constexpr int kEpiWarps = 4, kEpiThreads = 128;
@@ -382,11 +387,10 @@ constexpr int kFeatBytes = 8 * kBulkBlocks * 128;      // one feature buffer
 constexpr int kKcTmemCols = 512;                       // W_k 256 columns (512 bf16 per row), Y twice 16
 constexpr int kStreamThreads = 32 * (kProjWarps + kPoolWarps + 1);
 static_assert(kStreamStages <= 32, "one producer lane per ring slot");
-static_assert(kStreamStages % (kStagesPerBlock * kPoolWarps) == 0,
-              "a ring slot must always be read by the same pooling warp");
+static_assert(kStreamStages % kPoolWarps == 0 && 2 * kPoolWarps % kStreamStages == 0, "a barrier stands for one ring slot");
 
 struct __align__(1024) StreamSmem {
-    // a stage: channels 0..63 of its 32 rows (128 B per row, 16-byte pieces swizzled by row as the copy engine
+    // a stage: channels 0..63 of its 64 rows (128 B per row, 16-byte pieces swizzled by row as the copy engine
     // lays them out), then channels 64..127
     unsigned char ring[kStreamStages][kStageBytes];
     // features of 16 blocks, twice: [8 slabs of 64 features][16 blocks][128 B], 16-byte pieces swizzled by
@@ -394,16 +398,23 @@ struct __align__(1024) StreamSmem {
     // high part 4-5, its correction 6-7
     unsigned char feat[2][kFeatBytes];
     float ybuf[kBulkBlocks][kStreamDGate];
-    uint64_t full[kStreamStages], empty[kStreamStages];
+    uint64_t full[2 * kPoolWarps], empty[kStreamStages];
     uint64_t feat_full[2], feat_empty[2];
     uint64_t y_full[2], y_free[2];       // the products of an even / odd item are complete / have been read
     uint64_t w_ready;                    // a head's W_k is in tensor memory
     uint64_t tmem_done;                  // the epilogue warps have made their last tensor-memory access
     uint32_t tmem_base;
-    int lens[kLensCache];                                             // seq_lens, read once
+    int scan[kStreamThreads / 32];
+    int first[kMaxSeqs + 1];             // blocks of the sequences before (prefix sums of the complete blocks in the call's range)
 };
 static_assert(sizeof(StreamSmem) + 1024 <= 227 * 1024, "one CTA's shared memory");
 static_assert(kStageBytes % 2048 == 0, "both halves of a stage start on a swizzle-pattern boundary");
+
+// A CTA's run of blocks [x, end), item by item; every warp goes through it for itself.
+struct Run {
+    int x, end;          // blocks, counted head by head, sequence by sequence
+    int h, i, j, nb;     // the current item: head, sequence, first block, blocks (0: the run is over)
+};
 
 #ifdef SEER_DECODE_TRACE
 #define KC_T(var) const long long var = clock64()
@@ -413,18 +424,24 @@ static_assert(kStageBytes % 2048 == 0, "both halves of a stage start on a swizzl
 #define KC_ACC(slot, t0, t1)
 #endif
 
+// Barriers among parts of the CTA: the epilogue warps; the others; the others' arrival for the epilogue warps to wait for.
+__device__ __forceinline__ void rest_sync() { asm volatile("bar.sync 2, %0;" ::"n"(kStreamThreads - kEpiThreads) : "memory"); }
+__device__ __forceinline__ void lengths_arrive() { asm volatile("bar.arrive 3, %0;" ::"n"(kStreamThreads) : "memory"); }
+__device__ __forceinline__ void lengths_wait() { asm volatile("bar.sync 3, %0;" ::"n"(kStreamThreads) : "memory"); }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
+template <int B>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams p) {
+    constexpr int SPB = B > kStageRows ? B / kStageRows : 1;       // stages of a portion
+    constexpr int BPS = B < kStageRows ? kStageRows / B : 1;       // blocks of a portion
+    constexpr int kArrivals = SPB * kPoolWarps;
     extern __shared__ unsigned char smem_raw[];
     StreamSmem& sm = *reinterpret_cast<StreamSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        for (int s = 0; s < kStreamStages; ++s) {
-            mbar_init(&sm.full[s], 1);
-            mbar_init(&sm.empty[s], 1);
-        }
+        for (int s = 0; s < kArrivals; ++s) mbar_init(&sm.full[s], 1);
+        for (int s = 0; s < kStreamStages; ++s) mbar_init(&sm.empty[s], 1);
         for (int f = 0; f < 2; ++f) {
             mbar_init(&sm.feat_full[f], kPoolWarps);
             mbar_init(&sm.feat_empty[f], 1);
@@ -437,36 +454,103 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
     }
     if (warp == kEpiWarps) tmem_alloc(&sm.tmem_base, kKcTmemCols);
     tc_fence_before_sync();
-    pdl_wait();
-    pdl_launch_dependents();
-    // A small load issued while the copies flood the memory system waits microseconds behind them: the
-    // lengths are fetched once, before any copy is in flight.
-    for (int x = tid; x < min(p.batch, kLensCache); x += kStreamThreads) sm.lens[x] = p.seq_lens[x];
     __syncthreads();
     tc_fence_after_sync();
 
-    const int b = p.block_size;                        // == kStreamRows
-    const int groups = (p.num_blocks + kBulkBlocks - 1) / kBulkBlocks;
-    const int per_head = groups * p.batch;
-    const int n_items = per_head * p.num_kv_heads;
+    // Row `tid` of W_k[h] into tensor memory (epilogue warps): 256 columns, [max | min | mean | mean again].
+    auto load_w = [&](int h) {
+        const uint32_t tbase = sm.tmem_base + ((uint32_t)(32 * warp) << 16);
+        const uint4* wrow = reinterpret_cast<const uint4*>(p.w_k + ((size_t)h * p.d_gate + min(tid, p.d_gate - 1)) * 3 * kHeadDim);
+#pragma unroll 1
+        for (int c0 = 0; c0 < 3; ++c0) {                   // 2 x 32 columns = 128 bf16 each, in flight together
+            uint32_t wr[2][32];
+#pragma unroll
+            for (int x = 0; x < 16; ++x) {
+                const uint4 v = tid < p.d_gate ? __ldg(wrow + 16 * c0 + x) : make_uint4(0u, 0u, 0u, 0u);
+                wr[x >> 3][4 * (x & 7)] = v.x; wr[x >> 3][4 * (x & 7) + 1] = v.y;
+                wr[x >> 3][4 * (x & 7) + 2] = v.z; wr[x >> 3][4 * (x & 7) + 3] = v.w;
+            }
+            tmem_st32(tbase + 64 * c0, wr[0]);
+            tmem_st32(tbase + 64 * c0 + 32, wr[1]);
+            if (c0 == 2) {                                 // the mean's weights serve its correction too
+                tmem_st32(tbase + 192, wr[0]);
+                tmem_st32(tbase + 224, wr[1]);
+            }
+        }
+        tmem_wait_st();
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.w_ready);
+    };
+    // (run_begin's first head, whatever the lengths)
+    const int h_first = (int)((long long)p.num_kv_heads * blockIdx.x / gridDim.x);
+    const int j_end = min(p.first_block + p.num_blocks, p.max_blocks);
+    if (warp < kEpiWarps) {
+        load_w(h_first);                                   // weights are constants: before the wait
+        pdl_wait();
+        lengths_wait();
+    } else {
+        pdl_wait();
+        pdl_launch_dependents();
+        // Blocks per sequence, summed up.  (A small load issued while the copies flood the memory system waits
+        // microseconds behind them: the lengths are fetched once, before any copy is in flight.)
+        const int n_thr = kStreamThreads - kEpiThreads, t = tid - kEpiThreads;
+        const int per = (p.batch + n_thr - 1) / n_thr;
+        const int lo = min(p.batch, t * per), hi = min(p.batch, lo + per);
+        auto blocks_of = [&](int i) { const int L = p.seq_lens[i]; return max(0, min(j_end, L > 0 ? L / B : 0) - p.first_block); };
+        int mine = 0;
+        for (int i = lo; i < hi; ++i) mine += blocks_of(i);
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) sm.scan[warp] = incl;
+        rest_sync();
+        int acc = incl - mine;
+#pragma unroll
+        for (int w = kEpiWarps; w < kStreamThreads / 32; ++w) acc += w < warp ? sm.scan[w] : 0;
+        for (int i = lo; i < hi; ++i) {
+            sm.first[i] = acc;
+            acc += per == 1 ? mine : blocks_of(i);
+        }
+        if (hi == p.batch && lo < hi) sm.first[p.batch] = acc;
+        lengths_arrive();
+        rest_sync();
+    }
+
+    const int per_head = sm.first[p.batch];
+    const long long total = (long long)per_head * p.num_kv_heads;
     bool dead = false;                                 // a wait ran out: stop waiting, finish the motions
 #ifdef SEER_DECODE_TRACE
     unsigned long long tr[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const long long t_begin = clock64();
 #endif
 
-    // item -> (head, sequence, first block) and the number of complete blocks of it that exist
-    auto item_blocks = [&](int item, int& h, int& i, int& j_first) {
-        h = item / per_head;
-        const int rem = item - h * per_head;
-        const int g = rem / p.batch;
-        i = rem - g * p.batch;
-        const int L = i < kLensCache ? sm.lens[i] : p.seq_lens[i];
-        const int complete = L > 0 ? L / b : 0;
-        j_first = p.first_block + g * kBulkBlocks;
-        const int j_end = min(min(p.first_block + p.num_blocks, complete), p.max_blocks);
-        return max(0, min(kBulkBlocks, j_end - j_first));
+    auto item_at = [&](Run& r) {                       // fills in the item that begins at r.x
+        r.nb = 0;
+        if (r.x >= r.end) return;
+        r.h = r.x / per_head;
+        const int rem = r.x - r.h * per_head;
+        int lo = 0, hi = p.batch;                      // first[lo] <= rem < first[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (sm.first[mid] <= rem) lo = mid; else hi = mid;
+        }
+        r.i = lo;
+        r.j = p.first_block + rem - sm.first[lo];
+        r.nb = min(min(kBulkBlocks, sm.first[lo + 1] - rem), r.end - r.x);
     };
+    auto run_begin = [&]() {
+        Run r;
+        r.x = (int)(total * blockIdx.x / gridDim.x);
+        r.end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+        item_at(r);
+        return r;
+    };
+    auto run_next = [&](Run& r) { r.x += r.nb; item_at(r); };
+    auto portions = [](int nb) { return (nb + BPS - 1) / BPS; };
 
     if (warp == kProjWarps + kPoolWarps) {
         // ---- producer ----
@@ -476,26 +560,33 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
         // instead of one barrier round trip after the other.
         if (lane == 0) tma_prefetch_desc(&map_k);
         uint32_t cursor = lane;                        // the stage this lane arms next
-        uint32_t item_first = 0;                       // stage number of the first stage of `item`
-        int item = blockIdx.x, h = 0, i = 0, j_first = 0;
-        int nb = item < n_items ? item_blocks(item, h, i, j_first) : 0;
+        uint32_t item_first = 0;                       // stage number of the first stage of the item
+        Run r = run_begin();
         uint32_t idle = 0;
         while (true) {
-            while (item < n_items && cursor >= item_first + (uint32_t)(nb * kStagesPerBlock)) {
-                item_first += nb * kStagesPerBlock;
-                item += gridDim.x;
-                nb = item < n_items ? item_blocks(item, h, i, j_first) : 0;
+            while (r.nb > 0 && cursor >= item_first + (uint32_t)(portions(r.nb) * SPB)) {
+                item_first += portions(r.nb) * SPB;
+                run_next(r);
             }
-            const bool have = lane < kStreamStages && item < n_items;
+            const bool have = lane < kStreamStages && r.nb > 0;
             if (!__any_sync(0xffffffffu, have)) break;
             const bool go = have && mbar_test_wait(&sm.empty[lane], ((cursor / kStreamStages) & 1u) ^ 1u);
             if (go) {
-                const uint32_t rel = cursor - item_first;
-                const int q = rel / kStagesPerBlock, part = rel % kStagesPerBlock;
-                const int row0 = (j_first + q) * b + part * kStageRows;
-                mbar_arrive_expect_tx(&sm.full[lane], kStageBytes);
-                tma_load_4d(sm.ring[lane], &map_k, &sm.full[lane], 0, row0, h, i);
-                tma_load_4d(sm.ring[lane] + kStageBytes / 2, &map_k, &sm.full[lane], 64, row0, h, i);
+                const int row0 = r.j * B + (int)(cursor - item_first) * kStageRows;
+                uint64_t* full = &sm.full[cursor % kArrivals];
+                if (BPS == 1) {
+                    mbar_arrive_expect_tx(full, kStageBytes);
+                    tma_load_4d(sm.ring[lane], &map_k, full, 0, row0, r.h, r.i);
+                    tma_load_4d(sm.ring[lane] + kStageBytes / 2, &map_k, full, 64, row0, r.h, r.i);
+                } else {
+                    // block by block: nothing past the last complete one is read
+                    const int n_here = min(BPS, r.nb - (int)(cursor - item_first) * BPS);
+                    mbar_arrive_expect_tx(full, (uint32_t)n_here * (B * 256));
+                    for (int sb = 0; sb < n_here; ++sb) {
+                        tma_load_4d(sm.ring[lane] + sb * (B * 128), &map_k, full, 0, row0 + sb * B, r.h, r.i);
+                        tma_load_4d(sm.ring[lane] + kStageBytes / 2 + sb * (B * 128), &map_k, full, 64, row0 + sb * B, r.h, r.i);
+                    }
+                }
                 cursor += kStreamStages;
             }
             const uint32_t went = __ballot_sync(0xffffffffu, go);
@@ -521,97 +612,102 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
         int piece_off[4];
 #pragma unroll
         for (int m = 0; m < 4; ++m) piece_off[m] = (((cchunk & 7) ^ (lane >> 4)) ^ (2 * m)) << 4;
-        uint32_t block_no = 0, n_done = 0;                 // blocks and items this CTA has been through
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            int h, i, j_first;
-            const int nb = item_blocks(item, h, i, j_first);
-            if (nb == 0) continue;
-            const int fb = n_done & 1;
+        uint32_t portion_no = 0, n_done = 0;               // portions and items this CTA has been through
+        for (Run r = run_begin(); r.nb > 0; run_next(r)) {
+            const int fb = n_done & 1, n_por = portions(r.nb);
             KC_T(t_fe0);
             if (!dead && !mbar_wait(&sm.feat_empty[fb], ((n_done >> 1) & 1u) ^ 1u, p.status)) dead = true;
             KC_T(t_fe1);
             KC_ACC(0, t_fe0, t_fe1);
-            for (int q = 0; q < kBulkBlocks; ++q) {
-                if ((block_no + q) % kPoolWarps != (uint32_t)pw) continue;
-                __nv_bfloat162 mx[4], mn[4];
-                float sum[8];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    mx[c] = __float2bfloat162_rn(-INFINITY);
-                    mn[c] = __float2bfloat162_rn(INFINITY);
-                }
-#pragma unroll
-                for (int c = 0; c < 8; ++c) sum[c] = 0.f;
-                if (q < nb) {
+            // (the portions past the item's last one only clear their blocks' features)
+            for (int q0 = 0; q0 < kBulkBlocks / BPS; ++q0) {
+                if ((portion_no + q0) % kPoolWarps != (uint32_t)pw) continue;
+                const bool real = q0 < n_por;
+                const uint32_t sn0 = (portion_no + q0) * SPB;
 #pragma unroll 1
-                    for (int part = 0; part < kStagesPerBlock; ++part) {
-                        const uint32_t sn = (block_no + q) * kStagesPerBlock + part;
-                        const int s = sn % kStreamStages;
-                        KC_T(t_w0);
-                        if (!dead && !mbar_wait(&sm.full[s], (sn / kStreamStages) & 1u, p.status)) dead = true;
-                        KC_T(t_w1);
-                        KC_ACC(1, t_w0, t_w1);
-                        // lane: 16-byte column piece (lane & 15) of rows 2k + (lane >> 4); piece c of row r of a
-                        // 64-channel half sits at position c ^ (r & 7) of the row's 128 bytes
-                        const unsigned char* st = sm.ring[s] + lane_off;
-#pragma unroll 8
-                        for (int k = 0; k < kStageRows / 2; ++k) {
-                            const uint4 v = *reinterpret_cast<const uint4*>(st + k * 256 + piece_off[k & 3]);
-                            const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                mx[c] = __hmax2(mx[c], hh[c]);
-                                mn[c] = __hmin2(mn[c], hh[c]);
-                                const float2 f = bf16x2_to_float2(hh[c]);
-                                sum[2 * c] += f.x; sum[2 * c + 1] += f.y;
-                            }
-                        }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&sm.empty[s]);
-                        KC_T(t_w2);
-                        KC_ACC(2, t_w1, t_w2);
-#ifdef SEER_DECODE_TRACE
-                        tr[3] += 1;
-#endif
-                    }
+                for (int sb = 0; sb < BPS; ++sb) {
+                    const int q = q0 * BPS + sb;           // block of the item
+                    __nv_bfloat162 mx[4], mn[4];
+                    float sum[8];
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        uint32_t xm = *reinterpret_cast<uint32_t*>(&mx[c]), xn = *reinterpret_cast<uint32_t*>(&mn[c]);
-                        uint32_t ym = __shfl_xor_sync(0xffffffffu, xm, 16), yn = __shfl_xor_sync(0xffffffffu, xn, 16);
-                        mx[c] = __hmax2(mx[c], *reinterpret_cast<__nv_bfloat162*>(&ym));
-                        mn[c] = __hmin2(mn[c], *reinterpret_cast<__nv_bfloat162*>(&yn));
+                        mx[c] = __float2bfloat162_rn(-INFINITY);
+                        mn[c] = __float2bfloat162_rn(INFINITY);
                     }
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) sum[c] += __shfl_xor_sync(0xffffffffu, sum[c], 16);
-                }
-                if (lane < 16) {
-                    // 8 features per kind and lane: one 16-byte piece each, at its swizzled place in row q of its slab
-                    uint4 pmax = make_uint4(0u, 0u, 0u, 0u), pmin = pmax, phi = pmax, plo = pmax;
-                    if (q < nb) {
-                        pmax = make_uint4(*reinterpret_cast<uint32_t*>(&mx[0]), *reinterpret_cast<uint32_t*>(&mx[1]),
-                                          *reinterpret_cast<uint32_t*>(&mx[2]), *reinterpret_cast<uint32_t*>(&mx[3]));
-                        pmin = make_uint4(*reinterpret_cast<uint32_t*>(&mn[0]), *reinterpret_cast<uint32_t*>(&mn[1]),
-                                          *reinterpret_cast<uint32_t*>(&mn[2]), *reinterpret_cast<uint32_t*>(&mn[3]));
-                        uint32_t hi[4], lo[4];
+                    for (int c = 0; c < 8; ++c) sum[c] = 0.f;
+                    if (real) {
+#pragma unroll 1
+                        for (int part = 0; part < SPB; ++part) {
+                            const uint32_t sn = sn0 + part;
+                            const int s = sn % kStreamStages;
+                            KC_T(t_w0);
+                            if (sb == 0 && !dead && !mbar_wait(&sm.full[sn % kArrivals], (sn / kArrivals) & 1u, p.status)) dead = true;
+                            KC_T(t_w1);
+                            KC_ACC(1, t_w0, t_w1);
+                            // lane: 16-byte column piece (lane & 15) of rows 2k + (lane >> 4); piece c of row r of a
+                            // 64-channel half sits at position c ^ (r & 7) of the row's 128 bytes
+                            constexpr int kRowsHere = BPS > 1 ? B : kStageRows;
+                            const unsigned char* st = sm.ring[s] + sb * (kRowsHere * 128) + lane_off;
+#pragma unroll 8
+                            for (int k = 0; k < kRowsHere / 2; ++k) {
+                                const uint4 v = *reinterpret_cast<const uint4*>(st + k * 256 + piece_off[k & 3]);
+                                const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
-                        for (int c = 0; c < 8; c += 2) {
-                            const float a0 = sum[c] * (1.f / kStreamRows), a1 = sum[c + 1] * (1.f / kStreamRows);
-                            const __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
-                            hi[c >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-                            const float2 hf = bf16x2_to_float2(h2);
-                            lo[c >> 1] = pack_bf16x2(a0 - hf.x, a1 - hf.y);
+                                for (int c = 0; c < 4; ++c) {
+                                    mx[c] = __hmax2(mx[c], hh[c]);
+                                    mn[c] = __hmin2(mn[c], hh[c]);
+                                    const float2 f = bf16x2_to_float2(hh[c]);
+                                    sum[2 * c] += f.x; sum[2 * c + 1] += f.y;
+                                }
+                            }
+                            __syncwarp();
+                            if (lane == 0 && sb == BPS - 1) mbar_arrive(&sm.empty[s]);
+                            KC_T(t_w2);
+                            KC_ACC(2, t_w1, t_w2);
+#ifdef SEER_DECODE_TRACE
+                            tr[3] += 1;
+#endif
                         }
-                        phi = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                        plo = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            uint32_t xm = *reinterpret_cast<uint32_t*>(&mx[c]), xn = *reinterpret_cast<uint32_t*>(&mn[c]);
+                            uint32_t ym = __shfl_xor_sync(0xffffffffu, xm, 16), yn = __shfl_xor_sync(0xffffffffu, xn, 16);
+                            mx[c] = __hmax2(mx[c], *reinterpret_cast<__nv_bfloat162*>(&ym));
+                            mn[c] = __hmin2(mn[c], *reinterpret_cast<__nv_bfloat162*>(&yn));
+                        }
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) sum[c] += __shfl_xor_sync(0xffffffffu, sum[c], 16);
                     }
-                    unsigned char* f0 = sm.feat[fb] + (cchunk >> 3) * (kBulkBlocks * 128) + q * 128 + (((cchunk & 7) ^ (q & 7)) << 4);
-                    *reinterpret_cast<uint4*>(f0) = pmax;
-                    *reinterpret_cast<uint4*>(f0 + 2 * kBulkBlocks * 128) = pmin;
-                    *reinterpret_cast<uint4*>(f0 + 4 * kBulkBlocks * 128) = phi;
-                    *reinterpret_cast<uint4*>(f0 + 6 * kBulkBlocks * 128) = plo;
+                    if (lane < 16) {
+                        // 8 features per kind and lane: one 16-byte piece each, at its swizzled place in row q of its slab
+                        uint4 pmax = make_uint4(0u, 0u, 0u, 0u), pmin = pmax, phi = pmax, plo = pmax;
+                        if (q < r.nb) {
+                            pmax = make_uint4(*reinterpret_cast<uint32_t*>(&mx[0]), *reinterpret_cast<uint32_t*>(&mx[1]),
+                                              *reinterpret_cast<uint32_t*>(&mx[2]), *reinterpret_cast<uint32_t*>(&mx[3]));
+                            pmin = make_uint4(*reinterpret_cast<uint32_t*>(&mn[0]), *reinterpret_cast<uint32_t*>(&mn[1]),
+                                              *reinterpret_cast<uint32_t*>(&mn[2]), *reinterpret_cast<uint32_t*>(&mn[3]));
+                            uint32_t hi[4], lo[4];
+#pragma unroll
+                            for (int c = 0; c < 8; c += 2) {
+                                const float a0 = sum[c] * (1.f / B), a1 = sum[c + 1] * (1.f / B);
+                                const __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
+                                hi[c >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+                                const float2 hf = bf16x2_to_float2(h2);
+                                lo[c >> 1] = pack_bf16x2(a0 - hf.x, a1 - hf.y);
+                            }
+                            phi = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                            plo = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                        }
+                        unsigned char* f0 = sm.feat[fb] + (cchunk >> 3) * (kBulkBlocks * 128) + q * 128 + (((cchunk & 7) ^ (q & 7)) << 4);
+                        *reinterpret_cast<uint4*>(f0) = pmax;
+                        *reinterpret_cast<uint4*>(f0 + 2 * kBulkBlocks * 128) = pmin;
+                        *reinterpret_cast<uint4*>(f0 + 4 * kBulkBlocks * 128) = phi;
+                        *reinterpret_cast<uint4*>(f0 + 6 * kBulkBlocks * 128) = plo;
+                    }
                 }
             }
-            block_no += nb;
+            portion_no += n_por;
             ++n_done;
             fence_proxy_async_smem();              // the tensor cores read the features through the asynchronous proxy
             __syncwarp();
@@ -626,10 +722,8 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
         constexpr uint32_t idesc = tc_idesc_bf16(128, kBulkBlocks, false);
         int h_held = -1;
         uint32_t n_done = 0, n_heads = 0;
-        for (int item = blockIdx.x; item < n_items && !dead; item += gridDim.x) {
-            int h, i, j_first;
-            const int nb = item_blocks(item, h, i, j_first);
-            if (nb == 0) continue;
+        for (Run r = run_begin(); r.nb > 0 && !dead; run_next(r)) {
+            const int h = r.h;
             if (h != h_held) {
                 // the epilogue warps put the new head's rows in place (after the last products of the old one)
                 if (!mbar_wait(&sm.w_ready, n_heads & 1u, p.status)) { dead = true; break; }
@@ -660,32 +754,14 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
         tmem_dealloc(tbase, kKcTmemCols);
     } else if (warp < kEpiWarps) {
         // ---- epilogue: W_k into tensor memory, products out of it, rotation, store ----
-        const int r = tid;                            // row of W_k[h] and of Y, lane of tensor memory
+        const int row = tid;                          // row of W_k[h] and of Y, lane of tensor memory
         const uint32_t tbase = sm.tmem_base + ((uint32_t)(32 * warp) << 16);
-        int h_held = -1;
+        int h_held = h_first;
         uint32_t n_done = 0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            int h, i, j_first;
-            const int nb = item_blocks(item, h, i, j_first);
-            if (nb == 0) continue;
+        for (Run r = run_begin(); r.nb > 0; run_next(r)) {
+            const int h = r.h, i = r.i, nb = r.nb, j_first = r.j;
             if (h != h_held) {
-                // (every product that used the old rows is complete: this thread has read the last of them)
-                const uint4* wrow = reinterpret_cast<const uint4*>(p.w_k + ((size_t)h * p.d_gate + min(r, p.d_gate - 1)) * 3 * kHeadDim);
-#pragma unroll 1
-                for (int c0 = 0; c0 < 8; ++c0) {          // 8 x 32 columns = 512 bf16: [max | min | avg | avg again]
-                    uint32_t wr[32];
-                    const int src = (c0 < 6 ? c0 : c0 - 2) * 8;   // (16-byte pieces of the row; the mean's weights serve its correction too)
-#pragma unroll
-                    for (int x = 0; x < 8; ++x) {
-                        const uint4 v = r < p.d_gate ? __ldg(wrow + src + x) : make_uint4(0u, 0u, 0u, 0u);
-                        wr[4 * x] = v.x; wr[4 * x + 1] = v.y; wr[4 * x + 2] = v.z; wr[4 * x + 3] = v.w;
-                    }
-                    tmem_st32(tbase + 32 * c0, wr);
-                }
-                tmem_wait_st();
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm.w_ready);
+                load_w(h);                                 // (every product that used the old rows is complete: this thread has read the last of them)
                 h_held = h;
             }
             const int fb = n_done & 1;
@@ -703,7 +779,7 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.y_free[fb]);
 #pragma unroll
-            for (int q = 0; q < kBulkBlocks; ++q) sm.ybuf[q][r] = __uint_as_float(y[q]);
+            for (int q = 0; q < kBulkBlocks; ++q) sm.ybuf[q][row] = __uint_as_float(y[q]);
             epi_sync();
             const int half = p.d_gate / 2;
             const int u = i * p.num_kv_heads + h;
@@ -719,7 +795,7 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
                         float sn, cs;
-                        rope_sincos((double)j * (double)b, p.inv_freq[c0 + e + k], &sn, &cs);
+                        rope_sincos((double)j * (double)B, p.inv_freq[c0 + e + k], &sn, &cs);
                         const float a = sm.ybuf[q][c0 + e + k], bb = sm.ybuf[q][c0 + e + k + half];
                         r0[k] = a * cs - bb * sn;
                         r1[k] = bb * cs + a * sn;
@@ -749,12 +825,31 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
 
 }  // namespace
 
+// (Strides of zero -- one set of keys for several heads or sequences -- are left to the plain kernel: a tensor map need not
+// take them.)
 bool kcomp_bulk_streams(const KcompParams& p) {
-    const int U = p.batch * p.num_kv_heads;
-    const int gx = (p.num_blocks + kBulkBlocks - 1) / kBulkBlocks;
-    return p.first_block >= 0 && p.block_size == kStreamRows && p.d_gate <= kStreamDGate && !p.rows_block_local &&
-           (long long)gx * U >= 2LL * p.sm_count;
+    return p.first_block >= 0 && p.num_blocks > 0 && p.d_gate <= kStreamDGate && !p.rows_block_local && p.batch <= kMaxSeqs &&
+           p.stride_batch > 0 && p.stride_head > 0 &&
+           (long long)p.num_blocks * p.batch * p.num_kv_heads < (1ll << 30) &&
+           (long long)(p.first_block + (long long)p.num_blocks) * p.block_size < (1ll << 31);
 }
+
+namespace {
+template <int B>
+cudaError_t launch_stream(const KcompParams& p, const CUtensorMap& map_k, cudaStream_t stream) {
+    static bool configured[kMaxDevices] = {};
+    const int slot = current_device_slot();
+    if (!configured[slot]) {
+        const cudaError_t e = cudaFuncSetAttribute(kcomp_stream_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StreamSmem) + 1024);
+        if (e != cudaSuccess) return e;
+        configured[slot] = true;
+    }
+    // a CTA less per head or so keeps every run within one head
+    const int per_head = p.sm_count / p.num_kv_heads;
+    const int grid = 20 * per_head * p.num_kv_heads >= 19 * p.sm_count ? per_head * p.num_kv_heads : p.sm_count;
+    return launch_pdl(kcomp_stream_kernel<B>, dim3(grid), dim3(kStreamThreads), sizeof(StreamSmem) + 1024, stream, map_k, p);
+}
+}  // namespace
 
 cudaError_t launch_kcomp_append(const KcompParams& p, const CUtensorMap* map_k, cudaStream_t stream, int* launched) {
     const int U = p.batch * p.num_kv_heads;
@@ -769,18 +864,10 @@ cudaError_t launch_kcomp_append(const KcompParams& p, const CUtensorMap* map_k, 
         const int gx = (p.num_blocks + kBulkBlocks - 1) / kBulkBlocks;
         if (gx <= 0) return cudaSuccess;
         if (map_k && kcomp_bulk_streams(p)) {
-            static bool attr_set[64] = {};
-            int dev = 0;
-            cudaError_t e = cudaGetDevice(&dev);
-            if (e != cudaSuccess) return e;
-            if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-                e = cudaFuncSetAttribute(kcomp_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(StreamSmem) + 1024);
-                if (e != cudaSuccess) return e;
-                if (dev >= 0 && dev < 64) attr_set[dev] = true;
-            }
-            e = launch_pdl(kcomp_stream_kernel, dim3(min(p.sm_count, gx * U), 1, 1), dim3(kStreamThreads),
-                           sizeof(StreamSmem) + 1024, stream, *map_k, p);
+            const cudaError_t e = p.block_size == 128  ? launch_stream<128>(p, *map_k, stream)
+                                  : p.block_size == 64 ? launch_stream<64>(p, *map_k, stream)
+                                  : p.block_size == 32 ? launch_stream<32>(p, *map_k, stream)
+                                                       : launch_stream<16>(p, *map_k, stream);
             *launched = 1;
             return e;
         }

@@ -437,7 +437,8 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
     constexpr int BPS = B < kStageRows ? kStageRows / B : 1;       // blocks of a portion
     constexpr int kArrivals = SPB * kPoolWarps;
     extern __shared__ unsigned char smem_raw[];
-    StreamSmem& sm = *reinterpret_cast<StreamSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // (aligned by an offset, not by a cast through an integer: the compiler then still knows the accesses for shared ones)
+    StreamSmem& sm = *reinterpret_cast<StreamSmem*>(smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         for (int s = 0; s < kArrivals; ++s) mbar_init(&sm.full[s], 1);

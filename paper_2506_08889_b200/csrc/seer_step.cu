@@ -259,7 +259,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     using Smem = StepSmem<NW, MULTI>;
     constexpr int kWorkers = Z::kWorkers, kStages = Z::kStages, kArrivals = Z::kArrivals, kRows = Z::kRows;
     extern __shared__ unsigned char smem_raw[];
-    Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // (aligned by an offset, not by a cast through an integer: the compiler then still knows the accesses for shared ones)
+    Smem& sm = *reinterpret_cast<Smem*>(smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023));
     cg::cluster_group cluster = cg::this_cluster();
     const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), s_shift = 31 - __clz(S);
     const int u = blockIdx.y, i = u / p.num_kv_heads, h = u - i * p.num_kv_heads;

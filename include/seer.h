@@ -337,8 +337,8 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
  * blocks (Sec. 3.3).  The results are those of the three calls
  *     seer_kcomp_append(.., first_block = -1) ; seer_gate_select(.., scores_in = NULL) ; seer_sparse_decode
  * on `stream`, with one host round trip instead of three.  (With few tiles per list, as in
- * seer_sparse_decode, and at most 16384 compressed keys per sequence, gate and attention are one launch;
- * the append follows.  Otherwise the launches go out as gate, attention, append: the block that has just filled is the sequence's last block, which the gate takes without
+ * seer_sparse_decode, and at most 16384 compressed keys per sequence, gate, attention and append are one
+ * launch.  Otherwise the launches go out as gate, attention, append: the block that has just filled is the sequence's last block, which the gate takes without
  * scoring it, so the entry the append writes is first read in the next step.  When gate->max_blocks
  * blocks cover kv->max_seq_len, the attention kernel knows every list's length from the sequence
  * lengths and the budget; the gate kernel then marks each list as it finishes it and the attention

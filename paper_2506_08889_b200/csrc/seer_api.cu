@@ -689,9 +689,9 @@ seer_status seer_gate_select_threshold(seer_ctx* ctx, const seer_shape* shape, c
                               scores_out, stream);
 }
 
-static seer_status kcomp_append_common(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate, const int32_t* seq_lens,
-                                       const void* k_nope, int64_t stride_batch, int64_t stride_head, int64_t stride_token,
-                                       int rows_block_local, int first_block, int num_blocks, int wait_at_end, void* stream) {
+static seer_status kcomp_check(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate, const int32_t* seq_lens,
+                               const void* k_nope, int64_t stride_batch, int64_t stride_head, int64_t stride_token,
+                               int rows_block_local, int first_block, int num_blocks) {
     if (!ctx) return SEER_ERR_INVALID_ARG;
     seer_status st = check_shape(ctx, shape);
     if (st != SEER_OK) return st;
@@ -710,6 +710,15 @@ static seer_status kcomp_append_common(seer_ctx* ctx, const seer_shape* shape, c
     if (first_block >= 0 && num_blocks < 0) return fail(ctx, SEER_ERR_INVALID_ARG, "num_blocks is negative");
     if (first_block >= 0 && rows_block_local && num_blocks > 1)
         return fail(ctx, SEER_ERR_INVALID_ARG, "a block-local buffer holds one block only");
+    return SEER_OK;
+}
+
+static seer_status kcomp_append_common(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate, const int32_t* seq_lens,
+                                       const void* k_nope, int64_t stride_batch, int64_t stride_head, int64_t stride_token,
+                                       int rows_block_local, int first_block, int num_blocks, int wait_at_end, void* stream) {
+    seer_status st = kcomp_check(ctx, shape, gate, seq_lens, k_nope, stride_batch, stride_head, stride_token, rows_block_local,
+                                 first_block, num_blocks);
+    if (st != SEER_OK) return st;
     cudaError_t ce = cudaSetDevice(ctx->device);
     if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "cudaSetDevice: %s", cudaGetErrorString(ce));
 
@@ -770,6 +779,23 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
                                rows_block_local, first_block, num_blocks, 0, stream);
 }
 
+// The append of a one-launch step goes with it.  (With arguments that it does not take it stays a call of its own, which
+// says so after the step.)
+static bool append_in_step(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const seer_gate* gate, const void* k_nope,
+                           int64_t stride_batch, int64_t stride_head, int64_t stride_token, int rows_block_local, int q_len,
+                           GateParams* gp) {
+    if (!k_nope || kcomp_check(ctx, shape, gate, kv->seq_lens, k_nope, stride_batch, stride_head, stride_token, rows_block_local,
+                               -q_len, 1) != SEER_OK)
+        return false;
+    gp->k_nope = static_cast<const __nv_bfloat16*>(k_nope);
+    gp->w_k = static_cast<const __nv_bfloat16*>(gate->w_k);
+    gp->k_stride_batch = stride_batch;
+    gp->k_stride_head = stride_head;
+    gp->k_stride_token = stride_token;
+    gp->k_rows_block_local = rows_block_local;
+    return true;
+}
+
 // Short steps are one launch: every (sequence, KV head) unit has a cluster of its own.
 static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const seer_gate* gate, int q_len,
                              int token_budget, int max_sel) {
@@ -810,7 +836,10 @@ seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_
                                   nullptr, 1, &gp);
     const StepPlan plan = st == SEER_OK ? plan_of_step(ctx, shape, kv, gate, 1, token_budget, max_sel) : StepPlan{0, 1, 0};
     if (plan.S > 0) {
+        const bool appended = append_in_step(ctx, shape, kv, gate, k_nope, k_nope_stride_batch, k_nope_stride_head,
+                                             k_nope_stride_token, k_nope_rows_block_local, 1, &gp);
         st = decode_common(ctx, shape, kv, q, 1, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, plan);
+        if (appended) k_nope = nullptr;
     } else {
         if (st == SEER_OK) st = gate_launch(ctx, gp, stream);
         if (st != SEER_OK) {
@@ -843,7 +872,10 @@ seer_status seer_decode_step_multi(seer_ctx* ctx, const seer_shape* shape, const
     if (st != SEER_OK) return st;
     const StepPlan plan = plan_of_step(ctx, shape, kv, gate, q_len, token_budget, max_sel);
     if (plan.S > 0) {
+        const bool appended = append_in_step(ctx, shape, kv, gate, k_nope, k_nope_stride_batch, k_nope_stride_head,
+                                             k_nope_stride_token, k_nope_rows_block_local, q_len, &gp);
         st = decode_common(ctx, shape, kv, q, q_len, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, plan);
+        if (appended) k_nope = nullptr;
     } else {
         st = gate_launch(ctx, gp, stream);
         if (st != SEER_OK) return st;

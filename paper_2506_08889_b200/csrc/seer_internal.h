@@ -118,6 +118,11 @@ struct GateParams {
     float threshold;
     unsigned int* status;
     int* tickets;                   // [B*Hkv], zero between launches
+    // One-launch step: the block that has just filled, if any, is compressed in the same launch (see KcompParams).
+    const __nv_bfloat16* k_nope;    // null: no append
+    const __nv_bfloat16* w_k;
+    int64_t k_stride_batch, k_stride_head, k_stride_token;
+    int k_rows_block_local;
     int* list_flags;                // non-null: list_gen is stored (release) to list_flags[u] once unit u's list is written
     int list_gen;
     double inv_freq[kMaxDGate / 2]; // rope_theta^(-2c/d_gate), computed on the host in double

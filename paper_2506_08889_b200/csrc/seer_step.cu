@@ -7,6 +7,7 @@
 //   1. gate (GATE): the unit's gate query, spread over the cluster's warps, into every CTA's shared memory; the
 //      scores of the CTA's keys into the first CTA's; selection there; every listed tile's number into the
 //      shared memory of the CTA that will read it (tile t belongs to CTA t mod S);
+//      meanwhile other CTAs of the cluster compress the block that has just filled, if one has;
 //      list (!GATE): the CTA reads its tiles' numbers from the caller's list, or counts them off (dense);
 //   2. tiles: one producer warp keeps a ring of three 64-token K/V stages in flight; eight consumer warps, two
 //      groups of four, take alternate tiles, a warp 16 tokens (the same tensor-core steps as decode_kernel);
@@ -74,6 +75,7 @@ struct __align__(1024) StepSmem {
     float warp_red[NW];
     uint32_t list_key[32];
     int list_j[32];
+    float feat[3 * kHeadDim];                              // pooled features of the block that has just filled
     uint32_t pre_min, pre_max;                             // smallest and largest key of a candidate
     uint32_t prefix;
     int rem, bin_cnt, list_n, last_eq;
@@ -245,6 +247,113 @@ __device__ __forceinline__ void select_threshold(Smem& sm, const float* sc, int 
     }
     worker_sync<NW>();
     j_eq = sm.last_eq;
+}
+
+// The compressed key of block j of the unit, which has just filled, by warps 0..7 of some of the cluster's CTAs: part
+// `part` of `parts` of the rotary pairs.  The same sums in the same order as seer_kcomp.cu's append, so the same entry.
+// (256 threads meet at barrier 2.)
+__device__ __forceinline__ void append_block(const GateParams& g, float* feat, int u, int i, int h, int j, int part, int parts) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = g.block_size, half = g.d_gate / 2;
+    uint4 wv[4][2];
+    auto load_rows = [&](int pair) {                       // rows of W_k[h] of the rotary pairs `pair`, `pair` + 1
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = min(pair + (k & 1), half - 1) + (k >> 1) * half;
+            const uint4* wrow = reinterpret_cast<const uint4*>(g.w_k + ((size_t)h * g.d_gate + r) * 3 * kHeadDim);
+            wv[k][0] = __ldg(wrow + lane);
+            wv[k][1] = lane < 16 ? __ldg(wrow + 32 + lane) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    const int first = 2 * (part * 8 + warp), step = 2 * 8 * parts;
+    if (first < half) load_rows(first);
+    // warp: 16 channels; lane: eight of them, rows lane / 2, lane / 2 + 16, ...
+    const int c8 = 2 * warp + (lane & 1), rg = lane >> 1;
+    const __nv_bfloat16* src = g.k_nope + (size_t)i * g.k_stride_batch + (size_t)h * g.k_stride_head +
+                               (g.k_rows_block_local ? 0 : (size_t)j * b) * g.k_stride_token + 8 * c8;
+    __nv_bfloat162 mx[4], mn[4];
+    float sum[8];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) { mx[c] = __float2bfloat162_rn(-INFINITY); mn[c] = __float2bfloat162_rn(INFINITY); }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c] = 0.f;
+#pragma unroll 4
+    for (int r = rg; r < b; r += 16) {
+        const uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)r * g.k_stride_token);
+        const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            mx[c] = __hmax2(mx[c], hh[c]);
+            mn[c] = __hmin2(mn[c], hh[c]);
+            const float2 f = bf16x2_to_float2(hh[c]);
+            sum[2 * c] += f.x;
+            sum[2 * c + 1] += f.y;
+        }
+    }
+#pragma unroll
+    for (int off = 2; off < 32; off <<= 1) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t a = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<uint32_t*>(&mx[c]), off);
+            const uint32_t d = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<uint32_t*>(&mn[c]), off);
+            mx[c] = __hmax2(mx[c], *reinterpret_cast<const __nv_bfloat162*>(&a));
+            mn[c] = __hmin2(mn[c], *reinterpret_cast<const __nv_bfloat162*>(&d));
+        }
+    }
+    // (row groups 2w and 2w + 1 first, then those pairs one after the other)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float pair = sum[c] + __shfl_xor_sync(0xffffffffu, sum[c], 2);
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += __shfl_sync(0xffffffffu, pair, 4 * w + (lane & 1));
+        sum[c] = s / (float)b;
+    }
+    if (lane < 2) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float2 a = bf16x2_to_float2(mx[c]), d = bf16x2_to_float2(mn[c]);
+            feat[8 * c8 + 2 * c] = a.x;
+            feat[8 * c8 + 2 * c + 1] = a.y;
+            feat[kHeadDim + 8 * c8 + 2 * c] = d.x;
+            feat[kHeadDim + 8 * c8 + 2 * c + 1] = d.y;
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) feat[2 * kHeadDim + 8 * c8 + c] = sum[c];
+    }
+    asm volatile("bar.sync 2, 256;" ::: "memory");
+    __nv_bfloat16* dst = const_cast<__nv_bfloat16*>(g.kcomp) + ((size_t)u * g.max_blocks + j) * g.d_gate;
+    for (int pair = first; pair < half; pair += step) {
+        float acc[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            acc[k] = 0.f;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const int ch = lane + 32 * x;
+                const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&wv[k][x]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float2 w = bf16x2_to_float2(hh[c]);
+                    acc[k] = fmaf(w.x, ch < 48 ? feat[8 * ch + 2 * c] : 0.f, acc[k]);
+                    acc[k] = fmaf(w.y, ch < 48 ? feat[8 * ch + 2 * c + 1] : 0.f, acc[k]);
+                }
+            }
+        }
+        if (pair + step < half) load_rows(pair + step);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
+        if (lane < 2 && pair + lane < half) {
+            const int c = pair + lane;
+            const float a = lane ? acc[1] : acc[0], d = lane ? acc[3] : acc[2];
+            float sn, cs;
+            rope_sincos((double)j * (double)b, g.inv_freq[c], &sn, &cs);
+            dst[c] = __float2bfloat16(a * cs - d * sn);
+            dst[c + half] = __float2bfloat16(d * cs + a * sn);
+        }
+    }
 }
 
 // grid (S, units), cluster (S, 1, 1).  Short calls are bound by latency: 8 units x 64 blocks (16.8 MB, 2.6 us at memory
@@ -555,6 +664,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         fence_proxy_async_smem();                          // the ring's memory goes over to the copy engine
         __syncwarp();
         cluster_arrive();
+        // The other CTAs have nothing to do until the lists are out: up to four of them compress the block that has just
+        // filled.  (Nothing in this step reads its entry.)
+        if (g.k_nope && rank > 0 && rank <= 4 && warp < 8 && blockIdx.z == 0 && L >= g.block_size && L % g.block_size < q_len &&
+            L / g.block_size <= g.max_blocks)
+            append_block(g, sm.feat, u, i, h, L / g.block_size - 1, rank - 1, min(S - 1, 4));
     } else {
         pdl_wait();
         L = p.seq_lens[i];
@@ -853,6 +967,12 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             const size_t row = out_row(r);
             *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
             if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+        }
+        if constexpr (GATE) {                              // (a cluster of one CTA has nobody to leave the append to)
+            const GateParams& g = ga.g;
+            if (g.k_nope && S == 1 && warp < 8 && blockIdx.z == 0 && L >= g.block_size && L % g.block_size < q_len &&
+                L / g.block_size <= g.max_blocks)
+                append_block(g, sm.feat, u, i, h, L / g.block_size - 1, 0, 1);
         }
     }
 }

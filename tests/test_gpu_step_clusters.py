@@ -172,6 +172,44 @@ def test_step_multi(ctx, case):
     assert ctx.device_status() == binding.SEER_OK
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,T,b,dg,local", [
+    (1, 4, 1, 1, 64, 128, True),          # clusters of 16: four CTAs share the entry
+    (3, 16, 2, 1, 128, 256, False),
+    (20, 32, 8, 1, 32, 64, True),         # 160 units: one CTA each
+    (14, 32, 8, 2, 16, 128, False),       # 112 units: clusters of two
+    (2, 40, 8, 8, 64, 128, False),        # 40 rows: two clusters a unit, one of which appends
+])
+def test_step_appends_the_same_entry(ctx, B, Hq, Hkv, T, b, dg, local):
+    d, S, seed = 128, 1024, 77
+    nb = S // b
+    lens = np.array([(S, S - b + T - 1, S - 2 * b + T, 3 * b, b, b - 1, 0)[i % 7] for i in range(B)], np.int32)
+    q, qn = (synth.normal_bf16((B, T, Hq, d), seed, x, DEV) for x in ("q", "qn"))
+    _, k, v = make_qkv(B, Hq, Hkv, S, d, seed, DEV)
+    kn = synth.normal_bf16((B, Hkv, b if local else S, d), seed, "kn", DEV)
+    wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), seed, "wq", DEV, std=0.02)
+    wk = synth.normal_bf16((Hkv, dg, 3 * d), seed, "wk", DEV, std=0.02)
+    kc = synth.normal_bf16((B, Hkv, nb, dg), seed, "kc", DEV)
+    kc2 = kc.clone()
+    shape = binding.make_shape(B, Hq, Hkv, d, b, SCALE)
+    lens_t = torch.as_tensor(lens, device=DEV)
+    kv = binding.make_kv(k, v, lens_t)
+    idx = torch.zeros((B, Hkv, 4), dtype=torch.int32, device=DEV)
+    cnt = torch.zeros((B, Hkv), dtype=torch.int32, device=DEV)
+    out = torch.empty((B, T, Hq, d), dtype=torch.bfloat16, device=DEV)
+    gate = binding.make_gate(dg, THETA, wq, wk, kc, nb)
+    before = ctx.launch_count()
+    if T == 1:
+        ctx.seer_decode_step(shape, kv, gate, q, qn, kn, 4 * b, idx, cnt, 4, out, None, rows_block_local=local)
+    else:
+        ctx.seer_decode_step_multi(shape, kv, gate, q, qn, T, kn, 4 * b, idx, cnt, 4, out, None, rows_block_local=local)
+    if ctx.one_launch:
+        assert ctx.launch_count() - before == 1
+    ctx.seer_kcomp_append(shape, binding.make_gate(dg, THETA, None, wk, kc2, nb), lens_t, kn, rows_block_local=local, first_block=-T)
+    torch.cuda.synchronize()
+    assert torch.equal(kc, kc2)
+    assert ctx.device_status() == binding.SEER_OK
+
+
 @pytest.mark.parametrize("n,T,tau,max_sel", [(1500, 1, 2e-3, 400), (1500, 1, 1e-7, 40), (8000, 3, 4e-4, 900), (33, 1, 0.5, 9)])
 def test_threshold_gate(ctx, n, T, tau, max_sel):
     # the lists against the threshold rule applied to the scores that the gate gives out; a block within rounding of

@@ -409,7 +409,7 @@ def run_ours(args):
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": round(e2e_ms, 5)},
             "gpu_launches": int(launches),
             "clocks": clocks,
-            "roofline": {"bound": "hbm", "kernel": "decode_kernel<sparse>", "achieved": round(kern_gbs, 1),
+            "roofline": {"bound": "hbm", "kernel": "seer_sparse_decode (step_cluster_kernel at batch 8, decode_kernel above 128 tiles per CTA)", "achieved": round(kern_gbs, 1),
                          "peak": peak, "unit": "GB/s", "frac": round(kern_gbs / peak, 4), "peak_kind": f"of {peak_kind}",
                          "frac_of_nominal_8000": round(kern_gbs / NOMINAL_HBM_GBS, 4),
                          "algorithmic_bytes_per_launch": decode_bytes, "us_per_launch": round(sparse_ms * 1e3, 2),

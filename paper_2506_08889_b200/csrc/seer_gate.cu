@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(kGateThreads, 2) gate_cluster_kernel(const Gat
         kv[k] = pc < total ? __ldg(kc + pc) : make_uint4(0u, 0u, 0u, 0u);
     }
     GATE_STAMP(2);
-    cluster.sync();
+    cluster_sync();
     GATE_STAMP(3);
     // ---- 2. scores of this slice, into the first CTA's shared memory ---------------------------
     const int n_cand = min(max(0, L - q_len) / p.block_size, p.max_blocks);   // blocks before the query tokens' own
@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(kGateThreads, 2) gate_cluster_kernel(const Gat
         atomicMax(cluster.map_shared_rank(&sm.pre_max, 0), kmx);
     }
     GATE_STAMP(4);
-    cluster.sync();
+    cluster_sync();
     GATE_STAMP(5);
     // ---- 3. selection by the first CTA ----------------------------------------------------------
     if (slice != 0) return;

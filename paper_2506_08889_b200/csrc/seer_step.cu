@@ -503,7 +503,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         };
         constexpr int kPieces = kWorkers * kBatch;
         if (!producer) request(kPieces);                   // the second batch, into registers
-        cluster.sync();
+        cluster_sync();
         // ---- scores, into the first CTA's shared memory --------------------------------------------------------
         // A thread holds one piece of each of eight keys; reduce8 leaves every lane with the sum of one of the keys
         // (that of its piece number krev).
@@ -565,7 +565,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 atomicMax(cluster.map_shared_rank(&sm.pre_max, 0), kmx);
             }
         }
-        cluster.sync();
+        cluster_sync();
         // ---- selection, by the first CTA ----------------------------------------------------------------------------
         if (rank == 0 && !producer) {
             int32_t* dst = g.block_idx + (size_t)u * g.max_sel;
@@ -662,7 +662,6 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         if (!p.q) return;                                  // the gate alone
         fence_proxy_async_smem();                          // the ring's memory goes over to the copy engine
-        __syncwarp();
         cluster_arrive();
         // The other CTAs have nothing to do until the lists are out: up to four of them compress the block that has just
         // filled.  (Nothing in this step reads its entry.)
@@ -939,8 +938,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             if (lane < S) cluster.map_shared_rank(&sm.recv_ml[0][0], lane)[rank * kRows + r] = make_float2(M, l);
         }
     }
-    __syncwarp();
-    cluster.sync();
+    cluster_sync();
     if (!producer) {
         const int c_shift = 7 - s_shift;
         const int pairs = rows << (c_shift - 1);        // channel pairs of this CTA's slice, all rows

@@ -1,0 +1,27 @@
+"""Rules of the CUDA sources whose breach a run need not show, checked in the text."""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2506_08889_b200", "csrc")
+
+
+def _sources():
+    """File name -> its text without comments."""
+    found = {}
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        with open(path) as f:
+            found[os.path.basename(path)] = re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+    return found
+
+
+def test_aligned_cluster_barriers_bring_the_warp_together_first():
+    # barrier.cluster.*.aligned behind a branch of some lanes (a rotary pair that two lanes finish, predicated copies)
+    # is undefined unless the lanes have met again
+    wrapped = 0
+    for name, text in _sources().items():
+        assert "cluster.sync()" not in text, name
+        for m in re.finditer(r"barrier\.cluster\.", text):
+            assert re.search(r"__syncwarp\(\);\s*asm volatile\(\"$", text[:m.start()]), (name, text[m.start():m.start() + 40])
+            wrapped += 1
+    assert wrapped == 2

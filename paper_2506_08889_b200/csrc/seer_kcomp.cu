@@ -487,8 +487,10 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
     const int h_first = (int)((long long)p.num_kv_heads * blockIdx.x / gridDim.x);
     const int j_end = min(p.first_block + p.num_blocks, p.max_blocks);
     if (warp < kEpiWarps) {
-        load_w(h_first);                                   // weights are constants: before the wait
+        // (into L2 only, which follows later writes: the kernel before this one may be the one that makes W_k)
+        if (tid < p.d_gate) prefetch_l2(p.w_k + ((size_t)h_first * p.d_gate + tid) * 3 * kHeadDim, 3 * kHeadDim * 2);
         pdl_wait();
+        load_w(h_first);
         lengths_wait();
     } else {
         pdl_wait();

@@ -25,3 +25,20 @@ def test_aligned_cluster_barriers_bring_the_warp_together_first():
             assert re.search(r"__syncwarp\(\);\s*asm volatile\(\"$", text[:m.start()]), (name, text[m.start():m.start() + 40])
             wrapped += 1
     assert wrapped == 2
+
+
+def _kernel(name):
+    """The text of a kernel, from its name to the next kernel's."""
+    for text in _sources().values():
+        m = re.search(r"\n%s\(|__global__[^;{]*\b%s\(" % (name, name), text)
+        if m:
+            end = text.find("__global__", m.end())
+            return text[m.end():end if end > 0 else len(text)]
+    raise AssertionError(name)
+
+
+def test_weights_are_read_after_the_wait_for_the_kernel_before():
+    # that kernel may be the one that writes them
+    text = _kernel("kcomp_stream_kernel")
+    calls = [m.start() for m in re.finditer(r"\bload_w\(", text)]
+    assert calls and min(calls) > text.index("pdl_wait()")

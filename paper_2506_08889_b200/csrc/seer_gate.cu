@@ -520,8 +520,8 @@ __global__ void __launch_bounds__(kGateThreads, 2) gate_score_select_kernel(cons
 // ---- the whole gate of one unit in one thread-block cluster -------------------------------------
 // grid (S, B*Hkv) with cluster (S, 1, 1): the S CTAs of a cluster share one (sequence, KV head) unit.
 //   1. Every warp of the cluster takes rotary pairs of the Q branch (rows c and c + d_gate/2 of
-//      W_q[h]; the rows of its first pair are requested before the kernel waits for its
-//      predecessor, W_q being a constant), applies RoPE and stores the two results into the
+//      W_q[h]; the rows of its first pair are asked into L2 before the kernel waits for its
+//      predecessor), applies RoPE and stores the two results into the
 //      shared memory of all S CTAs (distributed shared memory).
 //   2. Each CTA scores its slice of the compressed keys (requested right after the wait, so they
 //      travel during step 1) and stores the scores into the shared memory of the cluster's first CTA.
@@ -544,18 +544,11 @@ __global__ void __launch_bounds__(kGateThreads, 2) gate_cluster_kernel(const Gat
     // CTA signals its start here and waits for the others just before step 1's remote stores.
     cluster_arrive();
     // Work items of the projection: (query token t, rotary pair c), item = t * half + c, dealt to the
-    // cluster's warps round robin.  W_q rows of this warp's first item: constants, requested before the wait.
+    // cluster's warps round robin.  W_q rows of this warp's first item: asked into L2 before the wait and no further,
+    // as the kernel before this one may be the one that makes them.
     const int n_items = q_len * half;
-    uint4 wv[2][NIT];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const uint4* wrow = reinterpret_cast<const uint4*>(p.w_q + ((size_t)h * p.d_gate + gw % half + k * half) * n);
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) {
-            const int ch = lane + 32 * it;
-            wv[k][it] = (gw < n_items && ch < chunks) ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
+    const __nv_bfloat16* w_first = p.w_q + ((size_t)h * p.d_gate + gw % half) * n;
+    if (gw < n_items && lane < 2) prefetch_l2(w_first + (size_t)lane * half * n, 2 * n);
     // The slice's compressed keys are asked into L2 meanwhile (a hint only; they are read after the
     // wait): entries of complete earlier blocks do not change any more, so in a decode step the
     // key stream overlaps the predecessor kernel.
@@ -580,10 +573,20 @@ __global__ void __launch_bounds__(kGateThreads, 2) gate_cluster_kernel(const Gat
     const int total = (j1 - j0) * lpk;
     constexpr int kBatch = 8;
     uint4* staged = reinterpret_cast<uint4*>(sc_all + ((p.max_blocks + 3) & ~3));     // [kBatch * 512] pieces
-    // The small loads the projection waits for -- the sequence length and the pre-RoPE queries of this
+    // The small loads the projection waits for -- the sequence length, W_q and the pre-RoPE queries of this
     // warp's first work item -- are requested before the keys: behind 128 KB of key requests they would
     // come back microseconds later.
     const int L = __ldg(p.seq_lens + i);
+    uint4 wv[2][NIT];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint4* wrow = reinterpret_cast<const uint4*>(w_first + (size_t)k * half * n);
+#pragma unroll
+        for (int it = 0; it < NIT; ++it) {
+            const int ch = lane + 32 * it;
+            wv[k][it] = (gw < n_items && ch < chunks) ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
     uint4 xv0[NIT];
     {
         const int t0 = gw / half;

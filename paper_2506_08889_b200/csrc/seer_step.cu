@@ -420,7 +420,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
             }
         };
-        if (!producer && t_first < q_len) load_w(c_first);     // constants, requested before the wait
+        // (W_q into L2 only, which follows later writes: the kernel before this one may be the one that makes it)
+        if (!producer && t_first < q_len && lane < 2) prefetch_l2(g.w_q + ((size_t)h * g.d_gate + c_first + lane * half) * n, 2 * n);
         if (rank == 0) {
             for (int x = tid; x < kBins; x += Z::kThreads) sm.hist[x] = 0;
             if (tid == 0) { sm.pre_min = 0xffffffffu; sm.pre_max = 0u; sm.list_n = 0; }
@@ -443,7 +444,10 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         uint4* staged = reinterpret_cast<uint4*>(sm.ring[2]);      // [kBatch * kWorkers]
         float* sc_all = reinterpret_cast<float*>(sm.ring[0]);
         if (!producer) {
-            if (t_first < q_len) load_x(t_first);
+            if (t_first < q_len) {
+                load_w(c_first);
+                load_x(t_first);
+            }
             // the first batch of keys travels during the projection (entries past n_i - 1 exist in memory: harmless)
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) {

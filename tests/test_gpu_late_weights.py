@@ -31,9 +31,11 @@ def late_copy():
     return run
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
+@pytest.fixture(scope="module", params=["1", "0"], ids=["clusters", "chain"])
+def ctx(request):
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setenv("SEER_STEP_CLUSTERS", request.param)      # read when a context is created
+        c = binding.Context(0)
     yield c
     c.close()
 
@@ -57,4 +59,44 @@ def test_build(ctx, late_copy, b, dg):
         torch.cuda.synchronize()
         got.append(kc)
     assert torch.equal(*got) and got[0].any()
+    assert ctx.device_status() == binding.SEER_OK
+
+
+@pytest.mark.parametrize("n,T,dg", [(300, 1, 128), (300, 3, 64), (4000, 1, 256), (9000, 1, 128)])
+def test_gate_and_step(ctx, late_copy, n, T, dg):
+    B, Hq, Hkv, d, b, max_sel = 2, 16, 4, 128, 16, 20
+    lens = torch.as_tensor(np.array([n * b, n * b // 2 + 5], np.int32), device=DEV)
+    q, qn = (synth.normal_bf16((B, T, Hq, d), 72, x, DEV) for x in ("q", "qn"))
+    k, v = (synth.normal_bf16((B, Hkv, n * b, d), 72, x, DEV) for x in ("k", "v"))
+    kn = synth.normal_bf16((B, Hkv, b, d), 72, "kn", DEV)
+    wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), 72, "wq", DEV, std=0.02)
+    wk = synth.normal_bf16((Hkv, dg, 3 * d), 72, "wk", DEV, std=0.02)
+    kc0 = synth.normal_bf16((B, Hkv, n, dg), 72, "kc", DEV)
+    shape = binding.make_shape(B, Hq, Hkv, d, b, 0.0884)
+    kv = binding.make_kv(k, v, lens)
+    for step in (False, True):
+        got = []
+        for late in (False, True):
+            w = torch.zeros(wq.numel() + wk.numel(), dtype=torch.bfloat16, device=DEV)
+            wq_in, wk_in = w[:wq.numel()].view(wq.shape), w[wq.numel():].view(wk.shape)
+            kc = kc0.clone()
+            gate = binding.make_gate(dg, THETA, wq_in, wk_in, kc, n)
+            idx = torch.zeros((B, Hkv, max_sel), dtype=torch.int32, device=DEV)
+            cnt = torch.zeros((B, Hkv), dtype=torch.int32, device=DEV)
+            out = torch.zeros((B, T, Hq, d), dtype=torch.bfloat16, device=DEV)
+            both = torch.cat([wq.flatten(), wk.flatten()])
+            if not late:
+                w.copy_(both)
+            torch.cuda.synchronize()
+            if late:
+                late_copy(w, both)
+            if step:
+                ctx.seer_decode_step_multi(shape, kv, gate, q, qn, T, kn, max_sel * b, idx, cnt, max_sel, out, None, rows_block_local=True)
+            else:
+                ctx.seer_gate_select_multi(shape, gate, lens, qn, None, T, max_sel * b, idx, cnt, max_sel)
+            torch.cuda.synchronize()
+            got.append((idx, cnt, out, kc))
+        for x, y in zip(*got):
+            assert torch.equal(x, y)
+        assert (got[0][3] != kc0).any() == step and got[0][0].any()
     assert ctx.device_status() == binding.SEER_OK

@@ -39,6 +39,7 @@ def _kernel(name):
 
 def test_weights_are_read_after_the_wait_for_the_kernel_before():
     # that kernel may be the one that writes them
-    text = _kernel("kcomp_stream_kernel")
-    calls = [m.start() for m in re.finditer(r"\bload_w\(", text)]
-    assert calls and min(calls) > text.index("pdl_wait()")
+    for name, load in (("kcomp_stream_kernel", r"\bload_w\("), ("step_cluster_kernel", r"\bload_w\("), ("gate_cluster_kernel", r"__ldg\(")):
+        text = _kernel(name)
+        calls = [m.start() for m in re.finditer(load, text)]
+        assert calls and min(calls) > text.index("pdl_wait()"), name

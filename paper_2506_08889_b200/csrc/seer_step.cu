@@ -30,6 +30,7 @@ constexpr int kTileBytes = 2 * kHalfTileBytes;             // one K or V tile: 1
 constexpr int kStageBytes = 2 * kTileBytes;                // K + V
 constexpr int kMaxS = 16;
 constexpr int kCodes = 256;                                // tile (or gathered block) numbers that a CTA holds
+constexpr int kListed = kStageBytes / 4;                   // scored blocks that the first CTA's list holds
 constexpr int kBins = 1024;                                // histogram of the selection
 constexpr int kMergeStride = 132;                          // floats per row of a warp's partial (bank spread)
 constexpr int kBatch = 8;                                  // 16-byte pieces of compressed keys per thread in flight
@@ -83,7 +84,7 @@ struct __align__(1024) StepSmem {
 static_assert(sizeof(StepSmem<8, true>) + 1024 <= 113 * 1024, "two CTAs per SM");
 static_assert(sizeof(StepSmem<16, true>) + 1024 <= 227 * 1024, "one CTA per SM");
 static_assert(kStepMaxBlocks * 4 <= 2 * kStageBytes && kBatch * 256 * 16 <= kStageBytes && kBatch * 512 * 16 <= 3 * kStageBytes, "the gate's use of the ring");
-static_assert(kCodes * kMaxS <= kStageBytes / 4, "the list behind the scores");
+static_assert(kCodes * kMaxS <= kListed, "the list behind the scores");
 
 template <int NW>
 __device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory"); }
@@ -464,7 +465,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         int need = 0;                                      // (threshold method: known once the scores are)
         if (n_i > 0 && !g.threshold_mode) {
             const int k = min(max(g.token_budget / g.block_size, 1), min(n_i, g.max_sel));
-            need = max(0, min(k - n_forced, n_cand));
+            // (kListed: only a sequence longer than max_seq_len, which the host's rule went by, gets that far)
+            need = max(0, min(min(k - n_forced, n_cand), kListed));
             n_blocks = need + n_forced;
         }
         // pieces that matter: up to the last run of keys with a candidate
@@ -573,7 +575,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         // ---- selection, by the first CTA ----------------------------------------------------------------------------
         if (rank == 0 && !producer) {
             int32_t* dst = g.block_idx + (size_t)u * g.max_sel;
-            int* list = reinterpret_cast<int*>(sm.ring[2]);      // the listed blocks, ascending (the host's rule bounds their number)
+            int* list = reinterpret_cast<int*>(sm.ring[2]);      // [kListed] the scored blocks of the list, ascending
             const int words = ((n_cand + 31) / 32 + NW - 1) / NW;      // 32 candidates each, per warp
             uint32_t thr;
             int j_eq;
@@ -598,7 +600,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 z = sum_all(z);
 #pragma unroll 4
                 for (int j = tid; j < n_cand; j += kWorkers) above += __expf(sc_all[j] - mx) > g.threshold * z ? 1.f : 0.f;
-                need = max(0, min(min((int)(sum_all(above) + 0.5f), g.max_sel - n_forced), n_cand));
+                need = max(0, min(min((int)(sum_all(above) + 0.5f), g.max_sel - n_forced), min(n_cand, kListed)));
                 n_blocks = n_i > 0 ? need + n_forced : 0;
             }
             select_threshold<NW>(sm, sc_all, n_cand, need, words, warp, lane, thr, j_eq);
@@ -640,16 +642,12 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 at = pos + all_low + incl_high - (in_both - in_low);
                 for (unsigned m = taken[1]; m; m &= m - 1) list[at++] = j_low + 1024 + __ffs(m) - 1;
             }
-            if (tid == 0) {
-                if (n_i > 0) {
-                    for (int x = 0; x < n_forced; ++x) list[need + x] = n_i - n_forced + x;
-                }
-                if (blockIdx.z == 0) g.block_cnt[u] = n_blocks;
-            }
+            if (tid == 0 && blockIdx.z == 0) g.block_cnt[u] = n_blocks;
             worker_sync<NW>();
-            // entry e of the list is block j: into the caller's list, and to the CTA that reads its tile(s)
+            // entry e of the list is block j (the last ones: the blocks taken without a score): into the caller's list, and
+            // to the CTA that reads its tile(s)
             for (int e = tid; e < g.max_sel; e += kWorkers) {
-                const int j = e < n_blocks ? list[e] : -1;
+                const int j = e < need ? list[e] : e < n_blocks ? n_i - n_blocks + e : -1;
                 if (blockIdx.z == 0) dst[e] = j;
                 if (e >= n_blocks || !p.q) continue;
                 if (p.blocks_per_tile == 1) {
@@ -699,6 +697,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     if (producer) {
         if (GATE) cluster_wait();                          // the tiles' numbers are in place
         pdl_launch_dependents();
+        if (GATE && n_local < n_mine && lane == 0) raise_status(p.status, DEV_BAD_INDEX);      // (a sequence longer than max_seq_len: tiles are left out)
         const int n_i = (L + p.block_size - 1) >> p.bs_shift;
         for (int base = 0; base < n_local; base += 32) {
             const int it = base + lane;

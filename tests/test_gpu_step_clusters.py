@@ -253,3 +253,33 @@ def test_bad_entries_are_skipped_and_reported(ctx):
     good = np.where((idx >= 0) & (idx < 16), idx, -1).astype(np.int32)
     check_attention(out, lse, *ref_sparse(bits(q), bits(k), bits(v), lens, good, cnt, b, SCALE), what="bad entries")
     assert ctx.device_status() == binding.SEER_ERR_BAD_INDEX
+
+
+def test_a_sequence_longer_than_said_stays_within_the_lists_memory(ctx):
+    # seq_lens above max_seq_len, by which the one-launch form was chosen: its list in shared memory holds 8192 scored
+    # blocks; it is cut there, the tiles left out are reported, and the next step is as good as any
+    if not ctx.one_launch:
+        pytest.skip("the chain keeps its lists in global memory")
+    n, b, d, dg, S = 9000, 16, 128, 128, 4096
+    q, k, v = make_qkv(1, 4, 1, S, d, 55, DEV)
+    qn = synth.normal_bf16((1, 4, d), 55, "qn", DEV)
+    wq = synth.normal_bf16((1, dg, 4 * d), 55, "wq", DEV, std=0.02)
+    kc = synth.normal_bf16((1, 1, n, dg), 55, "kc", DEV)
+    shape, gate = binding.make_shape(1, 4, 1, d, b, SCALE), binding.make_gate(dg, THETA, wq, None, kc, n)
+    out = torch.empty((1, 4, d), dtype=torch.bfloat16, device=DEV)
+    lse = torch.empty((1, 4), dtype=torch.float32, device=DEV)
+    for L in (n * b - 3, S):
+        lens_t = torch.tensor([L], dtype=torch.int32, device=DEV)
+        kv = binding.make_kv(k, v, lens_t, max_seq_len=S)
+        idx = torch.full((1, 1, n + 8), 55, dtype=torch.int32, device=DEV)
+        cnt = torch.zeros((1, 1), dtype=torch.int32, device=DEV)
+        ctx.seer_decode_step(shape, kv, gate, q, qn, None, n * b, idx, cnt, n, out, lse)
+        sc = torch.zeros((1, 1, n), dtype=torch.float32, device=DEV)
+        idx2, cnt2 = torch.zeros_like(idx[..., :n]), torch.zeros_like(cnt)
+        ctx.seer_gate_select(shape, gate, lens_t, qn, None, n * b, idx2, cnt2, n, scores_out=sc)
+        torch.cuda.synchronize()
+        want_idx, want_cnt = oracle.select(sc.cpu().numpy(), np.array([L], np.int32), b, (8192 + 1) * b, n)
+        assert np.array_equal(cnt.cpu().numpy(), want_cnt) and np.array_equal(idx.flatten()[:n].cpu().numpy(), want_idx.flatten())
+        assert (idx.flatten()[n:] == 55).all()
+        assert ctx.device_status() == (binding.SEER_OK if L == S else binding.SEER_ERR_BAD_INDEX)
+    check_attention(out, lse, *ref_sparse(bits(q), bits(k), bits(v), np.array([S], np.int32), want_idx, want_cnt, b, SCALE), what="afterwards")

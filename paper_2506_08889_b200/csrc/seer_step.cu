@@ -500,11 +500,12 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         }
         uint4 kv[kBatch];
+        // (through L2, not the read-only path: the entry that this launch appends, or the step before it did, is among them)
         auto request = [&](int cb) {
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) {
                 const int pc = cb + k * kWorkers + tid, j = block_of(pc >> lpk_shift);
-                kv[k] = pc < total && j < g.max_blocks ? __ldg(kc + ((size_t)j << lpk_shift) + csub) : make_uint4(0u, 0u, 0u, 0u);
+                kv[k] = pc < total && j < g.max_blocks ? __ldcg(kc + ((size_t)j << lpk_shift) + csub) : make_uint4(0u, 0u, 0u, 0u);
             }
         };
         constexpr int kPieces = kWorkers * kBatch;

@@ -283,3 +283,42 @@ def test_a_sequence_longer_than_said_stays_within_the_lists_memory(ctx):
         assert (idx.flatten()[n:] == 55).all()
         assert ctx.device_status() == (binding.SEER_OK if L == S else binding.SEER_ERR_BAD_INDEX)
     check_attention(out, lse, *ref_sparse(bits(q), bits(k), bits(v), np.array([S], np.int32), want_idx, want_cnt, b, SCALE), what="afterwards")
+
+
+@pytest.mark.parametrize("B,Hkv,T", [(20, 8, 1), (2, 4, 1), (20, 8, 2)])      # one CTA a unit (128 keys staged, the next 128 in registers), eight, one
+def test_steps_that_fill_a_block_each_without_a_pause(ctx, B, Hkv, T):
+    # step s fills block first + s, which step s + 1 has among its candidates; an entry that is not there yet has scores
+    # that would show in the list
+    b, d, dg, nb, first, steps, g = 16, 128, 128, 512, 150, 24, 2
+    S, Hq, max_sel = nb * b, Hkv * 2, 90
+    qs, qns = (synth.normal_bf16((2, B, T, Hq, d), 66, x, DEV) for x in ("q", "qn"))
+    k, v = (synth.normal_bf16((B, Hkv, S, d), 66, x, DEV) for x in ("k", "v"))
+    kn = synth.normal_bf16((steps, B, Hkv, b, d), 66, "kn", DEV)
+    wq = synth.normal_bf16((Hkv, dg, g * d), 66, "wq", DEV, std=0.02)
+    wk = synth.normal_bf16((Hkv, dg, 3 * d), 66, "wk", DEV, std=0.02)
+    kc = synth.normal_bf16((B, Hkv, nb, dg), 66, "kc", DEV)
+    kc[:, :, first:] *= 100
+    kc2 = kc.clone()
+    shape = binding.make_shape(B, Hq, Hkv, d, b, SCALE)
+    lens = [torch.full((B,), (first + s + 1) * b, dtype=torch.int32, device=DEV) for s in range(steps)]
+    kvs = [binding.make_kv(k, v, x) for x in lens]
+    gate, gate2 = binding.make_gate(dg, THETA, wq, wk, kc, nb), binding.make_gate(dg, THETA, wq, wk, kc2, nb)
+    idx = torch.zeros((2, steps, B, Hkv, max_sel), dtype=torch.int32, device=DEV)
+    cnt = torch.zeros((2, steps, B, Hkv), dtype=torch.int32, device=DEV)
+    out = torch.empty((B, T, Hq, d), dtype=torch.bfloat16, device=DEV)
+    torch.cuda.synchronize()
+    for s in range(steps):
+        args = (shape, kvs[s], gate, qs[s & 1], qns[s & 1])
+        more = (kn[s], max_sel * b, idx[0, s], cnt[0, s], max_sel, out)
+        if T == 1:
+            ctx.seer_decode_step(*args, *more, rows_block_local=True)
+        else:
+            ctx.seer_decode_step_multi(*args, T, *more, rows_block_local=True)
+    for s in range(steps):
+        torch.cuda.synchronize()
+        ctx.seer_kcomp_append(shape, gate2, lens[s], kn[s], rows_block_local=True, first_block=-T)
+        torch.cuda.synchronize()
+        ctx.seer_gate_select_multi(shape, gate2, lens[s], qns[s & 1], None, T, max_sel * b, idx[1, s], cnt[1, s], max_sel)
+    torch.cuda.synchronize()
+    assert torch.equal(idx[0], idx[1]) and torch.equal(cnt[0], cnt[1]) and torch.equal(kc, kc2)
+    assert ctx.device_status() == binding.SEER_OK

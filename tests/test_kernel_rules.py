@@ -43,3 +43,8 @@ def test_weights_are_read_after_the_wait_for_the_kernel_before():
         text = _kernel(name)
         calls = [m.start() for m in re.finditer(load, text)]
         assert calls and min(calls) > text.index("pdl_wait()"), name
+
+
+def test_the_one_launch_step_reads_no_compressed_key_through_the_read_only_path():
+    # it appends one in the same launch, and the next step starts under its end
+    assert not re.search(r"__ldg\(\s*kc\b", _kernel("step_cluster_kernel"))

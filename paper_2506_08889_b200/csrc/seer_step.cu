@@ -595,12 +595,13 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     return r;
                 };
                 const float mx = key_score(sm.pre_max);
+                auto weight = [&](int j) { const float s = sc_all[j]; return s == s ? __expf(s - mx) : 0.f; };     // (NaN: as minus infinity)
                 float z = 0.f, above = 0.f;
 #pragma unroll 4
-                for (int j = tid; j < n_cand; j += kWorkers) z += __expf(sc_all[j] - mx);
+                for (int j = tid; j < n_cand; j += kWorkers) z += weight(j);
                 z = sum_all(z);
 #pragma unroll 4
-                for (int j = tid; j < n_cand; j += kWorkers) above += __expf(sc_all[j] - mx) > g.threshold * z ? 1.f : 0.f;
+                for (int j = tid; j < n_cand; j += kWorkers) above += weight(j) > g.threshold * z ? 1.f : 0.f;
                 need = max(0, min(min((int)(sum_all(above) + 0.5f), g.max_sel - n_forced), min(n_cand, kListed)));
                 n_blocks = n_i > 0 ? need + n_forced : 0;
             }

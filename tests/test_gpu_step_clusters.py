@@ -238,6 +238,33 @@ def test_threshold_gate(ctx, n, T, tau, max_sel):
     assert ctx.device_status() == binding.SEER_OK
 
 
+@pytest.mark.parametrize("bad", [[float("nan")], [float("nan"), float("-inf")], []])
+def test_threshold_gate_gives_no_weight_to_a_nan(ctx, bad):
+    # a compressed key that is not a number has no probability, and takes none from the others
+    B, Hq, Hkv, d, dg, b, n, tau, max_sel = 1, 8, 2, 128, 128, 32, 700, 3e-3, 300
+    lens = np.array([n * b - 3], np.int32)
+    qn = synth.normal_bf16((B, Hq, d), 62, "qn", DEV)
+    wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), 62, "wq", DEV, std=0.03)
+    kc = synth.normal_bf16((B, Hkv, n, dg), 62, "kc", DEV)
+    for j, x in enumerate(bad):
+        kc[:, :, 10 + 7 * j::40] = x                        # (minus infinity times both signs: NaN too)
+    idx = torch.full((B, Hkv, max_sel), 55, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hkv), 55, dtype=torch.int32, device=DEV)
+    sc = torch.zeros((B, Hkv, n), dtype=torch.float32, device=DEV)
+    gate = binding.make_gate(dg, THETA, wq, None, kc, n)
+    ctx.seer_gate_select_threshold(binding.make_shape(B, Hq, Hkv, d, b, SCALE), gate, torch.as_tensor(lens, device=DEV), qn, None, tau,
+                                   idx, cnt, max_sel, scores_out=sc)
+    torch.cuda.synchronize()
+    sc = sc.cpu().numpy()
+    assert np.isnan(sc).any() == bool(bad)
+    want_idx, want_cnt, probs = oracle.select_threshold_multi(np.where(np.isnan(sc), -np.inf, sc).astype(np.float32), lens, b, tau, 1, max_sel)
+    idx, cnt = idx.cpu().numpy(), cnt.cpu().numpy()
+    for h in range(Hkv):
+        got, want = set(idx[0, h, :cnt[0, h]].tolist()), set(want_idx[0, h, :want_cnt[0, h]].tolist())
+        assert len(want) > 20 and all(abs(probs[0, h, j] - tau) <= 1e-5 * tau + 1e-9 for j in got ^ want), (h, got ^ want)
+    assert ctx.device_status() == binding.SEER_OK
+
+
 def test_bad_entries_are_skipped_and_reported(ctx):
     B, Hq, Hkv, b, S, d = 1, 8, 2, 64, 1024, 128
     q, k, v = make_qkv(B, Hq, Hkv, S, d, 17, DEV)

@@ -115,9 +115,9 @@ typedef struct {
  * (workspace_bytes, 0 = a default of 64 MiB; partial results of split
  * sequences, gate scratch, status words).  *out is NULL on failure.
  * Read from the environment at creation: SEER_DECODE_WIDE_VARIANT,
- * SEER_STEP_LIST_FLAGS (under seer_decode_step) and SEER_STEP_CLUSTERS (0:
- * single-token calls never take the one-launch form for short lists, below);
- * read at the
+ * SEER_STEP_LIST_FLAGS (under seer_decode_step) and SEER_STEP_CLUSTERS (0: no
+ * call -- gate, attention or step, of one or several query tokens -- takes the
+ * one-launch form of short calls, below); read at the
  * process's first gate call: SEER_GATE_WIDEN (0: the gate's clusters keep one
  * CTA per 512 compressed keys also when there are few sequences; n: they may be
  * widened while all of them fit the SMs at n CTAs each, default 2).  Also at
@@ -129,7 +129,12 @@ typedef struct {
  * (q_len * group) have two kernels: 16 = on the tcgen05 tensor cores with S, P,
  * O and the queries in tensor memory, 8 = mma.sync.  Unset, up to 48 rows take
  * the first and more rows the second (the faster one each, as measured).
- * Results agree within the decode tolerance. */
+ * Results agree within the decode tolerance.
+ * The one-launch form of short calls has no such choices: where one of the other
+ * five switches is set (to any value), the calls that it is about do not take it
+ * -- the work split: attention and steps; SEER_DECODE_WIDE_VARIANT (8 or 16):
+ * those of 17 to 64 rows; SEER_STEP_LIST_FLAGS: seer_decode_step;
+ * SEER_GATE_WIDEN (looked for at creation): the gate and steps. */
 seer_status seer_create(seer_ctx** out, int device, size_t workspace_bytes);
 /* Frees the workspace.  The caller must have synchronised the streams used. */
 void seer_destroy(seer_ctx* ctx);

@@ -53,6 +53,10 @@ struct seer_ctx {
     int list_gen_last;          // the last such number handed out
     int use_list_flags;         // 0: the attention kernel of a step waits for the whole gate kernel instead (SEER_STEP_LIST_FLAGS=0)
     int use_clusters;           // 0: short calls, too, go through the kernels of long ones (SEER_STEP_CLUSTERS=0)
+    // A switch that chooses among the forms of those kernels was set: the calls that it is about go through them.
+    int chain_attention;        // SEER_DECODE_POOL_DIV, SEER_DECODE_MIN_TILES: attention, steps (and wide_variant != 0: those of more than 16 rows)
+    int chain_step;             // SEER_STEP_LIST_FLAGS: steps of one query token
+    int chain_gate;             // SEER_GATE_WIDEN: the gate, steps
     int wide_variant;           // kernel variant code for more than 16 rows per unit: 16 (tcgen05), 8 (mma.sync), 0 (by size)
     int rope_d_gate;            // the rotary frequencies of the last gate width and theta seen (0: none yet)
     float rope_theta;
@@ -318,7 +322,7 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
 #ifdef SEER_DECODE_TRACE
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
-    if (!gate && ctx->use_clusters && ctx->list_gen == 0 && ctx->sel_from_lens == 0)
+    if (!gate && ctx->use_clusters && !ctx->chain_attention && !(wide && ctx->wide_variant) && ctx->list_gen == 0 && ctx->sel_from_lens == 0)
         plan = step_plan(U, q_len * group, !sparse, max_tiles / U, 0, 0);
     if (plan.S > 0) {
         p.rows = plan.rows;
@@ -366,11 +370,12 @@ seer_status seer_create(seer_ctx** out, int device, size_t workspace_bytes) {
     }
     ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
     ctx->pool_div = 4;
-    if (const char* e = getenv("SEER_DECODE_POOL_DIV")) ctx->pool_div = atoi(e);
+    if (const char* e = getenv("SEER_DECODE_POOL_DIV")) { ctx->pool_div = atoi(e); ctx->chain_attention = 1; }
     ctx->min_tiles = 4;
-    if (const char* e = getenv("SEER_DECODE_MIN_TILES")) ctx->min_tiles = atoi(e);
+    if (const char* e = getenv("SEER_DECODE_MIN_TILES")) { ctx->min_tiles = atoi(e); ctx->chain_attention = 1; }
     ctx->use_list_flags = 1;
-    if (const char* e = getenv("SEER_STEP_LIST_FLAGS")) ctx->use_list_flags = atoi(e) != 0;
+    if (const char* e = getenv("SEER_STEP_LIST_FLAGS")) { ctx->use_list_flags = atoi(e) != 0; ctx->chain_step = 1; }
+    if (getenv("SEER_GATE_WIDEN")) ctx->chain_gate = 1;
     ctx->use_clusters = 1;
     if (const char* e = getenv("SEER_STEP_CLUSTERS")) ctx->use_clusters = atoi(e) != 0;
     ctx->wide_variant = 0;      // chosen by the number of rows
@@ -627,7 +632,7 @@ static seer_status gate_prepare(seer_ctx* ctx, const seer_shape* shape, const se
 
 static seer_status gate_launch(seer_ctx* ctx, const GateParams& p, void* stream) {
     int launched = 0;
-    if (ctx->use_clusters && !p.scores_in && !p.list_flags && gate_one_kernel(p.max_blocks)) {
+    if (ctx->use_clusters && !ctx->chain_gate && !p.scores_in && !p.list_flags && gate_one_kernel(p.max_blocks)) {
         // the gate of the one-launch step by itself, while its clusters are resident all at once
         const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, false, 0, 0, p.max_blocks);
         if (plan.S > 0) {
@@ -799,14 +804,17 @@ static bool append_in_step(seer_ctx* ctx, const seer_shape* shape, const seer_kv
 // Short steps are one launch: every (sequence, KV head) unit has a cluster of its own.
 static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const seer_gate* gate, int q_len,
                              int token_budget, int max_sel) {
-    if (!ctx->use_clusters || gate->max_blocks > kStepMaxBlocks) return StepPlan{0, 1, 0};
+    const int rows = q_len * (shape->num_q_heads / shape->num_kv_heads);
+    if (!ctx->use_clusters || gate->max_blocks > kStepMaxBlocks || ctx->chain_attention || ctx->chain_gate || (q_len == 1 && ctx->chain_step) ||
+        (ctx->wide_variant && rows > 16 && shape->block_size >= kTileTokens))
+        return StepPlan{0, 1, 0};
     const long long bs = shape->block_size, cap = kv->max_seq_len > 0 ? (kv->max_seq_len + bs - 1) / bs : 1;
     long long blocks = token_budget / bs > 1 ? token_budget / bs : 1;
     if (q_len > 1 && blocks < 2) blocks = 2;               // (two blocks can hold query tokens)
     if (blocks > max_sel) blocks = max_sel;
     if (blocks > cap) blocks = cap;
     const long long tiles = (blocks * bs + kTileTokens - 1) / kTileTokens;
-    return step_plan(shape->batch * shape->num_kv_heads, q_len * (shape->num_q_heads / shape->num_kv_heads), false, tiles,
+    return step_plan(shape->batch * shape->num_kv_heads, rows, false, tiles,
                      bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles, gate->max_blocks);
 }
 

@@ -203,8 +203,9 @@ seer_status seer_dense_decode(seer_ctx* ctx, const seer_shape* shape, const seer
  * The selected blocks of all (sequence, KV head) pairs are cut into 64-token
  * tiles and dealt out evenly over the CTAs; pieces of one pair meet in a
  * log-sum-exp combine done by the last CTA to finish (no second launch).  With
- * few tiles per pair -- max_sel decides, at most 64 per CTA -- every pair has a
- * thread-block cluster of its own instead, which combines in shared memory.
+ * few tiles per pair -- max_sel decides, for dense calls max_seq_len: at most 18
+ * per CTA in clusters of one CTA up to 48 in clusters of sixteen -- every pair has
+ * a thread-block cluster of its own instead, which combines in shared memory.
  * A list with no valid entry gives out = 0, lse = -inf.
  * block_idx, block_cnt and seq_lens may be written by the kernel launched just
  * before this call on the stream: they are read only once that kernel has completed.
@@ -341,8 +342,8 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
  * and token-budget selection (Eq. 1a/1c, Sec. 3.1), block-sparse decode over the selected
  * blocks (Sec. 3.3).  The results are those of the three calls
  *     seer_kcomp_append(.., first_block = -1) ; seer_gate_select(.., scores_in = NULL) ; seer_sparse_decode
- * on `stream`, with one host round trip instead of three.  (With few tiles per list, as in
- * seer_sparse_decode, and at most 16384 compressed keys per sequence, gate, attention and append are one
+ * on `stream`, with one host round trip instead of three.  (With at most 64 tiles per CTA of the lists'
+ * clusters and at most 16384 compressed keys per sequence, gate, attention and append are one
  * launch.  Otherwise the launches go out as gate, attention, append: the block that has just filled is the sequence's last block, which the gate takes without
  * scoring it, so the entry the append writes is first read in the next step.  When gate->max_blocks
  * blocks cover kv->max_seq_len, the attention kernel knows every list's length from the sequence

@@ -323,7 +323,7 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
     if (!gate && ctx->use_clusters && !ctx->chain_attention && !(wide && ctx->wide_variant) && ctx->list_gen == 0 && ctx->sel_from_lens == 0)
-        plan = step_plan(U, q_len * group, !sparse, max_tiles / U, 0, 0);
+        plan = step_plan(U, q_len * group, max_tiles / U, 0, 0);
     if (plan.S > 0) {
         p.rows = plan.rows;
         ce = launch_step_cluster(mk_copy, *mv, p, gate, plan, static_cast<cudaStream_t>(stream));
@@ -634,7 +634,7 @@ static seer_status gate_launch(seer_ctx* ctx, const GateParams& p, void* stream)
     int launched = 0;
     if (ctx->use_clusters && !ctx->chain_gate && !p.scores_in && !p.list_flags && gate_one_kernel(p.max_blocks)) {
         // the gate of the one-launch step by itself, while its clusters are resident all at once
-        const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, false, 0, 0, p.max_blocks);
+        const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, 0, 0, p.max_blocks);
         if (plan.S > 0) {
             CUtensorMap none;
             DecodeParams d;
@@ -814,7 +814,7 @@ static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     if (blocks > max_sel) blocks = max_sel;
     if (blocks > cap) blocks = cap;
     const long long tiles = (blocks * bs + kTileTokens - 1) / kTileTokens;
-    return step_plan(shape->batch * shape->num_kv_heads, rows, false, tiles,
+    return step_plan(shape->batch * shape->num_kv_heads, rows, tiles,
                      bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles, gate->max_blocks);
 }
 

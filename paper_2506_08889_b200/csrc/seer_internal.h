@@ -58,7 +58,7 @@ struct DecodeParams {
     int blocks_per_tile;            // 64 / block_size for blocks of 16 or 32 tokens (a tile gathers several listed blocks), else 1
     int bs_shift, tpb_shift, bpt_shift;   // log2 of block_size, tiles_per_block, blocks_per_tile
     unsigned int kvh_magic;         // ceil(2^32 / num_kv_heads), 0 for one KV head: unit / num_kv_heads by __umulhi
-    int group_magic;                // ceil(2^16 / group): r / group = (r * group_magic) >> 16 for r < 16
+    int group_magic;                // ceil(2^16 / group): r / group = (r * group_magic) >> 16 for r < 64
     int q_len;                      // query tokens per sequence (the last q_len cached tokens), 1 for plain decoding
     int t_base, t_cnt;              // this launch handles query tokens t_base .. t_base + t_cnt - 1
     int rows;                       // t_cnt * group: rows on the MMA N side, <= 8 * (N-tiles of the kernel)
@@ -131,12 +131,12 @@ struct GateParams {
 constexpr int kStepMaxBlocks = 16384;   // compressed keys per unit that its gate holds in shared memory
 // How a call of `units` units of `rows` (query token, head) rows whose lists are at most max_tiles tiles long runs as one
 // launch.  With the gate: max_keys compressed keys per unit, max_codes tiles or, if these are smaller, blocks per unit;
-// else 0.
+// else 0.  (max_tiles = 0: the gate alone.)
 struct StepPlan {
     int S;                              // CTAs per cluster; 0: not a short call
     int parts, rows;                    // clusters per unit, which have `rows` of its rows each (the last one the rest)
 };
-StepPlan step_plan(int units, int rows, bool dense, long long max_tiles, long long max_codes, int max_keys);
+StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes, int max_keys);
 // g == nullptr: attention only, over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.
 cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
                                 const StepPlan& plan, cudaStream_t stream);

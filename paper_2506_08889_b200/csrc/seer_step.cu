@@ -1037,15 +1037,28 @@ int resident_clusters(bool wide, int k) {
 // something to do each.  Measured against the kernels of long calls, us a call (a step's append included):
 //     step, 8 KV heads, budget 4096, 1 / 2 / 4 sequences     23.3 -> 16.9, 25.3 -> 19.8, 31.6 -> 28.8
 //     step of batch 8 at 128k, 205 blocks (51 tiles a CTA)   98.4 -> 85.0
-//     given lists, 16 ragged sequences, blocks of 128        52.8 -> 45.8
-//     one 4 x 512-block list set (64 tiles a CTA)            93.5 -> 86.2
 //     four query tokens, 20 rows, 4 sequences, budget 4096   63.2 -> 38.6;  64 rows 92.3 -> 75.2;  8 rows, 1 sequence 27.2 -> 19.0
 //     threshold gate alone in front of given lists, 4 sequences of 48k, blocks of 32: 42.5 -> 35.0 with both
-// The line at 128 tiles a CTA (64 for dense calls): beyond it the gain is below 3 %, and a batch of very uneven lengths,
-// whose tiles the other kernel spreads over all SMs, could lose (256 dense tiles, lengths 1 : 8: 185 -> 196).  With a few
-// more CTAs than SMs the SMs that hold two of them are the last to finish (80 units, 64 tiles a CTA, 160 CTAs: 65 -> 67;
-// 32 tiles: 40.8 -> 37.5), so the line is at 32 there.
-StepPlan step_plan(int units, int rows, bool dense, long long max_tiles, long long max_codes, int max_keys) {
+// A cluster's CTAs go through their unit's tiles by themselves; the decode kernel's CTAs share all tiles.  The rule sees
+// the longest list that there can be, not how uneven the lists are, and one long sequence among short ones leaves most
+// clusters idle.  us a call, decode kernel -> clusters, 8 KV heads; one sequence's lists long / half of them / all, by the
+// tiles a CTA of a long one:
+//     lists, 24 sequences (S = 1)    16: 13.3 -> 12.2 / 20.4 -> 14.0 / 34.1 -> 21.9    32: 13.7 -> 18.8 / 35 -> 26.6 / 50 -> 37.7
+//            16 sequences (S = 2)    16: 12.8 -> 11.9 / 20.9 -> 15.3 / 32.2 -> 25.7    32: 14.5 -> 18.9 / 37.5 -> 28.4 / 53.9 -> 46.0
+//             8 sequences (S = 4)    16: 13.9 -> 12.2 / 19.8 -> 14.7 / 30.6 -> 25.6    32: 17.4 -> 19.8 / 35.9 -> 27.8 / 52.5 -> 45.0
+//             4 sequences (S = 8)    32: 21.3 -> 21.8 / 34.9 -> 27.7 / 53.8 -> 45.8    64: 38.4 -> 41.2 / 54.5 -> 48.2 / 91.4 -> 83.7
+//            16 sequences, 20 rows (S = 1)
+//                                    16: 21.6 -> 18.8 / 27.6 -> 19.3 / 25.7 -> 20.1    32: 22.4 -> 30.7 / 39.7 -> 32.1 / 56.3 -> 33.5
+//     steps, 16 sequences (S = 2)    64: 31.7 -> 46.8 / 72.3 -> 58.6 / 103 -> 93      128: 45.3 -> 82.7 / 108 -> 103 / 178 -> 173
+//             8 sequences (S = 4)    64: 35.6 -> 47.4 / 69.6 -> 56.6 / 101 -> 91      128: 57.1 -> 80.6 / 105 -> 101 / 176 -> 172
+// Given lists and dense calls, whose lengths follow the sequences', keep to where one long sequence does not lose: 16 + 2 S
+// tiles a CTA (a decode call pays for its parts whatever its size, and more the longer its longest unit is).  The lists of a
+// step are all as long as the budget but for sequences shorter than that: the line is at 64, where all but the most uneven
+// batches gain; at 128 the even ones gain 3 % and the uneven ones lose up to half.  With a few more CTAs than SMs the SMs
+// that hold two of them are the last to finish (80 units, 64 tiles a CTA, 160 CTAs: 65 -> 67; 32 tiles: 40.8 -> 37.5), so
+// the line is at 32 there.  149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles
+// a CTA 45.9 -> 33.8, 52.7 -> 39.1, 59.3 -> 43.1; 64 tiles 93.5 -> 82.1, 108 -> 96, 127 -> 109.
+StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes, int max_keys) {
     const bool wide = rows > 16;
     StepPlan plan = {0, 1, rows};
     if (rows > 64) return plan;
@@ -1060,7 +1073,7 @@ StepPlan step_plan(int units, int rows, bool dense, long long max_tiles, long lo
         if (k > 0 && S > max_tiles && 128ll * S > max_keys) continue;      // a CTA would have nothing to do
         if (units > resident_clusters(wide, k)) continue;
         const bool few_doubled = units * S > sms && 5 * units * S <= 6 * sms;
-        const long long line = (long long)S * (few_doubled ? 32 : dense ? 64 : 128);
+        const long long line = (long long)S * min(max_keys > 0 ? 64 : 16 + 2 * S, few_doubled ? 32 : 64);
         if (max_tiles <= line && max_codes <= (long long)S * kCodes) plan.S = S;
         break;
     }

@@ -24,3 +24,16 @@ def pytest_collection_modifyitems(config, items):
     for it in items:
         if "gpu" in it.keywords:
             it.add_marker(skip)
+
+
+@pytest.fixture(scope="module", params=["clusters", "chain"])
+def ctx(request):
+    """A context that takes the one-launch form of short calls, and one whose every call goes through the kernels of long
+    ones: most sizes that a test can afford are short, and both kinds of kernels serve the same entry points."""
+    from paper_2506_08889_b200 import binding
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setenv("SEER_STEP_CLUSTERS", "1" if request.param == "clusters" else "0")      # read when a context is created
+        c = binding.Context(0)
+    c.one_launch = request.param == "clusters"
+    yield c
+    c.close()

@@ -12,13 +12,6 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
-    yield c
-    c.close()
-
-
 def _run_sparse(ctx, q, k, v, lens, idx, cnt, b, scale, page_table=None, page_size=0, max_seq_len=None,
                 use_cnt=True):
     B, Hq, d = q.shape
@@ -231,8 +224,8 @@ def test_host_side_argument_checks(ctx):
 
 
 def test_result_does_not_depend_on_how_the_work_is_cut(ctx, monkeypatch):
-    # the same launch with work stealing (default) and with a purely static split, on a case large
-    # enough for stealing to happen: both within the parity bound of the oracle, and of each other
+    # the same launch with work stealing (the decode kernel's default) or by clusters, and with a purely static split, on a
+    # case large enough for stealing to happen: both within the parity bound of the oracle, and of each other
     B, Hq, Hkv, d, b, S = 4, 10, 2, 128, 64, 32768
     lens = np.array([S, S - 1000, S // 2 + 17, S - 64], np.int32)
     q, k, v = make_qkv(B, Hq, Hkv, S, d, 123, DEV)

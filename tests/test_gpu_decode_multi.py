@@ -12,22 +12,19 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.fixture(scope="module", params=["mma.sync", "tcgen05"])
+@pytest.fixture(scope="module", params=["mma.sync", "tcgen05", "clusters"])
 def ctx(request):
-    """Every test of this file runs twice: units of 17 to 64 rows take the rows-on-M kernel, which exists as an
+    """Every test of this file runs three times.  Units of 17 to 64 rows take the rows-on-M kernel, which exists as an
     mma.sync variant and as a tcgen05 variant (S, P, O and the queries in tensor memory); a context created with
-    SEER_DECODE_WIDE_VARIANT=8 or 16 takes that one at every size (unset: tcgen05 up to 48 rows).  Up to 16 rows
-    both runs take the same kernels."""
-    import os
-    old = os.environ.get("SEER_DECODE_WIDE_VARIANT")
-    os.environ["SEER_DECODE_WIDE_VARIANT"] = "16" if request.param == "tcgen05" else "8"
-    try:
-        c = binding.Context(0)
-    finally:
-        if old is None:
-            del os.environ["SEER_DECODE_WIDE_VARIANT"]
+    SEER_DECODE_WIDE_VARIANT=8 or 16 takes that one at every size (unset: tcgen05 up to 48 rows).  Up to 16 rows, both of
+    these runs take the decode kernel with the tokens on M.  The third takes the one-launch form wherever it is allowed."""
+    with pytest.MonkeyPatch.context() as mp:
+        if request.param == "clusters":
+            mp.delenv("SEER_DECODE_WIDE_VARIANT", raising=False)
         else:
-            os.environ["SEER_DECODE_WIDE_VARIANT"] = old
+            mp.setenv("SEER_DECODE_WIDE_VARIANT", "16" if request.param == "tcgen05" else "8")
+        mp.setenv("SEER_STEP_CLUSTERS", "1" if request.param == "clusters" else "0")
+        c = binding.Context(0)
     yield c
     c.close()
 

@@ -14,13 +14,6 @@ DEV = "cuda:0"
 THETA = 1.0e6
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
-    yield c
-    c.close()
-
-
 def test_largest_unit_count_ragged_short_sequences(ctx):
     # batch * num_kv_heads = 65528 of at most 65535; every unit has one to three blocks
     B, Hq, Hkv, d, b, S = 8191, 16, 8, 128, 64, 192

@@ -16,13 +16,6 @@ DEV = "cuda:0"
 THETA = 1.0e6
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
-    yield c
-    c.close()
-
-
 def _bf16_ulp_close(got_bits, want_f64):
     got = synth.bits_to_bf16(got_bits).to(torch.float64).numpy()
     bad = np.abs(got - want_f64) > kc_tolerance(want_f64)
@@ -530,8 +523,8 @@ def test_steps_back_to_back_with_and_without_the_list_marks(monkeypatch):
     """Many seer_decode_step calls in a row without a synchronisation, the queries alternating between two
     draws (so that consecutive steps select different blocks and a mark or a list left by an earlier step
     would give a wrong result), on ragged lengths: every step's lists are the oracle's selection on the
-    scores the gate computes, every output the oracle's attention over those lists -- with the per-unit
-    marks between the gate and the attention kernel (default) and with SEER_STEP_LIST_FLAGS=0."""
+    scores the gate computes, every output the oracle's attention over those lists -- as one launch, with the
+    per-unit marks between the gate and the attention kernel, and with SEER_STEP_LIST_FLAGS=0."""
     B, Hq, Hkv, d, dg, b, S = 4, 8, 2, 128, 128, 64, 8192
     nb = S // b
     lens = np.array([S, S - 5 * b - 9, 40 * b + 1, 3 * b], np.int32)
@@ -578,14 +571,13 @@ def test_steps_back_to_back_with_and_without_the_list_marks(monkeypatch):
             check_attention(outs[s], lses[s], o_w, l_w, a_w, what=f"step {s}")
         assert c.device_status() == binding.SEER_OK
 
-    with_marks = binding.Context(0)
-    try:
-        run(with_marks)
-    finally:
-        with_marks.close()
-    monkeypatch.setenv("SEER_STEP_LIST_FLAGS", "0")             # read when a context is created
-    without = binding.Context(0)
-    try:
-        run(without)
-    finally:
-        without.close()
+    # (each switch is read when a context is created; with the marks switch set, 0 or 1, steps are never one launch)
+    for switch, value in ((None, None), ("SEER_STEP_LIST_FLAGS", "1"), ("SEER_STEP_LIST_FLAGS", "0"), ("SEER_STEP_CLUSTERS", "0")):
+        with monkeypatch.context() as mp:
+            if switch:
+                mp.setenv(switch, value)
+            c = binding.Context(0)
+        try:
+            run(c)
+        finally:
+            c.close()

@@ -31,15 +31,6 @@ def late_copy():
     return run
 
 
-@pytest.fixture(scope="module", params=["1", "0"], ids=["clusters", "chain"])
-def ctx(request):
-    with pytest.MonkeyPatch.context() as mp:
-        mp.setenv("SEER_STEP_CLUSTERS", request.param)      # read when a context is created
-        c = binding.Context(0)
-    yield c
-    c.close()
-
-
 @pytest.mark.parametrize("b,dg", [(16, 128), (32, 64), (64, 128), (128, 128), (64, 256)])
 def test_build(ctx, late_copy, b, dg):
     B, Hkv, S, d = 2, 8, 2048, 128

@@ -14,13 +14,6 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
-    yield c
-    c.close()
-
-
 def _draw(case):
     r = synth.np_rng(7000 + case, "config")
     b = int(r.choice([16, 32, 64, 128]))

@@ -14,13 +14,6 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
-    yield c
-    c.close()
-
-
 @pytest.mark.parametrize("T", [1, 3])
 def test_sparse_decode_repeated_launches_agree(ctx, T):
     B, Hq, Hkv, d, b, S = 2, 40, 8, 128, 64, 32768

@@ -14,13 +14,6 @@ DEV = "cuda:0"
 THETA = 1.0e6
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
-    yield c
-    c.close()
-
-
 def _sparse(ctx, q, k, v, lens, idx, cnt, b, scale, **kw):
     B, Hq, d = q.shape
     shape = binding.make_shape(B, Hq, k.shape[1], d, b, scale)

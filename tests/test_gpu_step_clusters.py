@@ -17,16 +17,6 @@ THETA = 1.0e6
 SCALE = 0.0884
 
 
-@pytest.fixture(scope="module", params=["1", "0"], ids=["clusters", "chain"])
-def ctx(request):
-    with pytest.MonkeyPatch.context() as mp:
-        mp.setenv("SEER_STEP_CLUSTERS", request.param)      # read when a context is created
-        c = binding.Context(0)
-    c.one_launch = request.param == "1"
-    yield c
-    c.close()
-
-
 CASES = [
     # B, Hq, Hkv, b, d_gate, S, page, scores, [(budget in blocks, max_sel)]
     (1, 5, 1, 64, 128, 4096 - 13, 0, "random", [(8, 8), (1, 3), (200, 64)]),            # few units, S up to 16, 64 tiles

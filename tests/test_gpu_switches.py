@@ -1,40 +1,53 @@
-"""Which kernels a call takes under the environment's switches: by default short calls are one launch; a switch that chooses
-among the forms of the other kernels is never passed over without a word."""
+"""Which kernels a call takes: short calls are one launch of the cluster kernel up to its lines, and never where a switch of the
+environment is set that chooses among the other kernels.  The kernels' names come from the profiler's activity records; a
+process of its own takes them, all at once (this file run as a program)."""
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
 
-from paper_2506_08889_b200 import binding, synth
-from util import bits, check_attention, kernels_of, make_qkv, ref_dense
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+sys.path[:0] = [ROOT, os.path.join(ROOT, "tests")]
+
+from paper_2506_08889_b200 import binding, synth  # noqa: E402
+from util import bits, check_attention, make_qkv, ref_dense  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 SWITCHES = ("SEER_STEP_CLUSTERS", "SEER_DECODE_WIDE_VARIANT", "SEER_STEP_LIST_FLAGS", "SEER_GATE_WIDEN", "SEER_DECODE_POOL_DIV",
             "SEER_DECODE_MIN_TILES")
-ALL = {"gate", "sparse", "dense", "sparse_wide", "step", "step_multi", "step_wide"}
-
-
-@pytest.mark.parametrize("switch,value,chain", [
+CALLS = ("gate", "sparse", "dense", "sparse_rows15", "sparse_wide", "step", "step_multi", "step_wide")
+ATTENTION = set(CALLS) - {"gate"}
+SETTINGS = [                              # a switch, its value, the calls that do not take the one-launch form then
     (None, None, set()),
     ("SEER_STEP_CLUSTERS", "1", set()),
-    ("SEER_STEP_CLUSTERS", "0", ALL),
+    ("SEER_STEP_CLUSTERS", "0", set(CALLS)),
     ("SEER_DECODE_WIDE_VARIANT", "8", {"sparse_wide", "step_wide"}),
     ("SEER_DECODE_WIDE_VARIANT", "16", {"sparse_wide", "step_wide"}),
     ("SEER_STEP_LIST_FLAGS", "0", {"step"}),
     ("SEER_STEP_LIST_FLAGS", "1", {"step"}),
     ("SEER_GATE_WIDEN", "2", {"gate", "step", "step_multi", "step_wide"}),
-    ("SEER_DECODE_POOL_DIV", "0", ALL - {"gate"}),
-    ("SEER_DECODE_MIN_TILES", "4", ALL - {"gate"}),
-])
-def test_calls_take_the_kernels_that_a_switch_is_about(monkeypatch, switch, value, chain):
-    for name in SWITCHES:
-        monkeypatch.delenv(name, raising=False)
-    if switch:
-        monkeypatch.setenv(switch, value)
+    ("SEER_DECODE_POOL_DIV", "0", ATTENTION),
+    ("SEER_DECODE_MIN_TILES", "4", ATTENTION),
+]
+LINES = [                                 # a call, its sequences, the tiles of its one long list, whether clusters take it
+    # two hundred units of one CTA each: 18 tiles a CTA for lists and dense calls, 64 for a step
+    ("sparse", 25, 18, True), ("sparse", 25, 19, False), ("dense", 25, 18, True), ("dense", 25, 19, False),
+    ("step", 25, 64, True), ("step", 25, 65, False),
+    # sixty-four units of four CTAs: 24
+    ("sparse", 8, 96, True), ("sparse", 8, 97, False),
+]
+
+
+def _switch_calls(c):
     B, Hq, Hkv, d, dg, b, S, n = 2, 10, 2, 128, 128, 64, 2048, 8
     q1, k, v = make_qkv(B, Hq, Hkv, S, d, 31, DEV)
     q4 = synth.normal_bf16((B, 4, Hq, d), 31, "q4", DEV)
-    q2 = q4[:, :2].contiguous()
+    q2, q3 = q4[:, :2].contiguous(), q4[:, :3].contiguous()
     wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), 31, "wq", DEV, std=0.02)
     kc = synth.normal_bf16((B, Hkv, S // b, dg), 31, "kc", DEV)
     lens = torch.as_tensor(np.array([S, S - 100], np.int32), device=DEV)
@@ -42,42 +55,20 @@ def test_calls_take_the_kernels_that_a_switch_is_about(monkeypatch, switch, valu
     kv = binding.make_kv(k, v, lens)
     idx = torch.zeros((B, Hkv, n), dtype=torch.int32, device=DEV)
     cnt = torch.zeros((B, Hkv), dtype=torch.int32, device=DEV)
-    c = binding.Context(0)
-    try:
-        calls = {
-            "gate": lambda: c.seer_gate_select(shape, gate, lens, q1, None, n * b, idx, cnt, n),
-            "sparse": lambda: c.seer_sparse_decode(shape, kv, q1, idx, cnt, n, torch.empty_like(q1)),
-            "dense": lambda: c.seer_dense_decode(shape, kv, q1, torch.empty_like(q1)),
-            "sparse_wide": lambda: c.seer_sparse_decode_multi(shape, kv, q4, 4, idx, cnt, n, torch.empty_like(q4)),
-            "step": lambda: c.seer_decode_step(shape, kv, gate, q1, q1, None, n * b, idx, cnt, n, torch.empty_like(q1), None),
-            "step_multi": lambda: c.seer_decode_step_multi(shape, kv, gate, q2, q2, 2, None, n * b, idx, cnt, n, torch.empty_like(q2), None),
-            "step_wide": lambda: c.seer_decode_step_multi(shape, kv, gate, q4, q4, 4, None, n * b, idx, cnt, n, torch.empty_like(q4), None),
-        }
-        for name, call in calls.items():
-            call()
-            took = kernels_of(call)
-            assert took, "no kernel seen"
-            if name not in chain:
-                want = ["step_cluster_kernel"]
-            else:                                           # (the part of a step that the switch is not about may be either)
-                gate_part = "gate_cluster_kernel" if switch in ("SEER_STEP_CLUSTERS", "SEER_GATE_WIDEN") else "_cluster_kernel"
-                attention_part = "_kernel" if switch == "SEER_GATE_WIDEN" else "decode_kernel"
-                want = [gate_part] if name == "gate" else [gate_part, attention_part] if "step" in name else [attention_part]
-            assert len(took) == len(want) and all(w in t for w, t in zip(want, took)), (name, took)
-        assert c.device_status() == binding.SEER_OK
-    finally:
-        c.close()
+    return {
+        "gate": lambda: c.seer_gate_select(shape, gate, lens, q1, None, n * b, idx, cnt, n),
+        "sparse": lambda: c.seer_sparse_decode(shape, kv, q1, idx, cnt, n, torch.empty_like(q1)),
+        "dense": lambda: c.seer_dense_decode(shape, kv, q1, torch.empty_like(q1)),
+        "sparse_rows15": lambda: c.seer_sparse_decode_multi(shape, kv, q3, 3, idx, cnt, n, torch.empty_like(q3)),
+        "sparse_wide": lambda: c.seer_sparse_decode_multi(shape, kv, q4, 4, idx, cnt, n, torch.empty_like(q4)),
+        "step": lambda: c.seer_decode_step(shape, kv, gate, q1, q1, None, n * b, idx, cnt, n, torch.empty_like(q1), None),
+        "step_multi": lambda: c.seer_decode_step_multi(shape, kv, gate, q2, q2, 2, None, n * b, idx, cnt, n, torch.empty_like(q2), None),
+        "step_wide": lambda: c.seer_decode_step_multi(shape, kv, gate, q4, q4, 4, None, n * b, idx, cnt, n, torch.empty_like(q4), None),
+    }
 
 
-@pytest.mark.parametrize("kind,B,tiles,clusters", [
-    # two hundred units of one CTA each: 18 tiles a CTA for lists and dense calls, 64 for a step
-    ("sparse", 25, 18, True), ("sparse", 25, 19, False), ("dense", 25, 18, True), ("dense", 25, 19, False),
-    ("step", 25, 64, True), ("step", 25, 65, False),
-    # sixty-four units of four CTAs: 24
-    ("sparse", 8, 96, True), ("sparse", 8, 97, False),
-])
-def test_lines_between_the_one_launch_form_and_the_decode_kernel(kind, B, tiles, clusters):
-    # one long sequence among short ones, which is what the lines are there for; both sides against the oracle
+def _line_call(c, kind, B, tiles):
+    """One long sequence among short ones, every block listed: the call, and its output to be checked."""
     Hq, Hkv, d, dg, b = 16, 8, 128, 64, 64
     S = tiles * b
     lens = np.array([S - 5] + [(64, 1, 200, 0)[i % 4] for i in range(B - 1)], np.int32)
@@ -91,16 +82,83 @@ def test_lines_between_the_one_launch_form_and_the_decode_kernel(kind, B, tiles,
     cnt = torch.as_tensor(n.astype(np.int32)[:, None].repeat(Hkv, 1), device=DEV)
     out = torch.full((B, Hq, d), float("nan"), dtype=torch.bfloat16, device=DEV)
     lse = torch.full((B, Hq), float("nan"), dtype=torch.float32, device=DEV)
-    c = binding.Context(0)
-    try:
-        call = {"sparse": lambda: c.seer_sparse_decode(shape, kv, q, idx, cnt, tiles, out, lse),
-                "dense": lambda: c.seer_dense_decode(shape, kv, q, out, lse),
-                "step": lambda: c.seer_decode_step(shape, kv, gate, q, q, None, tiles * b, idx, cnt, tiles, out, lse)}[kind]
+    call = {"sparse": lambda: c.seer_sparse_decode(shape, kv, q, idx, cnt, tiles, out, lse),
+            "dense": lambda: c.seer_dense_decode(shape, kv, q, out, lse),
+            "step": lambda: c.seer_decode_step(shape, kv, gate, q, q, None, tiles * b, idx, cnt, tiles, out, lse)}[kind]
+    return call, lambda: check_attention(out, lse, *ref_dense(bits(q), bits(k), bits(v), lens, 0.1), what=kind)
+
+
+def _kernels_of(call):
+    from torch.autograd import DeviceType
+    from torch.profiler import ProfilerActivity, profile
+    call()
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
         call()
         torch.cuda.synchronize()
-        check_attention(out, lse, *ref_dense(bits(q), bits(k), bits(v), lens, 0.1), what=kind)
-        took = kernels_of(call)
-        assert "decode_kernel" not in took[-1] if clusters else "decode_kernel" in took[-1], took
+    found = sorted((e.time_range.start, e.name) for e in prof.events() if e.device_type == DeviceType.CUDA)
+    return [name for _, name in found if "seer" in name and "kernel" in name]
+
+
+def _main():
+    seen = {"switches": [], "lines": []}
+    for switch, value, _ in SETTINGS:
+        for name in SWITCHES:
+            os.environ.pop(name, None)
+        if switch:
+            os.environ[switch] = value                      # read when a context is created
+        c = binding.Context(0)
+        seen["switches"].append({name: _kernels_of(call) for name, call in _switch_calls(c).items()})
+        c.close()
+    for name in SWITCHES:
+        os.environ.pop(name, None)
+    c = binding.Context(0)
+    seen["lines"] = [_kernels_of(_line_call(c, kind, B, tiles)[0]) for kind, B, tiles, _ in LINES]
+    c.close()
+    print(json.dumps(seen))
+
+
+@pytest.fixture(scope="module")
+def seen():
+    done = subprocess.run([sys.executable, os.path.abspath(__file__)], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stderr[-2000:]
+    found = json.loads(done.stdout.strip().splitlines()[-1])
+    if not any(found["lines"]):
+        pytest.skip("no activity records here")
+    return found
+
+
+@pytest.mark.parametrize("at", range(len(SETTINGS)), ids=["%s-%s" % s[:2] for s in SETTINGS])
+def test_calls_take_the_kernels_that_a_switch_is_about(seen, at):
+    switch, value, chain = SETTINGS[at]
+    for name, took in seen["switches"][at].items():
+        if name not in chain:
+            want = ["step_cluster_kernel"]
+        else:
+            # (the part of a step that the switch is not about may be either; decode_kernel<sparse, paged, tiles of rows,
+            # small blocks, tensor memory>)
+            gate = "gate_cluster_kernel" if switch in ("SEER_STEP_CLUSTERS", "SEER_GATE_WIDEN") else "_cluster_kernel"
+            rows = "8, false, false" if value == "8" else "8, false, true" if "wide" in name else "2, false, false" if name[-2:] in ("15", "ti") else "1, false, false"
+            attention = "_kernel" if switch == "SEER_GATE_WIDEN" else "decode_kernel<%s, false, %s>" % ("false" if name == "dense" else "true", rows)
+            want = [gate] if name == "gate" else [gate, attention] if "step" in name else [attention]
+        assert len(took) == len(want) and all(w in t for w, t in zip(want, took)), (name, want, took)
+
+
+@pytest.mark.parametrize("at", range(len(LINES)), ids=["%s-%d-%d" % s[:3] for s in LINES])
+def test_lines_between_the_one_launch_form_and_the_decode_kernel(seen, at):
+    kind, B, tiles, clusters = LINES[at]
+    took = seen["lines"][at]
+    assert ("decode_kernel" in took[-1]) != clusters and (len(took) == 1) == (clusters or kind != "step"), took
+    c = binding.Context(0)
+    try:
+        call, check = _line_call(c, kind, B, tiles)
+        call()
+        torch.cuda.synchronize()
+        check()
         assert c.device_status() == binding.SEER_OK
     finally:
         c.close()
+
+
+if __name__ == "__main__":
+    _main()

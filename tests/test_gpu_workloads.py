@@ -17,13 +17,6 @@ DEV = "cuda:0"
 SEED = synth.BASE_SEED
 
 
-@pytest.fixture(scope="module")
-def ctx():
-    c = binding.Context(0)
-    yield c
-    c.close()
-
-
 def _kv(w, tag):
     shape = (w.batch, w.num_kv_heads, w.seq_len, w.head_dim)
     return (synth.normal_bf16(shape, SEED, tag + "k", DEV), synth.normal_bf16(shape, SEED, tag + "v", DEV))

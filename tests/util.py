@@ -112,15 +112,3 @@ def to_paged(k, v, page_size, seed):
     kp[table.reshape(-1).long()] = kb
     vp[table.reshape(-1).long()] = vb
     return kp, vp, table.to(torch.int32).contiguous()
-
-
-def kernels_of(call):
-    """Names of the CUDA kernels that call() launches, in order."""
-    from torch.autograd import DeviceType
-    from torch.profiler import ProfilerActivity, profile
-    torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
-        call()
-        torch.cuda.synchronize()
-    found = sorted((e.time_range.start, e.name) for e in prof.events() if e.device_type == DeviceType.CUDA)
-    return [name for _, name in found if "kernel" in name and "seer" in name]

@@ -185,6 +185,17 @@ seer_status get_map(seer_ctx* ctx, const void* base, const uint64_t dims[4], con
     return SEER_OK;
 }
 
+// A decode launch carries counters that the host advances per call (the stamp of its partial results, the
+// number its step's list marks must show): replayed from a captured graph they would repeat, and partials or
+// marks left by the previous replay would pass for this one's.  Refuse rather than compute wrong results.
+seer_status refuse_capture(seer_ctx* ctx, void* stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
+        return fail(ctx, SEER_ERR_UNSUPPORTED,
+                    "the stream is being captured: decode launches carry per-call counters and cannot be replayed from a graph");
+    return SEER_OK;
+}
+
 seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const void* q, int q_len,
                           const int32_t* block_idx, const int32_t* block_cnt, int max_sel, bool sparse,
                           void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0}) {
@@ -221,15 +232,8 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
 
     cudaError_t ce = cudaSetDevice(ctx->device);
     if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "cudaSetDevice: %s", cudaGetErrorString(ce));
-    // A decode launch carries counters that the host advances per call (the stamp of its partial results, the
-    // number its step's list marks must show): replayed from a captured graph they would repeat, and partials or
-    // marks left by the previous replay would pass for this one's.  Refuse rather than compute wrong results.
-    {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
-            return fail(ctx, SEER_ERR_UNSUPPORTED,
-                        "the stream is being captured: decode launches carry per-call counters and cannot be replayed from a graph");
-    }
+    st = refuse_capture(ctx, stream);
+    if (st != SEER_OK) return st;
     // Query tokens share a launch while (tokens x group) fits the kernel's 16 rows; more tokens
     // take further launches over the same lists (each reads the selected K/V once).
     // Up to 16 rows ride on the MMA's N side (tokens on M); more than 16 rows (with blocks of 64 or 128 tokens)
@@ -849,6 +853,7 @@ seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_
         st = decode_common(ctx, shape, kv, q, 1, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, plan);
         if (appended) k_nope = nullptr;
     } else {
+        if (st == SEER_OK) st = refuse_capture(ctx, stream);   // (before the gate, which could be captured, is enqueued)
         if (st == SEER_OK) st = gate_launch(ctx, gp, stream);
         if (st != SEER_OK) {
             ctx->list_gen = 0;
@@ -885,7 +890,8 @@ seer_status seer_decode_step_multi(seer_ctx* ctx, const seer_shape* shape, const
         st = decode_common(ctx, shape, kv, q, q_len, block_idx, block_cnt, max_sel, true, out, lse, stream, &gp, plan);
         if (appended) k_nope = nullptr;
     } else {
-        st = gate_launch(ctx, gp, stream);
+        st = refuse_capture(ctx, stream);
+        if (st == SEER_OK) st = gate_launch(ctx, gp, stream);
         if (st != SEER_OK) return st;
         st = seer_sparse_decode_multi(ctx, shape, kv, q, q_len, block_idx, block_cnt, max_sel, out, lse, stream);
     }

@@ -318,3 +318,45 @@ def test_decode_refuses_a_stream_that_is_being_captured(ctx):
     ref = ref_dense(bits(q), bits(k), bits(v), lens, 0.0884)
     check_attention(out, None, ref[0], None, ref[2], what="after the capture")
     assert ctx.device_status() == binding.SEER_OK
+
+
+@pytest.mark.parametrize("q_len", [1, 2])
+def test_step_on_a_stream_that_is_being_captured_enqueues_nothing(ctx, q_len):
+    # not its gate either, which by itself could be captured
+    B, Hq, Hkv, d, b, S, n = 1, 4, 1, 128, 64, 1024, 4
+    q, k, v = make_qkv(B, q_len * Hq, Hkv, S, d, 6, DEV)
+    wq = synth.normal_bf16((Hkv, d, Hq * d), 6, "wq", DEV, std=0.02)
+    kc = synth.normal_bf16((B, Hkv, S // b, d), 6, "kc", DEV)
+    lens_t = torch.as_tensor(np.array([S - 1], np.int32), device=DEV)
+    shape, gate = binding.make_shape(B, Hq, Hkv, d, b, 0.0884), binding.make_gate(d, 1.0e6, wq, None, kc, S // b)
+    kv = binding.make_kv(k, v, lens_t)
+    idx = torch.full((B, Hkv, n), -7, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hkv), -7, dtype=torch.int32, device=DEV)
+    out, fill = torch.zeros_like(q), torch.zeros(8, device=DEV)
+
+    def step(**kw):
+        if q_len == 1:
+            ctx.seer_decode_step(shape, kv, gate, q, q, None, n * b, idx, cnt, n, out, **kw)
+        else:
+            ctx.seer_decode_step_multi(shape, kv, gate, q, q, q_len, None, n * b, idx, cnt, n, out, **kw)
+
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    before = ctx.launch_count()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        graph.capture_begin()
+        try:
+            fill.add_(1.0)
+            with pytest.raises(binding.SeerError) as e:
+                step(stream=side)
+            assert e.value.status == binding.SEER_ERR_UNSUPPORTED
+        finally:
+            graph.capture_end()
+    assert ctx.launch_count() == before
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (idx == -7).all() and (cnt == -7).all()
+    step()
+    torch.cuda.synchronize()
+    assert (cnt == n).all() and ctx.device_status() == binding.SEER_OK

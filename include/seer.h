@@ -226,10 +226,12 @@ seer_status seer_sparse_decode(seer_ctx* ctx, const seer_shape* shape, const see
  * as it serves all heads of the group.  q_len = 1 is seer_sparse_decode / seer_dense_decode.
  *  q   [B,q_len,Hq,d] bf16 contiguous;  out [B,q_len,Hq,d] bf16;  lse [B,q_len,Hq] fp32 or NULL.
  * A query that sees no listed token (also every query at a negative position, when
- * L_i < q_len) gets out = 0, lse = -inf.  All tokens share one launch -- and the selected K/V
- * are read once for all of them -- while q_len * (Hq/Hkv) <= 64 (with blocks of 16 or 32 tokens:
- * <= 16); beyond that the call issues one launch per 64 (16) rows on the stream.  Other
- * arguments, errors and the treatment of the lists as in the single-token calls.
+ * L_i < q_len) gets out = 0, lse = -inf.  q_len * (Hq/Hkv) is at most 64, and all tokens share
+ * one launch, which reads the selected K/V once for all of them -- except where lists of blocks of
+ * 16 or 32 tokens are too long for the one-launch form of short calls: there a launch takes the
+ * tokens that make up to 16 rows, and the call issues as many as it needs on the stream.  (The
+ * one-launch form gives more than 32 rows two clusters, the second of which reads K/V again.)
+ * Other arguments, errors and the treatment of the lists as in the single-token calls.
  */
 seer_status seer_sparse_decode_multi(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv,
                                      const void* q, int q_len, const int32_t* block_idx,
@@ -344,8 +346,9 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
  *     seer_kcomp_append(.., first_block = -1) ; seer_gate_select(.., scores_in = NULL) ; seer_sparse_decode
  * on `stream`, with one host round trip instead of three.  (With at most 64 tiles per CTA of the lists'
  * clusters and at most 16384 compressed keys per sequence, gate, attention and append are one
- * launch.  Otherwise the launches go out as gate, attention, append: the block that has just filled is the sequence's last block, which the gate takes without
- * scoring it, so the entry the append writes is first read in the next step.  When gate->max_blocks
+ * launch.  Otherwise the launches go out as gate, attention, append: the block that has just filled is
+ * the sequence's last block, which the gate takes without scoring it, so the entry the append writes is
+ * first read in the next step.  When gate->max_blocks
  * blocks cover kv->max_seq_len, the attention kernel knows every list's length from the sequence
  * lengths and the budget; the gate kernel then marks each list as it finishes it and the attention
  * kernel starts on a sequence's blocks as soon as that list is marked, with a bounded wait that ends
@@ -383,8 +386,9 @@ seer_status seer_decode_step_multi(seer_ctx* ctx, const seer_shape* shape, const
  * of HBM to its own pool at start-up and forbids cudaMalloc afterwards (a late allocation can
  * fail, or stall the GPU, under its memory plan), or code that runs inside a region where the
  * CUDA allocator must not be entered.  seer_create allocates a workspace, so those callers
- * cannot have a context.  This call computes exactly what seer_gate_select computes from
- * q_nope (same kernels, same results) but keeps the scratch it needs -- per-unit tickets, the gate
+ * cannot have a context.  This call computes what seer_gate_select computes from q_nope (the
+ * same sums in the same order, by the kernels that seer_gate_select takes where the one-launch form of
+ * short calls does not do) but keeps the scratch it needs -- per-unit tickets, the gate
  * query, and the block scores unless scores_out is given -- in an array of
  * SEER_STATIC_SCRATCH_BYTES that is part of the library image.  Every GPU on which the library
  * is used holds one copy of that array from first use until the process exits.

@@ -229,11 +229,15 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 // Programmatic dependent launch.  Every kernel of the library is launched with the stream-
-// serialisation attribute: it may start while its predecessor in the stream is still running,
-// and touches nothing in global memory before pdl_wait(), which returns once every earlier
-// kernel has completed.  pdl_launch_dependents() lets the next kernel start its own set-up; a
-// kernel calls it only after its own pdl_wait(), so a dependent never overlaps a kernel two
-// places back.  Launched without the attribute both calls do nothing.
+// serialisation attribute: it may start while its predecessor in the stream is still running.
+// Before pdl_wait(), which returns once every earlier kernel has completed, it asks for L2
+// prefetches at most.  pdl_launch_dependents() lets the next kernel start its own set-up; a kernel
+// calls it only after its own pdl_wait(), so a dependent never overlaps a kernel two places back,
+// and what was final before the predecessor was launched is so for it, too.  On that rests what
+// the kernels inside one call do before their wait: the two-kernel gate's scores request the
+// first keys, a chained step's attention reads the lengths and makes its schedule, and its append
+// (kcomp_kernel, wait_at_end) does all its work and calls the two the other way round.
+// Launched without the attribute both calls do nothing.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 

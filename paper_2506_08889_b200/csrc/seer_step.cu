@@ -357,10 +357,12 @@ __device__ __forceinline__ void append_block(const GateParams& g, float* feat, i
     }
 }
 
-// grid (S, units), cluster (S, 1, 1).  Short calls are bound by latency: 8 units x 64 blocks (16.8 MB, 2.6 us at memory
-// speed) take 13 us from the first read to the last write, of which the gate query 1.5, the scores 1.0, the selection
-// and the lists 3.3, the tiles 2.5, the combine 2.2 and four cluster barriers 0.5 to 1.0 each.  Longer ones by memory: 64
-// units x 205 blocks (430 MB) 70 us, 6.2 TB/s; CTAs that share a unit read neighbouring blocks at the same time.
+// grid (S, units), cluster (S, 1, 1).  Short calls are bound by latency: a step of 8 units x 64 blocks (16.8 MB, 2.6 us at
+// memory speed) takes 14.5 us.  Time stamps in the kernel (which make it a microsecond or two longer; medians over the CTAs,
+// from the first read on) put 1.9 us on the gate query, 1.0 on the barrier behind it, 3.7 on the scores, 0.6 on the barrier,
+// 1.5 on the selection, 2.1 on the lists and their barrier, 2.6 on the tiles, 1.0 on the warps' combine, 1.0 on the barrier,
+// 0.9 on the output.  Longer ones by memory: of a step of 64 units x 205 blocks (430 MB; 83.5 us) the tiles take 66 us,
+// 6.5 TB/s, from the first CTA's first to the last one's last; CTAs that share a unit read neighbouring blocks at the same time.
 template <int NW, bool GATE, bool MULTI>
 __global__ void __launch_bounds__(Size<NW, MULTI>::kThreads, NW == 8 ? 2 : 1)
 step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,

@@ -198,7 +198,7 @@ seer_status refuse_capture(seer_ctx* ctx, void* stream) {
 
 seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const void* q, int q_len,
                           const int32_t* block_idx, const int32_t* block_cnt, int max_sel, bool sparse,
-                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0}) {
+                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0, false}) {
     // (gate: the whole step in one launch, by `plan`)
     if (!ctx) return SEER_ERR_INVALID_ARG;
     seer_status st = check_shape(ctx, shape);
@@ -636,25 +636,11 @@ static seer_status gate_prepare(seer_ctx* ctx, const seer_shape* shape, const se
 
 static seer_status gate_launch(seer_ctx* ctx, const GateParams& p, void* stream) {
     int launched = 0;
-    if (ctx->use_clusters && !ctx->chain_gate && !p.scores_in && !p.list_flags && gate_one_kernel(p.max_blocks)) {
-        // the gate of the one-launch step by itself, while its clusters are resident all at once
-        const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, 0, 0, p.max_blocks);
-        if (plan.S > 0) {
-            CUtensorMap none;
-            DecodeParams d;
-            memset(&none, 0, sizeof none);
-            memset(&d, 0, sizeof d);
-            d.seq_lens = p.seq_lens;
-            d.num_kv_heads = p.num_kv_heads;
-            d.num_units = p.batch * p.num_kv_heads;
-            d.group = p.group;
-            d.q_len = p.q_len;
-            d.rows = plan.rows;
-            const cudaError_t ce = launch_step_cluster(none, none, d, &p, plan, static_cast<cudaStream_t>(stream));
-            if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "gate launch: %s", cudaGetErrorString(ce));
-            ctx->launches += 1;
-            return SEER_OK;
-        }
+    cudaError_t cluster_err = cudaSuccess;
+    if (ctx->use_clusters && !ctx->chain_gate && launch_gate_cluster(p, static_cast<cudaStream_t>(stream), &cluster_err)) {
+        if (cluster_err != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "gate launch: %s", cudaGetErrorString(cluster_err));
+        ctx->launches += 1;
+        return SEER_OK;
     }
     const cudaError_t ce = launch_gate_select(p, static_cast<cudaStream_t>(stream), &launched);
     ctx->launches += launched;

@@ -135,11 +135,15 @@ constexpr int kStepMaxBlocks = 16384;   // compressed keys per unit that its gat
 struct StepPlan {
     int S;                              // CTAs per cluster; 0: not a short call
     int parts, rows;                    // clusters per unit, which have `rows` of its rows each (the last one the rest)
+    bool wide;                          // 16 worker warps per CTA, one CTA per SM (else 8 and two)
 };
 StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes, int max_keys);
 // g == nullptr: attention only, over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.
 cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
                                 const StepPlan& plan, cudaStream_t stream);
+// The gate by itself as one launch of such clusters (at most 8192 compressed keys per unit), while they are resident all at
+// once; false: not that size, and nothing has been launched.
+bool launch_gate_cluster(const GateParams& p, cudaStream_t stream, cudaError_t* err);
 // Launches the scoring kernels (unless scores_in is given) and the selection kernel.
 // Returns the number of kernels launched through *launched.
 cudaError_t launch_gate_select(const GateParams& p, cudaStream_t stream, int* launched);

@@ -5,16 +5,23 @@
 // a fence and a ticket and read back by the last CTA.  Here the S CTAs (S = 1 .. 16) of a unit's cluster share
 // the unit from its first byte to its output:
 //   1. gate (GATE): the unit's gate query, spread over the cluster's warps, into every CTA's shared memory; the
-//      scores of the CTA's keys into the first CTA's; selection there; every listed tile's number into the
-//      shared memory of the CTA that will read it (tile t belongs to CTA t mod S);
-//      meanwhile other CTAs of the cluster compress the block that has just filled, if one has;
+//      scores of each CTA's keys into every CTA's; every CTA selects for itself, and keeps the listed tiles that it
+//      reads (tile t belongs to CTA t mod S); meanwhile the producer warps compress the block that has just filled,
+//      if one has;
 //      list (!GATE): the CTA reads its tiles' numbers from the caller's list, or counts them off (dense);
 //   2. tiles: one producer warp keeps a ring of three 64-token K/V stages in flight; eight consumer warps, two
 //      groups of four, take alternate tiles, a warp 16 tokens (the same tensor-core steps as decode_kernel);
 //   3. combine: the warps' partials meet in shared memory, the CTA's go, a slice of the channels each, to the
-//      cluster's CTAs, which write their slice of the output after one cluster barrier.
-// Nothing between the steps leaves the SMs, and no CTA waits for another except at the cluster's hardware barrier.
+//      cluster's CTAs, which write their slice of the output.
+// Nothing between the steps leaves the SMs.  What one CTA stores into another's shared memory (queries, scores, partials)
+// carries its own completion: the store counts its bytes down on an mbarrier of the receiver, which knows how many there
+// will be.  A CTA thus waits for what it reads and for nothing else.  The cluster's hardware barrier, whose release first
+// waits for all of a thread's stores to be acknowledged, is used twice: before the first of these stores, and at the end,
+// so that no CTA leaves while one is under way.
 #include <cooperative_groups.h>
+
+#include <cstring>
+#include <type_traits>
 
 #include "seer_gate_device.cuh"
 #include "seer_internal.h"
@@ -30,11 +37,11 @@ constexpr int kTileBytes = 2 * kHalfTileBytes;             // one K or V tile: 1
 constexpr int kStageBytes = 2 * kTileBytes;                // K + V
 constexpr int kMaxS = 16;
 constexpr int kCodes = 256;                                // tile (or gathered block) numbers that a CTA holds
-constexpr int kListed = kStageBytes / 4;                   // scored blocks that the first CTA's list holds
+constexpr int kListed = 8192;                              // most scored blocks of a list
 constexpr int kBins = 1024;                                // histogram of the selection
+constexpr int kFew = 1024;                                 // candidates (and key tiles) that its short list holds
 constexpr int kMergeStride = 132;                          // floats per row of a warp's partial (bank spread)
-constexpr int kBatch = 8;                                  // 16-byte pieces of compressed keys per thread in flight
-constexpr int kChunkKeys = 32;                             // keys are dealt to the cluster's CTAs in runs of 32
+constexpr int kKeyTile = 16;                               // keys are dealt to the cluster's warps in tiles of 16
 constexpr int kMaxQLen = 8;
 
 // Two sizes.  NW = 8 worker warps (gate, consumers, combine) and a ring of three stages: two CTAs per SM, up to 16
@@ -50,113 +57,183 @@ struct Size {
 template <int NW, bool MULTI>
 struct __align__(1024) StepSmem {
     using Z = Size<NW, MULTI>;
-    // K/V ring.  Before the first tile is asked for, the gate's: the scores of the unit (first CTA; up to
-    // kStepMaxBlocks) in stages 0 and 1, the staged first batch of keys behind them, the list of the taken blocks in
-    // its place later.  After the last tile: the warps' partials.
+    // K/V ring.  Before the first tile is asked for, the gate's: the scores of the unit (up to kStepMaxBlocks) in stages 0
+    // and 1, GateScratch behind them.  After the last tile: the warps' partials.
     unsigned char ring[Z::kStages][kStageBytes];
-    // What the gate uses until the lists are out, and what arrives from the cluster's CTAs after their last tile.
-    union {
-        float qg[MULTI ? kMaxQLen : 1][kMaxDGate];         // gate queries
-        __align__(16) float recv_o[Z::kRows * kHeadDim];   // [source CTA][row][this CTA's slice of the channels]
-    };
-    union {
-        __align__(16) int hist[kBins + 4];                 // selection (first CTA); the one past the last is for nobody
-        float2 recv_ml[kMaxS][Z::kRows];                   // [source CTA][row]: max, sum
-    };
+    // what the cluster's CTAs send after their last tile (a fast one while this one still selects: memory of its own)
+    __align__(16) float recv_o[Z::kRows * kHeadDim];       // [source CTA][row][this CTA's slice of the channels]
+    float2 recv_ml[kMaxS][Z::kRows];                       // [source CTA][row]: max, sum
     float2 warp_ml[NW][8];
     // Tile n arrives in stage n % kStages and is announced on full[n % kArrivals].  The consumer groups that share a
     // tile's rows take all of one residue of the tile numbers, at their own pace, and every barrier belongs to one
     // residue, so its groups follow all of its phases.  (With a barrier per stage a group would miss the others' phases
     // and could take one that is two back for the one that it waits for.)
     uint64_t full[Z::kArrivals], empty[Z::kStages];
+    uint64_t got_query, got_scores, got_feat, got_parts;   // bytes from the cluster's CTAs
     int meta[Z::kArrivals];                                // tokens from the tile's first row on (blocks of 16 or 32 tokens: per block, 8 bits each)
     int codes[kCodes];                                     // GATE: this CTA's tiles: 64-token tile numbers, or the gathered blocks
-    // selection (first CTA)
+    // selection
     int warp_tot[NW];
     float warp_red[NW];
+    uint32_t warp_min[NW], warp_max[NW];                   // ... and of a warp's candidates
     uint32_t list_key[32];
     int list_j[32];
-    float feat[3 * kHeadDim];                              // pooled features of the block that has just filled
+    __align__(16) float feat[3 * kHeadDim];                // pooled features of the block that has just filled
+    __align__(16) float feat_own[3][16];                   // those of 16 channels, on their way to the cluster's CTAs
     uint32_t pre_min, pre_max;                             // smallest and largest key of a candidate
     uint32_t prefix;
-    int rem, bin_cnt, list_n, last_eq;
+    int rem, bin_cnt, list_n, tile_n, few_n, last_eq, no_list;
 };
 static_assert(sizeof(StepSmem<8, true>) + 1024 <= 113 * 1024, "two CTAs per SM");
 static_assert(sizeof(StepSmem<16, true>) + 1024 <= 227 * 1024, "one CTA per SM");
-static_assert(kStepMaxBlocks * 4 <= 2 * kStageBytes && kBatch * 256 * 16 <= kStageBytes && kBatch * 512 * 16 <= 3 * kStageBytes, "the gate's use of the ring");
-static_assert(kCodes * kMaxS <= kListed, "the list behind the scores");
+// The gate's part of the ring (stage 2).
+struct GateScratch {
+    // Gate queries, from all CTAs: each channel in three bf16 parts (high, middle, low), which together are the fp32 number
+    // exactly, two channels a word.  (Rows 64 bytes longer than the channels: neighbouring parts are in different banks.)
+    __align__(16) uint32_t parts[kMaxQLen][3][kMaxDGate / 2 + 16];
+    float sums[16][16][8];                                 // partial sums of the gate query: [warp][row][token]
+    __align__(16) int hist[kBins];                         // selection
+};
+// ... and of the selection, when the queries have been used.
+struct ShortList {
+    unsigned taken[kStepMaxBlocks / 32];                   // a bit per candidate
+    float tile_max[kStepMaxBlocks / kKeyTile];             // largest score of a key tile
+    int tile[kFew];                                        // the tiles that may have a taken one
+    float score[kFew];                                     // their candidates that may be taken
+    int j[kFew];
+};
+static_assert(sizeof(ShortList) <= offsetof(GateScratch, hist) && kStepMaxBlocks / kKeyTile <= kFew, "the short list's place");
+static_assert(kStepMaxBlocks <= 64 * 256, "a bit per candidate of a lane");
+static_assert(kStepMaxBlocks * 4 <= 2 * kStageBytes && sizeof(GateScratch) <= kStageBytes, "the gate's use of the ring");
 
+// Barriers among the worker warps, and between them and the producer.  The aligned forms are for a warp whose lanes are
+// together; behind a loop or branch of some lanes they need not be, so they are brought together here.
 template <int NW>
-__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory"); }
+__device__ __forceinline__ void worker_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory");
+}
+template <int NW>
+__device__ __forceinline__ void tiles_listed_arrive() {
+    __syncwarp();
+    asm volatile("bar.arrive 3, %0;" ::"n"(32 * NW + 32) : "memory");
+}
+template <int NW>
+__device__ __forceinline__ void tiles_listed_wait() {
+    __syncwarp();
+    asm volatile("bar.sync 3, %0;" ::"n"(32 * NW + 32) : "memory");
+}
+
+// ... and whether one of the worker threads says so
+template <int NW>
+__device__ __forceinline__ bool worker_any(bool x) {
+    uint32_t any;
+    __syncwarp();
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(any)
+        : "r"((uint32_t)x), "n"(32 * NW)
+        : "memory");
+    return any != 0;
+}
 
 template <bool GATE>
 struct GateArg { GateParams g; };
 template <>
 struct GateArg<false> {};
 
-// The selection of the token budget's `need` best of the candidates [0, n_cand), by the first CTA's worker warps.
-// Leaves (thr, j_eq): candidate j is taken if its key is above thr, or equal to it and j <= j_eq.  Comparisons only:
-// the lower block number wins a tie, NaN is below every number.  A histogram over a monotone linear map of
-// [min, max] leaves a few candidates in the boundary bin, which every warp ranks for itself; crowded bins and ranges
-// that are not finite take radix passes over key - min instead.
-template <int NW, typename Smem>
-__device__ __forceinline__ void select_threshold(Smem& sm, const float* sc, int n_cand, int need, int words, int warp, int lane,
-                                                 uint32_t& thr, int& j_eq) {
+// ---- stores into a CTA of the cluster (addr, bar: of its shared memory, cluster_addr), counted on its mbarrier ----------
+__device__ __forceinline__ uint32_t cluster_addr(const void* mine, int rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void send_u32(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send_f32x2(uint32_t addr, float2 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_f32x4(uint32_t addr, float4 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_min(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.min.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_max(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.max.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
+                 : "memory");
+}
+// Bounded wait for what the cluster's CTAs have sent (the first and only phase of `bar`).
+__device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status) {
+    uint32_t ok = 0;
+    for (uint32_t it = 0; it < (1u << 24) && !ok; ++it) {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar))
+            : "memory");
+        if (!ok && it > 64) __nanosleep(64);
+    }
+    if (!ok) raise_status(status, DEV_TIMEOUT);
+    __syncwarp();                                          // (the lanes need not have left the loop together)
+    return ok != 0;
+}
+
+// The selection of the `need` best of the candidates [0, n_cand), by a CTA's worker warps: take(e, j) for the e-th of them in
+// block order.  Comparisons only: the lower block number wins a tie, NaN is below every number.  A histogram over a
+// monotone linear map of [min, max] leaves a few candidates in the boundary bin, which every warp ranks for itself;
+// crowded bins and ranges that are not finite take radix passes over key - min instead.  With many candidates for few
+// places a short list comes first: the need-th largest of the key tiles' maxima is a bound that at least `need`
+// candidates reach, and few others do.
+// What bounds it: this code runs once per call, by two warps a scheduler, so that its time is the number of instructions
+// on its longest path (some ten cycles each, mostly their fetch) and not the candidates; hence rolled loops, whose
+// bodies stay in the instruction buffers, and one candidate a lane and turn.
+template <int NW, typename Smem, typename Take>
+__device__ __forceinline__ void select_blocks(Smem& sm, GateScratch& gs, const float* sc, int n_cand, int need, int warp, int lane, Take&& take) {
+    constexpr int kThreads = 32 * NW, kPer = kBins / kThreads;
     const int tid = 32 * warp + lane;
-    if (need >= n_cand) { thr = 0u; j_eq = 0x7fffffff; return; }
-    if (need <= 0) { thr = 0xffffffffu; j_eq = -1; return; }
-    const uint32_t kmin = sm.pre_min, kmax = sm.pre_max;
-    const float smin = key_score(kmin), smax = key_score(kmax);
-    const float range = smax - smin, scale = (kBins - 1.f) / range;
-    const int j0 = warp * words * 32 + lane;               // this lane's candidates: j0, j0 + 32, ...
-    // (four at a time, without branches: their loads go out together)
-    auto each = [&](auto&& fn) {
-#pragma unroll 1
-        for (int e = 0; e < words; e += 4) {
-            float v[4];
+    int* hist = gs.hist;
+    if (need <= 0) return;
+    // candidate j is taken if its key is above thr, or equal to it and j <= j_eq
+    uint32_t thr = 0u;
+    int j_eq = 0x7fffffff;
+    // the warps' totals before this one's
+    auto before = [&]() -> int { return __reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_tot[lane] : 0); };
+    auto scan = [&](int v) -> int {                        // inclusive, over the warp
 #pragma unroll
-            for (int x = 0; x < 4; ++x) v[x] = sc[min(j0 + 32 * (e + x), n_cand - 1)];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) fn((e + x < words) & (j0 + 32 * (e + x) < n_cand), score_key(v[x]), j0 + 32 * (e + x));
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += t;
         }
+        return v;
     };
-    // The same for passes in any order, on the scores themselves: neighbouring blocks have similar scores, so the lanes of
-    // a warp take candidates that are far apart (lane l has run l of `run` blocks, from its own place in it on: no bank
-    // conflicts); side by side, their additions to the histogram would queue for a few bins.
-    const int run = (n_cand + 31) / 32, rot = (run & 1) ? 0 : lane % run;
-    auto each_spread = [&](auto&& fn) {
-#pragma unroll 1
-        for (int q = warp; q < run; q += 4 * NW) {
-            float v[4];
-            int jj[4];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                int at = q + x * NW + rot;
-                at -= at >= run ? run : 0;
-                jj[x] = q + x * NW < run ? min(lane * run + at, n_cand) : n_cand;      // (n_cand: none)
-                v[x] = sc[min(jj[x], n_cand - 1)];
-            }
-            fn(v, jj);
-        }
-    };
-    // thread t owns a few bins, from kBins-1-kPer*t downwards: finds the bin that straddles the rem-th best key
-    constexpr int kPer = kBins / (32 * NW);
+    // thread t owns kPer bins, from kBins-1-kPer*t downwards: finds the bin that straddles the rem-th best
     auto find_bin = [&](int rem) {
         worker_sync<NW>();
         int c[kPer], mine = 0;
-#pragma unroll
-        for (int x = 0; x < kPer; ++x) { c[x] = sm.hist[kBins - 1 - kPer * tid - x]; mine += c[x]; }
-        int incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
+        if constexpr (kPer == 4) {
+            const int4 v = *reinterpret_cast<const int4*>(hist + kBins - 4 * (tid + 1));
+            c[0] = v.w; c[1] = v.z; c[2] = v.y; c[3] = v.x;
+        } else {
+            const int2 v = *reinterpret_cast<const int2*>(hist + kBins - 2 * (tid + 1));
+            c[0] = v.y; c[1] = v.x;
         }
+#pragma unroll
+        for (int x = 0; x < kPer; ++x) mine += c[x];
+        const int incl = scan(mine);
         if (lane == 31) sm.warp_tot[warp] = incl;
         worker_sync<NW>();
-        int above = incl - mine;
-#pragma unroll
-        for (int w2 = 0; w2 < NW; ++w2) above += w2 < warp ? sm.warp_tot[w2] : 0;
+        int above = incl - mine + before();
         if (above < rem && rem <= above + mine) {
 #pragma unroll
             for (int x = 0; x < kPer; ++x) {
@@ -170,161 +247,334 @@ __device__ __forceinline__ void select_threshold(Smem& sm, const float* sc, int 
         }
         worker_sync<NW>();
     };
-    if (smin > -INFINITY && range > 0.f && range < INFINITY && scale < INFINITY) {
-        // (every score is finite here; -0 and +0 have the same bin)
-        auto bin_of = [&](float s, int j) -> int { return j < n_cand ? min(kBins - 1, (int)((s - smin) * scale)) : kBins; };
-        each_spread([&](const float (&v)[4], const int (&j)[4]) {
+    auto clear_bins = [&]() {                              // (a thread's own ones)
 #pragma unroll
-            for (int x = 0; x < 4; ++x) atomicAdd(&sm.hist[bin_of(v[x], j[x])], 1);
-        });
-        find_bin(need);
-        const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
-        if (cnt <= 32) {
-            each_spread([&](const float (&v)[4], const int (&j)[4]) {
-                bool in[4], any = false;
+        for (int x = 0; x < kPer; ++x) hist[kBins - 1 - kPer * tid - x] = 0;
+    };
+    auto enlist = [&](float v, int j) {
+        const int slot = atomicAdd(&sm.list_n, 1) & 31;
+        sm.list_key[slot] = score_key(v);
+        sm.list_j[slot] = j;
+    };
+    // the `rem`-th best of the `cnt` <= 32 listed candidates, found by every warp for itself
+    auto rank_list = [&](int rem, int cnt) {
+        const uint32_t key = lane < cnt ? sm.list_key[lane] : 0u;
+        const int j = lane < cnt ? sm.list_j[lane] : 0x7fffffff;
+        int rank = 0;
+#pragma unroll 1
+        for (int m = 0; m < cnt; ++m) {
+            const uint32_t km = __shfl_sync(0xffffffffu, key, m);
+            const int jm = __shfl_sync(0xffffffffu, j, m);
+            rank += km > key || (km == key && jm < j);
+        }
+        const int src = __ffs(__ballot_sync(0xffffffffu, lane < cnt && rank == rem - 1)) - 1;
+        thr = __shfl_sync(0xffffffffu, key, src);
+        j_eq = __shfl_sync(0xffffffffu, j, src);
+    };
+    if (need < n_cand) {
+        const uint32_t kmin = sm.pre_min, kmax = sm.pre_max;
+        const float smin = key_score(kmin), smax = key_score(kmax);
+        const float range = smax - smin, scale = (kBins - 1.f) / range;
+        const bool finite = smin > -INFINITY && range > 0.f && range < INFINITY && scale < INFINITY;
+        // (every candidate's score is finite then; -0 and +0 have the same bin)
+        auto bin_of = [&](float s) -> int { return min(kBins - 1, (int)((s - smin) * scale)); };
+        bool found = false;
+        // Up to eight candidates a thread: they stay in its registers from the histogram to the list.
+        auto in_registers = [&](auto q_c) -> bool {
+            constexpr int Q = decltype(q_c)::value;
+            const int j0 = 4 * Q * tid, end = (n_cand + kKeyTile - 1) & ~(kKeyTile - 1);
+            float v[4 * Q];
+            int b[4 * Q];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) any |= in[x] = bin_of(v[x], j[x]) == bin;
-                if (any) {
+            for (int x = 0; x < Q; ++x) {
+                const float4 f = j0 + 4 * x < end ? *reinterpret_cast<const float4*>(sc + j0 + 4 * x)
+                                                  : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                v[4 * x] = f.x; v[4 * x + 1] = f.y; v[4 * x + 2] = f.z; v[4 * x + 3] = f.w;
+            }
+            // (minus infinity, behind the last candidate, has a negative bin)
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        if (in[x]) {
-                            const int slot = atomicAdd(&sm.list_n, 1);
-                            sm.list_key[slot] = score_key(v[x]);
-                            sm.list_j[slot] = j[x];
-                        }
+            for (int k = 0; k < 4 * Q; ++k) {
+                b[k] = bin_of(v[k]);
+                if (b[k] >= 0) atomicAdd(&hist[b[k]], 1);
+            }
+            find_bin(need);
+            const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
+            if (cnt > 32) return false;
+#pragma unroll
+            for (int k = 0; k < 4 * Q; ++k)
+                if (b[k] == bin) enlist(v[k], j0 + k);
+            worker_sync<NW>();
+            rank_list(rem, cnt);
+            const float last = key_score(thr);
+            unsigned taken = 0u;
+#pragma unroll
+            for (int k = 0; k < 4 * Q; ++k) taken |= (unsigned)((v[k] > last) | ((v[k] == last) & (j0 + k <= j_eq))) << k;
+            const int mine = __popc(taken), incl = scan(mine);
+            if (lane == 31) sm.warp_tot[warp] = incl;
+            worker_sync<NW>();
+            int at = incl - mine + before();
+#pragma unroll 1
+            for (; taken; taken &= taken - 1) take(at++, j0 + __ffs(taken) - 1);
+            return true;
+        };
+        if (finite && n_cand <= 8 * kThreads) {
+            if (n_cand <= 4 * kThreads ? in_registers(std::integral_constant<int, 1>()) : in_registers(std::integral_constant<int, 2>())) return;
+        }
+        // The short list: from 4096 candidates on, for one place in 32 or fewer.  15625 candidates, 127 places: scores to list
+        // 4.5 us, where the histogram over all candidates and the list in one CTA took 12.3.
+        if (finite && n_cand >= 4096 && n_cand > 8 * kThreads && 32 * need <= n_cand) {
+            ShortList& sl = *reinterpret_cast<ShortList*>(&gs);
+            const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile;
+            for (int x = tid; x < kStepMaxBlocks / 32; x += kThreads) sl.taken[x] = 0u;
+            // (places of the last tile behind the last candidate hold minus infinity)
+#pragma unroll 1
+            for (int t = tid; t < n_tiles; t += kThreads) {
+                const float4* src = reinterpret_cast<const float4*>(sc + kKeyTile * t);
+                float best = -INFINITY;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {              // (neighbouring lanes begin at different banks)
+                    const float4 v = src[x ^ ((lane >> 1) & 3)];
+                    best = fmaxf(best, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                }
+                sl.tile_max[t] = best;
+                atomicAdd(&hist[bin_of(best)], 1);
+            }
+            find_bin(need);
+            const int bound = (int)sm.prefix;
+            clear_bins();
+#pragma unroll 1
+            for (int t = tid; t < n_tiles; t += kThreads)
+                if (bin_of(sl.tile_max[t]) >= bound) sl.tile[atomicAdd(&sm.tile_n, 1)] = t;
+            worker_sync<NW>();
+            // bins of their own for the few, from about the bound's bin to the largest score
+            const float lo = smin + (float)bound / scale, fine = (kBins - 1.f) / (smax - lo);
+            auto fine_of = [&](float s) -> int { return max(0, min(kBins - 1, (int)((s - lo) * fine))); };
+            const int total = kKeyTile * sm.tile_n;
+            if (fine > 0.f && fine < INFINITY) {
+#pragma unroll 1
+                for (int x = tid; x < total; x += kThreads) {
+                    const int j = kKeyTile * sl.tile[x / kKeyTile] + (x & (kKeyTile - 1));
+                    const float v = sc[j];
+                    if (bin_of(v) >= bound) {
+                        const int slot = atomicAdd(&sm.few_n, 1);
+                        if (slot < kFew) { sl.score[slot] = v; sl.j[slot] = j; }
+                        atomicAdd(&hist[fine_of(v)], 1);
                     }
                 }
-            });
-            worker_sync<NW>();
-            const uint32_t key = lane < cnt ? sm.list_key[lane] : 0u;
-            const int j = lane < cnt ? sm.list_j[lane] : 0x7fffffff;
-            int rank = 0;
-            for (int m = 0; m < cnt; ++m) {
-                const uint32_t km = __shfl_sync(0xffffffffu, key, m);
-                const int jm = __shfl_sync(0xffffffffu, j, m);
-                rank += km > key || (km == key && jm < j);
+                find_bin(need);
+                const int few = sm.few_n, bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
+                if (few <= kFew && cnt <= 32) {
+#pragma unroll 1
+                    for (int e = tid; e < few; e += kThreads)
+                        if (fine_of(sl.score[e]) == bin) enlist(sl.score[e], sl.j[e]);
+                    worker_sync<NW>();
+                    rank_list(rem, cnt);
+#pragma unroll 1
+                    for (int e = tid; e < few; e += kThreads) {
+                        const uint32_t key = score_key(sl.score[e]);
+                        const int j = sl.j[e];
+                        if (key > thr || (key == thr && j <= j_eq)) atomicOr(&sl.taken[j >> 5], 1u << (j & 31));
+                    }
+                    worker_sync<NW>();
+                    // a thread's words of the bits, in order
+                    const int per = (kStepMaxBlocks / 32 + kThreads - 1) / kThreads;
+                    int mine = 0;
+                    for (int x = 0; x < per; ++x) mine += __popc(sl.taken[per * tid + x]);
+                    const int incl = scan(mine);
+                    if (lane == 31) sm.warp_tot[warp] = incl;
+                    worker_sync<NW>();
+                    int at = incl - mine + before();
+                    for (int x = 0; x < per; ++x)
+                        for (unsigned m = sl.taken[per * tid + x]; m; m &= m - 1) take(at++, 32 * (per * tid + x) + __ffs(m) - 1);
+                    return;
+                }
+                clear_bins();                              // (crowded, too: all candidates then)
             }
-            const int src = __ffs(__ballot_sync(0xffffffffu, lane < cnt && rank == rem - 1)) - 1;
-            thr = __shfl_sync(0xffffffffu, key, src);
-            j_eq = __shfl_sync(0xffffffffu, j, src);
-            return;
+            worker_sync<NW>();
+        }
+        if (finite && n_cand > 8 * kThreads) {
+            // Neighbouring blocks have similar scores: the lanes of a warp take candidates that are far apart (lane l has
+            // run l of an odd number of blocks: no bank conflicts); side by side, their additions would queue for a few bins.
+            const int run = ((n_cand + 31) / 32) | 1;
+            auto each_spread = [&](auto&& fn) {
+                int j = lane * run + warp;
+                float v = sc[min(j, n_cand - 1)];
+#pragma unroll 1
+                for (int q = warp; q < run; q += NW) {
+                    const float next = sc[min(j + NW, n_cand - 1)];      // (on its way while this one is worked on)
+                    if (j < n_cand) fn(v, j);
+                    v = next;
+                    j += NW;
+                }
+            };
+            each_spread([&](float v, int) { atomicAdd(&hist[bin_of(v)], 1); });
+            find_bin(need);
+            const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
+            if (cnt <= 32) {
+                each_spread([&](float v, int j) { if (bin_of(v) == bin) enlist(v, j); });
+                worker_sync<NW>();
+                rank_list(rem, cnt);
+                found = true;
+            }
+        }
+        if (!found) {
+            const int words = (n_cand + 32 * NW - 1) / (32 * NW), j0 = warp * words * 32 + lane;
+            auto each = [&](auto&& fn) {
+#pragma unroll 1
+                for (int e = 0; e < words; ++e) {
+                    const int j = j0 + 32 * e;
+                    fn(j < n_cand, score_key(sc[min(j, n_cand - 1)]), j);
+                }
+            };
+            // radix passes of ten bits over key - kmin
+            int bits_left = 32 - __clz(max(kmax - kmin, 1u)), rem = need;
+            uint32_t prefix = 0u;
+            while (bits_left > 0) {
+                const int wbits = min(10, bits_left), shift = bits_left - wbits;
+                clear_bins();
+                worker_sync<NW>();
+                each([&](bool ok, uint32_t key, int) {
+                    const uint32_t rel = key - kmin;
+                    if (ok && (uint32_t)((unsigned long long)rel >> (shift + wbits)) == prefix)        // (shift + wbits can be 32)
+                        atomicAdd(&hist[(rel >> shift) & ((1u << wbits) - 1u)], 1);
+                });
+                find_bin(rem);
+                prefix = (prefix << wbits) | sm.prefix;
+                rem = sm.rem;
+                bits_left = shift;
+            }
+            thr = kmin + prefix;
+            // the rem-th candidate whose key equals thr, in block order (a warp's candidates are one run of blocks)
+            int n_eq = 0;
+            each([&](bool ok, uint32_t key, int) { n_eq += __popc(__ballot_sync(0xffffffffu, ok && key == thr)); });
+            worker_sync<NW>();                             // (everybody has read the last pass's totals)
+            if (lane == 0) sm.warp_tot[warp] = n_eq;
+            worker_sync<NW>();
+            int eq_before = before();
+            if (eq_before < rem && rem <= eq_before + n_eq) {
+                each([&](bool ok, uint32_t key, int j) {
+                    const bool eq = ok && key == thr;
+                    const unsigned m = __ballot_sync(0xffffffffu, eq);
+                    if (eq && eq_before + __popc(m & ((1u << lane) - 1u)) == rem - 1) sm.last_eq = j;
+                    eq_before += __popc(m);
+                });
+            }
+            worker_sync<NW>();
+            j_eq = sm.last_eq;
         }
     }
-    // radix passes of ten bits over key - kmin
-    int bits_left = 32 - __clz(max(kmax - kmin, 1u)), rem = need;
-    uint32_t prefix = 0u;
-    while (bits_left > 0) {
-        const int wbits = min(10, bits_left), shift = bits_left - wbits;
-#pragma unroll
-        for (int x = 0; x < kPer; ++x) sm.hist[kPer * tid + x] = 0;
-        worker_sync<NW>();
-        each([&](bool ok, uint32_t key, int) {
-            const uint32_t rel = key - kmin;
-            if (ok && (uint32_t)((unsigned long long)rel >> (shift + wbits)) == prefix)        // (shift + wbits can be 32)
-                atomicAdd(&sm.hist[(rel >> shift) & ((1u << wbits) - 1u)], 1);
-        });
-        find_bin(rem);
-        prefix = (prefix << wbits) | sm.prefix;
-        rem = sm.rem;
-        bits_left = shift;
+    // the taken ones in order: a warp has a run of blocks, a lane every 32nd of them
+    const int words = (n_cand + 32 * NW - 1) / (32 * NW), j0 = warp * words * 32 + lane;
+    unsigned long long mine = 0ull;
+#pragma unroll 2
+    for (int e = 0; e < words; ++e) {
+        const int j = j0 + 32 * e;
+        const uint32_t key = score_key(sc[min(j, n_cand - 1)]);
+        if ((j < n_cand) & ((key > thr) | ((key == thr) & (j <= j_eq)))) mine |= 1ull << e;
     }
-    thr = kmin + prefix;
-    // the rem-th candidate whose key equals thr, in block order (a warp's candidates are one run of blocks)
-    int n_eq = 0;
-    each([&](bool ok, uint32_t key, int) { n_eq += __popc(__ballot_sync(0xffffffffu, ok && key == thr)); });
-    worker_sync<NW>();                                         // (everybody has read the last pass's totals)
-    if (lane == 0) sm.warp_tot[warp] = n_eq;
+    const int all = __reduce_add_sync(0xffffffffu, __popcll(mine));
+    if (lane == 0) sm.warp_tot[warp] = all;
     worker_sync<NW>();
-    int before = 0;
-#pragma unroll
-    for (int w2 = 0; w2 < NW; ++w2) before += w2 < warp ? sm.warp_tot[w2] : 0;
-    if (before < rem && rem <= before + n_eq) {
-        each([&](bool ok, uint32_t key, int j) {
-            const bool eq = ok && key == thr;
-            const unsigned m = __ballot_sync(0xffffffffu, eq);
-            if (eq && before + __popc(m & ((1u << lane) - 1u)) == rem - 1) sm.last_eq = j;
-            before += __popc(m);
-        });
+    int at = before();
+#pragma unroll 1
+    for (int e = 0; e < words; ++e) {
+        const bool in = (mine >> e) & 1ull;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (in) take(at + __popc(m & ((1u << lane) - 1u)), j0 + 32 * e);
+        at += __popc(m);
     }
-    worker_sync<NW>();
-    j_eq = sm.last_eq;
 }
 
-// The compressed key of block j of the unit, which has just filled, by warps 0..7 of some of the cluster's CTAs: part
-// `part` of `parts` of the rotary pairs.  The same sums in the same order as seer_kcomp.cu's append, so the same entry.
-// (256 threads meet at barrier 2.)
-__device__ __forceinline__ void append_block(const GateParams& g, float* feat, int u, int i, int h, int j, int part, int parts) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b = g.block_size, half = g.d_gate / 2;
-    uint4 wv[4][2];
-    auto load_rows = [&](int pair) {                       // rows of W_k[h] of the rotary pairs `pair`, `pair` + 1
+// The compressed key of block j of the unit, which has just filled, in two parts.  The same sums in the same order as
+// seer_kcomp.cu's append, so the same entry.  First the pooled features, by the producer warps of the cluster, which have
+// nothing else to do while the gate is at work: 16 channels at a time, to every CTA of the cluster.
+template <typename Smem>
+__device__ __forceinline__ void append_pool(const GateParams& g, Smem& sm, int i, int h, int j, int rank, int S) {
+    const int lane = threadIdx.x & 31, b = g.block_size;
+    const __nv_bfloat16* src = g.k_nope + (size_t)i * g.k_stride_batch + (size_t)h * g.k_stride_head +
+                               (g.k_rows_block_local ? 0 : (size_t)j * b) * g.k_stride_token;
+    const int rg = lane >> 1;                              // lane: eight channels, rows lane / 2, lane / 2 + 16, ...
+#pragma unroll 1
+    for (int w0 = rank; w0 < 8; w0 += S) {
+        const int c8 = 2 * w0 + (lane & 1);
+        __nv_bfloat162 mx[4], mn[4];
+        float sum[8];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) { mx[c] = __float2bfloat162_rn(-INFINITY); mn[c] = __float2bfloat162_rn(INFINITY); }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) sum[c] = 0.f;
+#pragma unroll 4
+        for (int r = rg; r < b; r += 16) {
+            const uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)r * g.k_stride_token + 8 * c8);
+            const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                mx[c] = __hmax2(mx[c], hh[c]);
+                mn[c] = __hmin2(mn[c], hh[c]);
+                const float2 f = bf16x2_to_float2(hh[c]);
+                sum[2 * c] += f.x;
+                sum[2 * c + 1] += f.y;
+            }
+        }
+#pragma unroll
+        for (int off = 2; off < 32; off <<= 1) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint32_t a = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<uint32_t*>(&mx[c]), off);
+                const uint32_t d = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<uint32_t*>(&mn[c]), off);
+                mx[c] = __hmax2(mx[c], *reinterpret_cast<const __nv_bfloat162*>(&a));
+                mn[c] = __hmin2(mn[c], *reinterpret_cast<const __nv_bfloat162*>(&d));
+            }
+        }
+        // (row groups 2w and 2w + 1 first, then those pairs one after the other)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const float pair = sum[c] + __shfl_xor_sync(0xffffffffu, sum[c], 2);
+            float s = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) s += __shfl_sync(0xffffffffu, pair, 4 * w + (lane & 1));
+            sum[c] = s / (float)b;
+        }
+        if (lane < 2) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float2 a = bf16x2_to_float2(mx[c]), d = bf16x2_to_float2(mn[c]);
+                *reinterpret_cast<float2*>(&sm.feat_own[0][8 * lane + 2 * c]) = a;
+                *reinterpret_cast<float2*>(&sm.feat_own[1][8 * lane + 2 * c]) = d;
+                *reinterpret_cast<float2*>(&sm.feat_own[2][8 * lane + 2 * c]) = make_float2(sum[2 * c], sum[2 * c + 1]);
+            }
+        }
+        __syncwarp();
+        if (lane < S) {                                    // lane r to CTA r of the cluster
+            const uint32_t to = cluster_addr(sm.feat + 16 * w0, lane), bar = cluster_addr(&sm.got_feat, lane);
+#pragma unroll 1
+            for (int x = 0; x < 12; ++x)
+                send_f32x4(to + (x >> 2) * (kHeadDim * 4) + (x & 3) * 16, *reinterpret_cast<const float4*>(&sm.feat_own[x >> 2][4 * (x & 3)]), bar);
+        }
+        __syncwarp();
+    }
+}
+
+// Then the projection, by the worker warps of all CTAs, while their first tiles travel: two rotary pairs at a time.
+template <int NW, typename Smem>
+__device__ __forceinline__ void append_project(const GateParams& g, Smem& sm, int u, int h, int j, int rank, int S) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = g.d_gate / 2;
+    const int ppc = half / S;                              // pairs of this CTA (an even number)
+    if (2 * warp >= ppc) return;
+    const float* feat = sm.feat;
+    __nv_bfloat16* dst = const_cast<__nv_bfloat16*>(g.kcomp) + ((size_t)u * g.max_blocks + j) * g.d_gate;
+    bool waited = false;
+#pragma unroll 1
+    for (int pair = rank * ppc + 2 * warp; pair < (rank + 1) * ppc; pair += 2 * NW) {
+        uint4 wv[4][2];                                    // rows of W_k[h] of the rotary pairs `pair`, `pair` + 1
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int r = min(pair + (k & 1), half - 1) + (k >> 1) * half;
+            const int r = pair + (k & 1) + (k >> 1) * half;
             const uint4* wrow = reinterpret_cast<const uint4*>(g.w_k + ((size_t)h * g.d_gate + r) * 3 * kHeadDim);
             wv[k][0] = __ldg(wrow + lane);
             wv[k][1] = lane < 16 ? __ldg(wrow + 32 + lane) : make_uint4(0u, 0u, 0u, 0u);
         }
-    };
-    const int first = 2 * (part * 8 + warp), step = 2 * 8 * parts;
-    if (first < half) load_rows(first);
-    // warp: 16 channels; lane: eight of them, rows lane / 2, lane / 2 + 16, ...
-    const int c8 = 2 * warp + (lane & 1), rg = lane >> 1;
-    const __nv_bfloat16* src = g.k_nope + (size_t)i * g.k_stride_batch + (size_t)h * g.k_stride_head +
-                               (g.k_rows_block_local ? 0 : (size_t)j * b) * g.k_stride_token + 8 * c8;
-    __nv_bfloat162 mx[4], mn[4];
-    float sum[8];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) { mx[c] = __float2bfloat162_rn(-INFINITY); mn[c] = __float2bfloat162_rn(INFINITY); }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) sum[c] = 0.f;
-#pragma unroll 4
-    for (int r = rg; r < b; r += 16) {
-        const uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)r * g.k_stride_token);
-        const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            mx[c] = __hmax2(mx[c], hh[c]);
-            mn[c] = __hmin2(mn[c], hh[c]);
-            const float2 f = bf16x2_to_float2(hh[c]);
-            sum[2 * c] += f.x;
-            sum[2 * c + 1] += f.y;
-        }
-    }
-#pragma unroll
-    for (int off = 2; off < 32; off <<= 1) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint32_t a = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<uint32_t*>(&mx[c]), off);
-            const uint32_t d = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<uint32_t*>(&mn[c]), off);
-            mx[c] = __hmax2(mx[c], *reinterpret_cast<const __nv_bfloat162*>(&a));
-            mn[c] = __hmin2(mn[c], *reinterpret_cast<const __nv_bfloat162*>(&d));
-        }
-    }
-    // (row groups 2w and 2w + 1 first, then those pairs one after the other)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        const float pair = sum[c] + __shfl_xor_sync(0xffffffffu, sum[c], 2);
-        float s = 0.f;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) s += __shfl_sync(0xffffffffu, pair, 4 * w + (lane & 1));
-        sum[c] = s / (float)b;
-    }
-    if (lane < 2) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float2 a = bf16x2_to_float2(mx[c]), d = bf16x2_to_float2(mn[c]);
-            feat[8 * c8 + 2 * c] = a.x;
-            feat[8 * c8 + 2 * c + 1] = a.y;
-            feat[kHeadDim + 8 * c8 + 2 * c] = d.x;
-            feat[kHeadDim + 8 * c8 + 2 * c + 1] = d.y;
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) feat[2 * kHeadDim + 8 * c8 + c] = sum[c];
-    }
-    asm volatile("bar.sync 2, 256;" ::: "memory");
-    __nv_bfloat16* dst = const_cast<__nv_bfloat16*>(g.kcomp) + ((size_t)u * g.max_blocks + j) * g.d_gate;
-    for (int pair = first; pair < half; pair += step) {
+        if (!waited) waited = wait_sent(&sm.got_feat, g.status);
         float acc[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -341,28 +591,131 @@ __device__ __forceinline__ void append_block(const GateParams& g, float* feat, i
                 }
             }
         }
-        if (pair + step < half) load_rows(pair + step);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
-        if (lane < 2 && pair + lane < half) {
+        if (lane < 2) {
             const int c = pair + lane;
             const float a = lane ? acc[1] : acc[0], d = lane ? acc[3] : acc[2];
             float sn, cs;
-            rope_sincos((double)j * (double)b, g.inv_freq[c], &sn, &cs);
+            rope_sincos((double)j * (double)g.block_size, g.inv_freq[c], &sn, &cs);
             dst[c] = __float2bfloat16(a * cs - d * sn);
             dst[c + half] = __float2bfloat16(d * cs + a * sn);
         }
     }
 }
 
-// grid (S, units), cluster (S, 1, 1).  Short calls are bound by latency: a step of 8 units x 64 blocks (16.8 MB, 2.6 us at
-// memory speed) takes 14.5 us.  Time stamps in the kernel (which make it a microsecond or two longer; medians over the CTAs,
-// from the first read on) put 1.9 us on the gate query, 1.0 on the barrier behind it, 3.7 on the scores, 0.6 on the barrier,
-// 1.5 on the selection, 2.1 on the lists and their barrier, 2.6 on the tiles, 1.0 on the warps' combine, 1.0 on the barrier,
-// 0.9 on the output.  Longer ones by memory: of a step of 64 units x 205 blocks (430 MB; 83.5 us) the tiles take 66 us,
-// 6.5 TB/s, from the first CTA's first to the last one's last; CTAs that share a unit read neighbouring blocks at the same time.
+// sin and cos like rope_sincos, with what the reduced angle loses when it is rounded to fp32 put back (first order): the
+// gate query is made of MMAs' sums, whose accumulation cuts off, and gets back here what they lose.
+__device__ __forceinline__ void rope_sincos_wide(double pos, double inv_freq, double* sn, double* cs) {
+    double turns = pos * inv_freq * 0.15915494309189535;   // 1 / (2 pi)
+    turns = 2. * (turns - rint(turns));
+    const float x = (float)turns;
+    float s, c;
+    sincospif(x, &s, &c);
+    const double rest = (turns - (double)x) * 3.14159265358979324;
+    *sn = (double)s + (double)c * rest;
+    *cs = (double)c - (double)s * rest;
+}
+
+// The score of one key by plain dot products (whole warp; the largest over the query tokens): for a key or gate query that
+// is not finite, where the parts of the query (score_keys) would make NaN of what is an infinity.
+__device__ __noinline__ float score_key_plain(const uint4* key, const GateScratch& gs, int q_len, int d_gate, int lane) {
+    const uint4 kv = lane < d_gate / 8 ? __ldcg(key + lane) : make_uint4(0u, 0u, 0u, 0u);
+    float best = -INFINITY;
+    for (int t = 0; t < q_len; ++t) {
+        float a = 0.f;
+        if (lane < d_gate / 8) {
+            float q[8];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float2 hi = bf16x2_to_float2(gs.parts[t][0][4 * lane + c]), mid = bf16x2_to_float2(gs.parts[t][1][4 * lane + c]),
+                             low = bf16x2_to_float2(gs.parts[t][2][4 * lane + c]);
+                q[2 * c] = hi.x + (mid.x + low.x);
+                q[2 * c + 1] = hi.y + (mid.y + low.y);
+            }
+            a = dot8(kv, q);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        best = q_len > 1 ? fmaxf(best, a) : a;
+    }
+    return best;
+}
+
+// Scores of this warp's key tiles, by MMAs: tiles warp, warp + NW, ... of the CTA's run of the unit's tiles of 16 keys.  A
+// lane holds the pieces lane % 4 + 4 * x of keys lane / 4 and lane / 4 + 8,
+// straight from global memory: XU = min(XS, 4) of each key at a time (32 registers; keys of 256 channels in two halves).
+// The B operand is the gate queries: columns 4t .. 4t + 3 are query token t's channels, the high part in the first two (one
+// with the first and one with the last eight channels of an MMA, zero elsewhere: of sums half as long the MMA cuts off
+// less), the middle and low parts in the others.  Both operands' contraction index is permuted alike: piece x of a lane is
+// two MMAs' operand as it lies in memory.
+template <int XS, bool MULTI>
+struct KeyScores {
+    static constexpr int XU = XS < 4 ? XS : 4, kHalves = XS / XU, kDepth = 4 / XU;      // tiles requested ahead
+    uint4 a[kDepth][2 * XU];
+
+    __device__ __forceinline__ void request(int d, const uint4* kc, int tile, int half, int max_blocks, int lane) {
+        const int j = kKeyTile * tile + (lane >> 2);
+        const uint4* src = kc + (size_t)j * (4 * XS) + 16 * half + (lane & 3);
+#pragma unroll
+        for (int x = 0; x < XU; ++x) {
+            a[d][2 * x] = j < max_blocks ? __ldcg(src + 4 * x) : make_uint4(0u, 0u, 0u, 0u);
+            a[d][2 * x + 1] = j + 8 < max_blocks ? __ldcg(src + 32 * XS + 4 * x) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+    // The sums of rows lane / 4 and lane / 4 + 8 of the tile in a[d], the largest over the query tokens, the same in a row's
+    // four lanes; `odd`: one of the sums is not finite.  `more(half)` asks for a half of the tile; `next` for another tile.
+    template <typename More, typename Next>
+    __device__ __forceinline__ void sums(int d, const GateScratch& gs, int q_len, int lane, float& v0, float& v1, bool& odd, More&& more, Next&& next) {
+        v0 = v1 = -INFINITY;
+        odd = false;
+#pragma unroll 1
+        for (int nt = 0; 2 * nt < q_len; ++nt) {
+            // (each MMA begins at zero and its 16 products are added up outside: the MMA's own accumulation cuts off where the
+            // addition rounds to nearest)
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+            const int col = (lane >> 2) & 3, t = 2 * nt + (lane >> 4);
+            const uint32_t even = t < q_len && col != 1 ? 0xffffffffu : 0u, odd_w = t < q_len && col != 0 ? 0xffffffffu : 0u;
+            const uint4* bq = reinterpret_cast<const uint4*>(gs.parts[min(t, q_len - 1)][max(0, col - 1)]) + (lane & 3);
+#pragma unroll
+            for (int half = 0; half < kHalves; ++half) {
+                if (kHalves > 1 && (half > 0 || nt > 0)) more(half);
+#pragma unroll
+                for (int x = 0; x < XU; ++x) {
+                    const uint4 b = bq[4 * (half * XU + x)];
+                    const uint4 lo = a[d][2 * x], hi = a[d][2 * x + 1];
+                    const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
+                    float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma_bf16_16816(c0, a0, b.x & even, b.y & odd_w);
+                    mma_bf16_16816(c1, a1, b.z & even, b.w & odd_w);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) s[c] += c0[c] + c1[c];
+                }
+            }
+            if (2 * nt + 2 >= q_len) next();
+            // lanes 0 and 2 of a row's four have a token's high part, 1 and 3 its middle and low parts
+            float r0 = s[0] + s[1], r1 = s[2] + s[3];
+            r0 += __shfl_xor_sync(0xffffffffu, r0, 1);
+            r1 += __shfl_xor_sync(0xffffffffu, r1, 1);
+            odd |= !(fabsf(r0) < INFINITY) || !(fabsf(r1) < INFINITY);
+            if (2 * nt + ((lane >> 1) & 1) >= q_len) r0 = r1 = -INFINITY;
+            v0 = fmaxf(v0, fmaxf(r0, __shfl_xor_sync(0xffffffffu, r0, 2)));
+            v1 = fmaxf(v1, fmaxf(r1, __shfl_xor_sync(0xffffffffu, r1, 2)));
+            if (!MULTI) break;
+        }
+    }
+};
+
+// grid (S, units), cluster (S, 1, 1).  Short calls are bound by latency, and that by the number of instructions on the
+// longest path: all of this runs once, by two warps a scheduler, at some ten cycles an instruction.  A step of 8 units x 64
+// blocks (16.8 MB, 2.6 us at memory speed): by time stamps in the kernel (which make it a microsecond or two longer; medians
+// over the CTAs, from the first read on) the gate query is there after 2.8 us, the scores after 4.4, the list after 6.9, the
+// tiles from 8.4 to 10.1, the CTAs' parts after 11.7, the output after 13.  With a cluster barrier behind each of the first
+// three, the selection by one CTA and its lists stored into the others, it was 2.9, 7.2, 10.6, 11.8 to 13.3, 15.3, 16.2.
+// Longer calls by memory: of a step of 64 units x 205 blocks (430 MB) the tiles take 66 us, 6.5 TB/s, from the first CTA's
+// first to the last one's last; CTAs that share a unit read neighbouring blocks at the same time.
 template <int NW, bool GATE, bool MULTI>
 __global__ void __launch_bounds__(Size<NW, MULTI>::kThreads, NW == 8 ? 2 : 1)
 step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -385,203 +738,266 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     // eight rows are an MMA's N side: `tiles_n` consumer groups share a K/V tile, `paces` such teams take alternate tiles
     const int tiles_n = MULTI ? (rows + 7) >> 3 : 1;
     const int paces = MULTI ? Z::kGroups / tiles_n : Z::kGroups;
-    // (another CTA's shared memory is written only after the barrier this opens: it is then known to be running)
-    cluster_arrive();
     if (tid < kArrivals) {
         mbar_init(&sm.full[tid], 1);
         if (tid < kStages) mbar_init(&sm.empty[tid], 4 * tiles_n);
+        if (tid == 0) {
+            mbar_init(&sm.got_query, 1);
+            mbar_init(&sm.got_scores, 1);
+            mbar_init(&sm.got_feat, 1);
+            mbar_init(&sm.got_parts, 1);
+            sm.pre_min = 0xffffffffu;
+            sm.pre_max = 0u;
+            sm.list_n = sm.tile_n = sm.few_n = 0;
+            sm.no_list = 0;
+        }
         mbar_fence_init();
+        if (tid == 0) {
+            if constexpr (GATE) mbar_arrive_expect_tx(&sm.got_query, (uint32_t)(q_len * ga.g.d_gate * 6));
+            mbar_arrive_expect_tx(&sm.got_parts, (uint32_t)(rows * kHeadDim * 4 + S * rows * 8));
+        }
     }
+    // (another CTA's shared memory is written only after the barrier this opens: it is then known to be running, and its
+    // mbarriers are initialised)
+    cluster_arrive();
     if (producer && lane == 0 && p.q) {
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
     }
 
     int n_blocks = 0, L = 0;                               // listed blocks of the unit, cached tokens
+    int entry[4] = {-1, -1, -1, -1};                       // !GATE: the list's entries of this lane's first tile
+    bool dead = false;                                     // a wait ran out: go through the motions, the results are invalid
     if constexpr (GATE) {
         const GateParams& g = ga.g;
-        const int n = g.group * kHeadDim, chunks = n / 8, half = g.d_gate / 2;
-        const int nit = (chunks + 31) / 32;                // 16-byte pieces of a W_q row per lane (1..4)
-        const int gw = rank * NW + warp, n_gw = S * NW;
-        const int lpk_shift = g.d_gate == 64 ? 3 : g.d_gate == 128 ? 4 : 5, lpk = 1 << lpk_shift;   // lanes per key
-        const int csub = tid & (lpk - 1);
+        const int n = g.group * kHeadDim, half = g.d_gate / 2;
         const uint4* kc = reinterpret_cast<const uint4*>(g.kcomp + (size_t)u * g.max_blocks * g.d_gate);
-        // this CTA's key number lk (runs of kChunkKeys, dealt round robin) is block
-        auto block_of = [&](int lk) { return (((lk / kChunkKeys) << s_shift) + rank) * kChunkKeys + (lk & (kChunkKeys - 1)); };
-        // Rotary pairs (c, c + d_gate/2) of the gate query are dealt to the cluster's warps; with more warps than pairs
-        // several of them take a pair, for every t_step-th query token each.
-        const int c_step = min(n_gw, half), t_step = max(1, n_gw / half), t_first = gw / half, c_first = gw % half;
-        uint4 wv[2][4];
-        auto load_w = [&](int c) {
+        // Gate query: a CTA makes the rotary pairs (c, c + d_gate/2) c_first .. c_first + ppc of all query tokens, by MMAs of 16
+        // rows of W_q (eight pairs) by 8 tokens; the contraction, in units of 32 channels, is split over the warps that share
+        // a row tile (`slices` of them), whose partial sums meet in shared memory.  A lane holds pieces of 16 bytes as they lie
+        // in memory (channels 8 * (lane % 4) .. of a unit): the contraction index is permuted, in W_q and x alike.  What bounds
+        // it is the way of the first bytes and, for several query tokens, was the arithmetic: with a warp per pair and token by
+        // FMA the queries of four tokens were there after 7.2 us, now after 3.3.  (Each MMA begins at zero and the last sums
+        // and the rotation are in double: against 64 bits the scores are off by 1.21e-7 of their norm, by FMA 1.28e-7.)
+        const int ppc = half >> s_shift, c_first = rank * ppc;
+        const int mt_shift = 31 - __clz(min((ppc + 7) >> 3, NW)), slices = NW >> mt_shift, slice = warp >> mt_shift;
+        const int row8 = lane >> 2, units = n / 32;
+        uint4 wa[4], wb[4], xx[4];
+        auto load_w = [&](int m0, int u0) {
+            const int pair = 8 * (m0 + (warp & ((1 << mt_shift) - 1))) + row8;
+            const uint4* w = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + c_first + min(pair, ppc - 1)) * n) + (lane & 3);
+            const uint4* x = reinterpret_cast<const uint4*>(
+                g.q_nope + (((size_t)i * q_len + min(row8, q_len - 1)) * g.num_q_heads + (size_t)h * g.group) * kHeadDim) + (lane & 3);
+            const size_t step = (size_t)half * n / 8;
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const uint4* wrow = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + c + k * half) * n);
-#pragma unroll
-                for (int it = 0; it < 4; ++it) {
-                    const int ch = lane + 32 * it;
-                    wv[k][it] = it < nit && ch < chunks ? __ldg(wrow + ch) : make_uint4(0u, 0u, 0u, 0u);
-                }
+            for (int k = 0; k < 4; ++k) {
+                const int un = u0 + k * slices;
+                if (un >= units) break;
+                wa[k] = pair < ppc ? __ldg(w + 4 * un) : make_uint4(0u, 0u, 0u, 0u);
+                wb[k] = pair < ppc ? __ldg(w + 4 * un + step) : make_uint4(0u, 0u, 0u, 0u);
+                xx[k] = row8 < q_len ? __ldg(x + 4 * un) : make_uint4(0u, 0u, 0u, 0u);
             }
         };
         // (W_q into L2 only, which follows later writes: the kernel before this one may be the one that makes it)
-        if (!producer && t_first < q_len && lane < 2) prefetch_l2(g.w_q + ((size_t)h * g.d_gate + c_first + lane * half) * n, 2 * n);
-        if (rank == 0) {
-            for (int x = tid; x < kBins; x += Z::kThreads) sm.hist[x] = 0;
-            if (tid == 0) { sm.pre_min = 0xffffffffu; sm.pre_max = 0u; sm.list_n = 0; }
+        if (producer && lane < 2) prefetch_l2(g.w_q + ((size_t)h * g.d_gate + c_first + lane * half) * n, 2 * n * ppc);
+        float* sc_all = reinterpret_cast<float*>(sm.ring[0]);
+        GateScratch& gs = *reinterpret_cast<GateScratch*>(sm.ring[2]);
+        if (!producer) {
+            for (int x = tid; x < kBins; x += kWorkers) gs.hist[x] = 0;
         }
         pdl_wait();                                        // queries, lengths and compressed keys are final
         if (!p.q) pdl_launch_dependents();                 // (the gate alone has no work for which it wants the SMs)
         L = p.seq_lens[i];
-        uint4 xv[4];
-        auto load_x = [&](int t) {
-            const uint4* xsrc = reinterpret_cast<const uint4*>(
-                g.q_nope + (((size_t)i * q_len + t) * g.num_q_heads + (size_t)h * g.group) * kHeadDim);
-#pragma unroll
-            for (int it = 0; it < 4; ++it) {
-                const int ch = lane + 32 * it;
-                xv[it] = it < nit && ch < chunks ? __ldg(xsrc + ch) : make_uint4(0u, 0u, 0u, 0u);
-            }
-        };
-        const int all_chunks = (g.max_blocks + kChunkKeys - 1) / kChunkKeys;
-        const int total_cap = ((max(0, all_chunks - rank) + S - 1) >> s_shift) << (lpk_shift + 5);    // pieces, block numbers past the cache among them
-        uint4* staged = reinterpret_cast<uint4*>(sm.ring[2]);      // [kBatch * kWorkers]
-        float* sc_all = reinterpret_cast<float*>(sm.ring[0]);
-        if (!producer) {
-            if (t_first < q_len) {
-                load_w(c_first);
-                load_x(t_first);
-            }
-            // the first batch of keys travels during the projection (entries past n_i - 1 exist in memory: harmless)
-#pragma unroll
-            for (int k = 0; k < kBatch; ++k) {
-                const int pc = k * kWorkers + tid, j = block_of(pc >> lpk_shift);
-                if (pc < total_cap && j < g.max_blocks) cp_async16(staged + pc, kc + ((size_t)j << lpk_shift) + csub);
-            }
-        }
-        const int n_i = L > 0 ? (L + g.block_size - 1) / g.block_size : 0;
+        if (!producer) load_w(0, slice);
+        const int b_shift = 31 - __clz(g.block_size);
+        const int n_i = L > 0 ? (L + g.block_size - 1) >> b_shift : 0;
         // the blocks that hold a query token's own position, j_f .. n_i - 1 (one, the last, for a single token), are always
         // taken; the candidates are those before them
-        const int j_f = max(0, L - q_len) / g.block_size;
-        const int n_forced = min(n_i - j_f, g.max_sel);
-        const int n_cand = min(j_f, g.max_blocks);
+        const int j_f = max(0, L - q_len) >> b_shift;
+        int n_forced = min(n_i - j_f, g.max_sel);
+        int n_cand = min(j_f, g.max_blocks);
+        const bool appends = g.k_nope && blockIdx.z == 0 && L >= g.block_size && (L & (g.block_size - 1)) < q_len && (L >> b_shift) <= g.max_blocks;
         int need = 0;                                      // (threshold method: known once the scores are)
         if (n_i > 0 && !g.threshold_mode) {
-            const int k = min(max(g.token_budget / g.block_size, 1), min(n_i, g.max_sel));
+            const int k = min(max(g.token_budget >> b_shift, 1), min(n_i, g.max_sel));
             // (kListed: only a sequence longer than max_seq_len, which the host's rule went by, gets that far)
             need = max(0, min(min(k - n_forced, n_cand), kListed));
             n_blocks = need + n_forced;
         }
-        // pieces that matter: up to the last run of keys with a candidate
-        const int cand_chunks = (n_cand + kChunkKeys - 1) / kChunkKeys;
-        const int total = ((max(0, cand_chunks - rank) + S - 1) >> s_shift) << (lpk_shift + 5);
+        // This CTA's key tiles: a run of those with a candidate.  The producer warp asks for them into L2, so that they travel
+        // while the gate query is made.
+        const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile, per_cta = (n_tiles + S - 1) >> s_shift;
+        const int tile0 = min(rank * per_cta, n_tiles), my_tiles = min(per_cta, n_tiles - tile0);
+        // who selects: every CTA that will read tiles, or (the gate alone) the first one
+        const int n_sel = p.q ? S : 1, sel_shift = p.q ? s_shift : 0;
+        const bool selects = rank < n_sel;
+        if (producer) {
+            // (the tiles behind each warp's first; few requests to a lane, each of which takes the warp some fifty nanoseconds)
+            const int later = max(0, my_tiles - NW), step = (later + 31) >> 5;
+            if (lane * step < later) {
+                const int m = NW + lane * step, j = kKeyTile * (tile0 + m);
+                prefetch_l2(g.kcomp + ((size_t)u * g.max_blocks + j) * g.d_gate,
+                            min(kKeyTile * min(step, my_tiles - m), g.max_blocks - j) * g.d_gate * 2);
+            }
+            // (the scores of the other CTAs' key tiles, and from every CTA their smallest and largest key)
+            if (selects && lane == 0) mbar_arrive_expect_tx(&sm.got_scores, (uint32_t)((n_tiles - my_tiles) * kKeyTile * 4 + S * 8));
+            if (appends && lane < 3) {
+                if (lane == 0) mbar_arrive_expect_tx(&sm.got_feat, 3 * kHeadDim * 4);
+                else prefetch_l2(g.w_k + ((size_t)h * g.d_gate + c_first + (lane - 1) * half) * 3 * kHeadDim, ppc * 3 * kHeadDim * 2);
+            }
+        }
         cluster_wait();                                    // every CTA of the cluster has started
-        // ---- gate query: rotary pairs (c, c + d_gate/2) dealt to the cluster's warps --------------------------
+        // ---- gate query ------------------------------------------------------------------------------------------------
         if (!producer) {
-            for (int c = c_first; c < half; c += c_step) {
-                for (int t = t_first; t < q_len; t += t_step) {
-                    if (c != c_first && t == t_first) load_w(c);
-                    if (MULTI && (c != c_first || t != t_first)) load_x(t);
-                    float a = 0.f, b = 0.f;
+            float (*part)[16][8] = gs.sums;
+            for (int m0 = 0; 8 * m0 < ppc; m0 += NW) {
+                if (m0 > 0) {
+                    worker_sync<NW>();                     // (the partial sums have been read)
+                    load_w(m0, slice);
+                }
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};       // (each MMA from zero: KeyScores)
+#pragma unroll 1
+                for (int u0 = slice;;) {
 #pragma unroll
-                    for (int it = 0; it < 4; ++it) {
-                        if (it < nit) { a += dot8(wv[0][it], xv[it]); b += dot8(wv[1][it], xv[it]); }
-                    }
+                    for (int k = 0; k < 4; ++k) {
+                        if (u0 + k * slices >= units) break;
+                        const uint32_t a0[4] = {wa[k].x, wb[k].x, wa[k].y, wb[k].y}, a1[4] = {wa[k].z, wb[k].z, wa[k].w, wb[k].w};
+                        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+                        mma_bf16_16816(c0, a0, xx[k].x, xx[k].y);
+                        mma_bf16_16816(c1, a1, xx[k].z, xx[k].w);
 #pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        a += __shfl_xor_sync(0xffffffffu, a, off);
-                        b += __shfl_xor_sync(0xffffffffu, b, off);
+                        for (int c = 0; c < 4; ++c) acc[c] += c0[c] + c1[c];
                     }
-                    float sn, cs;                          // query token t sits at position L - q_len + t
-                    rope_sincos((double)max(L - q_len + t, 0), g.inv_freq[c], &sn, &cs);
-                    if (lane < S) {                        // lane r stores into CTA r of the cluster
-                        float* dst = cluster.map_shared_rank(&sm.qg[0][0], lane) + t * kMaxDGate;
-                        dst[c] = a * cs - b * sn;
-                        dst[c + half] = b * cs + a * sn;
+                    u0 += 4 * slices;
+                    if (u0 >= units) break;
+                    load_w(m0, u0);
+                }
+                *reinterpret_cast<float2*>(&part[warp][row8][2 * (lane & 3)]) = make_float2(acc[0], acc[1]);
+                *reinterpret_cast<float2*>(&part[warp][row8 + 8][2 * (lane & 3)]) = make_float2(acc[2], acc[3]);
+                worker_sync<NW>();
+                // a thread per pair, token and CTA that gets them
+                const int np_shift = 31 - __clz(min(ppc, 8 << mt_shift));
+#pragma unroll 1
+                for (int x = tid; x < (q_len << (np_shift + s_shift)); x += kWorkers) {
+                    const int to = x & (S - 1), pr = (x >> s_shift) & ((1 << np_shift) - 1), t = x >> (s_shift + np_shift);
+                    const int c = c_first + 8 * m0 + pr;
+                    double sn, cs;                         // query token t sits at position L - q_len + t
+                    rope_sincos_wide((double)max(L - q_len + t, 0), g.inv_freq[c], &sn, &cs);
+                    double a = 0., b = 0.;
+#pragma unroll 4
+                    for (int sl = 0; sl < slices; ++sl) {
+                        a += (double)part[(sl << mt_shift) + (pr >> 3)][pr & 7][t];
+                        b += (double)part[(sl << mt_shift) + (pr >> 3)][(pr & 7) + 8][t];
+                    }
+                    // A thread has channels c and c + d_gate/2, its neighbour S lanes on the ones next to them (c is even here and
+                    // odd there, or the other way round): the even one sends the words of the lower two channels, the other
+                    // one those of the upper two.
+                    float f0 = (float)(a * cs - b * sn), f1 = (float)(b * cs + a * sn);
+                    const bool upper = pr & 1;
+                    const float got = __shfl_xor_sync(0xffffffffu, upper ? f0 : f1, S);
+                    if (upper) f0 = got;
+                    else f1 = got;
+                    const uint32_t dst = cluster_addr(&gs.parts[t][0][(c >> 1) + (upper ? half >> 1 : 0)], to), bar = cluster_addr(&sm.got_query, to);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const uint32_t w = pack_bf16x2(f0, f1);
+                        send_u32(dst + k * (uint32_t)sizeof(gs.parts[0][0]), w, bar);
+                        const float2 r = bf16x2_to_float2(w);
+                        // (each difference is exact: the rest of a rounding to eight bits has at most the sixteen bits behind
+                        // them; what is not finite has no rest)
+                        f0 = fabsf(r.x) < INFINITY ? f0 - r.x : 0.f;
+                        f1 = fabsf(r.y) < INFINITY ? f1 - r.y : 0.f;
                     }
                 }
             }
         }
-        uint4 kv[kBatch];
-        // (through L2, not the read-only path: the entry that this launch appends, or the step before it did, is among them)
-        auto request = [&](int cb) {
+        // ---- scores, into the shared memory of the CTAs that select ------------------------------------------------
+        // (keys through L2, not the read-only path: the entry that this launch appends, or the step before it did, is among them)
+        auto scores = [&](auto xs_c) {
+            constexpr int XS = decltype(xs_c)::value;
+            using Keys = KeyScores<XS, MULTI>;
+            Keys ks;
+            constexpr int kDepth = Keys::kDepth;
+            auto request = [&](int d, int m, int half) {
+                if (m < my_tiles) ks.request(d, kc, tile0 + m, half, g.max_blocks, lane);
+            };
 #pragma unroll
-            for (int k = 0; k < kBatch; ++k) {
-                const int pc = cb + k * kWorkers + tid, j = block_of(pc >> lpk_shift);
-                kv[k] = pc < total && j < g.max_blocks ? __ldcg(kc + ((size_t)j << lpk_shift) + csub) : make_uint4(0u, 0u, 0u, 0u);
+            for (int d = 0; d < kDepth; ++d) request(d, warp + d * NW, 0);
+            if (!wait_sent(&sm.got_query, p.status)) dead = true;
+            const float inv = rsqrtf((float)g.d_gate);
+            uint32_t kmn = 0xffffffffu, kmx = 0u;
+#pragma unroll 1
+            for (int m0 = warp; m0 < my_tiles; m0 += kDepth * NW) {
+#pragma unroll
+                for (int d = 0; d < kDepth; ++d) {
+                    const int m = m0 + d * NW;
+                    if (m < my_tiles) {
+                        const int j0 = kKeyTile * (tile0 + m);
+                        float v0, v1;
+                        bool odd;
+                        ks.sums(d, gs, q_len, lane, v0, v1, odd, [&](int half) { request(d, m, half); },
+                                [&]() { request(d, m + kDepth * NW, 0); });
+                        // lane 4r has the score of key r, lane 4r + 1 (the others alike) that of key r + 8
+                        const int k_of = (lane >> 2) + 8 * (lane & 1), j = j0 + k_of;
+                        float v = (lane & 1) ? v1 : v0;
+                        unsigned odds = __ballot_sync(0xffffffffu, odd);
+                        if (odds) {
+#pragma unroll 1
+                            for (int k = 0; k < kKeyTile; ++k) {
+                                if (((odds >> (4 * (k & 7))) & 15u) && j0 + k < n_cand) {
+                                    const float x = score_key_plain(kc + (size_t)(j0 + k) * (4 * XS), gs, q_len, g.d_gate, lane);
+                                    if (k == k_of) v = x;
+                                }
+                            }
+                        }
+                        v *= inv;
+                        if ((lane & 2) == 0) {
+                            const bool ok = j < n_cand;
+                            sc_all[j] = ok ? v : -INFINITY;
+                            if (ok) {
+                                if (g.scores_user) g.scores_user[(size_t)u * g.max_blocks + j] = v;
+                                const uint32_t key = score_key(v);
+                                kmn = min(kmn, key);
+                                kmx = max(kmx, key);
+                            }
+                        }
+                    }
+                }
+            }
+            kmn = __reduce_min_sync(0xffffffffu, kmn);
+            kmx = __reduce_max_sync(0xffffffffu, kmx);
+            if (lane == 0) { sm.warp_min[warp] = kmn; sm.warp_max[warp] = kmx; }
+            worker_sync<NW>();
+            // four scores at a time to the others
+            const int to = tid & (n_sel - 1);
+            if (to != rank) {
+                const uint32_t dst = cluster_addr(sc_all + kKeyTile * tile0, to), bar = cluster_addr(&sm.got_scores, to);
+#pragma unroll 1
+                for (int c = tid >> sel_shift; c < 4 * my_tiles; c += kWorkers >> sel_shift)
+                    send_f32x4(dst + 16 * c, *reinterpret_cast<const float4*>(sc_all + kKeyTile * tile0 + 4 * c), bar);
+            }
+            if (warp == 0) {
+                kmn = __reduce_min_sync(0xffffffffu, lane < NW ? sm.warp_min[lane] : 0xffffffffu);
+                kmx = __reduce_max_sync(0xffffffffu, lane < NW ? sm.warp_max[lane] : 0u);
+                if (lane < n_sel) {
+                    const uint32_t bar = cluster_addr(&sm.got_scores, lane);
+                    send_min(cluster_addr(&sm.pre_min, lane), kmn, bar);
+                    send_max(cluster_addr(&sm.pre_max, lane), kmx, bar);
+                }
             }
         };
-        constexpr int kPieces = kWorkers * kBatch;
-        if (!producer) request(kPieces);                   // the second batch, into registers
-        cluster_sync();
-        // ---- scores, into the first CTA's shared memory --------------------------------------------------------
-        // A thread holds one piece of each of eight keys; reduce8 leaves every lane with the sum of one of the keys
-        // (that of its piece number krev).
-        if (!producer) {
-            float* sc0 = cluster.map_shared_rank(sc_all, 0);
-            const float inv = rsqrtf((float)g.d_gate);
-            const int krev = ((lane & 1) << 2) | (lane & 2) | ((lane >> 2) & 1);
-            const bool storer = (csub & ~7) == 0;
-            uint32_t kmn = 0xffffffffu, kmx = 0u;
-            float* sc_user = g.scores_user ? g.scores_user + (size_t)u * g.max_blocks : nullptr;
-            // (several query tokens: a key's score is the largest of its products with their gate queries)
-            auto score_batch = [&](auto&& piece, int cb) {
-                float best = -INFINITY;
-                for (int t = 0; t < q_len; ++t) {
-                    float qsub[8], acc[kBatch];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) qsub[c] = sm.qg[t][8 * csub + c];
-#pragma unroll
-                    for (int k = 0; k < kBatch; ++k) acc[k] = dot8(piece(k), qsub);
-                    const float x = reduce8(acc, lane, lpk);
-                    best = MULTI ? fmaxf(best, x) : x;
-                }
-                const float v = best * inv;
-                const int pc = cb + krev * kWorkers + tid, j = block_of(pc >> lpk_shift);
-                if (storer && pc < total && j < n_cand) {
-                    sc0[j] = v;
-                    if (sc_user) sc_user[j] = v;
-                    const uint32_t key = score_key(v);
-                    kmn = min(kmn, key);
-                    kmx = max(kmx, key);
-                }
-            };
-            for (int cb = 0; cb < total;) {
-                cp_async_wait_all();
-                score_batch([&](int k) {
-                    const int pc = k * kWorkers + tid;
-                    return cb + pc < total && block_of((cb + pc) >> lpk_shift) < g.max_blocks ? staged[pc] : make_uint4(0u, 0u, 0u, 0u);
-                }, cb);
-                cb += kPieces;
-                if (cb >= total) break;
-                // (batches alternate between the staged area and the registers; the one after the next is on its way)
-#pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    const int pc = cb + kPieces + k * kWorkers + tid, j = block_of(pc >> lpk_shift);
-                    if (pc < total && j < g.max_blocks) cp_async16(staged + k * kWorkers + tid, kc + ((size_t)j << lpk_shift) + csub);
-                }
-                score_batch([&](int k) { return kv[k]; }, cb);
-                cb += kPieces;
-                request(cb + kPieces);
-            }
-            cp_async_wait_all();
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                kmn = min(kmn, __shfl_xor_sync(0xffffffffu, kmn, off));
-                kmx = max(kmx, __shfl_xor_sync(0xffffffffu, kmx, off));
-            }
-            if (lane == 0 && kmn <= kmx) {
-                atomicMin(cluster.map_shared_rank(&sm.pre_min, 0), kmn);
-                atomicMax(cluster.map_shared_rank(&sm.pre_max, 0), kmx);
-            }
-        }
-        cluster_sync();
-        // ---- selection, by the first CTA ----------------------------------------------------------------------------
-        if (rank == 0 && !producer) {
+        if (producer) {
+        } else if (g.d_gate == 128) scores(std::integral_constant<int, 4>());
+        else if (g.d_gate == 64) scores(std::integral_constant<int, 2>());
+        else scores(std::integral_constant<int, 8>());
+        // ---- selection ---------------------------------------------------------------------------------------------
+        if (selects && !producer) {
             int32_t* dst = g.block_idx + (size_t)u * g.max_sel;
-            int* list = reinterpret_cast<int*>(sm.ring[2]);      // [kListed] the scored blocks of the list, ascending
-            const int words = ((n_cand + 31) / 32 + NW - 1) / NW;      // 32 candidates each, per warp
-            uint32_t thr;
-            int j_eq;
+            const bool lists = rank == 0 && blockIdx.z == 0;     // this CTA writes the caller's list, too
+            // (a wait that has run out for one thread has for all: no list then, and the producer warp is told)
+            dead = worker_any<NW>(!wait_sent(&sm.got_scores, p.status) || dead);
+            if (dead) n_cand = need = n_forced = n_blocks = 0;
+            if (dead && tid == 0) sm.no_list = 1;
             if (g.threshold_mode) {
                 // Threshold method (Sec. 3.1): softmax of the scores over the candidates; those above tau are the `above`
                 // highest-scoring ones (equal scores have equal probabilities), so only the number differs
@@ -607,75 +1023,53 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 need = max(0, min(min((int)(sum_all(above) + 0.5f), g.max_sel - n_forced), min(n_cand, kListed)));
                 n_blocks = n_i > 0 ? need + n_forced : 0;
             }
-            select_threshold<NW>(sm, sc_all, n_cand, need, words, warp, lane, thr, j_eq);
-            // which of the warp's candidates are taken: lane x keeps the words x and x + 32 (words <= 64)
-            const int jw = warp * words * 32 + lane;
-            unsigned taken[2] = {0u, 0u};
-#pragma unroll 1
-            for (int e = 0; e < words; e += 4) {
-                float v[4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) v[x] = sc_all[min(jw + 32 * (e + x), n_cand - 1)];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const int j = jw + 32 * (e + x);
-                    const uint32_t key = score_key(v[x]);
-                    const unsigned m = __ballot_sync(0xffffffffu, (e + x < words) & (j < n_cand) & ((key > thr) | ((key == thr) & (j <= j_eq))));
-                    if (lane == ((e + x) & 31)) { if (e + x < 32) taken[0] = m; else taken[1] = m; }
-                }
-            }
-            const int in_low = __popc(taken[0]), in_both = in_low + __popc(taken[1]);
-            int incl_low = in_low, incl_high = in_both - in_low;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int lo = __shfl_up_sync(0xffffffffu, incl_low, o), hi = __shfl_up_sync(0xffffffffu, incl_high, o);
-                if (lane >= o) { incl_low += lo; incl_high += hi; }
-            }
-            const int all_low = __shfl_sync(0xffffffffu, incl_low, 31);
-            worker_sync<NW>();
-            if (lane == 31) sm.warp_tot[warp] = incl_low + incl_high;
-            worker_sync<NW>();
-            int pos = 0;
-#pragma unroll
-            for (int w2 = 0; w2 < NW; ++w2) pos += w2 < warp ? sm.warp_tot[w2] : 0;
-            // every lane lists its own words' blocks
-            {
-                int at = pos + incl_low - in_low;
-                const int j_low = warp * words * 32 + 32 * lane;
-                for (unsigned m = taken[0]; m; m &= m - 1) list[at++] = j_low + __ffs(m) - 1;
-                at = pos + all_low + incl_high - (in_both - in_low);
-                for (unsigned m = taken[1]; m; m &= m - 1) list[at++] = j_low + 1024 + __ffs(m) - 1;
-            }
-            if (tid == 0 && blockIdx.z == 0) g.block_cnt[u] = n_blocks;
-            worker_sync<NW>();
-            // entry e of the list is block j (the last ones: the blocks taken without a score): into the caller's list, and
-            // to the CTA that reads its tile(s)
-            for (int e = tid; e < g.max_sel; e += kWorkers) {
-                const int j = e < need ? list[e] : e < n_blocks ? n_i - n_blocks + e : -1;
-                if (blockIdx.z == 0) dst[e] = j;
-                if (e >= n_blocks || !p.q) continue;
+            // entry e of the list is block j: its tile(s) among this CTA's, if they are
+            auto take = [&](int e, int j) {
+                if (lists) dst[e] = j;
+                if (!p.q) return;
                 if (p.blocks_per_tile == 1) {
                     for (int x = 0; x < p.tiles_per_block; ++x) {
                         const int t = (e << p.tpb_shift) + x;
-                        if ((t >> s_shift) < kCodes) cluster.map_shared_rank(sm.codes, t & (S - 1))[t >> s_shift] = (j << p.tpb_shift) + x;
+                        if ((t & (S - 1)) == rank && (t >> s_shift) < kCodes) sm.codes[t >> s_shift] = (j << p.tpb_shift) + x;
                     }
                 } else {
-                    const int t = e >> p.bpt_shift, sub = e & (p.blocks_per_tile - 1);
-                    const int at = ((t >> s_shift) << p.bpt_shift) + sub;
-                    if (at < kCodes) cluster.map_shared_rank(sm.codes, t & (S - 1))[at] = j;
+                    const int t = e >> p.bpt_shift, at = ((t >> s_shift) << p.bpt_shift) + (e & (p.blocks_per_tile - 1));
+                    if ((t & (S - 1)) == rank && at < kCodes) sm.codes[at] = j;
                 }
+            };
+            select_blocks<NW>(sm, gs, sc_all, n_cand, need, warp, lane, take);
+            // the last ones: the blocks taken without a score
+            if (tid < n_blocks - need) take(need + tid, n_i - n_blocks + need + tid);
+            if (lists) {
+                if (tid == 0) g.block_cnt[u] = n_blocks;
+                for (int e = n_blocks + tid; e < g.max_sel; e += kWorkers) dst[e] = -1;
             }
         }
-        if (!p.q) return;                                  // the gate alone
+        if (!p.q) {                                        // the gate alone
+            cluster_sync();                                // (as at the end)
+            return;
+        }
         fence_proxy_async_smem();                          // the ring's memory goes over to the copy engine
-        cluster_arrive();
-        // The other CTAs have nothing to do until the lists are out: up to four of them compress the block that has just
-        // filled.  (Nothing in this step reads its entry.)
-        if (g.k_nope && rank > 0 && rank <= 4 && warp < 8 && blockIdx.z == 0 && L >= g.block_size && L % g.block_size < q_len &&
-            L / g.block_size <= g.max_blocks)
-            append_block(g, sm.feat, u, i, h, L / g.block_size - 1, rank - 1, min(S - 1, 4));
+        if (producer) {
+            // (nothing in this step reads the entry of the block that has just filled)
+            if (appends) append_pool(g, sm, i, h, (L >> b_shift) - 1, rank, S);
+            tiles_listed_wait<NW>();
+            if (sm.no_list) n_blocks = 0;
+        } else {
+            tiles_listed_arrive<NW>();
+            if (appends) append_project<NW>(g, sm, u, h, (L >> b_shift) - 1, rank, S);
+        }
     } else {
         pdl_wait();
+        // (the first entries are asked for beside the count that says how many there are, not behind it)
+        if (producer && p.block_idx) {
+            const int t = (lane << s_shift) + rank;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const int e = p.blocks_per_tile > 1 ? (t << p.bpt_shift) + x : t >> p.tpb_shift;
+                if (x < p.blocks_per_tile) entry[x] = p.block_idx[(size_t)u * p.max_sel + min(e, p.max_sel - 1)];
+            }
+        }
         L = p.seq_lens[i];
         if (p.block_idx) {
             const int cnt = p.block_cnt ? p.block_cnt[u] : p.max_sel;      // (not behind the test on L: both loads in flight)
@@ -697,9 +1091,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         return ((size_t)i * q_len + tl) * p.num_q_heads + (size_t)h * p.group + (row0 + r - tl * p.group);
     };
     const int qd = lane & 3, rw = lane >> 2;
-    bool dead = false;                                     // a wait ran out: go through the motions, the results are invalid
     if (producer) {
-        if (GATE) cluster_wait();                          // the tiles' numbers are in place
         pdl_launch_dependents();
         if (GATE && n_local < n_mine && lane == 0) raise_status(p.status, DEV_BAD_INDEX);      // (a sequence longer than max_seq_len: tiles are left out)
         const int n_i = (L + p.block_size - 1) >> p.bs_shift;
@@ -719,14 +1111,18 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         } else if (small) {
                             const int e = (t << p.bpt_shift) + x;
                             if (e < n_blocks) {
-                                const int blk = GATE ? sm.codes[(it << p.bpt_shift) + x] : p.block_idx[(size_t)u * p.max_sel + e];
+                                const int blk = GATE ? sm.codes[(it << p.bpt_shift) + x] : base == 0 ? entry[x] : p.block_idx[(size_t)u * p.max_sel + e];
                                 if (!GATE && blk >= n_i) raise_status(p.status, DEV_BAD_INDEX);
                                 if (blk >= 0 && blk < n_i) tok0 = blk << p.bs_shift;
                             }
                         } else if (GATE) {
                             tok0 = sm.codes[it] * kTileTokens;
+                            if ((unsigned)tok0 >= (unsigned)(n_i << p.bs_shift)) {     // (never: the lists are this kernel's own)
+                                raise_status(p.status, DEV_BAD_INDEX);
+                                tok0 = -1;
+                            }
                         } else {
-                            const int blk = p.block_idx[(size_t)u * p.max_sel + (t >> p.tpb_shift)];
+                            const int blk = base == 0 ? entry[0] : p.block_idx[(size_t)u * p.max_sel + (t >> p.tpb_shift)];
                             if (blk >= n_i) raise_status(p.status, DEV_BAD_INDEX);
                             if (blk >= 0 && blk < n_i) tok0 = (blk << p.bs_shift) + (t & (p.tiles_per_block - 1)) * kTileTokens;
                         }
@@ -784,6 +1180,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         }
         if (!GATE) cluster_wait();                         // (the barrier opened at the top)
+        cluster_arrive();
     } else {
         const int group = warp >> 2, my_n = MULTI ? group % tiles_n : 0, pace = MULTI ? group / tiles_n : group;
         // Q^T B-fragments: this thread supplies row 8 * my_n + rw of the unit's queries
@@ -806,7 +1203,6 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (r < rows) back[c] = q_len - 1 - (((row0 + r) * p.group_magic) >> 16);
             }
         }
-        if (GATE) cluster_wait();
         pdl_launch_dependents();
         const int w4 = warp & 3;                           // which 16 of a tile's tokens
         float o[8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
@@ -940,46 +1336,42 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     acc.w = fmaf(v.w, f, acc.w);
                 }
             }
-            float* dst = cluster.map_shared_rank(sm.recv_o, c >> c_shift) + (((rank * kRows + r) << c_shift) | (c & ((1 << c_shift) - 1)));
-            *reinterpret_cast<float4*>(dst) = acc;
-            if (lane < S) cluster.map_shared_rank(&sm.recv_ml[0][0], lane)[rank * kRows + r] = make_float2(M, l);
+            const int to = c >> c_shift;
+            send_f32x4(cluster_addr(sm.recv_o + (((rank * kRows + r) << c_shift) | (c & ((1 << c_shift) - 1))), to), acc, cluster_addr(&sm.got_parts, to));
+            if (lane < S) send_f32x2(cluster_addr(&sm.recv_ml[rank][r], lane), make_float2(M, l), cluster_addr(&sm.got_parts, lane));
         }
     }
-    cluster_sync();
     if (!producer) {
+        wait_sent(&sm.got_parts, p.status);
+        cluster_arrive();
+        // S lanes per channel pair, one per source CTA
         const int c_shift = 7 - s_shift;
-        const int pairs = rows << (c_shift - 1);        // channel pairs of this CTA's slice, all rows
-        for (int x = tid; x < pairs; x += kWorkers) {
-            const int r = x >> (c_shift - 1), c = 2 * (x & ((1 << (c_shift - 1)) - 1));
-            float M = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f;
-            float2 ml[kMaxS];
-#pragma unroll
-            for (int s = 0; s < kMaxS; ++s) {
-                ml[s] = s < S ? sm.recv_ml[s][r] : make_float2(-INFINITY, 0.f);
-                M = fmaxf(M, ml[s].x);
+#pragma unroll 1
+        for (int x = tid; x < rows * (kHeadDim / 2); x += kWorkers) {
+            const int s = x & (S - 1), c = 2 * ((x >> s_shift) & ((1 << (c_shift - 1)) - 1)), r = x >> 6;
+            const float2 ml = sm.recv_ml[s][r], v = *reinterpret_cast<const float2*>(&sm.recv_o[((s * kRows + r) << c_shift) + c]);
+            float M = ml.x;
+#pragma unroll 1
+            for (int o = 1; o < S; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+            const float f = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - M);
+            float l = ml.y * f, a0 = v.x * f, a1 = v.y * f;
+#pragma unroll 1
+            for (int o = 1; o < S; o <<= 1) {
+                l += __shfl_xor_sync(0xffffffffu, l, o);
+                a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+                a1 += __shfl_xor_sync(0xffffffffu, a1, o);
             }
-#pragma unroll
-            for (int s = 0; s < kMaxS; ++s) {
-                if (s < S) {
-                    const float f = ml[s].x == -INFINITY ? 0.f : fast_exp2(ml[s].x - M);
-                    const float2 v = *reinterpret_cast<const float2*>(&sm.recv_o[((s * kRows + r) << c_shift) + c]);
-                    l = fmaf(ml[s].y, f, l);
-                    a0 = fmaf(v.x, f, a0);
-                    a1 = fmaf(v.y, f, a1);
-                }
+            if (s == 0) {
+                const float inv = l > 0.f ? 1.f / l : 0.f;
+                const size_t row = out_row(r);
+                *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
+                if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
             }
-            const float inv = l > 0.f ? 1.f / l : 0.f;
-            const size_t row = out_row(r);
-            *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
-            if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
-        }
-        if constexpr (GATE) {                              // (a cluster of one CTA has nobody to leave the append to)
-            const GateParams& g = ga.g;
-            if (g.k_nope && S == 1 && warp < 8 && blockIdx.z == 0 && L >= g.block_size && L % g.block_size < q_len &&
-                L / g.block_size <= g.max_blocks)
-                append_block(g, sm.feat, u, i, h, L / g.block_size - 1, 0, 1);
         }
     }
+    // No CTA leaves before every one has received all that was sent to it: neither the receiver's shared memory nor the
+    // sender's place in the cluster may be gone while a store is under way.
+    cluster_wait();
 }
 
 template <int NW, bool GATE, bool MULTI>
@@ -1039,6 +1431,7 @@ int resident_clusters(bool wide, int k) {
 // something to do each.  Measured against the kernels of long calls, us a call (a step's append included):
 //     step, 8 KV heads, budget 4096, 1 / 2 / 4 sequences     23.3 -> 16.9, 25.3 -> 19.8, 31.6 -> 28.8
 //     step of batch 8 at 128k, 205 blocks (51 tiles a CTA)   98.4 -> 85.0
+//     (as the step was when these were measured; its gate's parts have become shorter since)
 //     four query tokens, 20 rows, 4 sequences, budget 4096   63.2 -> 38.6;  64 rows 92.3 -> 75.2;  8 rows, 1 sequence 27.2 -> 19.0
 //     threshold gate alone in front of given lists, 4 sequences of 48k, blocks of 32: 42.5 -> 35.0 with both
 // A cluster's CTAs go through their unit's tiles by themselves; the decode kernel's CTAs share all tiles.  The rule sees
@@ -1061,10 +1454,11 @@ int resident_clusters(bool wide, int k) {
 // the line is at 32 there.  149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles
 // a CTA 45.9 -> 33.8, 52.7 -> 39.1, 59.3 -> 43.1; 64 tiles 93.5 -> 82.1, 108 -> 96, 127 -> 109.
 StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes, int max_keys) {
-    const bool wide = rows > 16;
-    StepPlan plan = {0, 1, rows};
+    // Above 8192 keys, too, 16 warps a CTA: twice the keys in flight per SM (8 units of 15626 keys: 39.5 -> 33.4 us a step).
+    const bool wide = rows > 16 || max_keys > 8192;
+    StepPlan plan = {0, 1, rows, wide};
     if (rows > 64) return plan;
-    if (wide) {
+    if (rows > 32) {
         plan.parts = (rows + 31) / 32;
         plan.rows = (rows + plan.parts - 1) / plan.parts;
     }
@@ -1100,9 +1494,27 @@ cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const 
 
 cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
                                 const StepPlan& plan, cudaStream_t stream) {
-    if (p.q_len == 1) return launch_of<8, false>(map_k, map_v, p, g, plan, stream);
-    return plan.parts * plan.rows <= 16 ? launch_of<8, true>(map_k, map_v, p, g, plan, stream)
-                                        : launch_of<16, true>(map_k, map_v, p, g, plan, stream);
+    if (plan.wide) return launch_of<16, true>(map_k, map_v, p, g, plan, stream);
+    return p.q_len == 1 ? launch_of<8, false>(map_k, map_v, p, g, plan, stream) : launch_of<8, true>(map_k, map_v, p, g, plan, stream);
+}
+
+bool launch_gate_cluster(const GateParams& p, cudaStream_t stream, cudaError_t* err) {
+    if (p.scores_in || p.list_flags || !gate_one_kernel(p.max_blocks)) return false;
+    const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, 0, 0, p.max_blocks);
+    if (plan.S == 0) return false;
+    CUtensorMap none;
+    DecodeParams d;
+    memset(&none, 0, sizeof none);
+    memset(&d, 0, sizeof d);
+    d.seq_lens = p.seq_lens;
+    d.num_kv_heads = p.num_kv_heads;
+    d.num_units = p.batch * p.num_kv_heads;
+    d.group = p.group;
+    d.q_len = p.q_len;
+    d.rows = plan.rows;
+    d.status = p.status;
+    *err = launch_step_cluster(none, none, d, &p, plan, stream);
+    return true;
 }
 
 }  // namespace seer

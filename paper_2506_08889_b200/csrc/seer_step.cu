@@ -646,29 +646,29 @@ __device__ __noinline__ float score_key_plain(const uint4* key, const GateScratc
 
 // Scores of this warp's key tiles, by MMAs: tiles warp, warp + NW, ... of the CTA's run of the unit's tiles of 16 keys.  A
 // lane holds the pieces lane % 4 + 4 * x of keys lane / 4 and lane / 4 + 8,
-// straight from global memory: XU = min(XS, 4) of each key at a time (32 registers; keys of 256 channels in two halves).
+// straight from global memory (32 registers; of keys of 256 channels 64).
 // The B operand is the gate queries: columns 4t .. 4t + 3 are query token t's channels, the high part in the first two (one
 // with the first and one with the last eight channels of an MMA, zero elsewhere: of sums half as long the MMA cuts off
 // less), the middle and low parts in the others.  Both operands' contraction index is permuted alike: piece x of a lane is
 // two MMAs' operand as it lies in memory.
 template <int XS, bool MULTI>
 struct KeyScores {
-    static constexpr int XU = XS < 4 ? XS : 4, kHalves = XS / XU, kDepth = 4 / XU;      // tiles requested ahead
-    uint4 a[kDepth][2 * XU];
+    static constexpr int kDepth = XS < 4 ? 4 / XS : 1;     // tiles requested ahead
+    uint4 a[kDepth][2 * XS];
 
-    __device__ __forceinline__ void request(int d, const uint4* kc, int tile, int half, int max_blocks, int lane) {
+    __device__ __forceinline__ void request(int d, const uint4* kc, int tile, int max_blocks, int lane) {
         const int j = kKeyTile * tile + (lane >> 2);
-        const uint4* src = kc + (size_t)j * (4 * XS) + 16 * half + (lane & 3);
+        const uint4* src = kc + (size_t)j * (4 * XS) + (lane & 3);
 #pragma unroll
-        for (int x = 0; x < XU; ++x) {
+        for (int x = 0; x < XS; ++x) {
             a[d][2 * x] = j < max_blocks ? __ldcg(src + 4 * x) : make_uint4(0u, 0u, 0u, 0u);
             a[d][2 * x + 1] = j + 8 < max_blocks ? __ldcg(src + 32 * XS + 4 * x) : make_uint4(0u, 0u, 0u, 0u);
         }
     }
     // The sums of rows lane / 4 and lane / 4 + 8 of the tile in a[d], the largest over the query tokens, the same in a row's
-    // four lanes; `odd`: one of the sums is not finite.  `more(half)` asks for a half of the tile; `next` for another tile.
-    template <typename More, typename Next>
-    __device__ __forceinline__ void sums(int d, const GateScratch& gs, int q_len, int lane, float& v0, float& v1, bool& odd, More&& more, Next&& next) {
+    // four lanes; `odd`: one of the sums is not finite.  `next` asks for another tile.
+    template <typename Next>
+    __device__ __forceinline__ void sums(int d, const GateScratch& gs, int q_len, int lane, float& v0, float& v1, bool& odd, Next&& next) {
         v0 = v1 = -INFINITY;
         odd = false;
 #pragma unroll 1
@@ -680,19 +680,15 @@ struct KeyScores {
             const uint32_t even = t < q_len && col != 1 ? 0xffffffffu : 0u, odd_w = t < q_len && col != 0 ? 0xffffffffu : 0u;
             const uint4* bq = reinterpret_cast<const uint4*>(gs.parts[min(t, q_len - 1)][max(0, col - 1)]) + (lane & 3);
 #pragma unroll
-            for (int half = 0; half < kHalves; ++half) {
-                if (kHalves > 1 && (half > 0 || nt > 0)) more(half);
+            for (int x = 0; x < XS; ++x) {
+                const uint4 b = bq[4 * x];
+                const uint4 lo = a[d][2 * x], hi = a[d][2 * x + 1];
+                const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
+                float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_bf16_16816(c0, a0, b.x & even, b.y & odd_w);
+                mma_bf16_16816(c1, a1, b.z & even, b.w & odd_w);
 #pragma unroll
-                for (int x = 0; x < XU; ++x) {
-                    const uint4 b = bq[4 * (half * XU + x)];
-                    const uint4 lo = a[d][2 * x], hi = a[d][2 * x + 1];
-                    const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
-                    float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma_bf16_16816(c0, a0, b.x & even, b.y & odd_w);
-                    mma_bf16_16816(c1, a1, b.z & even, b.w & odd_w);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) s[c] += c0[c] + c1[c];
-                }
+                for (int c = 0; c < 4; ++c) s[c] += c0[c] + c1[c];
             }
             if (2 * nt + 2 >= q_len) next();
             // lanes 0 and 2 of a row's four have a token's high part, 1 and 3 its middle and low parts
@@ -918,11 +914,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             using Keys = KeyScores<XS, MULTI>;
             Keys ks;
             constexpr int kDepth = Keys::kDepth;
-            auto request = [&](int d, int m, int half) {
-                if (m < my_tiles) ks.request(d, kc, tile0 + m, half, g.max_blocks, lane);
+            auto request = [&](int d, int m) {
+                if (m < my_tiles) ks.request(d, kc, tile0 + m, g.max_blocks, lane);
             };
 #pragma unroll
-            for (int d = 0; d < kDepth; ++d) request(d, warp + d * NW, 0);
+            for (int d = 0; d < kDepth; ++d) request(d, warp + d * NW);
             if (!wait_sent(&sm.got_query, p.status)) dead = true;
             const float inv = rsqrtf((float)g.d_gate);
             uint32_t kmn = 0xffffffffu, kmx = 0u;
@@ -935,8 +931,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         const int j0 = kKeyTile * (tile0 + m);
                         float v0, v1;
                         bool odd;
-                        ks.sums(d, gs, q_len, lane, v0, v1, odd, [&](int half) { request(d, m, half); },
-                                [&]() { request(d, m + kDepth * NW, 0); });
+                        ks.sums(d, gs, q_len, lane, v0, v1, odd, [&]() { request(d, m + kDepth * NW); });
                         // lane 4r has the score of key r, lane 4r + 1 (the others alike) that of key r + 8
                         const int k_of = (lane >> 2) + 8 * (lane & 1), j = j0 + k_of;
                         float v = (lane & 1) ? v1 : v0;
@@ -1344,29 +1339,32 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     if (!producer) {
         wait_sent(&sm.got_parts, p.status);
         cluster_arrive();
-        // S lanes per channel pair, one per source CTA
         const int c_shift = 7 - s_shift;
+        const int pairs = rows << (c_shift - 1);           // channel pairs of this CTA's slice, all rows
 #pragma unroll 1
-        for (int x = tid; x < rows * (kHeadDim / 2); x += kWorkers) {
-            const int s = x & (S - 1), c = 2 * ((x >> s_shift) & ((1 << (c_shift - 1)) - 1)), r = x >> 6;
-            const float2 ml = sm.recv_ml[s][r], v = *reinterpret_cast<const float2*>(&sm.recv_o[((s * kRows + r) << c_shift) + c]);
-            float M = ml.x;
-#pragma unroll 1
-            for (int o = 1; o < S; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-            const float f = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - M);
-            float l = ml.y * f, a0 = v.x * f, a1 = v.y * f;
-#pragma unroll 1
-            for (int o = 1; o < S; o <<= 1) {
-                l += __shfl_xor_sync(0xffffffffu, l, o);
-                a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-                a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+        for (int x = tid; x < pairs; x += kWorkers) {
+            const int r = x >> (c_shift - 1), c = 2 * (x & ((1 << (c_shift - 1)) - 1));
+            float M = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f;
+            float2 ml[kMaxS];
+#pragma unroll
+            for (int s = 0; s < kMaxS; ++s) {
+                ml[s] = s < S ? sm.recv_ml[s][r] : make_float2(-INFINITY, 0.f);
+                M = fmaxf(M, ml[s].x);
             }
-            if (s == 0) {
-                const float inv = l > 0.f ? 1.f / l : 0.f;
-                const size_t row = out_row(r);
-                *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
-                if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+#pragma unroll
+            for (int s = 0; s < kMaxS; ++s) {
+                if (s < S) {
+                    const float f = ml[s].x == -INFINITY ? 0.f : fast_exp2(ml[s].x - M);
+                    const float2 v = *reinterpret_cast<const float2*>(&sm.recv_o[((s * kRows + r) << c_shift) + c]);
+                    l = fmaf(ml[s].y, f, l);
+                    a0 = fmaf(v.x, f, a0);
+                    a1 = fmaf(v.y, f, a1);
+                }
             }
+            const float inv = l > 0.f ? 1.f / l : 0.f;
+            const size_t row = out_row(r);
+            *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
+            if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
         }
     }
     // No CTA leaves before every one has received all that was sent to it: neither the receiver's shared memory nor the

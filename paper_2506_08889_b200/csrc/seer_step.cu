@@ -279,7 +279,7 @@ __device__ __forceinline__ void select_blocks(Smem& sm, GateScratch& gs, const f
         // (every candidate's score is finite then; -0 and +0 have the same bin)
         auto bin_of = [&](float s) -> int { return min(kBins - 1, (int)((s - smin) * scale)); };
         bool found = false;
-        // Up to eight candidates a thread: they stay in its registers from the histogram to the list.
+        // Up to sixteen candidates a thread: they stay in its registers from the histogram to the list.
         auto in_registers = [&](auto q_c) -> bool {
             constexpr int Q = decltype(q_c)::value;
             const int j0 = 4 * Q * tid, end = (n_cand + kKeyTile - 1) & ~(kKeyTile - 1);
@@ -317,12 +317,15 @@ __device__ __forceinline__ void select_blocks(Smem& sm, GateScratch& gs, const f
             for (; taken; taken &= taken - 1) take(at++, j0 + __ffs(taken) - 1);
             return true;
         };
-        if (finite && n_cand <= 8 * kThreads) {
-            if (n_cand <= 4 * kThreads ? in_registers(std::integral_constant<int, 1>()) : in_registers(std::integral_constant<int, 2>())) return;
+        if (finite && n_cand <= 16 * kThreads) {
+            if (n_cand <= 4 * kThreads   ? in_registers(std::integral_constant<int, 1>())
+                : n_cand <= 8 * kThreads ? in_registers(std::integral_constant<int, 2>())
+                                         : in_registers(std::integral_constant<int, 4>()))
+                return;
         }
-        // The short list: from 4096 candidates on, for one place in 32 or fewer.  15625 candidates, 127 places: scores to list
+        // The short list: beyond that, for one place in 32 or fewer.  15625 candidates, 127 places: scores to list
         // 4.5 us, where the histogram over all candidates and the list in one CTA took 12.3.
-        if (finite && n_cand >= 4096 && n_cand > 8 * kThreads && 32 * need <= n_cand) {
+        if (finite && n_cand > 16 * kThreads && 32 * need <= n_cand) {
             ShortList& sl = *reinterpret_cast<ShortList*>(&gs);
             const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile;
             for (int x = tid; x < kStepMaxBlocks / 32; x += kThreads) sl.taken[x] = 0u;
@@ -392,7 +395,7 @@ __device__ __forceinline__ void select_blocks(Smem& sm, GateScratch& gs, const f
             }
             worker_sync<NW>();
         }
-        if (finite && n_cand > 8 * kThreads) {
+        if (finite && n_cand > 16 * kThreads) {
             // Neighbouring blocks have similar scores: the lanes of a warp take candidates that are far apart (lane l has
             // run l of an odd number of blocks: no bank conflicts); side by side, their additions would queue for a few bins.
             const int run = ((n_cand + 31) / 32) | 1;
@@ -804,6 +807,9 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         pdl_wait();                                        // queries, lengths and compressed keys are final
         if (!p.q) pdl_launch_dependents();                 // (the gate alone has no work for which it wants the SMs)
         L = p.seq_lens[i];
+        // (what the second round of loads reads of the queries, if there is one)
+        if (producer && lane < q_len && units > 4 * slices)
+            prefetch_l2(g.q_nope + (((size_t)i * q_len + lane) * g.num_q_heads + (size_t)h * g.group) * kHeadDim, 2 * n);
         if (!producer) load_w(0, slice);
         const int b_shift = 31 - __clz(g.block_size);
         const int n_i = L > 0 ? (L + g.block_size - 1) >> b_shift : 0;
@@ -1452,7 +1458,8 @@ int resident_clusters(bool wide, int k) {
 // the line is at 32 there.  149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles
 // a CTA 45.9 -> 33.8, 52.7 -> 39.1, 59.3 -> 43.1; 64 tiles 93.5 -> 82.1, 108 -> 96, 127 -> 109.
 StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes, int max_keys) {
-    // Above 8192 keys, too, 16 warps a CTA: twice the keys in flight per SM (8 units of 15626 keys: 39.5 -> 33.4 us a step).
+    // Above 8192 keys, too, 16 warps a CTA: twice the keys in flight per SM (a step of
+    // 8 units of 15626 keys 39.5 -> 33.4 us; of 16 units of 9375 keys, blocks of 16, 56.5 -> 49.6).
     const bool wide = rows > 16 || max_keys > 8192;
     StepPlan plan = {0, 1, rows, wide};
     if (rows > 64) return plan;

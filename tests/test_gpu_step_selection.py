@@ -1,4 +1,4 @@
-"""The one-launch step's lists where its selection changes form: candidates in registers (up to eight a thread), a histogram
+"""The one-launch step's lists where its selection changes form: candidates in registers (up to sixteen a thread), a histogram
 over all of them, the short list of many candidates, 16 worker warps above 8192 keys, crowded bins; and scores that are not
 finite, which leave the matrix instructions for plain products."""
 import math
@@ -35,15 +35,15 @@ def scores64(qn, wq, kc, L):
     (2, 4, 1, 128, 16, 1025, 40, ""),          # 1024 candidates: four a thread
     (2, 4, 1, 128, 16, 1026, 40, ""),          # 1025: eight
     (1, 5, 1, 64, 16, 2049, 700, ""),          # 2048
-    (1, 5, 1, 256, 16, 2050, 700, ""),         # 2049: the histogram over all
-    (2, 8, 1, 128, 32, 4096, 100, ""),         # 4095: as before, 4097: the short list
+    (1, 5, 1, 256, 16, 2050, 700, ""),         # 2049: sixteen
+    (2, 8, 1, 128, 32, 4096, 100, ""),         # 4095: as before; 4097: the short list
     (2, 8, 1, 128, 32, 4098, 127, ""),
-    (2, 8, 1, 128, 32, 4098, 129, ""),         # too many places for it
+    (2, 8, 1, 128, 32, 4098, 129, ""),         # too many places for it: the histogram over all
     (1, 4, 1, 128, 16, 8190, 60, "crowded"),   # a far outlier: neither list helps
     (1, 4, 1, 128, 16, 8194, 200, ""),         # 16 worker warps
     (1, 4, 1, 64, 16, 16384, 300, ""),         # the most keys
     (1, 4, 1, 128, 16, 16384, 2000, "ties"),
-    (2, 8, 3, 128, 64, 2050, 33, ""),          # 24 rows: 16 worker warps, eight candidates a thread
+    (2, 8, 3, 128, 64, 2050, 33, ""),          # 24 rows: 16 worker warps
     (1, 8, 8, 64, 64, 4100, 30, ""),           # 64 rows: two clusters a unit
 ])
 def test_lists_against_64_bit_scores(Hkv, g, T, dg, b, n, need, kind):

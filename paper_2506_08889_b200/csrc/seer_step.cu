@@ -43,6 +43,7 @@ constexpr int kFew = 1024;                                 // candidates (and ke
 constexpr int kMergeStride = 132;                          // floats per row of a warp's partial (bank spread)
 constexpr int kKeyTile = 16;                               // keys are dealt to the cluster's warps in tiles of 16
 constexpr int kMaxQLen = 8;
+constexpr int kKeySlots = 32;                              // most key tiles that a CTA has asked for at a time (a lane each)
 
 // Two sizes.  NW = 8 worker warps (gate, consumers, combine) and a ring of three stages: two CTAs per SM, up to 16
 // rows (8 without MULTI).  NW = 16 and five stages: one CTA per SM, up to 32 rows.
@@ -57,9 +58,9 @@ struct Size {
 template <int NW, bool MULTI>
 struct __align__(1024) StepSmem {
     using Z = Size<NW, MULTI>;
-    // K/V ring.  Before the first tile is asked for, the gate's: the scores of the unit (up to kStepMaxBlocks) in stages 0
-    // and 1, GateScratch behind them.  After the last tile: the warps' partials.
-    unsigned char ring[Z::kStages][kStageBytes];
+    // K/V ring.  Before the first tile is asked for, the gate's: the scores of the unit (up to kStepMaxBlocks) at its
+    // beginning, GateScratch at its end, compressed keys on their way between them.  After the last tile: the warps' partials.
+    unsigned char ring[Z::kStages * kStageBytes];
     // what the cluster's CTAs send after their last tile (a fast one while this one still selects: memory of its own)
     __align__(16) float recv_o[Z::kRows * kHeadDim];       // [source CTA][row][this CTA's slice of the channels]
     float2 recv_ml[kMaxS][Z::kRows];                       // [source CTA][row]: max, sum
@@ -69,6 +70,7 @@ struct __align__(1024) StepSmem {
     // residue, so its groups follow all of its phases.  (With a barrier per stage a group would miss the others' phases
     // and could take one that is two back for the one that it waits for.)
     uint64_t full[Z::kArrivals], empty[Z::kStages];
+    uint64_t key_full[kKeySlots];
     uint64_t got_query, got_scores, got_feat, got_parts;   // bytes from the cluster's CTAs
     int meta[Z::kArrivals];                                // tokens from the tile's first row on (blocks of 16 or 32 tokens: per block, 8 bits each)
     int codes[kCodes];                                     // GATE: this CTA's tiles: 64-token tile numbers, or the gathered blocks
@@ -86,15 +88,16 @@ struct __align__(1024) StepSmem {
 };
 static_assert(sizeof(StepSmem<8, true>) + 1024 <= 113 * 1024, "two CTAs per SM");
 static_assert(sizeof(StepSmem<16, true>) + 1024 <= 227 * 1024, "one CTA per SM");
-// The gate's part of the ring (stage 2).
+// The gate's part of the ring, at its end.
+template <int NW, bool MULTI>
 struct GateScratch {
     // Gate queries, from all CTAs: each channel in three bf16 parts (high, middle, low), which together are the fp32 number
     // exactly, two channels a word.  (Rows 64 bytes longer than the channels: neighbouring parts are in different banks.)
-    __align__(16) uint32_t parts[kMaxQLen][3][kMaxDGate / 2 + 16];
-    float sums[16][16][8];                                 // partial sums of the gate query: [warp][row][token]
+    __align__(16) uint32_t parts[MULTI ? kMaxQLen : 1][3][kMaxDGate / 2 + 16];
+    float sums[NW][16][8];                                 // partial sums of the gate query: [warp][row][token]
     __align__(16) int hist[kBins];                         // selection
 };
-// ... and of the selection, when the queries have been used.
+// ... and of the selection, when queries and keys have been used.
 struct ShortList {
     unsigned taken[kStepMaxBlocks / 32];                   // a bit per candidate
     float tile_max[kStepMaxBlocks / kKeyTile];             // largest score of a key tile
@@ -102,9 +105,17 @@ struct ShortList {
     float score[kFew];                                     // their candidates that may be taken
     int j[kFew];
 };
-static_assert(sizeof(ShortList) <= offsetof(GateScratch, hist) && kStepMaxBlocks / kKeyTile <= kFew, "the short list's place");
-static_assert(kStepMaxBlocks <= 64 * 256, "a bit per candidate of a lane");
-static_assert(kStepMaxBlocks * 4 <= 2 * kStageBytes && sizeof(GateScratch) <= kStageBytes, "the gate's use of the ring");
+template <int NW, bool MULTI>
+struct GatePlace {                                         // offsets in the ring
+    using Scratch = GateScratch<NW, MULTI>;
+    static constexpr int kRing = Size<NW, MULTI>::kStages * kStageBytes;
+    static constexpr int kScratch = kRing - (int)sizeof(Scratch);
+    static constexpr int kShort = kRing - (int)sizeof(Scratch::hist) - (int)sizeof(ShortList);
+    static_assert(offsetof(Scratch, hist) + sizeof(Scratch::hist) == sizeof(Scratch), "the histogram comes last");
+    static_assert(kScratch % 16 == 0 && kShort % 16 == 0 && kShort >= 4 * kStepMaxBlocks, "behind the scores");
+    static_assert(kScratch - 4 * kStepMaxBlocks - 64 >= 2 * kKeyTile * kMaxDGate, "room for a key tile whatever there is to score");
+};
+static_assert(kStepMaxBlocks / kKeyTile <= kFew && kStepMaxBlocks <= 64 * 256, "the short list's tiles; a bit per candidate of a lane");
 
 // Barriers among the worker warps, and between them and the producer.  The aligned forms are for a warp whose lanes are
 // together; behind a loop or branch of some lanes they need not be, so they are brought together here.
@@ -199,10 +210,9 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status) {
 // on its longest path (some ten cycles each, mostly their fetch) and not the candidates; hence rolled loops, whose
 // bodies stay in the instruction buffers, and one candidate a lane and turn.
 template <int NW, typename Smem, typename Take>
-__device__ __forceinline__ void select_blocks(Smem& sm, GateScratch& gs, const float* sc, int n_cand, int need, int warp, int lane, Take&& take) {
+__device__ __forceinline__ void select_blocks(Smem& sm, int* hist, ShortList& sl, const float* sc, int n_cand, int need, int warp, int lane, Take&& take) {
     constexpr int kThreads = 32 * NW, kPer = kBins / kThreads;
     const int tid = 32 * warp + lane;
-    int* hist = gs.hist;
     if (need <= 0) return;
     // candidate j is taken if its key is above thr, or equal to it and j <= j_eq
     uint32_t thr = 0u;
@@ -326,7 +336,6 @@ __device__ __forceinline__ void select_blocks(Smem& sm, GateScratch& gs, const f
         // The short list: beyond that, for one place in 32 or fewer.  15625 candidates, 127 places: scores to list
         // 4.5 us, where the histogram over all candidates and the list in one CTA took 12.3.
         if (finite && n_cand > 16 * kThreads && 32 * need <= n_cand) {
-            ShortList& sl = *reinterpret_cast<ShortList*>(&gs);
             const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile;
             for (int x = tid; x < kStepMaxBlocks / 32; x += kThreads) sl.taken[x] = 0u;
             // (places of the last tile behind the last candidate hold minus infinity)
@@ -624,7 +633,7 @@ __device__ __forceinline__ void rope_sincos_wide(double pos, double inv_freq, do
 
 // The score of one key by plain dot products (whole warp; the largest over the query tokens): for a key or gate query that
 // is not finite, where the parts of the query (score_keys) would make NaN of what is an infinity.
-__device__ __noinline__ float score_key_plain(const uint4* key, const GateScratch& gs, int q_len, int d_gate, int lane) {
+__device__ __noinline__ float score_key_plain(const uint4* key, const uint32_t (*parts)[3][kMaxDGate / 2 + 16], int q_len, int d_gate, int lane) {
     const uint4 kv = lane < d_gate / 8 ? __ldcg(key + lane) : make_uint4(0u, 0u, 0u, 0u);
     float best = -INFINITY;
     for (int t = 0; t < q_len; ++t) {
@@ -633,8 +642,8 @@ __device__ __noinline__ float score_key_plain(const uint4* key, const GateScratc
             float q[8];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const float2 hi = bf16x2_to_float2(gs.parts[t][0][4 * lane + c]), mid = bf16x2_to_float2(gs.parts[t][1][4 * lane + c]),
-                             low = bf16x2_to_float2(gs.parts[t][2][4 * lane + c]);
+                const float2 hi = bf16x2_to_float2(parts[t][0][4 * lane + c]), mid = bf16x2_to_float2(parts[t][1][4 * lane + c]),
+                             low = bf16x2_to_float2(parts[t][2][4 * lane + c]);
                 q[2 * c] = hi.x + (mid.x + low.x);
                 q[2 * c + 1] = hi.y + (mid.y + low.y);
             }
@@ -647,65 +656,76 @@ __device__ __noinline__ float score_key_plain(const uint4* key, const GateScratc
     return best;
 }
 
-// Scores of this warp's key tiles, by MMAs: tiles warp, warp + NW, ... of the CTA's run of the unit's tiles of 16 keys.  A
-// lane holds the pieces lane % 4 + 4 * x of keys lane / 4 and lane / 4 + 8,
-// straight from global memory (32 registers; of keys of 256 channels 64).
+// The key tiles of a CTA (a run of the unit's keys) on their way through the ring: tile m comes in slot m mod `n` and slot s
+// belongs to warp s mod NW.  A tile of 16 keys is two bulk copies, of its first and of its last eight keys; the second halves'
+// memory begins 64 bytes off a bank line, so that lanes that read the same channels of a key of either half read different
+// banks.  The producer warp asks for the slots' first tiles, a warp for its slots' others.  (What bounds the scores of many keys
+// is how many are under way while the queries are made.  With a tile a warp, in its registers -- 64 of them for keys of 256
+// channels, which spilled -- a step of batch 8 at 128k took 83.5 us and takes 82.7, with 64 blocks 40.3 and 38.6, of two
+// sequences of 90k with 256 channels 32.2 and 24.0.)
+struct KeySlots {
+    unsigned char *a, *b;                                  // the halves of slot 0
+    int n, shift;                                          // shift: log2 of a half's bytes
+
+    __device__ __forceinline__ void place(unsigned char* ring, int n_tiles, int end, int d_gate) {
+        const int first = (n_tiles * kKeyTile * 4 + 127) & ~127;
+        shift = 34 - __clz(2 * d_gate);
+        n = min((end - first - 64) >> (shift + 1), kKeySlots);
+        a = ring + first;
+        b = a + (n << shift) + 64;
+    }
+    __device__ __forceinline__ void request(int slot, uint64_t* full, const unsigned char* keys, int rows) const {      // rows: keys there are, from the tile's first one on
+        const int na = min(rows, 8) << (shift - 3), nb = max(0, min(rows, 16) - 8) << (shift - 3);
+        mbar_arrive_expect_tx(full, (uint32_t)(na + nb));
+        bulk_load(a + (slot << shift), keys, (uint32_t)na, full);
+        if (nb > 0) bulk_load(b + (slot << shift), keys + (1 << shift), (uint32_t)nb, full);
+    }
+};
+
+// The sums of a key tile, by MMAs: row r of the first eight of the A operand is key (r & 1) * 8 + r / 2, row r + 8 the key
+// four behind it.  A lane supplies the pieces lane % 4 + 4 * x of its rows' keys: `pieces` gives them.
 // The B operand is the gate queries: columns 4t .. 4t + 3 are query token t's channels, the high part in the first two (one
 // with the first and one with the last eight channels of an MMA, zero elsewhere: of sums half as long the MMA cuts off
 // less), the middle and low parts in the others.  Both operands' contraction index is permuted alike: piece x of a lane is
 // two MMAs' operand as it lies in memory.
-template <int XS, bool MULTI>
-struct KeyScores {
-    static constexpr int kDepth = XS < 4 ? 4 / XS : 1;     // tiles requested ahead
-    uint4 a[kDepth][2 * XS];
-
-    __device__ __forceinline__ void request(int d, const uint4* kc, int tile, int max_blocks, int lane) {
-        const int j = kKeyTile * tile + (lane >> 2);
-        const uint4* src = kc + (size_t)j * (4 * XS) + (lane & 3);
+// v0, v1: the sums of rows lane / 4 and lane / 4 + 8, the largest over the query tokens, the same in a row's four lanes; `odd`:
+// one of the sums is not finite.
+template <int XS, bool MULTI, typename Pieces>
+__device__ __forceinline__ void key_sums(Pieces&& pieces, const uint32_t (*parts)[3][kMaxDGate / 2 + 16], int q_len, int lane, float& v0, float& v1,
+                                         bool& odd) {
+    v0 = v1 = -INFINITY;
+    odd = false;
+#pragma unroll 1
+    for (int nt = 0; 2 * nt < q_len; ++nt) {
+        // (each MMA begins at zero and its 16 products are added up outside: the MMA's own accumulation cuts off where the
+        // addition rounds to nearest)
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        const int col = (lane >> 2) & 3, t = 2 * nt + (lane >> 4);
+        const uint32_t even = t < q_len && col != 1 ? 0xffffffffu : 0u, odd_w = t < q_len && col != 0 ? 0xffffffffu : 0u;
+        const uint4* bq = reinterpret_cast<const uint4*>(parts[min(t, q_len - 1)][max(0, col - 1)]) + (lane & 3);
 #pragma unroll
         for (int x = 0; x < XS; ++x) {
-            a[d][2 * x] = j < max_blocks ? __ldcg(src + 4 * x) : make_uint4(0u, 0u, 0u, 0u);
-            a[d][2 * x + 1] = j + 8 < max_blocks ? __ldcg(src + 32 * XS + 4 * x) : make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
-    // The sums of rows lane / 4 and lane / 4 + 8 of the tile in a[d], the largest over the query tokens, the same in a row's
-    // four lanes; `odd`: one of the sums is not finite.  `next` asks for another tile.
-    template <typename Next>
-    __device__ __forceinline__ void sums(int d, const GateScratch& gs, int q_len, int lane, float& v0, float& v1, bool& odd, Next&& next) {
-        v0 = v1 = -INFINITY;
-        odd = false;
-#pragma unroll 1
-        for (int nt = 0; 2 * nt < q_len; ++nt) {
-            // (each MMA begins at zero and its 16 products are added up outside: the MMA's own accumulation cuts off where the
-            // addition rounds to nearest)
-            float s[4] = {0.f, 0.f, 0.f, 0.f};
-            const int col = (lane >> 2) & 3, t = 2 * nt + (lane >> 4);
-            const uint32_t even = t < q_len && col != 1 ? 0xffffffffu : 0u, odd_w = t < q_len && col != 0 ? 0xffffffffu : 0u;
-            const uint4* bq = reinterpret_cast<const uint4*>(gs.parts[min(t, q_len - 1)][max(0, col - 1)]) + (lane & 3);
+            const uint4 b = bq[4 * x];
+            uint4 lo, hi;
+            pieces(x, lo, hi);
+            const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
+            float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16_16816(c0, a0, b.x & even, b.y & odd_w);
+            mma_bf16_16816(c1, a1, b.z & even, b.w & odd_w);
 #pragma unroll
-            for (int x = 0; x < XS; ++x) {
-                const uint4 b = bq[4 * x];
-                const uint4 lo = a[d][2 * x], hi = a[d][2 * x + 1];
-                const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
-                float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
-                mma_bf16_16816(c0, a0, b.x & even, b.y & odd_w);
-                mma_bf16_16816(c1, a1, b.z & even, b.w & odd_w);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) s[c] += c0[c] + c1[c];
-            }
-            if (2 * nt + 2 >= q_len) next();
-            // lanes 0 and 2 of a row's four have a token's high part, 1 and 3 its middle and low parts
-            float r0 = s[0] + s[1], r1 = s[2] + s[3];
-            r0 += __shfl_xor_sync(0xffffffffu, r0, 1);
-            r1 += __shfl_xor_sync(0xffffffffu, r1, 1);
-            odd |= !(fabsf(r0) < INFINITY) || !(fabsf(r1) < INFINITY);
-            if (2 * nt + ((lane >> 1) & 1) >= q_len) r0 = r1 = -INFINITY;
-            v0 = fmaxf(v0, fmaxf(r0, __shfl_xor_sync(0xffffffffu, r0, 2)));
-            v1 = fmaxf(v1, fmaxf(r1, __shfl_xor_sync(0xffffffffu, r1, 2)));
-            if (!MULTI) break;
+            for (int c = 0; c < 4; ++c) s[c] += c0[c] + c1[c];
         }
+        // lanes 0 and 2 of a row's four have a token's high part, 1 and 3 its middle and low parts
+        float r0 = s[0] + s[1], r1 = s[2] + s[3];
+        r0 += __shfl_xor_sync(0xffffffffu, r0, 1);
+        r1 += __shfl_xor_sync(0xffffffffu, r1, 1);
+        odd |= !(fabsf(r0) < INFINITY) || !(fabsf(r1) < INFINITY);
+        if (2 * nt + ((lane >> 1) & 1) >= q_len) r0 = r1 = -INFINITY;
+        v0 = fmaxf(v0, fmaxf(r0, __shfl_xor_sync(0xffffffffu, r0, 2)));
+        v1 = fmaxf(v1, fmaxf(r1, __shfl_xor_sync(0xffffffffu, r1, 2)));
+        if (!MULTI) break;
     }
-};
+}
 
 // grid (S, units), cluster (S, 1, 1).  Short calls are bound by latency, and that by the number of instructions on the
 // longest path: all of this runs once, by two warps a scheduler, at some ten cycles an instruction.  A step of 8 units x 64
@@ -722,6 +742,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     using Z = Size<NW, MULTI>;
     using Smem = StepSmem<NW, MULTI>;
     constexpr int kWorkers = Z::kWorkers, kStages = Z::kStages, kArrivals = Z::kArrivals, kRows = Z::kRows;
+    using Place = GatePlace<NW, MULTI>;
     extern __shared__ unsigned char smem_raw[];
     // (aligned by an offset, not by a cast through an integer: the compiler then still knows the accesses for shared ones)
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023));
@@ -737,8 +758,9 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     // eight rows are an MMA's N side: `tiles_n` consumer groups share a K/V tile, `paces` such teams take alternate tiles
     const int tiles_n = MULTI ? (rows + 7) >> 3 : 1;
     const int paces = MULTI ? Z::kGroups / tiles_n : Z::kGroups;
-    if (tid < kArrivals) {
-        mbar_init(&sm.full[tid], 1);
+    if (tid < 32) {
+        if (GATE) mbar_init(&sm.key_full[tid], 1);
+        if (tid < kArrivals) mbar_init(&sm.full[tid], 1);
         if (tid < kStages) mbar_init(&sm.empty[tid], 4 * tiles_n);
         if (tid == 0) {
             mbar_init(&sm.got_query, 1);
@@ -770,7 +792,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     if constexpr (GATE) {
         const GateParams& g = ga.g;
         const int n = g.group * kHeadDim, half = g.d_gate / 2;
-        const uint4* kc = reinterpret_cast<const uint4*>(g.kcomp + (size_t)u * g.max_blocks * g.d_gate);
+        const unsigned char* kc = reinterpret_cast<const unsigned char*>(g.kcomp + (size_t)u * g.max_blocks * g.d_gate);
         // Gate query: a CTA makes the rotary pairs (c, c + d_gate/2) c_first .. c_first + ppc of all query tokens, by MMAs of 16
         // rows of W_q (eight pairs) by 8 tokens; the contraction, in units of 32 channels, is split over the warps that share
         // a row tile (`slices` of them), whose partial sums meet in shared memory.  A lane holds pieces of 16 bytes as they lie
@@ -799,8 +821,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         };
         // (W_q into L2 only, which follows later writes: the kernel before this one may be the one that makes it)
         if (producer && lane < 2) prefetch_l2(g.w_q + ((size_t)h * g.d_gate + c_first + lane * half) * n, 2 * n * ppc);
-        float* sc_all = reinterpret_cast<float*>(sm.ring[0]);
-        GateScratch& gs = *reinterpret_cast<GateScratch*>(sm.ring[2]);
+        float* sc_all = reinterpret_cast<float*>(sm.ring);
+        auto& gs = *reinterpret_cast<typename Place::Scratch*>(sm.ring + Place::kScratch);
         if (!producer) {
             for (int x = tid; x < kBins; x += kWorkers) gs.hist[x] = 0;
         }
@@ -826,21 +848,16 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             need = max(0, min(min(k - n_forced, n_cand), kListed));
             n_blocks = need + n_forced;
         }
-        // This CTA's key tiles: a run of those with a candidate.  The producer warp asks for them into L2, so that they travel
-        // while the gate query is made.
+        // This CTA's key tiles: a run of those with a candidate.  The producer warp asks for them, as many as there are slots for
+        // and the others into L2, so that they travel while the gate query is made.
         const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile, per_cta = (n_tiles + S - 1) >> s_shift;
         const int tile0 = min(rank * per_cta, n_tiles), my_tiles = min(per_cta, n_tiles - tile0);
+        KeySlots slots;
+        slots.place(sm.ring, n_tiles, Place::kScratch, g.d_gate);
         // who selects: every CTA that will read tiles, or (the gate alone) the first one
         const int n_sel = p.q ? S : 1, sel_shift = p.q ? s_shift : 0;
         const bool selects = rank < n_sel;
         if (producer) {
-            // (the tiles behind each warp's first; few requests to a lane, each of which takes the warp some fifty nanoseconds)
-            const int later = max(0, my_tiles - NW), step = (later + 31) >> 5;
-            if (lane * step < later) {
-                const int m = NW + lane * step, j = kKeyTile * (tile0 + m);
-                prefetch_l2(g.kcomp + ((size_t)u * g.max_blocks + j) * g.d_gate,
-                            min(kKeyTile * min(step, my_tiles - m), g.max_blocks - j) * g.d_gate * 2);
-            }
             // (the scores of the other CTAs' key tiles, and from every CTA their smallest and largest key)
             if (selects && lane == 0) mbar_arrive_expect_tx(&sm.got_scores, (uint32_t)((n_tiles - my_tiles) * kKeyTile * 4 + S * 8));
             if (appends && lane < 3) {
@@ -849,6 +866,20 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         }
         cluster_wait();                                    // every CTA of the cluster has started
+        if (producer) {
+            const int ready = min(my_tiles, slots.n);
+            if (lane < ready) {
+                const int j = kKeyTile * (tile0 + lane);
+                slots.request(lane, &sm.key_full[lane], kc + ((size_t)j << (slots.shift - 3)), g.max_blocks - j);
+            }
+            // (few requests to a lane, each of which takes the warp some fifty nanoseconds)
+            const int later = my_tiles - ready, step = (later + 31) >> 5;
+            if (lane * step < later) {
+                const int m = ready + lane * step, j = kKeyTile * (tile0 + m);
+                prefetch_l2(kc + ((size_t)j << (slots.shift - 3)),
+                            min(kKeyTile * min(step, my_tiles - m), g.max_blocks - j) << (slots.shift - 3));
+            }
+        }
         // ---- gate query ------------------------------------------------------------------------------------------------
         if (!producer) {
             float (*part)[16][8] = gs.sums;
@@ -917,52 +948,85 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         // (keys through L2, not the read-only path: the entry that this launch appends, or the step before it did, is among them)
         auto scores = [&](auto xs_c) {
             constexpr int XS = decltype(xs_c)::value;
-            using Keys = KeyScores<XS, MULTI>;
-            Keys ks;
-            constexpr int kDepth = Keys::kDepth;
-            auto request = [&](int d, int m) {
-                if (m < my_tiles) ks.request(d, kc, tile0 + m, g.max_blocks, lane);
-            };
-#pragma unroll
-            for (int d = 0; d < kDepth; ++d) request(d, warp + d * NW);
-            if (!wait_sent(&sm.got_query, p.status)) dead = true;
             const float inv = rsqrtf((float)g.d_gate);
             uint32_t kmn = 0xffffffffu, kmx = 0u;
+            // this lane's first piece of its first key in slot 0; the second key is kOff bytes behind the first
+            const int rr = lane >> 2, k_of = 8 * (rr & 1) + (rr >> 1) + 4 * (lane & 1);
+            const unsigned char* at = ((rr & 1) ? slots.b : slots.a) + (rr >> 1) * (64 * XS) + 16 * (lane & 3);
+            constexpr int kOff = 4 * (64 * XS);
+            int slot = warp, use = 0;
+            bool asked = false;
 #pragma unroll 1
-            for (int m0 = warp; m0 < my_tiles; m0 += kDepth * NW) {
+            for (int m = warp < slots.n ? warp : my_tiles;;) {
+                const bool mine = m < my_tiles;
+                const int j0 = kKeyTile * (tile0 + m), j = j0 + k_of;
+                const unsigned char* here = at + (slot << slots.shift);
+                auto in_slot = [&](int x, uint4& lo, uint4& hi) {
+                    lo = *reinterpret_cast<const uint4*>(here + 64 * x);
+                    hi = *reinterpret_cast<const uint4*>(here + kOff + 64 * x);
+                };
+                auto refill = [&]() {
+                    __syncwarp();                          // (all lanes have read the slot)
+                    if (lane == 0 && m + slots.n < my_tiles) {
+                        const int jn = j0 + kKeyTile * slots.n;
+                        fence_proxy_async_smem();
+                        slots.request(slot, &sm.key_full[slot], kc + (size_t)jn * (64 * XS), g.max_blocks - jn);
+                    }
+                };
+                uint4 held[2 * XS];                        // (not of 256 channels, which would be half of the thread's registers)
+                if (mine) {
+                    if (__any_sync(0xffffffffu, !mbar_wait(&sm.key_full[slot], use & 1, p.status))) {
+                        dead = true;
+                        break;
+                    }
+                    if constexpr (XS < 8) {
 #pragma unroll
-                for (int d = 0; d < kDepth; ++d) {
-                    const int m = m0 + d * NW;
-                    if (m < my_tiles) {
-                        const int j0 = kKeyTile * (tile0 + m);
-                        float v0, v1;
-                        bool odd;
-                        ks.sums(d, gs, q_len, lane, v0, v1, odd, [&]() { request(d, m + kDepth * NW); });
-                        // lane 4r has the score of key r, lane 4r + 1 (the others alike) that of key r + 8
-                        const int k_of = (lane >> 2) + 8 * (lane & 1), j = j0 + k_of;
-                        float v = (lane & 1) ? v1 : v0;
-                        unsigned odds = __ballot_sync(0xffffffffu, odd);
-                        if (odds) {
+                        for (int x = 0; x < XS; ++x) in_slot(x, held[2 * x], held[2 * x + 1]);
+                        refill();
+                    }
+                }
+                if (!asked) {                              // (the first keys are there before the queries are)
+                    asked = true;
+                    if (!wait_sent(&sm.got_query, p.status)) dead = true;
+                }
+                if (!mine) break;
+                float v0, v1;
+                bool odd;
+                if constexpr (XS < 8) {
+                    key_sums<XS, MULTI>([&](int x, uint4& lo, uint4& hi) { lo = held[2 * x]; hi = held[2 * x + 1]; }, gs.parts, q_len, lane, v0, v1, odd);
+                } else {
+                    key_sums<XS, MULTI>(in_slot, gs.parts, q_len, lane, v0, v1, odd);
+                    refill();
+                }
+                // lane 4r has the score of row r, lane 4r + 1 (the others alike) that of row r + 8
+                float v = (lane & 1) ? v1 : v0;
+                const unsigned odds = __ballot_sync(0xffffffffu, odd);
+                if (odds) {
 #pragma unroll 1
-                            for (int k = 0; k < kKeyTile; ++k) {
-                                if (((odds >> (4 * (k & 7))) & 15u) && j0 + k < n_cand) {
-                                    const float x = score_key_plain(kc + (size_t)(j0 + k) * (4 * XS), gs, q_len, g.d_gate, lane);
-                                    if (k == k_of) v = x;
-                                }
-                            }
-                        }
-                        v *= inv;
-                        if ((lane & 2) == 0) {
-                            const bool ok = j < n_cand;
-                            sc_all[j] = ok ? v : -INFINITY;
-                            if (ok) {
-                                if (g.scores_user) g.scores_user[(size_t)u * g.max_blocks + j] = v;
-                                const uint32_t key = score_key(v);
-                                kmn = min(kmn, key);
-                                kmx = max(kmx, key);
-                            }
+                    for (int k = 0; k < kKeyTile; ++k) {
+                        if (((odds >> (4 * (2 * (k & 3) + (k >> 3)))) & 15u) && j0 + k < n_cand) {
+                            const float x = score_key_plain(reinterpret_cast<const uint4*>(kc + (size_t)(j0 + k) * (64 * XS)), gs.parts, q_len, g.d_gate, lane);
+                            if (k == k_of) v = x;
                         }
                     }
+                }
+                v *= inv;
+                if ((lane & 2) == 0) {
+                    const bool ok = j < n_cand;
+                    sc_all[j] = ok ? v : -INFINITY;
+                    if (ok) {
+                        if (g.scores_user) g.scores_user[(size_t)u * g.max_blocks + j] = v;
+                        const uint32_t key = score_key(v);
+                        kmn = min(kmn, key);
+                        kmx = max(kmx, key);
+                    }
+                }
+                slot += NW;
+                m += NW;
+                if (slot >= slots.n) {                     // (the tile behind the last slot's comes in slot 0)
+                    m += slots.n + warp - slot;
+                    slot = warp;
+                    ++use;
                 }
             }
             kmn = __reduce_min_sync(0xffffffffu, kmn);
@@ -1038,7 +1102,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     if ((t & (S - 1)) == rank && at < kCodes) sm.codes[at] = j;
                 }
             };
-            select_blocks<NW>(sm, gs, sc_all, n_cand, need, warp, lane, take);
+            select_blocks<NW>(sm, gs.hist, *reinterpret_cast<ShortList*>(sm.ring + Place::kShort), sc_all, n_cand, need, warp, lane, take);
             // the last ones: the blocks taken without a score
             if (tid < n_blocks - need) take(need + tid, n_i - n_blocks + need + tid);
             if (lists) {
@@ -1151,7 +1215,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (lane == s) {
                     const int st = it % kStages;
                     if (!dead && !mbar_wait(&sm.empty[st], ((it / kStages) & 1) ^ 1, p.status)) dead = true;
-                    unsigned char* dst = sm.ring[st];
+                    unsigned char* dst = sm.ring + st * kStageBytes;
                     uint64_t* full = &sm.full[it % kArrivals];
                     sm.meta[it % kArrivals] = nv_all;      // (the tile kArrivals back has been read: the one kStages back has, which came after it)
                     if (dead || n_sub == 0) {
@@ -1221,11 +1285,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             if (!dead && !mbar_wait(&sm.full[it % kArrivals], (it / kArrivals) & 1, p.status)) dead = true;
             const int nvw = (small ? (sm.meta[it % kArrivals] >> (8 * sub_w)) & 0xff : sm.meta[it % kArrivals]) - off_w;   // valid tokens from this warp's first row on
             if (nvw > 0 && !dead) {
-                const uint32_t kbase = smem_u32(sm.ring[st]), vbase = kbase + kTileBytes;
+                const uint32_t kbase = smem_u32(sm.ring + st * kStageBytes), vbase = kbase + kTileBytes;
                 if (nvw < 16) {
                     // ragged tail: rows past the sequence end may hold anything; this warp's are cleared in V, so that
                     // a zero probability times garbage cannot produce NaN
-                    unsigned char* vt = sm.ring[st] + kTileBytes;
+                    unsigned char* vt = sm.ring + st * kStageBytes + kTileBytes;
                     for (int x = lane; x < (16 - nvw) * 16; x += 32) {
                         const int r = 16 * w4 + nvw + (x >> 4), part = x & 15;
                         *reinterpret_cast<uint4*>(vt + (part >> 3) * kHalfTileBytes + r * 128 + ((part & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
@@ -1295,7 +1359,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], off);
         }
         worker_sync<NW>();                                     // every tile has been read: the ring is free
-        float* part = reinterpret_cast<float*>(sm.ring[0]) + warp * 8 * kMergeStride;
+        float* part = reinterpret_cast<float*>(sm.ring) + warp * 8 * kMergeStride;
 #pragma unroll
         for (int a = 0; a < 8; ++a) {
             const int d0 = 16 * a + rw;
@@ -1324,7 +1388,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 M = fmaxf(M, ml[x].x);
             }
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float* src = reinterpret_cast<const float*>(sm.ring[0]) + (r & 7) * kMergeStride + c;
+            const float* src = reinterpret_cast<const float*>(sm.ring) + (r & 7) * kMergeStride + c;
 #pragma unroll
             for (int x = 0; x < NW; ++x) {
                 if (x < n_part) {

@@ -327,7 +327,7 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
     if (!gate && ctx->use_clusters && !ctx->chain_attention && !(wide && ctx->wide_variant) && ctx->list_gen == 0 && ctx->sel_from_lens == 0)
-        plan = step_plan(U, q_len * group, max_tiles / U, 0, 0);
+        plan = step_plan(U, q_len * group, q_len, max_tiles / U, 0, 0);
     if (plan.S > 0) {
         p.rows = plan.rows;
         ce = launch_step_cluster(mk_copy, *mv, p, gate, plan, static_cast<cudaStream_t>(stream));
@@ -804,7 +804,7 @@ static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     if (blocks > max_sel) blocks = max_sel;
     if (blocks > cap) blocks = cap;
     const long long tiles = (blocks * bs + kTileTokens - 1) / kTileTokens;
-    return step_plan(shape->batch * shape->num_kv_heads, rows, tiles,
+    return step_plan(shape->batch * shape->num_kv_heads, rows, q_len, tiles,
                      bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles, gate->max_blocks);
 }
 

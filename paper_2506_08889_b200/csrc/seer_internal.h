@@ -137,7 +137,7 @@ struct StepPlan {
     int parts, rows;                    // clusters per unit, which have `rows` of its rows each (the last one the rest)
     bool wide;                          // 16 worker warps per CTA, one CTA per SM (else 8 and two)
 };
-StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes, int max_keys);
+StepPlan step_plan(int units, int rows, int q_len, long long max_tiles, long long max_codes, int max_keys);
 // g == nullptr: attention only, over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.
 cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
                                 const StepPlan& plan, cudaStream_t stream);

@@ -39,7 +39,7 @@ constexpr int kMaxS = 16;
 constexpr int kCodes = 256;                                // tile (or gathered block) numbers that a CTA holds
 constexpr int kListed = 8192;                              // most scored blocks of a list
 constexpr int kBins = 1024;                                // histogram of the selection
-constexpr int kFew = 1024;                                 // candidates (and key tiles) that its short list holds
+constexpr int kFew = 2048;                                 // candidates that its short list holds
 constexpr int kMergeStride = 132;                          // floats per row of a warp's partial (bank spread)
 constexpr int kKeyTile = 16;                               // keys are dealt to the cluster's warps in tiles of 16
 constexpr int kMaxQLen = 8;
@@ -98,24 +98,31 @@ struct GateScratch {
     __align__(16) int hist[kBins];                         // selection
 };
 // ... and of the selection, when queries and keys have been used.
-struct ShortList {
+struct Selected {
     unsigned taken[kStepMaxBlocks / 32];                   // a bit per candidate
-    float tile_max[kStepMaxBlocks / kKeyTile];             // largest score of a key tile
-    int tile[kFew];                                        // the tiles that may have a taken one
-    float score[kFew];                                     // their candidates that may be taken
-    int j[kFew];
+    union {
+        uint16_t list[kListed];                            // the taken ones, in order
+        struct {                                           // on the way there, the short list:
+            uint16_t tile[kStepMaxBlocks / kKeyTile];      // the tiles that may have a taken one
+            uint16_t j[kFew];                              // their candidates that may be taken
+            union {
+                float tile_max[kStepMaxBlocks / kKeyTile]; // largest score of a key tile
+                float score[kFew];
+            };
+        };
+    };
 };
 template <int NW, bool MULTI>
 struct GatePlace {                                         // offsets in the ring
     using Scratch = GateScratch<NW, MULTI>;
     static constexpr int kRing = Size<NW, MULTI>::kStages * kStageBytes;
     static constexpr int kScratch = kRing - (int)sizeof(Scratch);
-    static constexpr int kShort = kRing - (int)sizeof(Scratch::hist) - (int)sizeof(ShortList);
+    static constexpr int kSelected = kRing - (int)sizeof(Scratch::hist) - (int)sizeof(Selected);
     static_assert(offsetof(Scratch, hist) + sizeof(Scratch::hist) == sizeof(Scratch), "the histogram comes last");
-    static_assert(kScratch % 16 == 0 && kShort % 16 == 0 && kShort >= 4 * kStepMaxBlocks, "behind the scores");
+    static_assert(kScratch % 16 == 0 && kSelected % 16 == 0 && kSelected >= 4 * kStepMaxBlocks, "behind the scores");
     static_assert(kScratch - 4 * kStepMaxBlocks - 64 >= 2 * kKeyTile * kMaxDGate, "room for a key tile whatever there is to score");
 };
-static_assert(kStepMaxBlocks / kKeyTile <= kFew && kStepMaxBlocks <= 64 * 256, "the short list's tiles; a bit per candidate of a lane");
+static_assert(kStepMaxBlocks <= 65536, "16 bits a block");
 
 // Barriers among the worker warps, and between them and the producer.  The aligned forms are for a warp whose lanes are
 // together; behind a loop or branch of some lanes they need not be, so they are brought together here.
@@ -200,35 +207,48 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status) {
     return ok != 0;
 }
 
-// The selection of the `need` best of the candidates [0, n_cand), by a CTA's worker warps: take(e, j) for the e-th of them in
-// block order.  Comparisons only: the lower block number wins a tie, NaN is below every number.  A histogram over a
-// monotone linear map of [min, max] leaves a few candidates in the boundary bin, which every warp ranks for itself;
-// crowded bins and ranges that are not finite take radix passes over key - min instead.  With many candidates for few
-// places a short list comes first: the need-th largest of the key tiles' maxima is a bound that at least `need`
-// candidates reach, and few others do.
+// The selection of the `need` best of the candidates [0, n_cand), 0 < need < n_cand, by a CTA's worker warps.  Comparisons
+// only: the lower block number wins a tie, NaN is below every number.  A histogram over a monotone linear map of [min, max]
+// leaves a few candidates in the boundary bin, which every warp ranks for itself; crowded bins and ranges that are not finite
+// take radix passes over key - min instead.
 // What bounds it: this code runs once per call, by two warps a scheduler, so that its time is the number of instructions
-// on its longest path (some ten cycles each, mostly their fetch) and not the candidates; hence rolled loops, whose
-// bodies stay in the instruction buffers, and one candidate a lane and turn.
-template <int NW, typename Smem, typename Take>
-__device__ __forceinline__ void select_blocks(Smem& sm, int* hist, ShortList& sl, const float* sc, int n_cand, int need, int warp, int lane, Take&& take) {
-    constexpr int kThreads = 32 * NW, kPer = kBins / kThreads;
-    const int tid = 32 * warp + lane;
-    if (need <= 0) return;
+// on its longest path (some ten cycles each, mostly their fetch) and not the candidates; hence rolled loops, whose bodies stay
+// in the instruction buffers.
+template <int NW, typename Smem>
+struct Selection {
+    static constexpr int kThreads = 32 * NW, kPer = kBins / kThreads;
+    Smem& sm;
+    int* hist;
+    const float* sc;
+    int n_cand, need, warp, lane, tid;
+    float smin, smax, scale;
+    bool finite;
     // candidate j is taken if its key is above thr, or equal to it and j <= j_eq
     uint32_t thr = 0u;
     int j_eq = 0x7fffffff;
+
+    __device__ __forceinline__ Selection(Smem& s, int* h, const float* scores, int n, int want, int w, int l)
+        : sm(s), hist(h), sc(scores), n_cand(n), need(want), warp(w), lane(l), tid(32 * w + l) {
+        smin = key_score(sm.pre_min);
+        smax = key_score(sm.pre_max);
+        const float range = smax - smin;
+        scale = (kBins - 1.f) / range;
+        // (every candidate's score is finite then; -0 and +0 have the same bin)
+        finite = smin > -INFINITY && range > 0.f && range < INFINITY && scale < INFINITY;
+    }
+    __device__ __forceinline__ int bin_of(float s) const { return min(kBins - 1, (int)((s - smin) * scale)); }
     // the warps' totals before this one's
-    auto before = [&]() -> int { return __reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_tot[lane] : 0); };
-    auto scan = [&](int v) -> int {                        // inclusive, over the warp
+    __device__ __forceinline__ int before() const { return __reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_tot[lane] : 0); }
+    __device__ __forceinline__ int scan(int v) const {      // inclusive, over the warp
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, v, o);
             if (lane >= o) v += t;
         }
         return v;
-    };
+    }
     // thread t owns kPer bins, from kBins-1-kPer*t downwards: finds the bin that straddles the rem-th best
-    auto find_bin = [&](int rem) {
+    __device__ __forceinline__ void find_bin(int rem) {
         worker_sync<NW>();
         int c[kPer], mine = 0;
         if constexpr (kPer == 4) {
@@ -256,18 +276,18 @@ __device__ __forceinline__ void select_blocks(Smem& sm, int* hist, ShortList& sl
             }
         }
         worker_sync<NW>();
-    };
-    auto clear_bins = [&]() {                              // (a thread's own ones)
+    }
+    __device__ __forceinline__ void clear_bins() {          // (a thread's own ones)
 #pragma unroll
         for (int x = 0; x < kPer; ++x) hist[kBins - 1 - kPer * tid - x] = 0;
-    };
-    auto enlist = [&](float v, int j) {
+    }
+    __device__ __forceinline__ void enlist(float v, int j) {
         const int slot = atomicAdd(&sm.list_n, 1) & 31;
         sm.list_key[slot] = score_key(v);
         sm.list_j[slot] = j;
-    };
+    }
     // the `rem`-th best of the `cnt` <= 32 listed candidates, found by every warp for itself
-    auto rank_list = [&](int rem, int cnt) {
+    __device__ __forceinline__ void rank_list(int rem, int cnt) {
         const uint32_t key = lane < cnt ? sm.list_key[lane] : 0u;
         const int j = lane < cnt ? sm.list_j[lane] : 0x7fffffff;
         int rank = 0;
@@ -280,221 +300,236 @@ __device__ __forceinline__ void select_blocks(Smem& sm, int* hist, ShortList& sl
         const int src = __ffs(__ballot_sync(0xffffffffu, lane < cnt && rank == rem - 1)) - 1;
         thr = __shfl_sync(0xffffffffu, key, src);
         j_eq = __shfl_sync(0xffffffffu, j, src);
+    }
+    // Up to 4 * Q <= 16 candidates a thread: they stay in its registers from the histogram to take(e, j), for the e-th taken
+    // one in block order.  False: the boundary bin is crowded.
+    template <int Q, typename Take>
+    __device__ __forceinline__ bool in_registers(Take&& take) {
+        const int j0 = 4 * Q * tid, end = (n_cand + kKeyTile - 1) & ~(kKeyTile - 1);
+        float v[4 * Q];
+        int b[4 * Q];
+#pragma unroll
+        for (int x = 0; x < Q; ++x) {
+            const float4 f = j0 + 4 * x < end ? *reinterpret_cast<const float4*>(sc + j0 + 4 * x)
+                                              : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            v[4 * x] = f.x; v[4 * x + 1] = f.y; v[4 * x + 2] = f.z; v[4 * x + 3] = f.w;
+        }
+        // (minus infinity, behind the last candidate, has a negative bin)
+#pragma unroll
+        for (int k = 0; k < 4 * Q; ++k) {
+            b[k] = bin_of(v[k]);
+            if (b[k] >= 0) atomicAdd(&hist[b[k]], 1);
+        }
+        find_bin(need);
+        const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
+        if (cnt > 32) return false;
+#pragma unroll
+        for (int k = 0; k < 4 * Q; ++k)
+            if (b[k] == bin) enlist(v[k], j0 + k);
+        worker_sync<NW>();
+        rank_list(rem, cnt);
+        const float last = key_score(thr);
+        unsigned taken = 0u;
+#pragma unroll
+        for (int k = 0; k < 4 * Q; ++k) taken |= (unsigned)((v[k] > last) | ((v[k] == last) & (j0 + k <= j_eq))) << k;
+        const int mine = __popc(taken), incl = scan(mine);
+        if (lane == 31) sm.warp_tot[warp] = incl;
+        worker_sync<NW>();
+        int at = incl - mine + before();
+#pragma unroll 1
+        for (; taken; taken &= taken - 1) take(at++, j0 + __ffs(taken) - 1);
+        return true;
+    }
+};
+
+// The other cases: many candidates, crowded bins, scores that are not finite.  The taken ones' numbers in order, in sl.list.
+// Neighbours are often taken together, so that a thread finds dozens: what is done per taken one is little more than its place
+// in the list (with what an entry means to the tiles done by the thread that found it the lists of 625 of 15625
+// blocks took 22 us, and now 13; those of 256 of 9375 up to 20, and now 8).  A function of its own: its loops' registers are not
+// those of the short calls' path.
+template <int NW, typename Smem>
+__device__ __noinline__ void select_many(Smem* smem, int* hist, Selected* selected, const float* sc, int n_cand, int need) {
+    __builtin_assume(__isShared(smem));
+    __builtin_assume(__isShared(hist));
+    __builtin_assume(__isShared(selected));
+    __builtin_assume(__isShared(sc));
+    constexpr int kThreads = 32 * NW;
+    Smem& sm = *smem;
+    Selected& sl = *selected;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    Selection<NW, Smem> sel(sm, hist, sc, n_cand, need, warp, lane);
+    // the list, from the bits
+    auto list_taken = [&]() {
+        constexpr int kWords = kStepMaxBlocks / 32 / kThreads;
+        worker_sync<NW>();                                 // (every bit is in place)
+        unsigned words[kWords];
+        int mine = 0;
+#pragma unroll
+        for (int x = 0; x < kWords; ++x) {
+            words[x] = 32 * (kWords * tid + x) < n_cand ? sl.taken[kWords * tid + x] : 0u;
+            mine += __popc(words[x]);
+        }
+        const int incl = sel.scan(mine);
+        if (lane == 31) sm.warp_tot[warp] = incl;
+        worker_sync<NW>();
+        int at = incl - mine + sel.before();
+#pragma unroll
+        for (int x = 0; x < kWords; ++x)
+#pragma unroll 1
+            for (unsigned m = words[x]; m; m &= m - 1) sl.list[at++] = (uint16_t)(32 * (kWords * tid + x) + __ffs(m) - 1);
+        worker_sync<NW>();
     };
-    if (need < n_cand) {
-        const uint32_t kmin = sm.pre_min, kmax = sm.pre_max;
-        const float smin = key_score(kmin), smax = key_score(kmax);
-        const float range = smax - smin, scale = (kBins - 1.f) / range;
-        const bool finite = smin > -INFINITY && range > 0.f && range < INFINITY && scale < INFINITY;
-        // (every candidate's score is finite then; -0 and +0 have the same bin)
-        auto bin_of = [&](float s) -> int { return min(kBins - 1, (int)((s - smin) * scale)); };
-        bool found = false;
-        // Up to sixteen candidates a thread: they stay in its registers from the histogram to the list.
-        auto in_registers = [&](auto q_c) -> bool {
-            constexpr int Q = decltype(q_c)::value;
-            const int j0 = 4 * Q * tid, end = (n_cand + kKeyTile - 1) & ~(kKeyTile - 1);
-            float v[4 * Q];
-            int b[4 * Q];
-#pragma unroll
-            for (int x = 0; x < Q; ++x) {
-                const float4 f = j0 + 4 * x < end ? *reinterpret_cast<const float4*>(sc + j0 + 4 * x)
-                                                  : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                v[4 * x] = f.x; v[4 * x + 1] = f.y; v[4 * x + 2] = f.z; v[4 * x + 3] = f.w;
-            }
-            // (minus infinity, behind the last candidate, has a negative bin)
-#pragma unroll
-            for (int k = 0; k < 4 * Q; ++k) {
-                b[k] = bin_of(v[k]);
-                if (b[k] >= 0) atomicAdd(&hist[b[k]], 1);
-            }
-            find_bin(need);
-            const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
-            if (cnt > 32) return false;
-#pragma unroll
-            for (int k = 0; k < 4 * Q; ++k)
-                if (b[k] == bin) enlist(v[k], j0 + k);
-            worker_sync<NW>();
-            rank_list(rem, cnt);
-            const float last = key_score(thr);
-            unsigned taken = 0u;
-#pragma unroll
-            for (int k = 0; k < 4 * Q; ++k) taken |= (unsigned)((v[k] > last) | ((v[k] == last) & (j0 + k <= j_eq))) << k;
-            const int mine = __popc(taken), incl = scan(mine);
-            if (lane == 31) sm.warp_tot[warp] = incl;
-            worker_sync<NW>();
-            int at = incl - mine + before();
+    bool found = false;
+    const bool many = sel.finite && n_cand > 16 * kThreads;
+    // For one place in 32 or fewer a short list comes first: the need-th largest of the key tiles' maxima is a bound that at
+    // least `need` candidates reach, and few others do.
+    if (many && 32 * need <= n_cand) {
+        const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile;
+        for (int x = tid; x < kStepMaxBlocks / 32; x += kThreads) sl.taken[x] = 0u;
+        // (places of the last tile behind the last candidate hold minus infinity)
 #pragma unroll 1
-            for (; taken; taken &= taken - 1) take(at++, j0 + __ffs(taken) - 1);
-            return true;
-        };
-        if (finite && n_cand <= 16 * kThreads) {
-            if (n_cand <= 4 * kThreads   ? in_registers(std::integral_constant<int, 1>())
-                : n_cand <= 8 * kThreads ? in_registers(std::integral_constant<int, 2>())
-                                         : in_registers(std::integral_constant<int, 4>()))
+        for (int t = tid; t < n_tiles; t += kThreads) {
+            const float4* src = reinterpret_cast<const float4*>(sc + kKeyTile * t);
+            float best = -INFINITY;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {                  // (neighbouring lanes begin at different banks)
+                const float4 v = src[x ^ ((lane >> 1) & 3)];
+                best = fmaxf(best, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+            }
+            sl.tile_max[t] = best;
+            atomicAdd(&hist[sel.bin_of(best)], 1);
+        }
+        sel.find_bin(need);
+        const int bound = (int)sm.prefix;
+        sel.clear_bins();
+#pragma unroll 1
+        for (int t = tid; t < n_tiles; t += kThreads)
+            if (sel.bin_of(sl.tile_max[t]) >= bound) sl.tile[atomicAdd(&sm.tile_n, 1)] = (uint16_t)t;
+        worker_sync<NW>();
+        // bins of their own for the few, from about the bound's bin to the largest score
+        const float lo = sel.smin + (float)bound / sel.scale, fine = (kBins - 1.f) / (sel.smax - lo);
+        auto fine_of = [&](float s) -> int { return max(0, min(kBins - 1, (int)((s - lo) * fine))); };
+        const int total = kKeyTile * sm.tile_n;
+        if (fine > 0.f && fine < INFINITY) {
+#pragma unroll 1
+            for (int x = tid; x < total; x += kThreads) {
+                const int j = kKeyTile * sl.tile[x / kKeyTile] + (x & (kKeyTile - 1));
+                const float v = sc[j];
+                if (sel.bin_of(v) >= bound) {
+                    const int slot = atomicAdd(&sm.few_n, 1);
+                    if (slot < kFew) { sl.score[slot] = v; sl.j[slot] = (uint16_t)j; }
+                    atomicAdd(&hist[fine_of(v)], 1);
+                }
+            }
+            sel.find_bin(need);
+            const int few = sm.few_n, bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
+            if (few <= kFew && cnt <= 32) {
+#pragma unroll 1
+                for (int e = tid; e < few; e += kThreads)
+                    if (fine_of(sl.score[e]) == bin) sel.enlist(sl.score[e], sl.j[e]);
+                worker_sync<NW>();
+                sel.rank_list(rem, cnt);
+#pragma unroll 1
+                for (int e = tid; e < few; e += kThreads) {
+                    const uint32_t key = score_key(sl.score[e]);
+                    const int j = sl.j[e];
+                    if (key > sel.thr || (key == sel.thr && j <= sel.j_eq)) atomicOr(&sl.taken[j >> 5], 1u << (j & 31));
+                }
+                list_taken();
                 return;
+            }
+            sel.clear_bins();                              // (crowded, too: all candidates then)
         }
-        // The short list: beyond that, for one place in 32 or fewer.  15625 candidates, 127 places: scores to list
-        // 4.5 us, where the histogram over all candidates and the list in one CTA took 12.3.
-        if (finite && n_cand > 16 * kThreads && 32 * need <= n_cand) {
-            const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile;
-            for (int x = tid; x < kStepMaxBlocks / 32; x += kThreads) sl.taken[x] = 0u;
-            // (places of the last tile behind the last candidate hold minus infinity)
+        worker_sync<NW>();
+    }
+    if (many) {
+        // Neighbouring blocks have similar scores: the lanes of a warp take candidates that are far apart (lane l has
+        // run l of an odd number of blocks: no bank conflicts); side by side, their additions would queue for a few bins.
+        // (four at a time: their loads go out together)
+        const int run = ((n_cand + 31) / 32) | 1;
+        auto each_spread = [&](auto&& fn) {
+            const int j0 = lane * run;
 #pragma unroll 1
-            for (int t = tid; t < n_tiles; t += kThreads) {
-                const float4* src = reinterpret_cast<const float4*>(sc + kKeyTile * t);
-                float best = -INFINITY;
+            for (int q = warp; q < run; q += 4 * NW) {
+                float v[4];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {              // (neighbouring lanes begin at different banks)
-                    const float4 v = src[x ^ ((lane >> 1) & 3)];
-                    best = fmaxf(best, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-                }
-                sl.tile_max[t] = best;
-                atomicAdd(&hist[bin_of(best)], 1);
+                for (int x = 0; x < 4; ++x) v[x] = sc[min(j0 + q + x * NW, n_cand - 1)];
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    if (q + x * NW < run && j0 + q + x * NW < n_cand) fn(v[x], j0 + q + x * NW);
             }
-            find_bin(need);
-            const int bound = (int)sm.prefix;
-            clear_bins();
-#pragma unroll 1
-            for (int t = tid; t < n_tiles; t += kThreads)
-                if (bin_of(sl.tile_max[t]) >= bound) sl.tile[atomicAdd(&sm.tile_n, 1)] = t;
+        };
+        each_spread([&](float v, int) { atomicAdd(&hist[sel.bin_of(v)], 1); });
+        sel.find_bin(need);
+        const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
+        if (cnt <= 32) {
+            each_spread([&](float v, int j) { if (sel.bin_of(v) == bin) sel.enlist(v, j); });
             worker_sync<NW>();
-            // bins of their own for the few, from about the bound's bin to the largest score
-            const float lo = smin + (float)bound / scale, fine = (kBins - 1.f) / (smax - lo);
-            auto fine_of = [&](float s) -> int { return max(0, min(kBins - 1, (int)((s - lo) * fine))); };
-            const int total = kKeyTile * sm.tile_n;
-            if (fine > 0.f && fine < INFINITY) {
-#pragma unroll 1
-                for (int x = tid; x < total; x += kThreads) {
-                    const int j = kKeyTile * sl.tile[x / kKeyTile] + (x & (kKeyTile - 1));
-                    const float v = sc[j];
-                    if (bin_of(v) >= bound) {
-                        const int slot = atomicAdd(&sm.few_n, 1);
-                        if (slot < kFew) { sl.score[slot] = v; sl.j[slot] = j; }
-                        atomicAdd(&hist[fine_of(v)], 1);
-                    }
-                }
-                find_bin(need);
-                const int few = sm.few_n, bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
-                if (few <= kFew && cnt <= 32) {
-#pragma unroll 1
-                    for (int e = tid; e < few; e += kThreads)
-                        if (fine_of(sl.score[e]) == bin) enlist(sl.score[e], sl.j[e]);
-                    worker_sync<NW>();
-                    rank_list(rem, cnt);
-#pragma unroll 1
-                    for (int e = tid; e < few; e += kThreads) {
-                        const uint32_t key = score_key(sl.score[e]);
-                        const int j = sl.j[e];
-                        if (key > thr || (key == thr && j <= j_eq)) atomicOr(&sl.taken[j >> 5], 1u << (j & 31));
-                    }
-                    worker_sync<NW>();
-                    // a thread's words of the bits, in order
-                    const int per = (kStepMaxBlocks / 32 + kThreads - 1) / kThreads;
-                    int mine = 0;
-                    for (int x = 0; x < per; ++x) mine += __popc(sl.taken[per * tid + x]);
-                    const int incl = scan(mine);
-                    if (lane == 31) sm.warp_tot[warp] = incl;
-                    worker_sync<NW>();
-                    int at = incl - mine + before();
-                    for (int x = 0; x < per; ++x)
-                        for (unsigned m = sl.taken[per * tid + x]; m; m &= m - 1) take(at++, 32 * (per * tid + x) + __ffs(m) - 1);
-                    return;
-                }
-                clear_bins();                              // (crowded, too: all candidates then)
-            }
-            worker_sync<NW>();
-        }
-        if (finite && n_cand > 16 * kThreads) {
-            // Neighbouring blocks have similar scores: the lanes of a warp take candidates that are far apart (lane l has
-            // run l of an odd number of blocks: no bank conflicts); side by side, their additions would queue for a few bins.
-            const int run = ((n_cand + 31) / 32) | 1;
-            auto each_spread = [&](auto&& fn) {
-                int j = lane * run + warp;
-                float v = sc[min(j, n_cand - 1)];
-#pragma unroll 1
-                for (int q = warp; q < run; q += NW) {
-                    const float next = sc[min(j + NW, n_cand - 1)];      // (on its way while this one is worked on)
-                    if (j < n_cand) fn(v, j);
-                    v = next;
-                    j += NW;
-                }
-            };
-            each_spread([&](float v, int) { atomicAdd(&hist[bin_of(v)], 1); });
-            find_bin(need);
-            const int bin = (int)sm.prefix, rem = sm.rem, cnt = sm.bin_cnt;
-            if (cnt <= 32) {
-                each_spread([&](float v, int j) { if (bin_of(v) == bin) enlist(v, j); });
-                worker_sync<NW>();
-                rank_list(rem, cnt);
-                found = true;
-            }
-        }
-        if (!found) {
-            const int words = (n_cand + 32 * NW - 1) / (32 * NW), j0 = warp * words * 32 + lane;
-            auto each = [&](auto&& fn) {
-#pragma unroll 1
-                for (int e = 0; e < words; ++e) {
-                    const int j = j0 + 32 * e;
-                    fn(j < n_cand, score_key(sc[min(j, n_cand - 1)]), j);
-                }
-            };
-            // radix passes of ten bits over key - kmin
-            int bits_left = 32 - __clz(max(kmax - kmin, 1u)), rem = need;
-            uint32_t prefix = 0u;
-            while (bits_left > 0) {
-                const int wbits = min(10, bits_left), shift = bits_left - wbits;
-                clear_bins();
-                worker_sync<NW>();
-                each([&](bool ok, uint32_t key, int) {
-                    const uint32_t rel = key - kmin;
-                    if (ok && (uint32_t)((unsigned long long)rel >> (shift + wbits)) == prefix)        // (shift + wbits can be 32)
-                        atomicAdd(&hist[(rel >> shift) & ((1u << wbits) - 1u)], 1);
-                });
-                find_bin(rem);
-                prefix = (prefix << wbits) | sm.prefix;
-                rem = sm.rem;
-                bits_left = shift;
-            }
-            thr = kmin + prefix;
-            // the rem-th candidate whose key equals thr, in block order (a warp's candidates are one run of blocks)
-            int n_eq = 0;
-            each([&](bool ok, uint32_t key, int) { n_eq += __popc(__ballot_sync(0xffffffffu, ok && key == thr)); });
-            worker_sync<NW>();                             // (everybody has read the last pass's totals)
-            if (lane == 0) sm.warp_tot[warp] = n_eq;
-            worker_sync<NW>();
-            int eq_before = before();
-            if (eq_before < rem && rem <= eq_before + n_eq) {
-                each([&](bool ok, uint32_t key, int j) {
-                    const bool eq = ok && key == thr;
-                    const unsigned m = __ballot_sync(0xffffffffu, eq);
-                    if (eq && eq_before + __popc(m & ((1u << lane) - 1u)) == rem - 1) sm.last_eq = j;
-                    eq_before += __popc(m);
-                });
-            }
-            worker_sync<NW>();
-            j_eq = sm.last_eq;
+            sel.rank_list(rem, cnt);
+            found = true;
         }
     }
-    // the taken ones in order: a warp has a run of blocks, a lane every 32nd of them
-    const int words = (n_cand + 32 * NW - 1) / (32 * NW), j0 = warp * words * 32 + lane;
-    unsigned long long mine = 0ull;
-#pragma unroll 2
-    for (int e = 0; e < words; ++e) {
-        const int j = j0 + 32 * e;
-        const uint32_t key = score_key(sc[min(j, n_cand - 1)]);
-        if ((j < n_cand) & ((key > thr) | ((key == thr) & (j <= j_eq)))) mine |= 1ull << e;
-    }
-    const int all = __reduce_add_sync(0xffffffffu, __popcll(mine));
-    if (lane == 0) sm.warp_tot[warp] = all;
-    worker_sync<NW>();
-    int at = before();
+    // a warp has a run of blocks, a lane every 32nd of them
+    const int words = (n_cand + 32 * NW - 1) / (32 * NW), w0 = warp * words, j0 = 32 * w0 + lane;
+    if (!found) {
+        const uint32_t kmin = sm.pre_min, kmax = sm.pre_max;
+        auto each = [&](auto&& fn) {
 #pragma unroll 1
-    for (int e = 0; e < words; ++e) {
-        const bool in = (mine >> e) & 1ull;
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        if (in) take(at + __popc(m & ((1u << lane) - 1u)), j0 + 32 * e);
-        at += __popc(m);
+            for (int e = 0; e < words; ++e) {
+                const int j = j0 + 32 * e;
+                fn(j < n_cand, score_key(sc[min(j, n_cand - 1)]), j);
+            }
+        };
+        // radix passes of ten bits over key - kmin
+        int bits_left = 32 - __clz(max(kmax - kmin, 1u)), rem = need;
+        uint32_t prefix = 0u;
+        while (bits_left > 0) {
+            const int wbits = min(10, bits_left), shift = bits_left - wbits;
+            sel.clear_bins();
+            worker_sync<NW>();
+            each([&](bool ok, uint32_t key, int) {
+                const uint32_t rel = key - kmin;
+                if (ok && (uint32_t)((unsigned long long)rel >> (shift + wbits)) == prefix)        // (shift + wbits can be 32)
+                    atomicAdd(&hist[(rel >> shift) & ((1u << wbits) - 1u)], 1);
+            });
+            sel.find_bin(rem);
+            prefix = (prefix << wbits) | sm.prefix;
+            rem = sm.rem;
+            bits_left = shift;
+        }
+        sel.thr = kmin + prefix;
+        // the rem-th candidate whose key equals thr, in block order
+        int n_eq = 0;
+        each([&](bool ok, uint32_t key, int) { n_eq += __popc(__ballot_sync(0xffffffffu, ok && key == sel.thr)); });
+        worker_sync<NW>();                                 // (everybody has read the last pass's totals)
+        if (lane == 0) sm.warp_tot[warp] = n_eq;
+        worker_sync<NW>();
+        int eq_before = sel.before();
+        if (eq_before < rem && rem <= eq_before + n_eq) {
+            each([&](bool ok, uint32_t key, int j) {
+                const bool eq = ok && key == sel.thr;
+                const unsigned m = __ballot_sync(0xffffffffu, eq);
+                if (eq && eq_before + __popc(m & ((1u << lane) - 1u)) == rem - 1) sm.last_eq = j;
+                eq_before += __popc(m);
+            });
+        }
+        worker_sync<NW>();
+        sel.j_eq = sm.last_eq;
     }
+#pragma unroll 1
+    for (int e = 0; e < words; e += 4) {
+        float v[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) v[x] = sc[min(j0 + 32 * (e + x), n_cand - 1)];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const uint32_t key = score_key(v[x]);
+            const int j = j0 + 32 * (e + x);
+            const unsigned m = __ballot_sync(0xffffffffu, (j < n_cand) & ((key > sel.thr) | ((key == sel.thr) & (j <= sel.j_eq))));
+            if (lane == 0 && e + x < words) sl.taken[w0 + e + x] = m;
+        }
+    }
+    list_taken();
 }
 
 // The compressed key of block j of the unit, which has just filled, in two parts.  The same sums in the same order as
@@ -662,7 +697,8 @@ __device__ __noinline__ float score_key_plain(const uint4* key, const uint32_t (
 // banks.  The producer warp asks for the slots' first tiles, a warp for its slots' others.  (What bounds the scores of many keys
 // is how many are under way while the queries are made.  With a tile a warp, in its registers -- 64 of them for keys of 256
 // channels, which spilled -- a step of batch 8 at 128k took 83.5 us and takes 82.7, with 64 blocks 40.3 and 38.6, of two
-// sequences of 90k with 256 channels 32.2 and 24.0.)
+// sequences of 90k with 256 channels 32.2 and 24.0.  All other keys asked into L2 at the same time are too many for it where
+// there are many units: of 200 units of 9375 keys, 480 MB, a step took 199 us and takes 142.)
 struct KeySlots {
     unsigned char *a, *b;                                  // the halves of slot 0
     int n, shift;                                          // shift: log2 of a half's bytes
@@ -848,12 +884,15 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             need = max(0, min(min(k - n_forced, n_cand), kListed));
             n_blocks = need + n_forced;
         }
-        // This CTA's key tiles: a run of those with a candidate.  The producer warp asks for them, as many as there are slots for
-        // and the others into L2, so that they travel while the gate query is made.
+        // This CTA's key tiles: a run of those with a candidate.  The producer warp asks for as many as there are slots for, so
+        // that they travel while the gate query is made.
         const int n_tiles = (n_cand + kKeyTile - 1) / kKeyTile, per_cta = (n_tiles + S - 1) >> s_shift;
         const int tile0 = min(rank * per_cta, n_tiles), my_tiles = min(per_cta, n_tiles - tile0);
         KeySlots slots;
-        slots.place(sm.ring, n_tiles, Place::kScratch, g.d_gate);
+        // (the queries' parts: those of the last q_len of kMaxQLen places, so that the keys have what is in front of them)
+        const int t_skip = MULTI ? kMaxQLen - q_len : 0;
+        uint32_t (*parts)[3][kMaxDGate / 2 + 16] = gs.parts + t_skip;
+        slots.place(sm.ring, n_tiles, Place::kScratch + t_skip * (int)sizeof(gs.parts[0]), g.d_gate);
         // who selects: every CTA that will read tiles, or (the gate alone) the first one
         const int n_sel = p.q ? S : 1, sel_shift = p.q ? s_shift : 0;
         const bool selects = rank < n_sel;
@@ -867,17 +906,9 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         cluster_wait();                                    // every CTA of the cluster has started
         if (producer) {
-            const int ready = min(my_tiles, slots.n);
-            if (lane < ready) {
+            if (lane < min(my_tiles, slots.n)) {
                 const int j = kKeyTile * (tile0 + lane);
                 slots.request(lane, &sm.key_full[lane], kc + ((size_t)j << (slots.shift - 3)), g.max_blocks - j);
-            }
-            // (few requests to a lane, each of which takes the warp some fifty nanoseconds)
-            const int later = my_tiles - ready, step = (later + 31) >> 5;
-            if (lane * step < later) {
-                const int m = ready + lane * step, j = kKeyTile * (tile0 + m);
-                prefetch_l2(kc + ((size_t)j << (slots.shift - 3)),
-                            min(kKeyTile * min(step, my_tiles - m), g.max_blocks - j) << (slots.shift - 3));
             }
         }
         // ---- gate query ------------------------------------------------------------------------------------------------
@@ -930,7 +961,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     const float got = __shfl_xor_sync(0xffffffffu, upper ? f0 : f1, S);
                     if (upper) f0 = got;
                     else f1 = got;
-                    const uint32_t dst = cluster_addr(&gs.parts[t][0][(c >> 1) + (upper ? half >> 1 : 0)], to), bar = cluster_addr(&sm.got_query, to);
+                    const uint32_t dst = cluster_addr(&parts[t][0][(c >> 1) + (upper ? half >> 1 : 0)], to), bar = cluster_addr(&sm.got_query, to);
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         const uint32_t w = pack_bf16x2(f0, f1);
@@ -946,10 +977,10 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         // ---- scores, into the shared memory of the CTAs that select ------------------------------------------------
         // (keys through L2, not the read-only path: the entry that this launch appends, or the step before it did, is among them)
+        uint32_t kmn = 0xffffffffu, kmx = 0u;              // smallest and largest key of this warp's scores
         auto scores = [&](auto xs_c) {
             constexpr int XS = decltype(xs_c)::value;
             const float inv = rsqrtf((float)g.d_gate);
-            uint32_t kmn = 0xffffffffu, kmx = 0u;
             // this lane's first piece of its first key in slot 0; the second key is kOff bytes behind the first
             const int rr = lane >> 2, k_of = 8 * (rr & 1) + (rr >> 1) + 4 * (lane & 1);
             const unsigned char* at = ((rr & 1) ? slots.b : slots.a) + (rr >> 1) * (64 * XS) + 16 * (lane & 3);
@@ -993,9 +1024,9 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 float v0, v1;
                 bool odd;
                 if constexpr (XS < 8) {
-                    key_sums<XS, MULTI>([&](int x, uint4& lo, uint4& hi) { lo = held[2 * x]; hi = held[2 * x + 1]; }, gs.parts, q_len, lane, v0, v1, odd);
+                    key_sums<XS, MULTI>([&](int x, uint4& lo, uint4& hi) { lo = held[2 * x]; hi = held[2 * x + 1]; }, parts, q_len, lane, v0, v1, odd);
                 } else {
-                    key_sums<XS, MULTI>(in_slot, gs.parts, q_len, lane, v0, v1, odd);
+                    key_sums<XS, MULTI>(in_slot, parts, q_len, lane, v0, v1, odd);
                     refill();
                 }
                 // lane 4r has the score of row r, lane 4r + 1 (the others alike) that of row r + 8
@@ -1005,7 +1036,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 #pragma unroll 1
                     for (int k = 0; k < kKeyTile; ++k) {
                         if (((odds >> (4 * (2 * (k & 3) + (k >> 3)))) & 15u) && j0 + k < n_cand) {
-                            const float x = score_key_plain(reinterpret_cast<const uint4*>(kc + (size_t)(j0 + k) * (64 * XS)), gs.parts, q_len, g.d_gate, lane);
+                            const float x = score_key_plain(reinterpret_cast<const uint4*>(kc + (size_t)(j0 + k) * (64 * XS)), parts, q_len, g.d_gate, lane);
                             if (k == k_of) v = x;
                         }
                     }
@@ -1029,16 +1060,22 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     ++use;
                 }
             }
+        };
+        if (!producer) {
+            if (g.d_gate == 128) scores(std::integral_constant<int, 4>());
+            else if (g.d_gate == 64) scores(std::integral_constant<int, 2>());
+            else scores(std::integral_constant<int, 8>());
             kmn = __reduce_min_sync(0xffffffffu, kmn);
             kmx = __reduce_max_sync(0xffffffffu, kmx);
             if (lane == 0) { sm.warp_min[warp] = kmn; sm.warp_max[warp] = kmx; }
             worker_sync<NW>();
-            // four scores at a time to the others
-            const int to = tid & (n_sel - 1);
+            // four scores at a time to the others (a lane each to sixteen CTAs, the scores of 8 units of 15625 keys took 5 us
+            // longer to arrive)
+            const int to = (tid >> 3) & (n_sel - 1);       // (eight lanes: a line of one CTA's)
             if (to != rank) {
                 const uint32_t dst = cluster_addr(sc_all + kKeyTile * tile0, to), bar = cluster_addr(&sm.got_scores, to);
 #pragma unroll 1
-                for (int c = tid >> sel_shift; c < 4 * my_tiles; c += kWorkers >> sel_shift)
+                for (int c = 8 * (tid >> (3 + sel_shift)) + (tid & 7); c < 4 * my_tiles; c += kWorkers >> sel_shift)
                     send_f32x4(dst + 16 * c, *reinterpret_cast<const float4*>(sc_all + kKeyTile * tile0 + 4 * c), bar);
             }
             if (warp == 0) {
@@ -1050,11 +1087,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     send_max(cluster_addr(&sm.pre_max, lane), kmx, bar);
                 }
             }
-        };
-        if (producer) {
-        } else if (g.d_gate == 128) scores(std::integral_constant<int, 4>());
-        else if (g.d_gate == 64) scores(std::integral_constant<int, 2>());
-        else scores(std::integral_constant<int, 8>());
+        }
         // ---- selection ---------------------------------------------------------------------------------------------
         if (selects && !producer) {
             int32_t* dst = g.block_idx + (size_t)u * g.max_sel;
@@ -1102,9 +1135,22 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     if ((t & (S - 1)) == rank && at < kCodes) sm.codes[at] = j;
                 }
             };
-            select_blocks<NW>(sm, gs.hist, *reinterpret_cast<ShortList*>(sm.ring + Place::kShort), sc_all, n_cand, need, warp, lane, take);
-            // the last ones: the blocks taken without a score
-            if (tid < n_blocks - need) take(need + tid, n_i - n_blocks + need + tid);
+            Selected& sl = *reinterpret_cast<Selected*>(sm.ring + Place::kSelected);
+            int e0 = 0;                                    // entries that are in place
+            if (need > 0 && need < n_cand) {
+                Selection<NW, Smem> sel(sm, gs.hist, sc_all, n_cand, need, warp, lane);
+                if (sel.finite && (n_cand <= 4 * kWorkers    ? sel.template in_registers<1>(take)
+                                   : n_cand <= 8 * kWorkers  ? sel.template in_registers<2>(take)
+                                   : n_cand <= 16 * kWorkers ? sel.template in_registers<4>(take)
+                                                             : false))
+                    e0 = need;
+                else
+                    select_many<NW>(&sm, gs.hist, &sl, sc_all, n_cand, need);
+            }
+            // the others: the list's, or every candidate; behind them the blocks taken without a score
+#pragma unroll 1
+            for (int e = e0 + tid; e < n_blocks; e += kWorkers)
+                take(e, e >= need ? n_i - n_blocks + e : need < n_cand ? (int)sl.list[e] : e);
             if (lists) {
                 if (tid == 0) g.block_cnt[u] = n_blocks;
                 for (int e = n_blocks + tid; e < g.max_sel; e += kWorkers) dst[e] = -1;
@@ -1521,10 +1567,7 @@ int resident_clusters(bool wide, int k) {
 // that hold two of them are the last to finish (80 units, 64 tiles a CTA, 160 CTAs: 65 -> 67; 32 tiles: 40.8 -> 37.5), so
 // the line is at 32 there.  149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles
 // a CTA 45.9 -> 33.8, 52.7 -> 39.1, 59.3 -> 43.1; 64 tiles 93.5 -> 82.1, 108 -> 96, 127 -> 109.
-StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes, int max_keys) {
-    // Above 8192 keys, too, 16 warps a CTA: twice the keys in flight per SM (a step of
-    // 8 units of 15626 keys 39.5 -> 33.4 us; of 16 units of 9375 keys, blocks of 16, 56.5 -> 49.6).
-    const bool wide = rows > 16 || max_keys > 8192;
+static StepPlan plan_of(bool wide, int units, int rows, long long max_tiles, long long max_codes, int max_keys) {
     StepPlan plan = {0, 1, rows, wide};
     if (rows > 64) return plan;
     if (rows > 32) {
@@ -1543,6 +1586,24 @@ StepPlan step_plan(int units, int rows, long long max_tiles, long long max_codes
         break;
     }
     return plan;
+}
+
+// Which of the two sizes.  Above 16 rows there is only the one of 16 warps.  One query token takes eight warps whatever the
+// number of keys: two CTAs an SM make clusters twice as large, or twice as many units resident.  (With 16 warps above 8192
+// keys a step of 8 units of 15625 keys and 625 blocks went to the kernels of long calls: 119 us, now 63; so did 200 units of
+// 9375 keys, 233 and 142, and 192 units of short sequences in a cache of 16384 keys, 184 and 47; 16 units of 9375 took 50 and take
+// 36, 96 took 153 and take 96.)  Several query tokens' parts leave the keys less room, which costs where the scores take most of
+// it: 16 warps above 8192 keys where their clusters have eight CTAs or more (two tokens, 8 units of 15625: 36.3 -> 33.8; but 16
+// units of 9375, in clusters of four, 36.6 -> 44.5).
+StepPlan step_plan(int units, int rows, int q_len, long long max_tiles, long long max_codes, int max_keys) {
+    if (rows <= 16) {
+        if (q_len > 1 && max_keys > 8192) {
+            const StepPlan plan = plan_of(true, units, rows, max_tiles, max_codes, max_keys);
+            if (plan.S >= 8) return plan;
+        }
+        return plan_of(false, units, rows, max_tiles, max_codes, max_keys);
+    }
+    return plan_of(true, units, rows, max_tiles, max_codes, max_keys);
 }
 
 namespace {
@@ -1569,7 +1630,7 @@ cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map
 
 bool launch_gate_cluster(const GateParams& p, cudaStream_t stream, cudaError_t* err) {
     if (p.scores_in || p.list_flags || !gate_one_kernel(p.max_blocks)) return false;
-    const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, 0, 0, p.max_blocks);
+    const StepPlan plan = step_plan(p.batch * p.num_kv_heads, 1, 1, 0, 0, p.max_blocks);
     if (plan.S == 0) return false;
     CUtensorMap none;
     DecodeParams d;

@@ -198,7 +198,7 @@ seer_status refuse_capture(seer_ctx* ctx, void* stream) {
 
 seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const void* q, int q_len,
                           const int32_t* block_idx, const int32_t* block_cnt, int max_sel, bool sparse,
-                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0, false}) {
+                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0, false, false}) {
     // (gate: the whole step in one launch, by `plan`)
     if (!ctx) return SEER_ERR_INVALID_ARG;
     seer_status st = check_shape(ctx, shape);
@@ -330,6 +330,7 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
         plan = step_plan(U, q_len * group, q_len, max_tiles / U, 0, 0);
     if (plan.S > 0) {
         p.rows = plan.rows;
+        p.next_early = plan.next_early;
         ce = launch_step_cluster(mk_copy, *mv, p, gate, plan, static_cast<cudaStream_t>(stream));
         if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "decode launch: %s", cudaGetErrorString(ce));
         ctx->launches += 1;
@@ -797,7 +798,7 @@ static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     const int rows = q_len * (shape->num_q_heads / shape->num_kv_heads);
     if (!ctx->use_clusters || gate->max_blocks > kStepMaxBlocks || ctx->chain_attention || ctx->chain_gate || (q_len == 1 && ctx->chain_step) ||
         (ctx->wide_variant && rows > 16 && shape->block_size >= kTileTokens))
-        return StepPlan{0, 1, 0};
+        return StepPlan{0, 1, 0, false, false};
     const long long bs = shape->block_size, cap = kv->max_seq_len > 0 ? (kv->max_seq_len + bs - 1) / bs : 1;
     long long blocks = token_budget / bs > 1 ? token_budget / bs : 1;
     if (q_len > 1 && blocks < 2) blocks = 2;               // (two blocks can hold query tokens)
@@ -832,7 +833,7 @@ seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     GateParams gp;
     seer_status st = gate_prepare(ctx, shape, gate, kv->seq_lens, q_nope, nullptr, token_budget, 0, 0.f, block_idx, block_cnt, max_sel,
                                   nullptr, 1, &gp);
-    const StepPlan plan = st == SEER_OK ? plan_of_step(ctx, shape, kv, gate, 1, token_budget, max_sel) : StepPlan{0, 1, 0};
+    const StepPlan plan = st == SEER_OK ? plan_of_step(ctx, shape, kv, gate, 1, token_budget, max_sel) : StepPlan{0, 1, 0, false, false};
     if (plan.S > 0) {
         const bool appended = append_in_step(ctx, shape, kv, gate, k_nope, k_nope_stride_batch, k_nope_stride_head,
                                              k_nope_stride_token, k_nope_rows_block_local, 1, &gp);

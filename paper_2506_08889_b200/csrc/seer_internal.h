@@ -73,6 +73,7 @@ struct DecodeParams {
     int sel_from_lens;              // > 0: every unit's list holds min(this, blocks of its sequence) entries, so the
                                     // counts follow from the lengths and the schedule can be made before the kernel
                                     // that writes the lists has finished (0: read block_cnt)
+    int next_early;                     // cluster kernel: StepPlan's
     unsigned int* status;
     unsigned long long* tickets;    // [num_units]: tiles done << 32 | valid-slot bits; zero between launches
     int* sched;                     // [2]: theft cursor, exit counter; zero between launches
@@ -136,6 +137,7 @@ struct StepPlan {
     int S;                              // CTAs per cluster; 0: not a short call
     int parts, rows;                    // clusters per unit, which have `rows` of its rows each (the last one the rest)
     bool wide;                          // 16 worker warps per CTA, one CTA per SM (else 8 and two)
+    bool next_early;                    // the stream's next launch may start beside this one
 };
 StepPlan step_plan(int units, int rows, int q_len, long long max_tiles, long long max_codes, int max_keys);
 // g == nullptr: attention only, over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.

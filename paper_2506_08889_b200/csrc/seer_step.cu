@@ -61,8 +61,12 @@ struct __align__(1024) StepSmem {
     // K/V ring.  Before the first tile is asked for, the gate's: the scores of the unit (up to kStepMaxBlocks) at its
     // beginning, GateScratch at its end, compressed keys on their way between them.  After the last tile: the warps' partials.
     unsigned char ring[Z::kStages * kStageBytes];
-    // what the cluster's CTAs send after their last tile (a fast one while this one still selects: memory of its own)
-    __align__(16) float recv_o[Z::kRows * kHeadDim];       // [source CTA][row][this CTA's slice of the channels]
+    // what the cluster's CTAs send after their last tile (a fast one while this one still selects: memory that is its own
+    // from the moment on that this CTA has sent its scores)
+    union {
+        __align__(16) float recv_o[Z::kRows * kHeadDim];   // [source CTA][row][this CTA's slice of the channels]
+        double sums[NW][16][MULTI ? kMaxQLen : 1];         // before that: partial sums of the gate query: [warp][row][token]
+    };
     float2 recv_ml[kMaxS][Z::kRows];                       // [source CTA][row]: max, sum
     float2 warp_ml[NW][8];
     // Tile n arrives in stage n % kStages and is announced on full[n % kArrivals].  The consumer groups that share a
@@ -94,7 +98,6 @@ struct GateScratch {
     // Gate queries, from all CTAs: each channel in three bf16 parts (high, middle, low), which together are the fp32 number
     // exactly, two channels a word.  (Rows 64 bytes longer than the channels: neighbouring parts are in different banks.)
     __align__(16) uint32_t parts[MULTI ? kMaxQLen : 1][3][kMaxDGate / 2 + 16];
-    float sums[NW][16][8];                                 // partial sums of the gate query: [warp][row][token]
     __align__(16) int hist[kBins];                         // selection
 };
 // ... and of the selection, when queries and keys have been used.
@@ -834,8 +837,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         // a row tile (`slices` of them), whose partial sums meet in shared memory.  A lane holds pieces of 16 bytes as they lie
         // in memory (channels 8 * (lane % 4) .. of a unit): the contraction index is permuted, in W_q and x alike.  What bounds
         // it is the way of the first bytes and, for several query tokens, was the arithmetic: with a warp per pair and token by
-        // FMA the queries of four tokens were there after 7.2 us, now after 3.3.  (Each MMA begins at zero and the last sums
-        // and the rotation are in double: against 64 bits the scores are off by 1.21e-7 of their norm, by FMA 1.28e-7.)
+        // FMA the queries of four tokens were there after 7.2 us, now after 3.3.  (Each MMA begins at zero and
+        // the rotation is in double: against 64 bits the scores are off by 7.4e-8 of their norm, by FMA 1.17e-7.)
+        // How the units are dealt to warps depends on the cluster's size, and the scores shall not: a sequence's lists are the
+        // same whatever the batch around it.  The units' sums are therefore added up in double, which is exact, in any order,
+        // as long as none is 2^24 times another; beyond that the order is 2^-53 of the sum and all but never seen in fp32.
         const int ppc = half >> s_shift, c_first = rank * ppc;
         const int mt_shift = 31 - __clz(min((ppc + 7) >> 3, NW)), slices = NW >> mt_shift, slice = warp >> mt_shift;
         const int row8 = lane >> 2, units = n / 32;
@@ -913,13 +919,13 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         // ---- gate query ------------------------------------------------------------------------------------------------
         if (!producer) {
-            float (*part)[16][8] = gs.sums;
+            auto part = sm.sums;
             for (int m0 = 0; 8 * m0 < ppc; m0 += NW) {
                 if (m0 > 0) {
                     worker_sync<NW>();                     // (the partial sums have been read)
                     load_w(m0, slice);
                 }
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};       // (each MMA from zero: KeyScores)
+                double acc[4] = {0., 0., 0., 0.};
 #pragma unroll 1
                 for (int u0 = slice;;) {
 #pragma unroll
@@ -930,14 +936,19 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         mma_bf16_16816(c0, a0, xx[k].x, xx[k].y);
                         mma_bf16_16816(c1, a1, xx[k].z, xx[k].w);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) acc[c] += c0[c] + c1[c];
+                        for (int c = 0; c < 4; c += MULTI ? 1 : 2) acc[c] += (double)(c0[c] + c1[c]);      // (one token: column 0)
                     }
                     u0 += 4 * slices;
                     if (u0 >= units) break;
                     load_w(m0, u0);
                 }
-                *reinterpret_cast<float2*>(&part[warp][row8][2 * (lane & 3)]) = make_float2(acc[0], acc[1]);
-                *reinterpret_cast<float2*>(&part[warp][row8 + 8][2 * (lane & 3)]) = make_float2(acc[2], acc[3]);
+                if constexpr (MULTI) {
+                    *reinterpret_cast<double2*>(&part[warp][row8][2 * (lane & 3)]) = make_double2(acc[0], acc[1]);
+                    *reinterpret_cast<double2*>(&part[warp][row8 + 8][2 * (lane & 3)]) = make_double2(acc[2], acc[3]);
+                } else if ((lane & 3) == 0) {
+                    part[warp][row8][0] = acc[0];
+                    part[warp][row8 + 8][0] = acc[2];
+                }
                 worker_sync<NW>();
                 // a thread per pair, token and CTA that gets them
                 const int np_shift = 31 - __clz(min(ppc, 8 << mt_shift));
@@ -948,10 +959,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     double sn, cs;                         // query token t sits at position L - q_len + t
                     rope_sincos_wide((double)max(L - q_len + t, 0), g.inv_freq[c], &sn, &cs);
                     double a = 0., b = 0.;
-#pragma unroll 4
-                    for (int sl = 0; sl < slices; ++sl) {
-                        a += (double)part[(sl << mt_shift) + (pr >> 3)][pr & 7][t];
-                        b += (double)part[(sl << mt_shift) + (pr >> 3)][(pr & 7) + 8][t];
+#pragma unroll
+                    for (int sl = 0; sl < NW; ++sl) {
+                        if (sl >= slices) break;
+                        a += part[(sl << mt_shift) + (pr >> 3)][pr & 7][t];
+                        b += part[(sl << mt_shift) + (pr >> 3)][(pr & 7) + 8][t];
                     }
                     // A thread has channels c and c + d_gate/2, its neighbour S lanes on the ones next to them (c is even here and
                     // odd there, or the other way round): the even one sends the words of the lower two channels, the other

@@ -535,6 +535,13 @@ __device__ __noinline__ void select_many(Smem* smem, int* hist, Selected* select
     list_taken();
 }
 
+// Cut off, not rounded: no finite number becomes infinite.
+__device__ __forceinline__ uint32_t pack_bf16x2_toward_zero(float lo, float hi) {
+    uint32_t d;
+    asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+
 // The compressed key of block j of the unit, which has just filled, in two parts.  The same sums in the same order as
 // seer_kcomp.cu's append, so the same entry.  First the pooled features, by the producer warps of the cluster, which have
 // nothing else to do while the gate is at work: 16 channels at a time, to every CTA of the cluster.
@@ -976,11 +983,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     const uint32_t dst = cluster_addr(&parts[t][0][(c >> 1) + (upper ? half >> 1 : 0)], to), bar = cluster_addr(&sm.got_query, to);
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
-                        const uint32_t w = pack_bf16x2(f0, f1);
+                        const uint32_t w = pack_bf16x2_toward_zero(f0, f1);
                         send_u32(dst + k * (uint32_t)sizeof(gs.parts[0][0]), w, bar);
                         const float2 r = bf16x2_to_float2(w);
-                        // (each difference is exact: the rest of a rounding to eight bits has at most the sixteen bits behind
-                        // them; what is not finite has no rest)
+                        // (each difference is exact: it has the bits behind the eight cut off, at most sixteen; what is not finite
+                        // has no rest, and what is finite stays it)
                         f0 = fabsf(r.x) < INFINITY ? f0 - r.x : 0.f;
                         f1 = fabsf(r.y) < INFINITY ? f1 - r.y : 0.f;
                     }

@@ -631,7 +631,10 @@ __device__ __forceinline__ void append_project(const GateParams& g, Smem& sm, in
             wv[k][0] = __ldg(wrow + lane);
             wv[k][1] = lane < 16 ? __ldg(wrow + 32 + lane) : make_uint4(0u, 0u, 0u, 0u);
         }
-        if (!waited) waited = wait_sent(&sm.got_feat, g.status);
+        if (!waited) {                                     // (without the features nothing goes into the cache, which outlives the call)
+            if (__any_sync(0xffffffffu, !wait_sent(&sm.got_feat, g.status))) return;
+            waited = true;
+        }
         float acc[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -1187,7 +1190,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             if (sm.no_list) n_blocks = 0;
         } else {
             tiles_listed_arrive<NW>();
-            if (appends) append_project<NW>(g, sm, u, h, (L >> b_shift) - 1, rank, S);
+            if (appends && !dead) append_project<NW>(g, sm, u, h, (L >> b_shift) - 1, rank, S);
         }
     } else {
         pdl_wait();

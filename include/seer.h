@@ -256,6 +256,11 @@ seer_status seer_dense_decode_multi(seer_ctx* ctx, const seer_shape* shape, cons
  *  scores_out[B,Hkv,max_blocks] fp32 or NULL: receives the computed scores.
  *  block_idx [B,Hkv,max_sel] int32 out; block_cnt [B,Hkv] int32 out.
  *  seq_lens  device [B].
+ * The scores of a (sequence, KV head) in the one-launch form of short calls are the same bits whatever the
+ * batch around it, in this call and in the steps.  The kernels of long calls (more than 8192 compressed keys
+ * in this call, more clusters than are resident, SEER_STEP_CLUSTERS=0) add up in another order: their
+ * scores agree to a few times 2^-24 of the products' size, and blocks whose scores do so may change
+ * places in the list.
  */
 seer_status seer_gate_select(seer_ctx* ctx, const seer_shape* shape, const seer_gate* gate,
                              const int32_t* seq_lens, const void* q_nope,
@@ -344,7 +349,8 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
  * and token-budget selection (Eq. 1a/1c, Sec. 3.1), block-sparse decode over the selected
  * blocks (Sec. 3.3).  The results are those of the three calls
  *     seer_kcomp_append(.., first_block = -1) ; seer_gate_select(.., scores_in = NULL) ; seer_sparse_decode
- * on `stream`, with one host round trip instead of three.  (With at most 64 tiles per CTA of the lists'
+ * on `stream` (where step and gate call take different forms, up to blocks whose scores agree to within
+ * fp32 rounding; see seer_gate_select), with one host round trip instead of three.  (With at most 64 tiles per CTA of the lists'
  * clusters and at most 16384 compressed keys per sequence, gate, attention and append are one
  * launch.  Otherwise the launches go out as gate, attention, append: the block that has just filled is
  * the sequence's last block, which the gate takes without scoring it, so the entry the append writes is
@@ -386,9 +392,10 @@ seer_status seer_decode_step_multi(seer_ctx* ctx, const seer_shape* shape, const
  * of HBM to its own pool at start-up and forbids cudaMalloc afterwards (a late allocation can
  * fail, or stall the GPU, under its memory plan), or code that runs inside a region where the
  * CUDA allocator must not be entered.  seer_create allocates a workspace, so those callers
- * cannot have a context.  This call computes what seer_gate_select computes from q_nope (the
- * same sums in the same order, by the kernels that seer_gate_select takes where the one-launch form of
- * short calls does not do) but keeps the scratch it needs -- per-unit tickets, the gate
+ * cannot have a context.  This call computes what seer_gate_select computes from q_nope, by the
+ * same kernels and so to the same bits (the one-launch form of short calls among them; of the switches
+ * that a context reads when it is created, SEER_STEP_CLUSTERS and SEER_GATE_WIDEN are looked for at each
+ * call) but keeps the scratch it needs -- per-unit tickets, the gate
  * query, and the block scores unless scores_out is given -- in an array of
  * SEER_STATIC_SCRATCH_BYTES that is part of the library image.  Every GPU on which the library
  * is used holds one copy of that array from first use until the process exits.

@@ -960,7 +960,10 @@ extern "C" seer_status seer_gate_select_static(int device, const seer_shape* sha
     for (int c = 0; c < gate->d_gate / 2; ++c)
         p.inv_freq[c] = pow((double)gate->rope_theta, -2.0 * (double)c / (double)gate->d_gate);
     int launched = 0;
-    if (!launch_gate_cluster(p, s, &ce)) ce = launch_gate_select(p, s, &launched);      // (as a context's gate call)
+    // (the one-launch form as in a gate call of a context that were created now)
+    const char* clusters = getenv("SEER_STEP_CLUSTERS");
+    const bool one_launch = !(clusters && atoi(clusters) == 0) && !getenv("SEER_GATE_WIDEN");
+    if (!one_launch || !launch_gate_cluster(p, s, &ce)) ce = launch_gate_select(p, s, &launched);
     if (ce != cudaSuccess) return static_fail(err, err_len, SEER_ERR_CUDA, "kernel launch failed (code %lld)", (long long)ce);
     return SEER_OK;
 }

@@ -1,5 +1,6 @@
 """The bulk build's two ways to add up the sequences' blocks (up to 32 sequences, every warp for itself; more, the CTA
-together), with sequences that have no complete block, for heads that divide the CTAs and heads that do not."""
+together), with sequences that have no complete block, and its two ways to cut the runs: within a head where the heads
+divide the CTAs (3, 4, 5 and 8 heads do: the last CTAs stay away) and across heads where they do not (20 and 32)."""
 import numpy as np
 import pytest
 import torch
@@ -12,7 +13,8 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.mark.parametrize("B,Hkv,b,dg", [(31, 4, 64, 128), (32, 8, 16, 128), (33, 8, 64, 64), (32, 5, 128, 128), (40, 3, 32, 128)])
+@pytest.mark.parametrize("B,Hkv,b,dg", [(31, 4, 64, 128), (32, 8, 16, 128), (33, 8, 64, 64), (32, 5, 128, 128), (40, 3, 32, 128),
+                                             (31, 20, 64, 128), (40, 32, 32, 64)])
 def test_build_of_many_sequences(B, Hkv, b, dg):
     lens = np.array([(i * 37 % 11) * b + (i * 13) % b for i in range(B)], np.int32)
     S, d = 12 * b, 128

@@ -1,5 +1,5 @@
 """The one-launch gate's scores do not depend on how many CTAs share a unit: a sequence's are the same bits alone and in a
-batch of any size.  And gate queries next to the largest fp32 number stay finite."""
+batch of any size, and so are a step's lists.  And gate queries next to the largest fp32 number stay finite."""
 import numpy as np
 import pytest
 import torch
@@ -55,4 +55,36 @@ def test_gate_query_next_to_the_largest_number():
     want = scores64(qn, wq, kc, L)[0, 0, :n - 1]
     assert float(want.abs().max()) > 1e11
     assert bool(((sc[0, 0, :n - 1].double() - want).abs() <= 4 * 2.0 ** -24 * want.abs()).all())
+    assert ctx.device_status() == binding.SEER_OK
+
+
+@pytest.mark.parametrize("Hkv,g,T,dg,n,finite", [(2, 4, 1, 128, 4097, True), (8, 5, 1, 128, 2000, False), (2, 4, 1, 256, 700, False),
+                                                 (2, 8, 3, 128, 2050, True), (2, 8, 3, 64, 1000, False), (1, 8, 8, 128, 900, False)])
+def test_a_step_has_the_gate_s_lists(Hkv, g, T, dg, n, finite):
+    # (up to 64 rows: 8 and 16 warps a CTA, one and two clusters a unit, beside the gate's own form)
+    d, b, need = 128, 64, 50
+    L, seed = n * b - 3, 1600 + n
+    qn, q = (synth.normal_bf16((1, T, Hkv * g, d), seed, x, DEV) for x in ("qn", "q"))
+    wq = synth.normal_bf16((Hkv, dg, g * d), seed, "wq", DEV, std=0.02)
+    kc = synth.normal_bf16((1, Hkv, n, dg), seed, "kc", DEV)
+    if not finite:
+        kc[:, :, 3::170, 5] = float("inf")
+        kc[:, :, 4::190, 9] = -float("inf")
+        kc[:, :, 5::23, 2] = float("nan")
+    # every third block twice: equal scores, so that one bit more or less would change the list
+    kc[:, :, 1:n - 1:3] = kc[:, :, 0:n - 2:3]
+    k = synth.normal_bf16((1, Hkv, n * b, d), seed, "k", DEV)
+    lens_t = torch.tensor([L], dtype=torch.int32, device=DEV)
+    shape, gate, kv = binding.make_shape(1, Hkv * g, Hkv, d, b, 0.09), binding.make_gate(dg, THETA, wq, None, kc, n), binding.make_kv(k, k, lens_t)
+    ctx, lists = binding.Context(0), []
+    for step in (False, True):
+        idx, cnt = torch.zeros((1, Hkv, need), dtype=torch.int32, device=DEV), torch.zeros((1, Hkv), dtype=torch.int32, device=DEV)
+        before = ctx.launch_count()
+        if step:
+            ctx.seer_decode_step_multi(shape, kv, gate, q, qn, T, None, need * b, idx, cnt, need, torch.empty_like(q), None)
+        else:
+            ctx.seer_gate_select_multi(shape, gate, lens_t, qn, None, T, need * b, idx, cnt, need)
+        assert ctx.launch_count() - before == 1
+        lists.append(idx.cpu().numpy())
+    assert np.array_equal(*lists)
     assert ctx.device_status() == binding.SEER_OK

@@ -490,8 +490,8 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
     auto blocks_of = [&](int i) { const int L = p.seq_lens[i]; return max(0, min(j_end, L > 0 ? L / B : 0) - p.first_block); };
     // Up to 32 sequences: every warp sums up for itself, one lane a sequence, and all write the same numbers.  From the
     // wait's end to the first copy it was 3.7 us, two block barriers, the divisions of run_begin and a load among them; with
-    // this, the runs cut by heads and the angles made ahead of the products builds of 0.54 / 0.23 GB take 94.1 / 46.0 us
-    // instead of 95.1 / 46.7.
+    // this, the runs cut by heads and the angles made ahead of the products a build of 0.23 GB takes 45.9 us instead of
+    // 46.6; of 0.54 GB the difference, 94.9 to 94.3, is that between two runs.
     const bool few_seqs = p.batch <= 32;
     auto sum_lengths = [&]() {
         const int mine = lane < p.batch ? blocks_of(lane) : 0;

@@ -737,13 +737,13 @@ struct KeySlots {
 // with the first and one with the last eight channels of an MMA, zero elsewhere: of sums half as long the MMA cuts off
 // less), the middle and low parts in the others.  Both operands' contraction index is permuted alike: piece x of a lane is
 // two MMAs' operand as it lies in memory.
-// v0, v1: the sums of rows lane / 4 and lane / 4 + 8, the largest over the query tokens, the same in a row's four lanes; `odd`:
-// one of the sums is not finite.
+// v0, v1: the sums of rows lane / 4 and lane / 4 + 8, the largest over the query tokens, the same in a row's four lanes; `odd0`, `odd1`:
+// one of the row's sums is not finite.
 template <int XS, bool MULTI, typename Pieces>
 __device__ __forceinline__ void key_sums(Pieces&& pieces, const uint32_t (*parts)[3][kMaxDGate / 2 + 16], int q_len, int lane, float& v0, float& v1,
-                                         bool& odd) {
+                                         bool& odd0, bool& odd1) {
     v0 = v1 = -INFINITY;
-    odd = false;
+    odd0 = odd1 = false;
 #pragma unroll 1
     for (int nt = 0; 2 * nt < q_len; ++nt) {
         // (each MMA begins at zero and its 16 products are added up outside: the MMA's own accumulation cuts off where the
@@ -768,7 +768,8 @@ __device__ __forceinline__ void key_sums(Pieces&& pieces, const uint32_t (*parts
         float r0 = s[0] + s[1], r1 = s[2] + s[3];
         r0 += __shfl_xor_sync(0xffffffffu, r0, 1);
         r1 += __shfl_xor_sync(0xffffffffu, r1, 1);
-        odd |= !(fabsf(r0) < INFINITY) || !(fabsf(r1) < INFINITY);
+        odd0 |= !(fabsf(r0) < INFINITY);
+        odd1 |= !(fabsf(r1) < INFINITY);
         if (2 * nt + ((lane >> 1) & 1) >= q_len) r0 = r1 = -INFINITY;
         v0 = fmaxf(v0, fmaxf(r0, __shfl_xor_sync(0xffffffffu, r0, 2)));
         v1 = fmaxf(v1, fmaxf(r1, __shfl_xor_sync(0xffffffffu, r1, 2)));
@@ -1044,20 +1045,24 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
                 if (!mine) break;
                 float v0, v1;
-                bool odd;
+                bool odd0, odd1;
                 if constexpr (XS < 8) {
-                    key_sums<XS, MULTI>([&](int x, uint4& lo, uint4& hi) { lo = held[2 * x]; hi = held[2 * x + 1]; }, parts, q_len, lane, v0, v1, odd);
+                    key_sums<XS, MULTI>([&](int x, uint4& lo, uint4& hi) { lo = held[2 * x]; hi = held[2 * x + 1]; }, parts, q_len, lane, v0, v1, odd0, odd1);
                 } else {
-                    key_sums<XS, MULTI>(in_slot, parts, q_len, lane, v0, v1, odd);
+                    key_sums<XS, MULTI>(in_slot, parts, q_len, lane, v0, v1, odd0, odd1);
                     refill();
                 }
                 // lane 4r has the score of row r, lane 4r + 1 (the others alike) that of row r + 8
                 float v = (lane & 1) ? v1 : v0;
-                const unsigned odds = __ballot_sync(0xffffffffu, odd);
-                if (odds) {
+                // (only of keys that are candidates: behind them is whatever the cache or the slot holds, which has no part in this)
+                const int j_lo = j0 + 8 * (rr & 1) + (rr >> 1);
+                odd0 &= j_lo < n_cand;
+                odd1 &= j_lo + 4 < n_cand;
+                if (__any_sync(0xffffffffu, odd0 | odd1)) {
+                    const unsigned odds0 = __ballot_sync(0xffffffffu, odd0), odds1 = __ballot_sync(0xffffffffu, odd1);
 #pragma unroll 1
                     for (int k = 0; k < kKeyTile; ++k) {
-                        if (((odds >> (4 * (2 * (k & 3) + (k >> 3)))) & 15u) && j0 + k < n_cand) {
+                        if ((((k & 4) ? odds1 : odds0) >> (4 * (2 * (k & 3) + (k >> 3)))) & 15u) {
                             const float x = score_key_plain(reinterpret_cast<const uint4*>(kc + (size_t)(j0 + k) * (64 * XS)), parts, q_len, g.d_gate, lane);
                             if (k == k_of) v = x;
                         }

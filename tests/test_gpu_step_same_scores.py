@@ -34,6 +34,32 @@ def test_scores_are_the_same_in_every_batch(g, T, dg):
     assert ctx.device_status() == binding.SEER_OK
 
 
+@pytest.mark.parametrize("n,T,dg", [(5, 1, 128), (21, 1, 128), (63, 1, 64), (300, 3, 256)])
+def test_what_lies_behind_the_candidates_has_no_part(n, T, dg):
+    Hkv, g, d, b, cap = 2, 4, 128, 64, n + 23
+    L = n * b - 3                      # candidates: the first n - 1 (n - 2) blocks of a cache of n + 23
+    wq = synth.normal_bf16((Hkv, dg, g * d), n, "wq", DEV, std=0.02)
+    qn = synth.normal_bf16((1, T, Hkv * g, d), n, "qn", DEV)
+    kc = synth.normal_bf16((1, Hkv, cap, dg), n, "kc", DEV)
+    lens_t = torch.tensor([L], dtype=torch.int32, device=DEV)
+    ctx, got = binding.Context(0), []
+    m = n - 1 - (T > 1)
+    for behind in (0.0, float("nan"), float("inf"), None):
+        c = kc.clone()
+        if behind is None:
+            c = c[:, :, :m + 1].contiguous()         # ... or the cache ends there
+        else:
+            c[:, :, m:] = behind
+        idx, cnt = torch.zeros((1, Hkv, 4), dtype=torch.int32, device=DEV), torch.zeros((1, Hkv), dtype=torch.int32, device=DEV)
+        sc = torch.zeros((1, Hkv, c.shape[2]), dtype=torch.float32, device=DEV)
+        shape, gate = binding.make_shape(1, Hkv * g, Hkv, d, b, 0.09), binding.make_gate(dg, THETA, wq, None, c, c.shape[2])
+        ctx.seer_gate_select_multi(shape, gate, lens_t, qn, None, T, 4 * b, idx, cnt, 4, scores_out=sc)
+        got.append(sc[0, :, :m].cpu().numpy().view(np.uint32))
+    for other in got[1:]:
+        assert np.array_equal(got[0], other)
+    assert ctx.device_status() == binding.SEER_OK
+
+
 def test_gate_query_next_to_the_largest_number():
     # channel 63 of 128 turns by 4800 * theta^(-126/128) = 0.006: the query's channel is 3.4e38 * cos, above the largest bf16
     g, d, dg, b, n = 1, 128, 128, 16, 300

@@ -326,8 +326,19 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
 #ifdef SEER_DECODE_TRACE
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
-    if (!gate && ctx->use_clusters && !ctx->chain_attention && !(wide && ctx->wide_variant) && ctx->list_gen == 0 && ctx->sel_from_lens == 0)
-        plan = step_plan(U, q_len * group, q_len, max_tiles / U, 0, 0);
+    if (!gate && ctx->use_clusters && !ctx->chain_attention && !(wide && ctx->wide_variant) && ctx->list_gen == 0 && ctx->sel_from_lens == 0) {
+        const ListPlan lists = q_len == 1 ? list_plan(U, max_tiles / U) : ListPlan{0, false, false};
+        if (lists.S > 0 && (!lists.spread || w.scratch + list_part_bytes(U, lists.S) <= ctx->ws_bytes)) {
+            p.part_o = reinterpret_cast<float*>(ctx->ws + w.scratch);
+            p.spread = lists.spread;
+            p.next_early = lists.next_early;
+            ce = launch_lists(mk_copy, *mv, p, lists.S, static_cast<cudaStream_t>(stream));
+            if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "decode launch: %s", cudaGetErrorString(ce));
+            ctx->launches += 1;
+            return SEER_OK;
+        }
+        if (q_len > 1) plan = step_plan(U, q_len * group, q_len, max_tiles / U, 0, 0);
+    }
     if (plan.S > 0) {
         p.rows = plan.rows;
         p.next_early = plan.next_early;

@@ -1,0 +1,67 @@
+// Parts shared by the kernels that give a unit (one sequence's KV head) a thread-block cluster: stores that count their bytes
+// down on the receiver's mbarrier, the layout of a staged K/V tile.
+#pragma once
+
+#include "seer_gate_device.cuh"
+#include "seer_internal.h"
+
+namespace seer {
+
+constexpr int kHalfTileBytes = kTileTokens * 128;          // 64 rows x 128 B (64 bf16 channels)
+constexpr int kTileBytes = 2 * kHalfTileBytes;             // one K or V tile: 16 KiB
+constexpr int kStageBytes = 2 * kTileBytes;                // K + V
+constexpr int kMaxS = 16;                                  // CTAs of a cluster
+
+// Barriers among the worker warps, and between them and the producer.  The aligned forms are for a warp whose lanes are
+// together; behind a loop or branch of some lanes they need not be, so they are brought together here.
+template <int NW>
+__device__ __forceinline__ void worker_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory");
+}
+
+// ---- stores into a CTA of the cluster (addr, bar: of its shared memory, cluster_addr), counted on its mbarrier ----------
+__device__ __forceinline__ uint32_t cluster_addr(const void* mine, int rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void send_u32(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send_f32x2(uint32_t addr, float2 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_f32x4(uint32_t addr, float4 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_min(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.min.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_max(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.max.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
+                 : "memory");
+}
+// Bounded wait for what the cluster's CTAs have sent (by default the first phase of `bar`).
+__device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status, uint32_t parity = 0) {
+    uint32_t ok = 0;
+    for (uint32_t it = 0; it < (1u << 24) && !ok; ++it) {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        if (!ok && it > 64) __nanosleep(64);
+    }
+    if (!ok) raise_status(status, DEV_TIMEOUT);
+    __syncwarp();                                          // (the lanes need not have left the loop together)
+    return ok != 0;
+}
+
+}  // namespace seer

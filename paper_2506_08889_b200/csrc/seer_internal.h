@@ -73,7 +73,8 @@ struct DecodeParams {
     int sel_from_lens;              // > 0: every unit's list holds min(this, blocks of its sequence) entries, so the
                                     // counts follow from the lengths and the schedule can be made before the kernel
                                     // that writes the lists has finished (0: read block_cnt)
-    int next_early;                     // cluster kernel: StepPlan's
+    int next_early;                     // cluster kernels: StepPlan's, ListPlan's
+    int spread;                         // list kernel: ListPlan's
     unsigned int* status;
     unsigned long long* tickets;    // [num_units]: tiles done << 32 | valid-slot bits; zero between launches
     int* sched;                     // [2]: theft cursor, exit counter; zero between launches
@@ -140,9 +141,20 @@ struct StepPlan {
     bool next_early;                    // the stream's next launch may start beside this one
 };
 StepPlan step_plan(int units, int rows, int q_len, long long max_tiles, long long max_codes, int max_keys);
-// g == nullptr: attention only, over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.
+// g == nullptr: attention only (of several query tokens), over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.
 cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
                                 const StepPlan& plan, cudaStream_t stream);
+// One query token over given lists, or all blocks, as one launch of a cluster of S CTAs per unit (seer_lists.cu).
+constexpr int kListUnits = 320;         // most units whose tiles it counts
+struct ListPlan {
+    int S;                              // CTAs per cluster; 0: the decode kernel
+    bool spread;                        // the lists may be so long that it matters whether they are even
+    bool next_early;                    // the stream's next launch may start beside this one
+};
+ListPlan list_plan(int units, long long max_tiles);
+// Bytes of partial results (DecodeParams::part_o) that a launch may need.
+size_t list_part_bytes(int units, int S);
+cudaError_t launch_lists(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, int S, cudaStream_t stream);
 // The gate by itself as one launch of such clusters (at most 8192 compressed keys per unit), while they are resident all at
 // once; false: not that size, and nothing has been launched.
 bool launch_gate_cluster(const GateParams& p, cudaStream_t stream, cudaError_t* err);

@@ -1,0 +1,780 @@
+// Sparse decode over given lists, and dense decode, of one query token (up to eight heads per KV head): one launch of
+// thread-block clusters.
+//
+// Every (sequence, KV head) unit has S CTAs (two per SM) that meet in shared memory, as in the one-launch step: a producer
+// warp keeps a ring of three 64-token K/V stages in flight, eight consumer warps in two groups take alternate tiles, the
+// warps' partials and then the CTAs' (a slice of the channels each, by stores that count their bytes down on the
+// receiver's mbarrier) are merged without a trip through global memory.  How the work is dealt is decided in the kernel,
+// which alone knows the lists' lengths:
+//   even lists     cluster c takes unit c from end to end;
+//   uneven ones    every cluster takes its unit's first tiles, up to a line; what is left of the long units, laid end to end,
+//                  is dealt to the clusters whose own lists end well before it.  A cluster goes through its share piece by
+//                  piece, each a run of tiles of one unit; a unit of several pieces is put together from their partial
+//                  results, in global memory, by the CTAs that deliver the last one (rank r of the clusters has slice r of the
+//                  channels, so each slice is a matter of its own, with its own counter).
+// Every CTA comes to the same decision from the same numbers, so that nothing is waited for across clusters.
+//
+// What bounds it: memory, from the first tiles (2.8 us after the kernel may read its inputs) to the last; 128 ragged lists of 13 to
+// 102 tiles (247 MB) take 44.8 us, 52.6 by the decode kernel, whose CTAs make a schedule first and publish their partial
+// results with a fence and a ticket each; 64 lists of 103 tiles (216 MB) 37.9 and 47.1.  A CTA by itself is bound by its three
+// stages, of which the consumers hold one or two: 0.46 us a tile.
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
+#include "seer_cluster.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace seer {
+
+namespace {
+
+constexpr int kNW = 8;                                     // consumer warps; with the producer warp two CTAs per SM
+constexpr int kThreads = 32 * kNW + 32;
+constexpr int kStages = 3, kGroups = kNW / 4, kArrivals = kStages * kGroups;
+constexpr int kRows = kMaxGroup;
+
+struct __align__(1024) ListSmem {
+    unsigned char ring[kStages * kStageBytes];
+    // what the cluster's CTAs send after a piece's last tile, by turns: a CTA that sends its part of piece k + 2 has received all
+    // of piece k + 1, whose senders had read piece k's
+    __align__(16) float recv_o[2][kRows * kHeadDim];       // [source CTA][row][this CTA's slice of the channels]
+    float2 recv_ml[2][kMaxS][kRows];                       // [source CTA][row]: max, sum
+    float2 warp_ml[kNW][kRows];
+    // Tile n arrives in stage (n + pieces before) % kStages (behind a piece is a stage without a tile) and is announced on
+    // full[n % kArrivals]: a barrier belongs to one residue of the tile numbers and so to one consumer group, which follows all
+    // of its phases.
+    uint64_t full[kArrivals], empty[kStages];
+    // A stage, behind a piece, to put its partials together: given[piece % kStages].  (Pieces may be without a tile for a CTA; that
+    // of three before has been put together when a stage is given.)
+    uint64_t got_parts[2], dealt, given[kStages];
+    int meta[kArrivals];                                   // tokens from the tile's first row on (blocks of 16 or 32 tokens: per block, 8 bits each)
+    // uneven lists: how the tiles are dealt
+    int rest[kListUnits + 1];                              // tiles above the line of the units before
+    int room[kListUnits + 1];                              // tiles that the helpers before take (on the way there: the units' tiles)
+    int line, helpers, helper, is_last;                    // helper: number of this cluster among the helpers, or -1
+};
+static_assert(sizeof(ListSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
+
+__device__ __forceinline__ void consumers_sync() { worker_sync<kNW>(); }
+__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n) : "memory");
+}
+
+// A consumer warp's step over a staged K/V tile (as in the one-launch step, whose registers do not allow a copy of it that both
+// kernels share: 0.2 us of 14), for eight rows (query token, head) of the unit: the 16 tokens `w4` of the tile,
+// online softmax with running maximum m_run, sum l_run and output o of its own.  S^T = K . Q^T and O^T += V^T . P^T by mma.sync,
+// tokens (channels) on M, rows on N.
+// stage: K and V of the tile; bq: the Q^T fragments; nvw: valid tokens from this warp's first one on (at least one); back: newest
+// cached tokens that this thread's two rows may not see.
+__device__ __forceinline__ void tile_step(float (&o)[8][4], float (&m_run)[2], float (&l_run)[2], unsigned char* stage,
+                                          const uint32_t (&bq)[8][2], int nvw, const int (&back)[2], float scale_log2, int lane, int w4) {
+    const int rw = lane >> 2;
+    // lane-constant parts of the ldmatrix addresses (swizzle: 16-B chunk ^= row & 7)
+    const int k_row = 16 * w4 + ((lane >> 3) & 1) * 8 + (lane & 7), k_csel = lane >> 4;
+    const int v_row = 16 * w4 + ((lane >> 4) & 1) * 8 + (lane & 7), v_csel = (lane >> 3) & 1;
+    const int sw = lane & 7;
+    const uint32_t kbase = smem_u32(stage), vbase = kbase + kTileBytes;
+    if (nvw < 16) {
+        // ragged tail: rows past the sequence end may hold anything; this warp's are cleared in V, so that
+        // a zero probability times garbage cannot produce NaN
+        unsigned char* vt = stage + kTileBytes;
+        for (int x = lane; x < (16 - nvw) * 16; x += 32) {
+            const int r = 16 * w4 + nvw + (x >> 4), part = x & 15;
+            *reinterpret_cast<uint4*>(vt + (part >> 3) * kHalfTileBytes + r * 128 + ((part & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+    }
+    // ---- S^T = K . Q^T (four short accumulator chains) ----
+    float sa[4][4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) sa[x][0] = sa[x][1] = sa[x][2] = sa[x][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+        uint32_t a[4];
+        const int c8 = ((2 * ks) & 7) + k_csel;
+        ldmatrix_x4(a, kbase + (ks >> 2) * kHalfTileBytes + k_row * 128 + ((c8 ^ sw) << 4));
+        mma_bf16_16816(sa[ks & 3], a, bq[ks][0], bq[ks][1]);
+    }
+    float s[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) s[x] = ((sa[0][x] + sa[1][x]) + (sa[2][x] + sa[3][x])) * scale_log2;
+    const int lim0 = nvw - back[0], lim1 = nvw - back[1];      // tokens that a row sees of this warp's 16
+    if (rw >= lim0) s[0] = -INFINITY;
+    if (rw >= lim1) s[1] = -INFINITY;
+    if (rw + 8 >= lim0) s[2] = -INFINITY;
+    if (rw + 8 >= lim1) s[3] = -INFINITY;
+    // ---- online softmax over this warp's 16 tokens, per row (column of S^T) ----
+    float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
+#pragma unroll
+    for (int off = 4; off < 32; off <<= 1) {
+        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, off));
+        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, off));
+    }
+    const float mn0 = fmaxf(m_run[0], mx0), mn1 = fmaxf(m_run[1], mx1);
+    // a row that has seen nothing so far keeps max = -inf; exponents are then taken against 0
+    const float mb0 = mn0 == -INFINITY ? 0.f : mn0, mb1 = mn1 == -INFINITY ? 0.f : mn1;
+    const float al0 = fast_exp2(m_run[0] - mb0), al1 = fast_exp2(m_run[1] - mb1);
+    const bool same_max = __all_sync(0xffffffffu, m_run[0] == mn0 && m_run[1] == mn1);
+    m_run[0] = mn0;
+    m_run[1] = mn1;
+    const float p0 = fast_exp2(s[0] - mb0), p1 = fast_exp2(s[1] - mb1);
+    const float p2 = fast_exp2(s[2] - mb0), p3 = fast_exp2(s[3] - mb1);
+    l_run[0] = l_run[0] * al0 + (p0 + p2);
+    l_run[1] = l_run[1] * al1 + (p1 + p3);
+    if (!same_max) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a) { o[a][0] *= al0; o[a][1] *= al1; o[a][2] *= al0; o[a][3] *= al1; }
+    }
+    const uint32_t b0 = movmatrix_trans(pack_bf16x2(p0, p1));      // tokens 0-7 of the slice
+    const uint32_t b1 = movmatrix_trans(pack_bf16x2(p2, p3));      // tokens 8-15
+    // ---- O^T += V^T . P^T ----
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+        uint32_t f[4];
+        const int c8 = ((2 * a) & 7) + v_csel;
+        ldmatrix_x4_trans(f, vbase + (a >> 2) * kHalfTileBytes + v_row * 128 + ((c8 ^ sw) << 4));
+        mma_bf16_16816(o[a], f, b0, b1);
+    }
+}
+
+// Whether the lists are dealt.  In hundredths of a microsecond: a CTA that has the memory to itself gets through a tile in 0.46
+// us (three stages, of which one or two are being read); all CTAs together through one in 0.0047 us, taken as 0.004 because
+// the last ones are alone with their tiles; a deal costs 8 us: 2 to make it, 4 for the pieces' way through global memory, and
+// the helpers' second start.
+constexpr int kTileTime = 46, kPieceTiles = 8;             // (a piece costs a helper as much as so many tiles a CTA)
+__device__ __forceinline__ bool list_uneven(int total, int most, int units, int S) {
+    return kTileTime * (long long)most / S > max(2ll * total / 5, kTileTime * (long long)total / (units * S)) + 800;
+}
+
+// A cluster's piece of a unit: its tiles a .. b.  `x`, `end`: what is left of the cluster's share of the rest.
+struct Piece {
+    int u, a, b, n;                                        // n: tiles of the unit
+    int x, end;
+};
+
+// The place of x in the ascending v[0 .. n]: the last i < n with v[i] <= x.
+__device__ __forceinline__ int place_of(const int* v, int n, int x) {
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (v[mid] <= x) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// The deal, by one warp, whose lane l has the tiles of units l, l + 32, ... in n[]: the lowest line at which the helpers have
+// room below it for what is above it.  (Every cluster has the first tiles of its own unit, which are asked for before the
+// deal.  Few tiles are not worth a piece: a unit that ends a little above the line keeps what is its, a cluster with little
+// room is no helper, and where a helper's share ends a few tiles from a unit's end it ends there.)
+template <int COUNTS>
+__device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int units, int S, int cluster_id, int total, int most) {
+    const int lane = threadIdx.x & 31, cost = kPieceTiles * S, few = cost / 2;
+    auto above = [&](int line, int t) { return t - line >= few ? t - line : 0; };
+    auto below = [&](int line, int t) { return line - cost - t >= few ? line - cost - t : 0; };
+    int lo = max(total / units, kStages * S), hi = max(lo, most);      // (line `most`: nothing is above it)
+#pragma unroll 1
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        int free = 0;
+#pragma unroll
+        for (int k = 0; k < COUNTS; ++k)
+            if (lane + 32 * k < units) free += below(mid, n[k]) - above(mid, n[k]);
+        if (__reduce_add_sync(0xffffffffu, free) >= 0) hi = mid;
+        else lo = mid + 1;
+    }
+    const int line = lo;
+    int rest = 0, room = 0, helpers = 0;
+#pragma unroll
+    for (int k = 0; k < COUNTS; ++k) {
+        if (32 * k >= units) break;
+        const int v = lane + 32 * k;
+        const int over = v < units ? above(line, n[k]) : 0, mine = v < units ? below(line, n[k]) : 0;
+        int a = over, b = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int ta = __shfl_up_sync(0xffffffffu, a, o), tb = __shfl_up_sync(0xffffffffu, b, o);
+            if (lane >= o) { a += ta; b += tb; }
+        }
+        const unsigned has = __ballot_sync(0xffffffffu, mine > 0);
+        if (v < units) sm.rest[v] = rest + a - over;
+        if (mine > 0) {
+            const int at = helpers + __popc(has & ((1u << lane) - 1u));
+            sm.room[at] = room + b - mine;
+            if (v == cluster_id) sm.helper = at;
+        }
+        helpers += __popc(has);
+        rest += __shfl_sync(0xffffffffu, a, 31);
+        room += __shfl_sync(0xffffffffu, b, 31);
+    }
+    if (lane == 0) {
+        sm.rest[units] = rest;
+        sm.room[helpers] = room;
+        sm.helpers = helpers;
+        sm.line = line;
+    }
+    __syncwarp();
+    for (int k = lane; k < helpers; k += 32) {
+        const int x = sm.room[k];
+        if (x >= rest) break;
+        const int u = place_of(sm.rest, units, x), r0 = sm.rest[u], r1 = sm.rest[u + 1];
+        if (2 * (x - r0) < few) sm.room[k] = r0;
+        else if (2 * (r1 - x) < few) sm.room[k] = r1;
+    }
+    __syncwarp();
+}
+
+// grid (S, units), cluster (S, 1, 1).  SPREAD: the lists may be so long that it matters whether they are even.
+template <bool SPREAD>
+__device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p) {
+    extern __shared__ unsigned char smem_raw[];
+    // (aligned by an offset, not by a cast through an integer: the compiler then still knows the accesses for shared ones)
+    ListSmem& sm = *reinterpret_cast<ListSmem*>(smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023));
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), s_shift = 31 - __clz(S);
+    const int c_shift = 7 - s_shift;                       // log2 of the channels of a CTA's slice
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool producer = warp == kNW;
+    const int rows = p.group, cluster_id = blockIdx.y;
+    const uint32_t part_bytes = (uint32_t)(rows * kHeadDim * 4 + S * rows * 8);      // what a CTA receives per piece
+    if (tid < 32) {
+        if (tid < kArrivals) mbar_init(&sm.full[tid], 1);
+        if (tid < kStages) {
+            mbar_init(&sm.empty[tid], kNW);
+            mbar_init(&sm.given[tid], 1);
+        }
+        if (tid < 2) mbar_init(&sm.got_parts[tid], 1);
+        if (tid == 0) {
+            mbar_init(&sm.dealt, 1);
+            sm.line = 0x7fffffff;                          // (even lists)
+            sm.helper = -1;
+        }
+        mbar_fence_init();
+        if (tid < 2) mbar_arrive_expect_tx(&sm.got_parts[tid], part_bytes);
+    }
+    // (another CTA's shared memory is written only after the barrier this opens: it is then known to be running, and its
+    // mbarriers are initialised)
+    cluster_arrive();
+    if (producer && lane == 0) {
+        tma_prefetch_desc(&map_k);
+        tma_prefetch_desc(&map_v);
+    }
+    const bool dense = !p.block_idx;
+    const bool small = !dense && p.blocks_per_tile > 1;
+    auto sequence_of = [&](int u) { return p.kvh_magic ? (int)__umulhi((unsigned)u, p.kvh_magic) : u; };
+    // a unit's listed blocks, and its tiles
+    auto blocks_of = [&](int u, int L) -> int {
+        if (dense) return 0;
+        const int cnt = p.block_cnt ? p.block_cnt[u] : p.max_sel;          // (not behind a test on L: both loads in flight)
+        return L > 0 ? max(0, min(cnt, p.max_sel)) : 0;
+    };
+    auto tiles_of = [&](int n_blocks, int L) -> int {
+        if (dense) return L > 0 ? min((L + kTileTokens - 1) / kTileTokens, p.max_blocks_cap) : 0;
+        return small ? (n_blocks + p.blocks_per_tile - 1) >> p.bpt_shift : n_blocks << p.tpb_shift;
+    };
+    pdl_wait();
+    // (the first entries are asked for beside the count that says how many there are, not behind it)
+    int entry[4] = {-1, -1, -1, -1}, entry2[4] = {-1, -1, -1, -1};      // the list's entries of this lane's first tile, and of the second piece's
+    if (producer && !dense) {
+        const int t = (lane << s_shift) + rank;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int e = small ? (t << p.bpt_shift) + x : t >> p.tpb_shift;
+            if (x < p.blocks_per_tile) entry[x] = p.block_idx[(size_t)cluster_id * p.max_sel + min(e, p.max_sel - 1)];
+        }
+    }
+    Piece pc;
+    int L = p.seq_lens[sequence_of(cluster_id)], n_blocks = blocks_of(cluster_id, L);
+    pc.u = cluster_id;
+    pc.a = 0;
+    pc.b = pc.n = tiles_of(n_blocks, L);
+    pc.x = pc.end = 0;
+    __syncthreads();                                       // barriers initialised
+    // what the deal makes of this cluster's own unit, and its share of the rest
+    auto take_share = [&]() {
+        if (sm.line < 0x7fffffff && sm.rest[cluster_id + 1] > sm.rest[cluster_id]) pc.b = sm.line;
+        if (sm.helper >= 0) {
+            pc.x = sm.room[sm.helper];
+            pc.end = min(sm.room[sm.helper + 1], sm.rest[p.num_units]);
+        }
+    };
+    // on to the next piece; false: that was the last
+    auto next_piece = [&]() -> bool {
+        if (pc.x >= pc.end) return false;
+        pc.u = place_of(sm.rest, p.num_units, pc.x);       // (the last one that begins there: the others have nothing above the line)
+        const int r0 = sm.rest[pc.u], r1 = sm.rest[pc.u + 1], line = sm.line;
+        pc.a = line + pc.x - r0;
+        pc.x = min(r1, pc.end);
+        pc.b = line + pc.x - r0;
+        pc.n = line + r1 - r0;
+        return true;
+    };
+    auto mine_of = [&]() -> int { return max(0, pc.b - pc.a - rank + S - 1) >> s_shift; };      // this CTA's tiles of the piece
+    bool dead = false;                                     // a wait ran out: go through the motions, the results are invalid
+    int tiles_before = 0, pieces_before = 0;               // this CTA's tiles, and the cluster's pieces, before the current one
+    // (What is done for a piece is written once and compiled twice: for the cluster's own unit, which mostly is all there is, the
+    // numbers before it are known to be zero.)
+    using First = std::true_type;
+    using Later = std::false_type;
+    if (producer) {
+        if (p.next_early) pdl_launch_dependents();
+        // the deal is made (by a consumer warp); a helper's first piece is looked up at once
+        int L2 = 0, n_blocks2 = 0;
+        auto see_deal = [&]() {
+            if (!mbar_wait(&sm.dealt, 0, p.status)) dead = true;
+            __syncwarp();
+            take_share();
+            if (pc.x < pc.end) {
+                const int u = place_of(sm.rest, p.num_units, pc.x), t = sm.line + pc.x - sm.rest[u] + (lane << s_shift) + rank;
+                L2 = p.seq_lens[sequence_of(u)];
+                n_blocks2 = blocks_of(u, L2);
+                if (!dense) {
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        const int e = small ? (t << p.bpt_shift) + x : t >> p.tpb_shift;
+                        if (x < p.blocks_per_tile) entry2[x] = p.block_idx[(size_t)u * p.max_sel + min(e, p.max_sel - 1)];
+                    }
+                }
+            }
+        };
+        int tile0 = 0, piece = 0;
+        do {
+            if (SPREAD && piece > 0) {
+                const bool first = piece == 1;
+                L = first ? L2 : p.seq_lens[sequence_of(pc.u)];
+                n_blocks = first ? n_blocks2 : blocks_of(pc.u, L);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) entry[x] = entry2[x];
+            }
+            const int i = sequence_of(pc.u), h = pc.u - i * p.num_kv_heads;
+            int n_local = mine_of();
+            if (SPREAD && piece == 0 && n_local == 0) see_deal();
+            const int n_i = (L + p.block_size - 1) >> p.bs_shift;
+            const int32_t* list = p.block_idx + (size_t)pc.u * p.max_sel;
+            // (a CTA's first tiles do not depend on the deal)
+            const bool own = SPREAD && piece == 0;
+            for (int base = 0, count; base < n_local; base += count) {
+                count = !own || base > kStages ? 32 : base == 0 ? kStages : 32 - kStages;
+                const int it = base + lane;
+                int row[4] = {0, 0, 0, 0}, outer[4] = {0, 0, 0, 0}, nv_all = 0, n_sub = 0;
+                if (it < n_local) {
+                    const int t = pc.a + (it << s_shift) + rank;
+                    const int n_try = small ? p.blocks_per_tile : 1;
+                    const int span = small ? p.block_size : kTileTokens;
+                    const bool have = it < 32 && (!SPREAD || piece <= 1);
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        if (x < n_try) {
+                            int tok0 = -1;
+                            if (dense) {
+                                tok0 = t * kTileTokens;
+                            } else if (small) {
+                                const int e = (t << p.bpt_shift) + x;
+                                if (e < n_blocks) {
+                                    const int blk = have ? entry[x] : list[e];
+                                    if (blk >= n_i) raise_status(p.status, DEV_BAD_INDEX);
+                                    if (blk >= 0 && blk < n_i) tok0 = blk << p.bs_shift;
+                                }
+                            } else {
+                                const int blk = have ? entry[0] : list[t >> p.tpb_shift];
+                                if (blk >= n_i) raise_status(p.status, DEV_BAD_INDEX);
+                                if (blk >= 0 && blk < n_i) tok0 = (blk << p.bs_shift) + (t & (p.tiles_per_block - 1)) * kTileTokens;
+                            }
+                            int nv = tok0 >= 0 ? max(0, min(span, L - tok0)) : 0;
+                            if (nv > 0) {
+                                outer[x] = i;
+                                row[x] = tok0;
+                                if (p.page_table) {
+                                    const int pg = p.page_table[(size_t)i * p.page_table_stride + tok0 / p.page_size];
+                                    outer[x] = pg;
+                                    row[x] = tok0 % p.page_size;
+                                    if (pg < 0 || pg >= p.num_pages) { raise_status(p.status, DEV_BAD_INDEX); nv = 0; }
+                                }
+                            }
+                            nv_all |= nv << (8 * x);
+                            n_sub += nv > 0;
+                        }
+                    }
+                }
+                __syncwarp();
+                // lane s asks for tile s of the batch
+                const int m = min(count, n_local - base);
+                for (int s = 0; s < m; ++s) {
+                    if (lane == s) {
+                        const int n = tile0 + it, slot = n + piece, st = slot % kStages;
+                        if (!dead && !mbar_wait(&sm.empty[st], ((slot / kStages) & 1) ^ 1, p.status)) dead = true;
+                        unsigned char* dst = sm.ring + st * kStageBytes;
+                        uint64_t* full = &sm.full[n % kArrivals];
+                        sm.meta[n % kArrivals] = nv_all;   // (the tile kArrivals back has been read: a later one of its group had this stage or a later one)
+                        if (dead || n_sub == 0) {
+                            mbar_arrive(full);
+                        } else if (small) {
+                            const int sub_bytes = p.block_size * 128;      // one half (64 channels) of one block
+                            mbar_arrive_expect_tx(full, (uint32_t)(n_sub * 4 * sub_bytes));
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) {
+                                if ((nv_all >> (8 * x)) & 0xff) {
+                                    unsigned char* d2 = dst + x * sub_bytes;
+                                    tma_load_4d(d2, &map_k, full, 0, row[x], h, outer[x]);
+                                    tma_load_4d(d2 + kHalfTileBytes, &map_k, full, 64, row[x], h, outer[x]);
+                                    tma_load_4d(d2 + kTileBytes, &map_v, full, 0, row[x], h, outer[x]);
+                                    tma_load_4d(d2 + kTileBytes + kHalfTileBytes, &map_v, full, 64, row[x], h, outer[x]);
+                                }
+                            }
+                        } else {
+                            mbar_arrive_expect_tx(full, kStageBytes);
+                            tma_load_4d(dst, &map_k, full, 0, row[0], h, outer[0]);
+                            tma_load_4d(dst + kHalfTileBytes, &map_k, full, 64, row[0], h, outer[0]);
+                            tma_load_4d(dst + kTileBytes, &map_v, full, 0, row[0], h, outer[0]);
+                            tma_load_4d(dst + kTileBytes + kHalfTileBytes, &map_v, full, 64, row[0], h, outer[0]);
+                        }
+                    }
+                    __syncwarp();
+                }
+                dead = __any_sync(0xffffffffu, dead);
+                if (own && base == 0) {
+                    see_deal();
+                    n_local = mine_of();
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) entry[x] = __shfl_down_sync(0xffffffffu, entry[x], kStages);
+                }
+            }
+            if (!SPREAD) break;
+            // The slot behind a piece's last tile is the consumers': its stage is where they put their partials together.  They
+            // take it when the producer gives it, which it does, as with a tile, when the stage is free: every phase of its
+            // barrier is thus seen before the next one can end.  (Behind the last piece nobody asks for the stage again.)
+            tile0 += n_local;
+            if (pc.x < pc.end) {
+                const int slot = tile0 + piece;
+                if (!dead && !mbar_wait(&sm.empty[slot % kStages], ((slot / kStages) & 1) ^ 1, p.status)) dead = true;
+                dead = __any_sync(0xffffffffu, dead);
+                if (lane == 0) mbar_arrive(&sm.given[piece % kStages]);
+            }
+            ++piece;
+        } while (next_piece());
+        cluster_wait();                                    // (the barrier opened at the top)
+        cluster_arrive();
+    } else {
+        const int group = warp >> 2, w4 = warp & 3, qd = lane & 3, rw = lane >> 2;
+        // Q^T B-fragments: this thread supplies row rw of the unit's queries
+        uint32_t bq[8][2];
+        auto load_q = [&](int u) {
+            const int i = sequence_of(u), h = u - i * p.num_kv_heads;
+            const uint32_t* qrow = reinterpret_cast<const uint32_t*>(
+                p.q + ((size_t)i * p.num_q_heads + (size_t)h * p.group + (rw < rows ? rw : 0)) * kHeadDim);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                bq[ks][0] = rw < rows ? __ldg(qrow + 8 * ks + qd) : 0u;
+                bq[ks][1] = rw < rows ? __ldg(qrow + 8 * ks + 4 + qd) : 0u;
+            }
+        };
+        load_q(pc.u);
+        if (p.next_early) pdl_launch_dependents();
+        // blocks of 16 or 32 tokens: which of the gathered blocks this warp's rows belong to, and where in it
+        const int sub_w = !small ? 0 : p.block_size == 16 ? w4 : w4 >> 1;
+        const int off_w = !small ? 16 * w4 : p.block_size == 16 ? 0 : (w4 & 1) * 16;
+        constexpr int back[2] = {0, 0};
+        if (SPREAD && warp == 0) {
+            // The deal, while the first tiles travel.  The units' tiles, a few units a lane:
+            constexpr int kCounts = (kListUnits + 31) / 32;
+            int n[kCounts], len[kCounts], total = 0, most = 0;
+#pragma unroll
+            for (int k = 0; k < kCounts; ++k) {            // (all loads on their way before the first is looked at)
+                const int v = min(lane + 32 * k, p.num_units - 1);
+                len[k] = p.seq_lens[sequence_of(v)];
+                n[k] = p.block_cnt ? p.block_cnt[v] : p.max_sel;
+            }
+#pragma unroll
+            for (int k = 0; k < kCounts; ++k) {
+                n[k] = lane + 32 * k < p.num_units ? tiles_of(len[k] > 0 ? max(0, min(n[k], p.max_sel)) : 0, len[k]) : 0;
+                total += n[k];
+                most = max(most, n[k]);
+            }
+            total = __reduce_add_sync(0xffffffffu, total);
+            most = __reduce_max_sync(0xffffffffu, most);
+            if (list_uneven(total, most, p.num_units, S)) deal(sm, n, p.num_units, S, cluster_id, total, most);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.dealt);
+        }
+        if (SPREAD) {
+            mbar_wait(&sm.dealt, 0, p.status);             // (before the first tile is there)
+            __syncwarp();
+            take_share();
+        }
+        // false: that was the last piece
+        auto consume = [&](auto first_c) -> bool {
+            constexpr bool FIRST = decltype(first_c)::value;
+            const int tile0 = FIRST ? 0 : tiles_before, piece = FIRST ? 0 : pieces_before;
+            const int n_end = tile0 + mine_of();
+            float o[8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+#pragma unroll
+            for (int a = 0; a < 8; ++a) o[a][0] = o[a][1] = o[a][2] = o[a][3] = 0.f;
+            for (int n = FIRST ? group : tile0 + ((tile0 ^ group) & 1); n < n_end; n += kGroups) {
+                const int st = (n + piece) % kStages;
+                if (!dead && !mbar_wait(&sm.full[n % kArrivals], (n / kArrivals) & 1, p.status)) dead = true;
+                const int nvw = (small ? (sm.meta[n % kArrivals] >> (8 * sub_w)) & 0xff : sm.meta[n % kArrivals]) - off_w;   // valid tokens from this warp's first row on
+                if (nvw > 0 && !dead) tile_step(o, m_run, l_run, sm.ring + st * kStageBytes, bq, nvw, back, p.scale_log2, lane, w4);
+                __syncwarp();
+                if (lane == 0) mbar_arrive_n(&sm.empty[st], kNW / 4);
+            }
+            const bool more = SPREAD && pc.x < pc.end;
+            // ---- the warps' partials, then the CTAs' -----------------------------------------------------------------
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) {
+                l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], off);
+                l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], off);
+            }
+            const int st = (n_end + piece) % kStages, turn = piece & 1;
+            // [warp][row][channel]; the channel's place is swizzled by the row, so that a warp's stores meet different banks
+            float* parts = reinterpret_cast<float*>(sm.ring + st * kStageBytes);
+            if (more && !dead && !mbar_wait(&sm.given[piece % kStages], (piece / kStages) & 1, p.status)) dead = true;
+            consumers_sync();                              // every tile of the piece has been read: the slot's stage is free
+            float* part = parts + warp * (kRows * kHeadDim);
+            const int sw = qd << 3;
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                const int d0 = (16 * a + rw) ^ sw, d1 = (16 * a + rw + 8) ^ sw;
+                part[2 * qd * kHeadDim + d0] = o[a][0];
+                part[(2 * qd + 1) * kHeadDim + d0] = o[a][1];
+                part[2 * qd * kHeadDim + d1] = o[a][2];
+                part[(2 * qd + 1) * kHeadDim + d1] = o[a][3];
+            }
+            if (rw == 0) {
+                sm.warp_ml[warp][2 * qd] = make_float2(m_run[0], l_run[0]);
+                sm.warp_ml[warp][2 * qd + 1] = make_float2(m_run[1], l_run[1]);
+            }
+            __syncwarp();
+            if (FIRST) cluster_wait();                // every CTA of the cluster has started (the barrier opened at the top)
+            consumers_sync();
+            // a warp per row; lane: four channels
+            if (warp < rows) {
+                const int c = 4 * lane;
+                float M = -INFINITY, l = 0.f;
+                float2 ml[kNW];
+#pragma unroll
+                for (int x = 0; x < kNW; ++x) {
+                    ml[x] = sm.warp_ml[x][warp];
+                    M = fmaxf(M, ml[x].x);
+                }
+                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float* src = parts + warp * kHeadDim + (c ^ ((warp >> 1) << 3));
+#pragma unroll
+                for (int x = 0; x < kNW; ++x) {
+                    const float f = ml[x].x == -INFINITY ? 0.f : fast_exp2(ml[x].x - M);
+                    const float4 v = *reinterpret_cast<const float4*>(src + x * (kRows * kHeadDim));
+                    l = fmaf(ml[x].y, f, l);
+                    sum.x = fmaf(v.x, f, sum.x);
+                    sum.y = fmaf(v.y, f, sum.y);
+                    sum.z = fmaf(v.z, f, sum.z);
+                    sum.w = fmaf(v.w, f, sum.w);
+                }
+                const int to = c >> c_shift;
+                send_f32x4(cluster_addr(sm.recv_o[turn] + (((rank * kRows + warp) << c_shift) | (c & ((1 << c_shift) - 1))), to), sum,
+                           cluster_addr(&sm.got_parts[turn], to));
+                if (lane < S) send_f32x2(cluster_addr(&sm.recv_ml[turn][rank][warp], lane), make_float2(M, l), cluster_addr(&sm.got_parts[turn], lane));
+            }
+            const Piece done = pc;
+            if (more) {
+                next_piece();
+                load_q(pc.u);                              // (on their way under what follows)
+                fence_proxy_async_smem();                  // the stage goes over to the copy engine
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.empty[st]);
+            }
+            wait_sent(&sm.got_parts[turn], p.status, (piece >> 1) & 1);
+            if (!more) cluster_arrive();
+            else if (tid == 0) mbar_arrive_expect_tx(&sm.got_parts[turn], part_bytes);       // (for the piece after the next)
+            // ---- this CTA's slice of the channels: the output, or the piece's part of it --------------------------------
+            const int pairs = rows << (c_shift - 1);       // channel pairs of the slice, all rows
+            const bool whole = !SPREAD || done.b - done.a == done.n;
+            const int i = sequence_of(done.u), h = done.u - i * p.num_kv_heads;
+            // partial results in global memory: of the owner's piece and the helpers' (helper k's of unit u: k + u grows from one
+            // piece to the next), by rank: max and sum of the rows, then the sums
+            const int slice = 1 << c_shift, part_stride = 2 * kRows + (kRows << c_shift);
+            auto part_of = [&](int slot) { return p.part_o + (size_t)(slot * S + rank) * part_stride; };
+            auto write_out = [&](int r, int c, float M, float l, float a0, float a1) {
+                const float inv = l > 0.f ? 1.f / l : 0.f;
+                const size_t row = (size_t)i * p.num_q_heads + (size_t)h * p.group + r;
+                *reinterpret_cast<uint32_t*>(p.out + row * kHeadDim + (rank << c_shift) + c) = pack_bf16x2(a0 * inv, a1 * inv);
+                if (p.lse && rank == 0 && c == 0) p.lse[row] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+            };
+#pragma unroll 1
+            for (int x = tid; x < pairs; x += 32 * kNW) {
+                const int r = x >> (c_shift - 1), c = 2 * (x & ((slice >> 1) - 1));
+                float M = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f;
+                float2 ml[kMaxS];
+#pragma unroll
+                for (int s = 0; s < kMaxS; ++s) {
+                    ml[s] = s < S ? sm.recv_ml[turn][s][r] : make_float2(-INFINITY, 0.f);
+                    M = fmaxf(M, ml[s].x);
+                }
+#pragma unroll
+                for (int s = 0; s < kMaxS; ++s) {
+                    if (s < S) {
+                        const float f = ml[s].x == -INFINITY ? 0.f : fast_exp2(ml[s].x - M);
+                        const float2 v = *reinterpret_cast<const float2*>(&sm.recv_o[turn][((s * kRows + r) << c_shift) + c]);
+                        l = fmaf(ml[s].y, f, l);
+                        a0 = fmaf(v.x, f, a0);
+                        a1 = fmaf(v.y, f, a1);
+                    }
+                }
+                if (whole) {
+                    write_out(r, c, M, l, a0, a1);
+                } else {
+                    float* dst = part_of(done.a == 0 ? done.u : p.num_units + sm.helper + done.u);
+                    if (c == 0) *reinterpret_cast<float2*>(dst + 2 * r) = make_float2(M, l);
+                    *reinterpret_cast<float2*>(dst + 2 * kRows + (r << c_shift) + c) = make_float2(a0, a1);
+                }
+            }
+            if (!whole) {
+                // the helpers that have a piece of the unit; whoever counts the last puts the pieces together, in order
+                const int k_lo = place_of(sm.room, sm.helpers, sm.rest[done.u]), k_hi = place_of(sm.room, sm.helpers, sm.rest[done.u + 1] - 1);
+                int* count = reinterpret_cast<int*>(p.tickets) + done.u * kMaxS + rank;
+                __threadfence();
+                consumers_sync();
+                if (tid == 0) sm.is_last = atomicAdd(count, 1) == k_hi - k_lo + 1;
+                consumers_sync();
+                if (sm.is_last) {
+                    __threadfence();
+                    if (tid == 0) *count = 0;              // (as every launch finds it)
+#pragma unroll 1
+                    for (int x = tid; x < pairs; x += 32 * kNW) {
+                        const int r = x >> (c_shift - 1), c = 2 * (x & ((slice >> 1) - 1));
+                        float M = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f;
+#pragma unroll 1
+                        for (int k0 = k_lo - 1; k0 <= k_hi; k0 += 4) {
+                            float2 ml[4], v[4];            // (four pieces' numbers on their way at a time)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const int k = k0 + e;
+                                const float* src = part_of(k < k_lo ? done.u : p.num_units + min(k, k_hi) + done.u);
+                                ml[e] = k <= k_hi ? __ldcg(reinterpret_cast<const float2*>(src + 2 * r)) : make_float2(-INFINITY, 0.f);
+                                v[e] = k <= k_hi ? __ldcg(reinterpret_cast<const float2*>(src + 2 * kRows + (r << c_shift) + c)) : make_float2(0.f, 0.f);
+                            }
+                            float m = M;
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) m = fmaxf(m, ml[e].x);
+                            const float mb = m == -INFINITY ? 0.f : m, f = fast_exp2(M - mb);
+                            M = m;
+                            l *= f;
+                            a0 *= f;
+                            a1 *= f;
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float g = fast_exp2(ml[e].x - mb);
+                                l = fmaf(ml[e].y, g, l);
+                                a0 = fmaf(v[e].x, g, a0);
+                                a1 = fmaf(v[e].y, g, a1);
+                            }
+                        }
+                        write_out(r, c, M, l, a0, a1);
+                    }
+                }
+            }
+            tiles_before = n_end;
+            pieces_before = piece + 1;
+            return more;
+        };
+        bool more = consume(First());
+        if constexpr (SPREAD) {
+#pragma unroll 1
+            while (more) more = consume(Later());
+        }
+    }
+    // No CTA leaves before every one has received all that was sent to it: neither the receiver's shared memory nor the
+    // sender's place in the cluster may be gone while a store is under way.
+    cluster_wait();
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
+list_step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                         const __grid_constant__ DecodeParams p) {
+    list_body<false>(map_k, map_v, p);
+}
+__global__ void __launch_bounds__(kThreads, 2)
+dealt_decode_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                    const __grid_constant__ DecodeParams p) {
+    list_body<true>(map_k, map_v, p);
+}
+
+cudaLaunchConfig_t config_of(int S, int units, cudaStream_t stream, cudaLaunchAttribute (&attr)[2]) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S, units);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = sizeof(ListSmem) + 1024;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+template <typename Kernel>
+int resident_of(Kernel* kernel, int k) {
+    int n = 0;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ListSmem) + 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) {
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = config_of(1 << k, 1, nullptr, attr);
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
+    }
+    cudaGetLastError();                                    // (a refused size is no error of the caller's)
+    return n;
+}
+
+// Clusters of 2^k CTAs that the device holds at once, asked once per device; 0: it does not take such clusters.
+int resident_lists(int k) {
+    static int cached[kMaxDevices][5];                     // (value + 1; 0: not asked yet.  A race asks twice and stores the same)
+    int& c = cached[current_device_slot()][k];
+    if (c == 0) c = min(resident_of(list_step_cluster_kernel, k), resident_of(dealt_decode_kernel, k)) + 1;
+    return c - 1;
+}
+
+}  // namespace
+
+// As many CTAs per unit as keep every cluster resident at once and still have something to do each.  Above 128 tiles a CTA the
+// decode kernel, whose CTAs share all tiles throughout, is ahead where lists are ragged.  us a call, decode kernel -> clusters, 8
+// KV heads; all lists equally long / lengths spread evenly from an eighth on / one sequence's lists eight times the others':
+//     32 tiles a CTA      16 sequences (S = 2)  54.0 -> 43 / 40.8 -> 30.8 / 21.3 -> 20.4      24 (S = 1)  - / 39.3 -> 28.2 / 14.7 -> 19.1
+//                          8 sequences (S = 4)  47.0 -> 37.5 / 39.4 -> 31.8 / 24.8 -> 23.1    10 (S = 2)  - / 31.1 -> 24.6 / 16.5 -> 18.8
+//     48                  16 sequences          75.1 -> 64 / 50.8 -> 42.8 / 26.8 -> 26.5       8          73.8 -> 64.0 / 50.8 -> 44.4 / 32.4 -> 28.0
+//     128, dense           8 sequences           164 -> 154 / 105 -> 103
+//     192, dense           8 sequences           241 -> 228 / 147 -> 151
+//     256, dense           8 sequences           313 -> 305 / 193 -> 201
+// (One long sequence among short ones: as clusters without a deal 64 instead of 39 us where its lists have 102 tiles a CTA.)
+constexpr int kMostTiles = 128;
+ListPlan list_plan(int units, long long max_tiles) {
+    ListPlan plan = {0, false, false};
+    if (units > kListUnits || units * max_tiles >= (1ll << 30)) return plan;
+    for (int k = 4; k >= 0; --k) {
+        const int S = 1 << k;
+        if (k > 0 && S > max_tiles) continue;              // a CTA would have nothing to do
+        if (units > resident_lists(k)) continue;
+        if (max_tiles <= (long long)kMostTiles * S) plan.S = S;
+        plan.spread = max_tiles > (long long)S * (16 + 2 * S);       // (shorter lists gain nothing by a deal)
+        plan.next_early = 2 * units <= resident_lists(k);
+        break;
+    }
+    return plan;
+}
+
+size_t list_part_bytes(int units, int S) {
+    return (size_t)units * 3 * S * (2 * kRows + (size_t)kRows * kHeadDim / S) * sizeof(float);
+}
+
+cudaError_t launch_lists(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, int S, cudaStream_t stream) {
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = config_of(S, p.num_units, stream, attr);
+    return cudaLaunchKernelEx(&cfg, p.spread ? dealt_decode_kernel : list_step_cluster_kernel, map_k, map_v, p);
+}
+
+}  // namespace seer

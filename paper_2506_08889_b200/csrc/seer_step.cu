@@ -8,7 +8,7 @@
 //      scores of each CTA's keys into every CTA's; every CTA selects for itself, and keeps the listed tiles that it
 //      reads (tile t belongs to CTA t mod S); meanwhile the producer warps compress the block that has just filled,
 //      if one has;
-//      list (!GATE): the CTA reads its tiles' numbers from the caller's list, or counts them off (dense);
+//      list (!GATE, several query tokens): the CTA reads its tiles' numbers from the caller's list, or counts them off (dense);
 //   2. tiles: one producer warp keeps a ring of three 64-token K/V stages in flight; eight consumer warps, two
 //      groups of four, take alternate tiles, a warp 16 tokens (the same tensor-core steps as decode_kernel);
 //   3. combine: the warps' partials meet in shared memory, the CTA's go, a slice of the channels each, to the
@@ -23,8 +23,7 @@
 #include <cstring>
 #include <type_traits>
 
-#include "seer_gate_device.cuh"
-#include "seer_internal.h"
+#include "seer_cluster.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -32,10 +31,6 @@ namespace seer {
 
 namespace {
 
-constexpr int kHalfTileBytes = kTileTokens * 128;          // 64 rows x 128 B (64 bf16 channels)
-constexpr int kTileBytes = 2 * kHalfTileBytes;             // one K or V tile: 16 KiB
-constexpr int kStageBytes = 2 * kTileBytes;                // K + V
-constexpr int kMaxS = 16;
 constexpr int kCodes = 256;                                // tile (or gathered block) numbers that a CTA holds
 constexpr int kListed = 8192;                              // most scored blocks of a list
 constexpr int kBins = 1024;                                // histogram of the selection
@@ -127,13 +122,6 @@ struct GatePlace {                                         // offsets in the rin
 };
 static_assert(kStepMaxBlocks <= 65536, "16 bits a block");
 
-// Barriers among the worker warps, and between them and the producer.  The aligned forms are for a warp whose lanes are
-// together; behind a loop or branch of some lanes they need not be, so they are brought together here.
-template <int NW>
-__device__ __forceinline__ void worker_sync() {
-    __syncwarp();
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory");
-}
 template <int NW>
 __device__ __forceinline__ void tiles_listed_arrive() {
     __syncwarp();
@@ -165,50 +153,6 @@ template <bool GATE>
 struct GateArg { GateParams g; };
 template <>
 struct GateArg<false> {};
-
-// ---- stores into a CTA of the cluster (addr, bar: of its shared memory, cluster_addr), counted on its mbarrier ----------
-__device__ __forceinline__ uint32_t cluster_addr(const void* mine, int rank) {
-    uint32_t a;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ void send_u32(uint32_t addr, uint32_t v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void send_f32x2(uint32_t addr, float2 v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ void send_f32x4(uint32_t addr, float4 v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y),
-                 "f"(v.z), "f"(v.w), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ void send_min(uint32_t addr, uint32_t v, uint32_t bar) {
-    asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.min.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ void send_max(uint32_t addr, uint32_t v, uint32_t bar) {
-    asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.max.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
-                 : "memory");
-}
-// Bounded wait for what the cluster's CTAs have sent (the first and only phase of `bar`).
-__device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status) {
-    uint32_t ok = 0;
-    for (uint32_t it = 0; it < (1u << 24) && !ok; ++it) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(smem_u32(bar))
-            : "memory");
-        if (!ok && it > 64) __nanosleep(64);
-    }
-    if (!ok) raise_status(status, DEV_TIMEOUT);
-    __syncwarp();                                          // (the lanes need not have left the loop together)
-    return ok != 0;
-}
 
 // The selection of the `need` best of the candidates [0, n_cand), 0 < need < n_cand, by a CTA's worker warps.  Comparisons
 // only: the lower block number wins a tie, NaN is below every number.  A histogram over a monotone linear map of [min, max]
@@ -1560,8 +1504,7 @@ int resident_clusters(bool wide, int k) {
     int& c = cached[current_device_slot()][wide][k];
     if (c == 0) {
         c = wide ? min(resident_of<16, true, true>(k), resident_of<16, false, true>(k)) + 1
-                 : min(min(resident_of<8, true, false>(k), resident_of<8, false, false>(k)),
-                       min(resident_of<8, true, true>(k), resident_of<8, false, true>(k))) + 1;
+                 : min(resident_of<8, true, false>(k), min(resident_of<8, true, true>(k), resident_of<8, false, true>(k))) + 1;
     }
     return c - 1;
 }
@@ -1579,17 +1522,13 @@ int resident_clusters(bool wide, int k) {
 // the longest list that there can be, not how uneven the lists are, and one long sequence among short ones leaves most
 // clusters idle.  us a call, decode kernel -> clusters, 8 KV heads; one sequence's lists long / half of them / all, by the
 // tiles a CTA of a long one:
-//     lists, 24 sequences (S = 1)    16: 13.3 -> 12.2 / 20.4 -> 14.0 / 34.1 -> 21.9    32: 13.7 -> 18.8 / 35 -> 26.6 / 50 -> 37.7
-//            16 sequences (S = 2)    16: 12.8 -> 11.9 / 20.9 -> 15.3 / 32.2 -> 25.7    32: 14.5 -> 18.9 / 37.5 -> 28.4 / 53.9 -> 46.0
-//             8 sequences (S = 4)    16: 13.9 -> 12.2 / 19.8 -> 14.7 / 30.6 -> 25.6    32: 17.4 -> 19.8 / 35.9 -> 27.8 / 52.5 -> 45.0
-//             4 sequences (S = 8)    32: 21.3 -> 21.8 / 34.9 -> 27.7 / 53.8 -> 45.8    64: 38.4 -> 41.2 / 54.5 -> 48.2 / 91.4 -> 83.7
-//            16 sequences, 20 rows (S = 1)
+//     lists, 16 sequences, 20 rows (S = 1)
 //                                    16: 21.6 -> 18.8 / 27.6 -> 19.3 / 25.7 -> 20.1    32: 22.4 -> 30.7 / 39.7 -> 32.1 / 56.3 -> 33.5
 //     steps, 16 sequences (S = 2)    64: 31.7 -> 46.8 / 72.3 -> 58.6 / 103 -> 93      128: 45.3 -> 82.7 / 108 -> 103 / 178 -> 173
 //             8 sequences (S = 4)    64: 35.6 -> 47.4 / 69.6 -> 56.6 / 101 -> 91      128: 57.1 -> 80.6 / 105 -> 101 / 176 -> 172
-// Given lists and dense calls, whose lengths follow the sequences', keep to where one long sequence does not lose: 16 + 2 S
-// tiles a CTA (a decode call pays for its parts whatever its size, and more the longer its longest unit is).  The lists of a
-// step are all as long as the budget but for sequences shorter than that: the line is at 64, where all but the most uneven
+// Given lists and dense calls of several query tokens, whose lengths follow the sequences', keep to where one long sequence
+// does not lose much: 16 + 2 S tiles a CTA (a decode call pays for its parts whatever its size, and more the longer its longest
+// unit is; lists of one query token are dealt: seer_lists.cu).  The lists of a step are all as long as the budget but for sequences shorter than that: the line is at 64, where all but the most uneven
 // batches gain; at 128 the even ones gain 3 % and the uneven ones lose up to half.  With a few more CTAs than SMs the SMs
 // that hold two of them are the last to finish (80 units, 64 tiles a CTA, 160 CTAs: 65 -> 67; 32 tiles: 40.8 -> 37.5), so
 // the line is at 32 there.  149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles
@@ -1647,8 +1586,11 @@ cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const 
         const cudaLaunchConfig_t cfg = config_of<NW, true, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
         return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, MULTI>, map_k, map_v, p, GateArg<true>{*g});
     }
-    const cudaLaunchConfig_t cfg = config_of<NW, false, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
-    return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, false, MULTI>, map_k, map_v, p, GateArg<false>{});
+    if constexpr (MULTI) {
+        const cudaLaunchConfig_t cfg = config_of<NW, false, true>(plan.S, p.num_units, plan.parts, stream, attr);
+        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, false, true>, map_k, map_v, p, GateArg<false>{});
+    }
+    return cudaErrorInvalidValue;                          // (lists of one query token: seer_lists.cu)
 }
 
 }  // namespace

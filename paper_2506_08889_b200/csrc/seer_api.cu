@@ -198,7 +198,7 @@ seer_status refuse_capture(seer_ctx* ctx, void* stream) {
 
 seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const void* q, int q_len,
                           const int32_t* block_idx, const int32_t* block_cnt, int max_sel, bool sparse,
-                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0, false, false}) {
+                          void* out, float* lse, void* stream, const GateParams* gate = nullptr, StepPlan plan = {0, 1, 0, false, false, false}) {
     // (gate: the whole step in one launch, by `plan`)
     if (!ctx) return SEER_ERR_INVALID_ARG;
     seer_status st = check_shape(ctx, shape);
@@ -342,9 +342,20 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
     if (plan.S > 0) {
         p.rows = plan.rows;
         p.next_early = plan.next_early;
+        if (plan.spread) {                                 // (by the lengths both launches decide which of them does the attention)
+            const int k = gate->token_budget / shape->block_size;
+            p.sel_from_lens = k < 1 ? 1 : k < max_sel ? k : max_sel;
+        }
         ce = launch_step_cluster(mk_copy, *mv, p, gate, plan, static_cast<cudaStream_t>(stream));
         if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "decode launch: %s", cudaGetErrorString(ce));
         ctx->launches += 1;
+        if (plan.spread) {
+            p.part_o = reinterpret_cast<float*>(ctx->ws + w.scratch);
+            p.spread = 1;
+            ce = launch_lists(mk_copy, *mv, p, plan.S, static_cast<cudaStream_t>(stream));
+            if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "decode launch: %s", cudaGetErrorString(ce));
+            ctx->launches += 1;
+        }
         return SEER_OK;
     }
     for (int t0 = 0; t0 < q_len; t0 += tok_per_launch) {
@@ -809,15 +820,20 @@ static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     const int rows = q_len * (shape->num_q_heads / shape->num_kv_heads);
     if (!ctx->use_clusters || gate->max_blocks > kStepMaxBlocks || ctx->chain_attention || ctx->chain_gate || (q_len == 1 && ctx->chain_step) ||
         (ctx->wide_variant && rows > 16 && shape->block_size >= kTileTokens))
-        return StepPlan{0, 1, 0, false, false};
+        return StepPlan{0, 1, 0, false, false, false};
     const long long bs = shape->block_size, cap = kv->max_seq_len > 0 ? (kv->max_seq_len + bs - 1) / bs : 1;
     long long blocks = token_budget / bs > 1 ? token_budget / bs : 1;
     if (q_len > 1 && blocks < 2) blocks = 2;               // (two blocks can hold query tokens)
     if (blocks > max_sel) blocks = max_sel;
     if (blocks > cap) blocks = cap;
     const long long tiles = (blocks * bs + kTileTokens - 1) / kTileTokens;
-    return step_plan(shape->batch * shape->num_kv_heads, rows, q_len, tiles,
-                     bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles, gate->max_blocks);
+    const int U = shape->batch * shape->num_kv_heads;
+    StepPlan plan = step_plan(U, rows, q_len, tiles, bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles, gate->max_blocks);
+    if (plan.S > 0 && plan.spread) {
+        if (shape->batch == 1) plan.spread = false;        // (the heads' lists are equally long)
+        else if (list_plan(U, tiles).S != plan.S || ws_layout(U, 0, 0, 0).scratch + list_part_bytes(U, plan.S) > ctx->ws_bytes) plan.S = 0;
+    }
+    return plan;
 }
 
 seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_kv* kv, const seer_gate* gate,
@@ -844,7 +860,7 @@ seer_status seer_decode_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     GateParams gp;
     seer_status st = gate_prepare(ctx, shape, gate, kv->seq_lens, q_nope, nullptr, token_budget, 0, 0.f, block_idx, block_cnt, max_sel,
                                   nullptr, 1, &gp);
-    const StepPlan plan = st == SEER_OK ? plan_of_step(ctx, shape, kv, gate, 1, token_budget, max_sel) : StepPlan{0, 1, 0, false, false};
+    const StepPlan plan = st == SEER_OK ? plan_of_step(ctx, shape, kv, gate, 1, token_budget, max_sel) : StepPlan{0, 1, 0, false, false, false};
     if (plan.S > 0) {
         const bool appended = append_in_step(ctx, shape, kv, gate, k_nope, k_nope_stride_batch, k_nope_stride_head,
                                              k_nope_stride_token, k_nope_rows_block_local, 1, &gp);

@@ -64,4 +64,25 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status, u
     return ok != 0;
 }
 
+// Whether the lists are dealt.  In hundredths of a microsecond: a CTA that has the memory to itself gets through a tile in 0.46
+// us (three stages, of which one or two are being read); all CTAs together through one in 0.0047 us, taken as 0.004 because
+// the last ones are alone with their tiles; a deal costs 8 us: 2 to make it, 4 for the pieces' way through global memory, and
+// the helpers' second start.
+constexpr int kTileTime = 46, kPieceTiles = 8;             // (a piece costs a helper as much as so many tiles a CTA)
+__device__ __forceinline__ bool list_uneven(int total, int most, int units, int S) {
+    // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S)) + 800, without its divisions)
+    return 5ll * kTileTime * most * units > max(2ll * total * S * units, 5ll * kTileTime * total) + 4000ll * S * units;
+}
+// The same of a step's lists, as the sequences' lengths give them (whole warp).
+__device__ __forceinline__ bool step_uneven(const DecodeParams& p, int S) {
+    int total = 0, most = 0;
+    for (int i = threadIdx.x & 31; i < p.batch; i += 32) {
+        const int L = p.seq_lens[i], n = L > 0 ? min((L + p.block_size - 1) >> p.bs_shift, p.sel_from_lens) : 0;
+        const int tiles = p.blocks_per_tile > 1 ? (n + p.blocks_per_tile - 1) >> p.bpt_shift : n << p.tpb_shift;
+        total += tiles;
+        most = max(most, tiles);
+    }
+    return list_uneven(__reduce_add_sync(0xffffffffu, total) * p.num_kv_heads, __reduce_max_sync(0xffffffffu, most), p.num_units, S);
+}
+
 }  // namespace seer

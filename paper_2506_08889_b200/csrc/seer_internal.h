@@ -74,7 +74,7 @@ struct DecodeParams {
                                     // counts follow from the lengths and the schedule can be made before the kernel
                                     // that writes the lists has finished (0: read block_cnt)
     int next_early;                     // cluster kernels: StepPlan's, ListPlan's
-    int spread;                         // list kernel: ListPlan's
+    int spread;                         // list kernel: ListPlan's (sel_from_lens > 0: behind a step that has done even lists itself)
     unsigned int* status;
     unsigned long long* tickets;    // [num_units]: tiles done << 32 | valid-slot bits; zero between launches
     int* sched;                     // [2]: theft cursor, exit counter; zero between launches
@@ -139,12 +139,15 @@ struct StepPlan {
     int parts, rows;                    // clusters per unit, which have `rows` of its rows each (the last one the rest)
     bool wide;                          // 16 worker warps per CTA, one CTA per SM (else 8 and two)
     bool next_early;                    // the stream's next launch may start beside this one
+    bool spread;                        // a step whose lists may be so long that it matters whether they are even: the list kernel, with
+                                        // as many CTAs per unit, comes behind it
 };
 StepPlan step_plan(int units, int rows, int q_len, long long max_tiles, long long max_codes, int max_keys);
 // g == nullptr: attention only (of several query tokens), over p.block_idx (nullptr: all blocks).  p.q == nullptr: the gate only.
 cudaError_t launch_step_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g,
                                 const StepPlan& plan, cudaStream_t stream);
 // One query token over given lists, or all blocks, as one launch of a cluster of S CTAs per unit (seer_lists.cu).
+constexpr int kListTiles = 128;         // most tiles a CTA
 constexpr int kListUnits = 320;         // most units whose tiles it counts
 struct ListPlan {
     int S;                              // CTAs per cluster; 0: the decode kernel

@@ -140,15 +140,6 @@ __device__ __forceinline__ void tile_step(float (&o)[8][4], float (&m_run)[2], f
     }
 }
 
-// Whether the lists are dealt.  In hundredths of a microsecond: a CTA that has the memory to itself gets through a tile in 0.46
-// us (three stages, of which one or two are being read); all CTAs together through one in 0.0047 us, taken as 0.004 because
-// the last ones are alone with their tiles; a deal costs 8 us: 2 to make it, 4 for the pieces' way through global memory, and
-// the helpers' second start.
-constexpr int kTileTime = 46, kPieceTiles = 8;             // (a piece costs a helper as much as so many tiles a CTA)
-__device__ __forceinline__ bool list_uneven(int total, int most, int units, int S) {
-    return kTileTime * (long long)most / S > max(2ll * total / 5, kTileTime * (long long)total / (units * S)) + 800;
-}
-
 // A cluster's piece of a unit: its tiles a .. b.  `x`, `end`: what is left of the cluster's share of the rest.
 struct Piece {
     int u, a, b, n;                                        // n: tiles of the unit
@@ -275,6 +266,11 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         return small ? (n_blocks + p.blocks_per_tile - 1) >> p.bpt_shift : n_blocks << p.tpb_shift;
     };
     pdl_wait();
+    if (SPREAD && p.sel_from_lens > 0 && !step_uneven(p, S)) {     // (a step whose attention is done)
+        pdl_launch_dependents();
+        cluster_wait();
+        return;
+    }
     // (the first entries are asked for beside the count that says how many there are, not behind it)
     int entry[4] = {-1, -1, -1, -1}, entry2[4] = {-1, -1, -1, -1};      // the list's entries of this lane's first tile, and of the second piece's
     if (producer && !dense) {
@@ -751,7 +747,6 @@ int resident_lists(int k) {
 //     192, dense           8 sequences           241 -> 228 / 147 -> 151
 //     256, dense           8 sequences           313 -> 305 / 193 -> 201
 // (One long sequence among short ones: as clusters without a deal 64 instead of 39 us where its lists have 102 tiles a CTA.)
-constexpr int kMostTiles = 128;
 ListPlan list_plan(int units, long long max_tiles) {
     ListPlan plan = {0, false, false};
     if (units > kListUnits || units * max_tiles >= (1ll << 30)) return plan;
@@ -759,7 +754,7 @@ ListPlan list_plan(int units, long long max_tiles) {
         const int S = 1 << k;
         if (k > 0 && S > max_tiles) continue;              // a CTA would have nothing to do
         if (units > resident_lists(k)) continue;
-        if (max_tiles <= (long long)kMostTiles * S) plan.S = S;
+        if (max_tiles <= (long long)kListTiles * S) plan.S = S;
         plan.spread = max_tiles > (long long)S * (16 + 2 * S);       // (shorter lists gain nothing by a deal)
         plan.next_early = 2 * units <= resident_lists(k);
         break;

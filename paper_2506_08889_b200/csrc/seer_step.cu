@@ -729,7 +729,9 @@ __device__ __forceinline__ void key_sums(Pieces&& pieces, const uint32_t (*parts
 // three, the selection by one CTA and its lists stored into the others, it was 2.9, 7.2, 10.6, 11.8 to 13.3, 15.3, 16.2.
 // Longer calls by memory: of a step of 64 units x 205 blocks (430 MB) the tiles take 66 us, 6.5 TB/s, from the first CTA's
 // first to the last one's last; CTAs that share a unit read neighbouring blocks at the same time.
-template <int NW, bool GATE, bool MULTI>
+// SPREAD: the lists may be so long that it matters whether they are even; where they are not, the lists and the append are all
+// that is done here, and the list kernel behind this launch does the rest (else nothing).
+template <int NW, bool GATE, bool MULTI, bool SPREAD = false>
 __global__ void __launch_bounds__(Size<NW, MULTI>::kThreads, NW == 8 ? 2 : 1)
 step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ DecodeParams p, const __grid_constant__ GateArg<GATE> ga) {
@@ -824,7 +826,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             for (int x = tid; x < kBins; x += kWorkers) gs.hist[x] = 0;
         }
         pdl_wait();                                        // queries, lengths and compressed keys are final
-        if (!p.q && p.next_early) pdl_launch_dependents();     // (the gate alone has no work for which it wants the SMs)
+        if (!SPREAD && !p.q && p.next_early) pdl_launch_dependents();     // (the gate alone has no work for which it wants the SMs)
         L = p.seq_lens[i];
         // (what the second round of loads reads of the queries, if there is one)
         if (producer && lane < q_len && units > 4 * slices)
@@ -854,8 +856,10 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const int t_skip = MULTI ? kMaxQLen - q_len : 0;
         uint32_t (*parts)[3][kMaxDGate / 2 + 16] = gs.parts + t_skip;
         slots.place(sm.ring, n_tiles, Place::kScratch + t_skip * (int)sizeof(gs.parts[0]), g.d_gate);
+        const bool even = !SPREAD || !step_uneven(p, S);
+        auto attends = [&]() -> bool { return SPREAD ? even : p.q != nullptr; };
         // who selects: every CTA that will read tiles, or (the gate alone) the first one
-        const int n_sel = p.q ? S : 1, sel_shift = p.q ? s_shift : 0;
+        const int n_sel = attends() ? S : 1, sel_shift = attends() ? s_shift : 0;
         const bool selects = rank < n_sel;
         if (producer) {
             // (the scores of the other CTAs' key tiles, and from every CTA their smallest and largest key)
@@ -1095,7 +1099,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             // entry e of the list is block j: its tile(s) among this CTA's, if they are
             auto take = [&](int e, int j) {
                 if (lists) dst[e] = j;
-                if (!p.q) return;
+                if (!attends()) return;
                 if (p.blocks_per_tile == 1) {
                     for (int x = 0; x < p.tiles_per_block; ++x) {
                         const int t = (e << p.tpb_shift) + x;
@@ -1127,7 +1131,11 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 for (int e = n_blocks + tid; e < g.max_sel; e += kWorkers) dst[e] = -1;
             }
         }
-        if (!p.q) {                                        // the gate alone
+        if (!attends()) {                                  // the gate alone
+            if (SPREAD && appends) {
+                if (producer) append_pool(g, sm, i, h, (L >> b_shift) - 1, rank, S);
+                else if (!dead) append_project<NW>(g, sm, u, h, (L >> b_shift) - 1, rank, S);
+            }
             cluster_sync();                                // (as at the end)
             return;
         }
@@ -1459,11 +1467,12 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     cluster_wait();
 }
 
-template <int NW, bool GATE, bool MULTI>
+template <int NW, bool GATE, bool MULTI, bool SPREAD>
 cudaError_t configure() {
-    cudaError_t e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI, SPREAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(StepSmem<NW, MULTI>) + 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI, SPREAD>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
@@ -1485,14 +1494,14 @@ cudaLaunchConfig_t config_of(int S, int units, int parts, cudaStream_t stream, c
     return cfg;
 }
 
-template <int NW, bool GATE, bool MULTI>
+template <int NW, bool GATE, bool MULTI, bool SPREAD = false>
 int resident_of(int k) {
-    if (configure<NW, GATE, MULTI>() != cudaSuccess) return 0;
+    if (configure<NW, GATE, MULTI, SPREAD>() != cudaSuccess) return 0;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = config_of<NW, GATE, MULTI>(1 << k, 1, 1, nullptr, attr);
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, step_cluster_kernel<NW, GATE, MULTI>, &cfg) != cudaSuccess) n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, step_cluster_kernel<NW, GATE, MULTI, SPREAD>, &cfg) != cudaSuccess) n = 0;
     cudaGetLastError();                                    // (a refused size is no error of the caller's)
     return n;
 }
@@ -1504,7 +1513,8 @@ int resident_clusters(bool wide, int k) {
     int& c = cached[current_device_slot()][wide][k];
     if (c == 0) {
         c = wide ? min(resident_of<16, true, true>(k), resident_of<16, false, true>(k)) + 1
-                 : min(resident_of<8, true, false>(k), min(resident_of<8, true, true>(k), resident_of<8, false, true>(k))) + 1;
+                 : min(min(resident_of<8, true, false>(k), resident_of<8, true, false, true>(k)),
+                       min(resident_of<8, true, true>(k), resident_of<8, false, true>(k))) + 1;
     }
     return c - 1;
 }
@@ -1527,28 +1537,32 @@ int resident_clusters(bool wide, int k) {
 //     steps, 16 sequences (S = 2)    64: 31.7 -> 46.8 / 72.3 -> 58.6 / 103 -> 93      128: 45.3 -> 82.7 / 108 -> 103 / 178 -> 173
 //             8 sequences (S = 4)    64: 35.6 -> 47.4 / 69.6 -> 56.6 / 101 -> 91      128: 57.1 -> 80.6 / 105 -> 101 / 176 -> 172
 // Given lists and dense calls of several query tokens, whose lengths follow the sequences', keep to where one long sequence
-// does not lose much: 16 + 2 S tiles a CTA (a decode call pays for its parts whatever its size, and more the longer its longest
-// unit is; lists of one query token are dealt: seer_lists.cu).  The lists of a step are all as long as the budget but for sequences shorter than that: the line is at 64, where all but the most uneven
-// batches gain; at 128 the even ones gain 3 % and the uneven ones lose up to half.  With a few more CTAs than SMs the SMs
-// that hold two of them are the last to finish (80 units, 64 tiles a CTA, 160 CTAs: 65 -> 67; 32 tiles: 40.8 -> 37.5), so
-// the line is at 32 there.  149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles
-// a CTA 45.9 -> 33.8, 52.7 -> 39.1, 59.3 -> 43.1; 64 tiles 93.5 -> 82.1, 108 -> 96, 127 -> 109.
-static StepPlan plan_of(bool wide, int units, int rows, long long max_tiles, long long max_codes, int max_keys) {
-    StepPlan plan = {0, 1, rows, wide, false};
+// does not lose much: 16 + 2 S tiles a CTA (a decode call pays for its parts whatever its size, and more the longer its
+// longest unit is; lists of one query token are dealt: seer_lists.cu).  The lists of a step are all as long as the budget but for
+// sequences shorter than that: one launch up to 64 tiles a CTA, where all but the most uneven batches gain (80 units in 160
+// CTAs, twelve SMs with two of them: 48 tiles a CTA 78.6 -> 61.6, two query tokens 79.6 -> 64.7).  From there to 128 tiles
+// (line_spread: one query token) it is the sequences' lengths that decide, in the kernels: even lists are done in the one
+// launch, uneven ones by the list kernel behind it, which costs 5 us where it has nothing to do.  Chain -> two launches, all
+// lists long / lengths spread from 1/32 on / one of 410 tiles a unit among short ones:
+//     80 tiles a CTA, 8 sequences   129 -> 123 / 124 -> 111 / 79 -> 64        96, 10 sequences   114 -> 104 / 112 -> 94
+//     96, 16 sequences              150 -> 142 / 140 -> 125                   97, 10 sequences, blocks of 32   129 -> 104
+// 149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles a CTA 45.9 -> 33.8, 52.7 ->
+// 39.1, 59.3 -> 43.1; 64 tiles 93.5 -> 82.1, 108 -> 96, 127 -> 109.
+static StepPlan plan_of(bool wide, int units, int rows, long long max_tiles, long long max_codes, int max_keys, bool line_spread = false) {
+    StepPlan plan = {0, 1, rows, wide, false, false};
     if (rows > 64) return plan;
     if (rows > 32) {
         plan.parts = (rows + 31) / 32;
         plan.rows = (rows + plan.parts - 1) / plan.parts;
     }
-    const int sms = wide ? resident_clusters(true, 0) : resident_clusters(false, 0) / 2;
     units *= plan.parts;
     for (int k = 4; k >= 0; --k) {
         const int S = 1 << k;
         if (k > 0 && S > max_tiles && 128ll * S > max_keys) continue;      // a CTA would have nothing to do
         if (units > resident_clusters(wide, k)) continue;
-        const bool few_doubled = units * S > sms && 5 * units * S <= 6 * sms;
-        const long long line = (long long)S * min(max_keys > 0 ? 64 : 16 + 2 * S, few_doubled ? 32 : 64);
-        if (max_tiles <= line && max_codes <= (long long)S * kCodes) plan.S = S;
+        const long long line = (long long)S * (max_keys > 0 ? 64 : min(16 + 2 * S, 64));
+        plan.spread = line_spread && max_tiles > line && max_tiles <= (long long)S * kListTiles;
+        if ((max_tiles <= line || plan.spread) && max_codes <= (long long)S * kCodes) plan.S = S;
         // The next launch may start beside this one if both fit at once.  Otherwise its first clusters take places that the
         // last ones then lack: half the steps of 32 ragged units, in clusters of eight, had one to four clusters in a second
         // wave, 13 us late (mean 23.8 -> 22.6 us; threshold gate and lists 28.4 -> 27.8, batch 8 at 128k 82.7 -> 81.0).
@@ -1571,7 +1585,7 @@ StepPlan step_plan(int units, int rows, int q_len, long long max_tiles, long lon
             const StepPlan plan = plan_of(true, units, rows, max_tiles, max_codes, max_keys);
             if (plan.S >= 8) return plan;
         }
-        return plan_of(false, units, rows, max_tiles, max_codes, max_keys);
+        return plan_of(false, units, rows, max_tiles, max_codes, max_keys, q_len == 1 && max_keys > 0);
     }
     return plan_of(true, units, rows, max_tiles, max_codes, max_keys);
 }
@@ -1584,6 +1598,8 @@ cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const 
     cudaLaunchAttribute attr[2];
     if (g) {
         const cudaLaunchConfig_t cfg = config_of<NW, true, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
+        if constexpr (!MULTI)
+            if (plan.spread) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, false, true>, map_k, map_v, p, GateArg<true>{*g});
         return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, MULTI>, map_k, map_v, p, GateArg<true>{*g});
     }
     if constexpr (MULTI) {

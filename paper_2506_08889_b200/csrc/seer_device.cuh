@@ -114,6 +114,14 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t base, uint32_t cols) {
 // Orders tensor-core operations against the thread synchronisation (barrier wait or arrive) next to it.
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// One lane of a whole warp, for the instructions below that one thread issues.  Behind this choice the compiler knows them to be
+// issued once and keeps their operands in uniform registers; behind `lane == 0` every one of them cost about 110 cycles in moves
+// (32 of a bulk build's products 3600 cycles, 470 with this).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t chosen;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(chosen));
+    return chosen != 0;
+}
 // One arrival on the barrier once every MMA this thread has issued so far has completed.
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))

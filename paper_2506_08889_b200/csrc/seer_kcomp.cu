@@ -430,19 +430,49 @@ __device__ __forceinline__ void lengths_arrive() { asm volatile("bar.arrive 3, %
 __device__ __forceinline__ void lengths_wait() { asm volatile("bar.sync 3, %0;" ::"n"(kStreamThreads) : "memory"); }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
+// A block's features of one lane (eight channels: piece `cchunk`) to row q of a feature buffer: 16 bytes per kind, each at its
+// swizzled place in its slab; zeros where there is no such block.
+__device__ __forceinline__ void store_features(unsigned char* feat, int q, bool valid, int cchunk, const __nv_bfloat162 (&mx)[4],
+                                               const __nv_bfloat162 (&mn)[4], const float (&sum)[8], float inv_rows) {
+    uint4 pmax = make_uint4(0u, 0u, 0u, 0u), pmin = pmax, phi = pmax, plo = pmax;
+    if (valid) {
+        pmax = make_uint4(*reinterpret_cast<const uint32_t*>(&mx[0]), *reinterpret_cast<const uint32_t*>(&mx[1]),
+                          *reinterpret_cast<const uint32_t*>(&mx[2]), *reinterpret_cast<const uint32_t*>(&mx[3]));
+        pmin = make_uint4(*reinterpret_cast<const uint32_t*>(&mn[0]), *reinterpret_cast<const uint32_t*>(&mn[1]),
+                          *reinterpret_cast<const uint32_t*>(&mn[2]), *reinterpret_cast<const uint32_t*>(&mn[3]));
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) {
+            const float a0 = sum[c] * inv_rows, a1 = sum[c + 1] * inv_rows;
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
+            hi[c >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+            const float2 hf = bf16x2_to_float2(h2);
+            lo[c >> 1] = pack_bf16x2(a0 - hf.x, a1 - hf.y);
+        }
+        phi = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        plo = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
+    unsigned char* f0 = feat + (cchunk >> 3) * (kBulkBlocks * 128) + q * 128 + (((cchunk & 7) ^ (q & 7)) << 4);
+    *reinterpret_cast<uint4*>(f0) = pmax;
+    *reinterpret_cast<uint4*>(f0 + 2 * kBulkBlocks * 128) = pmin;
+    *reinterpret_cast<uint4*>(f0 + 4 * kBulkBlocks * 128) = phi;
+    *reinterpret_cast<uint4*>(f0 + 6 * kBulkBlocks * 128) = plo;
+}
+
 template <int B>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams p) {
     constexpr int SPB = B > kStageRows ? B / kStageRows : 1;       // stages of a portion
     constexpr int BPS = B < kStageRows ? kStageRows / B : 1;       // blocks of a portion
-    constexpr int kArrivals = SPB * kPoolWarps;
+    constexpr int SHARE = BPS > 2 ? BPS / 2 : 1;                   // portions of a stage: two blocks of 16 rows each
+    constexpr int kArrivals = SPB * SHARE * kPoolWarps;
     extern __shared__ unsigned char smem_raw[];
     // (aligned by an offset, not by a cast through an integer: the compiler then still knows the accesses for shared ones)
     StreamSmem& sm = *reinterpret_cast<StreamSmem*>(smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         for (int s = 0; s < kArrivals; ++s) mbar_init(&sm.full[s], 1);
-        for (int s = 0; s < kStreamStages; ++s) mbar_init(&sm.empty[s], 1);
+        for (int s = 0; s < kStreamStages; ++s) mbar_init(&sm.empty[s], SHARE);
         for (int f = 0; f < 2; ++f) {
             mbar_init(&sm.feat_full[f], kPoolWarps);
             mbar_init(&sm.feat_empty[f], 1);
@@ -651,14 +681,57 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
             if (!dead && !mbar_wait(&sm.feat_empty[fb], ((n_done >> 1) & 1u) ^ 1u, p.status)) dead = true;
             KC_T(t_fe1);
             KC_ACC(0, t_fe0, t_fe1);
-            // (the portions past the item's last one only clear their blocks' features)
-            for (int q0 = 0; q0 < kBulkBlocks / BPS; ++q0) {
+            // (the portions past the item's last stage only clear their blocks' features)
+            for (int q0 = 0; q0 < kBulkBlocks / BPS * SHARE; ++q0) {
                 if ((portion_no + q0) % kPoolWarps != (uint32_t)pw) continue;
-                const bool real = q0 < n_por;
-                const uint32_t sn0 = (portion_no + q0) * SPB;
-#pragma unroll 1
-                for (int sb = 0; sb < BPS; ++sb) {
-                    const int q = q0 * BPS + sb;           // block of the item
+                if constexpr (BPS > 1) {
+                    // Two blocks, one per half of the warp: a lane has eight channels of all of its block's rows, even and odd rows'
+                    // sums apart (added up as the two halves' are below, so the same bits as with half of the rows per lane and a
+                    // reduction).  Nothing is exchanged, and both blocks' features are made at once.
+                    const uint32_t sn = (portion_no + q0) / SHARE;
+                    const int s = sn % kStreamStages, sb = 2 * (q0 % SHARE) + (lane >> 4), q = 2 * q0 + (lane >> 4);
+                    __nv_bfloat162 mx[4], mn[4];
+                    float sum[8], odd[8];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        mx[c] = __float2bfloat162_rn(-INFINITY);
+                        mn[c] = __float2bfloat162_rn(INFINITY);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) sum[c] = odd[c] = 0.f;
+                    if (q0 / SHARE < n_por) {
+                        KC_T(t_w0);
+                        if (!dead && !mbar_wait(&sm.full[sn % kArrivals], (sn / kArrivals) & 1u, p.status)) dead = true;
+                        KC_T(t_w1);
+                        KC_ACC(1, t_w0, t_w1);
+                        const unsigned char* st = sm.ring[s] + (cchunk >> 3) * (kStageBytes / 2) + sb * (B * 128);
+                        const int piece = (cchunk & 7) << 4;
+#pragma unroll 8
+                        for (int row = 0; row < B; row += 2) {
+                            const uint4 v0 = *reinterpret_cast<const uint4*>(st + row * 128 + (piece ^ ((row & 7) << 4)));
+                            const uint4 v1 = *reinterpret_cast<const uint4*>(st + row * 128 + 128 + (piece ^ (((row & 7) + 1) << 4)));
+                            const __nv_bfloat162* h0 = reinterpret_cast<const __nv_bfloat162*>(&v0);
+                            const __nv_bfloat162* h1 = reinterpret_cast<const __nv_bfloat162*>(&v1);
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                mx[c] = __hmax2(mx[c], __hmax2(h0[c], h1[c]));
+                                mn[c] = __hmin2(mn[c], __hmin2(h0[c], h1[c]));
+                                const float2 f = bf16x2_to_float2(h0[c]), g = bf16x2_to_float2(h1[c]);
+                                sum[2 * c] += f.x; sum[2 * c + 1] += f.y;
+                                odd[2 * c] += g.x; odd[2 * c + 1] += g.y;
+                            }
+                        }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sm.empty[s]);
+                        KC_T(t_w2);
+                        KC_ACC(2, t_w1, t_w2);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) sum[c] += odd[c];
+                    }
+                    store_features(sm.feat[fb], q, q < r.nb, cchunk, mx, mn, sum, 1.f / B);
+                } else {
+                    const bool real = q0 < n_por;
+                    const uint32_t sn0 = (portion_no + q0) * SPB;
                     __nv_bfloat162 mx[4], mn[4];
                     float sum[8];
 #pragma unroll
@@ -674,15 +747,14 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
                             const uint32_t sn = sn0 + part;
                             const int s = sn % kStreamStages;
                             KC_T(t_w0);
-                            if (sb == 0 && !dead && !mbar_wait(&sm.full[sn % kArrivals], (sn / kArrivals) & 1u, p.status)) dead = true;
+                            if (!dead && !mbar_wait(&sm.full[sn % kArrivals], (sn / kArrivals) & 1u, p.status)) dead = true;
                             KC_T(t_w1);
                             KC_ACC(1, t_w0, t_w1);
                             // lane: 16-byte column piece (lane & 15) of rows 2k + (lane >> 4); piece c of row r of a
                             // 64-channel half sits at position c ^ (r & 7) of the row's 128 bytes
-                            constexpr int kRowsHere = BPS > 1 ? B : kStageRows;
-                            const unsigned char* st = sm.ring[s] + sb * (kRowsHere * 128) + lane_off;
+                            const unsigned char* st = sm.ring[s] + lane_off;
 #pragma unroll 8
-                            for (int k = 0; k < kRowsHere / 2; ++k) {
+                            for (int k = 0; k < kStageRows / 2; ++k) {
                                 const uint4 v = *reinterpret_cast<const uint4*>(st + k * 256 + piece_off[k & 3]);
                                 const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
@@ -694,7 +766,7 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
                                 }
                             }
                             __syncwarp();
-                            if (lane == 0 && sb == BPS - 1) mbar_arrive(&sm.empty[s]);
+                            if (lane == 0) mbar_arrive(&sm.empty[s]);
                             KC_T(t_w2);
                             KC_ACC(2, t_w1, t_w2);
 #ifdef SEER_DECODE_TRACE
@@ -711,35 +783,10 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
 #pragma unroll
                         for (int c = 0; c < 8; ++c) sum[c] += __shfl_xor_sync(0xffffffffu, sum[c], 16);
                     }
-                    if (lane < 16) {
-                        // 8 features per kind and lane: one 16-byte piece each, at its swizzled place in row q of its slab
-                        uint4 pmax = make_uint4(0u, 0u, 0u, 0u), pmin = pmax, phi = pmax, plo = pmax;
-                        if (q < r.nb) {
-                            pmax = make_uint4(*reinterpret_cast<uint32_t*>(&mx[0]), *reinterpret_cast<uint32_t*>(&mx[1]),
-                                              *reinterpret_cast<uint32_t*>(&mx[2]), *reinterpret_cast<uint32_t*>(&mx[3]));
-                            pmin = make_uint4(*reinterpret_cast<uint32_t*>(&mn[0]), *reinterpret_cast<uint32_t*>(&mn[1]),
-                                              *reinterpret_cast<uint32_t*>(&mn[2]), *reinterpret_cast<uint32_t*>(&mn[3]));
-                            uint32_t hi[4], lo[4];
-#pragma unroll
-                            for (int c = 0; c < 8; c += 2) {
-                                const float a0 = sum[c] * (1.f / B), a1 = sum[c + 1] * (1.f / B);
-                                const __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
-                                hi[c >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-                                const float2 hf = bf16x2_to_float2(h2);
-                                lo[c >> 1] = pack_bf16x2(a0 - hf.x, a1 - hf.y);
-                            }
-                            phi = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                            plo = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                        }
-                        unsigned char* f0 = sm.feat[fb] + (cchunk >> 3) * (kBulkBlocks * 128) + q * 128 + (((cchunk & 7) ^ (q & 7)) << 4);
-                        *reinterpret_cast<uint4*>(f0) = pmax;
-                        *reinterpret_cast<uint4*>(f0 + 2 * kBulkBlocks * 128) = pmin;
-                        *reinterpret_cast<uint4*>(f0 + 4 * kBulkBlocks * 128) = phi;
-                        *reinterpret_cast<uint4*>(f0 + 6 * kBulkBlocks * 128) = plo;
-                    }
+                    if (lane < 16) store_features(sm.feat[fb], q0, q0 < r.nb, cchunk, mx, mn, sum, 1.f / B);
                 }
             }
-            portion_no += n_por;
+            portion_no += n_por * SHARE;
             ++n_done;
             fence_proxy_async_smem();              // the tensor cores read the features through the asynchronous proxy
             __syncwarp();
@@ -767,10 +814,10 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
             // the Y buffer of two items ago has been read
             if (n_done >= 2 && !mbar_wait(&sm.y_free[fb], ((n_done - 2) >> 1) & 1u, p.status)) { dead = true; break; }
             __syncwarp();
-            if (lane == 0) {
+            if (elect_one()) {
                 tc_fence_after_sync();
                 const uint64_t fd = tc_smem_desc(smem_u32(sm.feat[fb]), 16, 1024);
-#pragma unroll 4
+#pragma unroll
                 for (int ks = 0; ks < 32; ++ks)
                     tc_mma_ts(tbase + 256 + 16 * fb, tbase + 8 * ks, fd + (uint64_t)(((ks >> 2) * (kBulkBlocks * 128) + (ks & 3) * 32) >> 4),
                               idesc, ks > 0);

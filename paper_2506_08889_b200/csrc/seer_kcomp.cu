@@ -474,7 +474,7 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
         for (int s = 0; s < kArrivals; ++s) mbar_init(&sm.full[s], 1);
         for (int s = 0; s < kStreamStages; ++s) mbar_init(&sm.empty[s], SHARE);
         for (int f = 0; f < 2; ++f) {
-            mbar_init(&sm.feat_full[f], kPoolWarps);
+            mbar_init(&sm.feat_full[f], BPS > 1 ? kBulkBlocks / 2 : kPoolWarps);      // (small blocks: the warps that have two of the item's)
             mbar_init(&sm.feat_empty[f], 1);
             mbar_init(&sm.y_full[f], 1);
             mbar_init(&sm.y_free[f], kEpiWarps);
@@ -675,15 +675,26 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
 #pragma unroll
         for (int m = 0; m < 4; ++m) piece_off[m] = (((cchunk & 7) ^ (lane >> 4)) ^ (2 * m)) << 4;
         uint32_t portion_no = 0, n_done = 0;               // portions and items this CTA has been through
+        bool skipped = false;
         for (Run r = run_begin(); r.nb > 0; run_next(r)) {
             const int fb = n_done & 1, n_por = portions(r.nb);
+            const int own = (int)((pw + kPoolWarps - portion_no % kPoolWarps) % kPoolWarps);       // this warp's first portion of the item
+            if (BPS > 1 && own >= kBulkBlocks / 2) {
+                // It has none of the eight.  (Never two items running without a look at the barrier, whose phases it has to
+                // follow: short items take the portions' numbers on by less than eight.)
+                if (skipped && !dead && !mbar_wait(&sm.feat_empty[fb], ((n_done >> 1) & 1u) ^ 1u, p.status)) dead = true;
+                skipped = !skipped;
+                portion_no += n_por * SHARE;
+                ++n_done;
+                continue;
+            }
+            skipped = false;
             KC_T(t_fe0);
             if (!dead && !mbar_wait(&sm.feat_empty[fb], ((n_done >> 1) & 1u) ^ 1u, p.status)) dead = true;
             KC_T(t_fe1);
             KC_ACC(0, t_fe0, t_fe1);
             // (the portions past the item's last stage only clear their blocks' features)
-            for (int q0 = 0; q0 < kBulkBlocks / BPS * SHARE; ++q0) {
-                if ((portion_no + q0) % kPoolWarps != (uint32_t)pw) continue;
+            for (int q0 = own; q0 < kBulkBlocks / BPS * SHARE; q0 += kPoolWarps) {
                 if constexpr (BPS > 1) {
                     // Two blocks, one per half of the warp: a lane has eight channels of all of its block's rows, even and odd rows'
                     // sums apart (added up as the two halves' are below, so the same bits as with half of the rows per lane and a

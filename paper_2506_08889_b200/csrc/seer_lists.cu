@@ -395,36 +395,48 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
                     }
                 }
                 __syncwarp();
-                // lane s asks for tile s of the batch
+                // tile s of the batch, which lane s has looked up, is asked for by an elected lane
                 const int m = min(count, n_local - base);
                 for (int s = 0; s < m; ++s) {
-                    if (lane == s) {
-                        const int n = tile0 + it, slot = n + piece, st = slot % kStages;
-                        if (!dead && !mbar_wait(&sm.empty[st], ((slot / kStages) & 1) ^ 1, p.status)) dead = true;
+                    const int n = tile0 + base + s, slot = n + piece, st = slot % kStages;
+                    const int nv = __shfl_sync(0xffffffffu, nv_all, s), subs = __shfl_sync(0xffffffffu, n_sub, s);
+                    int r[4], o[4];
+                    r[0] = __shfl_sync(0xffffffffu, row[0], s);
+                    o[0] = __shfl_sync(0xffffffffu, outer[0], s);
+                    if (small) {
+#pragma unroll
+                        for (int x = 1; x < 4; ++x) {
+                            r[x] = __shfl_sync(0xffffffffu, row[x], s);
+                            o[x] = __shfl_sync(0xffffffffu, outer[x], s);
+                        }
+                    }
+                    if (!dead && !mbar_wait(&sm.empty[st], ((slot / kStages) & 1) ^ 1, p.status)) dead = true;
+                    dead = __any_sync(0xffffffffu, dead);
+                    if (elect_one()) {
                         unsigned char* dst = sm.ring + st * kStageBytes;
                         uint64_t* full = &sm.full[n % kArrivals];
-                        sm.meta[n % kArrivals] = nv_all;   // (the tile kArrivals back has been read: a later one of its group had this stage or a later one)
-                        if (dead || n_sub == 0) {
+                        sm.meta[n % kArrivals] = nv;       // (the tile kArrivals back has been read: a later one of its group had this stage or a later one)
+                        if (dead || subs == 0) {
                             mbar_arrive(full);
                         } else if (small) {
                             const int sub_bytes = p.block_size * 128;      // one half (64 channels) of one block
-                            mbar_arrive_expect_tx(full, (uint32_t)(n_sub * 4 * sub_bytes));
+                            mbar_arrive_expect_tx(full, (uint32_t)(subs * 4 * sub_bytes));
 #pragma unroll
                             for (int x = 0; x < 4; ++x) {
-                                if ((nv_all >> (8 * x)) & 0xff) {
+                                if ((nv >> (8 * x)) & 0xff) {
                                     unsigned char* d2 = dst + x * sub_bytes;
-                                    tma_load_4d(d2, &map_k, full, 0, row[x], h, outer[x]);
-                                    tma_load_4d(d2 + kHalfTileBytes, &map_k, full, 64, row[x], h, outer[x]);
-                                    tma_load_4d(d2 + kTileBytes, &map_v, full, 0, row[x], h, outer[x]);
-                                    tma_load_4d(d2 + kTileBytes + kHalfTileBytes, &map_v, full, 64, row[x], h, outer[x]);
+                                    tma_load_4d(d2, &map_k, full, 0, r[x], h, o[x]);
+                                    tma_load_4d(d2 + kHalfTileBytes, &map_k, full, 64, r[x], h, o[x]);
+                                    tma_load_4d(d2 + kTileBytes, &map_v, full, 0, r[x], h, o[x]);
+                                    tma_load_4d(d2 + kTileBytes + kHalfTileBytes, &map_v, full, 64, r[x], h, o[x]);
                                 }
                             }
                         } else {
                             mbar_arrive_expect_tx(full, kStageBytes);
-                            tma_load_4d(dst, &map_k, full, 0, row[0], h, outer[0]);
-                            tma_load_4d(dst + kHalfTileBytes, &map_k, full, 64, row[0], h, outer[0]);
-                            tma_load_4d(dst + kTileBytes, &map_v, full, 0, row[0], h, outer[0]);
-                            tma_load_4d(dst + kTileBytes + kHalfTileBytes, &map_v, full, 64, row[0], h, outer[0]);
+                            tma_load_4d(dst, &map_k, full, 0, r[0], h, o[0]);
+                            tma_load_4d(dst + kHalfTileBytes, &map_k, full, 64, r[0], h, o[0]);
+                            tma_load_4d(dst + kTileBytes, &map_v, full, 0, r[0], h, o[0]);
+                            tma_load_4d(dst + kTileBytes + kHalfTileBytes, &map_v, full, 64, r[0], h, o[0]);
                         }
                     }
                     __syncwarp();

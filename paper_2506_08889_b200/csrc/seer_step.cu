@@ -731,7 +731,9 @@ __device__ __forceinline__ void key_sums(Pieces&& pieces, const uint32_t (*parts
 // first to the last one's last; CTAs that share a unit read neighbouring blocks at the same time.
 // SPREAD: the lists may be so long that it matters whether they are even; where they are not, the lists and the append are all
 // that is done here, and the list kernel behind this launch does the rest (else nothing).
-template <int NW, bool GATE, bool MULTI, bool SPREAD = false>
+// SMALL: lists of blocks of 16 or 32 tokens, four or two to a tile.  (Told apart at run time both kinds' look-ups and copies took
+// registers from one another, and spilled.)
+template <int NW, bool GATE, bool MULTI, bool SPREAD, bool SMALL>
 __global__ void __launch_bounds__(Size<NW, MULTI>::kThreads, NW == 8 ? 2 : 1)
 step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ DecodeParams p, const __grid_constant__ GateArg<GATE> ga) {
@@ -783,7 +785,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     }
 
     int n_blocks = 0, L = 0;                               // listed blocks of the unit, cached tokens
-    int entry[4] = {-1, -1, -1, -1};                       // !GATE: the list's entries of this lane's first tile
+    constexpr int kSubs = SMALL ? 4 : 1;                   // most blocks of a tile
+    int entry[kSubs] = {};                                 // !GATE: the list's entries of this lane's first tile
     bool dead = false;                                     // a wait ran out: go through the motions, the results are invalid
     if constexpr (GATE) {
         const GateParams& g = ga.g;
@@ -1100,7 +1103,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             auto take = [&](int e, int j) {
                 if (lists) dst[e] = j;
                 if (!attends()) return;
-                if (p.blocks_per_tile == 1) {
+                if constexpr (!SMALL) {
                     for (int x = 0; x < p.tiles_per_block; ++x) {
                         const int t = (e << p.tpb_shift) + x;
                         if ((t & (S - 1)) == rank && (t >> s_shift) < kCodes) sm.codes[t >> s_shift] = (j << p.tpb_shift) + x;
@@ -1155,8 +1158,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         if (producer && p.block_idx) {
             const int t = (lane << s_shift) + rank;
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int e = p.blocks_per_tile > 1 ? (t << p.bpt_shift) + x : t >> p.tpb_shift;
+            for (int x = 0; x < kSubs; ++x) {
+                const int e = SMALL ? (t << p.bpt_shift) + x : t >> p.tpb_shift;
                 if (x < p.blocks_per_tile) entry[x] = p.block_idx[(size_t)u * p.max_sel + min(e, p.max_sel - 1)];
             }
         }
@@ -1170,7 +1173,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 
     // ---- tiles ------------------------------------------------------------------------------------------------------
     const bool dense = !GATE && !p.block_idx;
-    const bool small = !dense && p.blocks_per_tile > 1;
+    constexpr bool small = SMALL;
     const int T = dense ? (L > 0 ? min((L + kTileTokens - 1) / kTileTokens, p.max_blocks_cap) : 0)
                         : small ? (n_blocks + p.blocks_per_tile - 1) >> p.bpt_shift : n_blocks << p.tpb_shift;
     const int n_mine = (max(0, T - rank) + S - 1) >> s_shift;
@@ -1187,13 +1190,13 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const int n_i = (L + p.block_size - 1) >> p.bs_shift;
         for (int base = 0; base < n_local; base += 32) {
             const int it = base + lane;
-            int row[4] = {0, 0, 0, 0}, outer[4] = {0, 0, 0, 0}, nv_all = 0, n_sub = 0;
+            int row[kSubs] = {}, outer[kSubs] = {}, nv_all = 0, n_sub = 0;
             if (it < n_local) {
                 const int t = (it << s_shift) + rank;
                 const int n_try = small ? p.blocks_per_tile : 1;
                 const int span = small ? p.block_size : kTileTokens;
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
+                for (int x = 0; x < kSubs; ++x) {
                     if (x < n_try) {
                         int tok0 = -1;
                         if (dense) {
@@ -1234,30 +1237,48 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
             }
             __syncwarp();
-            // lane s asks for tile s of the batch
+            // Tile s of the batch, which lane s has looked up.  With up to sixteen copies a tile (blocks of 16 or 32 tokens) an
+            // elected lane asks for them (see elect_one: 77 units, three query tokens, blocks of 16: 93.4 -> 82 us); with four
+            // lane s itself, as handing over what it knows takes longer (one sequence of 32k 13.4, elected 13.65).
             const int m = min(32, n_local - base);
             for (int s = 0; s < m; ++s) {
-                if (lane == s) {
-                    const int st = it % kStages;
-                    if (!dead && !mbar_wait(&sm.empty[st], ((it / kStages) & 1) ^ 1, p.status)) dead = true;
-                    unsigned char* dst = sm.ring + st * kStageBytes;
-                    uint64_t* full = &sm.full[it % kArrivals];
-                    sm.meta[it % kArrivals] = nv_all;      // (the tile kArrivals back has been read: the one kStages back has, which came after it)
-                    if (dead || n_sub == 0) {
-                        mbar_arrive(full);
-                    } else if (small) {
-                        const int sub_bytes = p.block_size * 128;      // one half (64 channels) of one block
-                        mbar_arrive_expect_tx(full, (uint32_t)(n_sub * 4 * sub_bytes));
+                const int n = base + s, st = n % kStages;
+                unsigned char* dst = sm.ring + st * kStageBytes;
+                uint64_t* full = &sm.full[n % kArrivals];
+                if constexpr (SMALL) {
+                    const int nv = __shfl_sync(0xffffffffu, nv_all, s), subs = __shfl_sync(0xffffffffu, n_sub, s);
+                    int r[4], o[4];
 #pragma unroll
-                        for (int x = 0; x < 4; ++x) {
-                            if ((nv_all >> (8 * x)) & 0xff) {
-                                unsigned char* d2 = dst + x * sub_bytes;
-                                tma_load_4d(d2, &map_k, full, 0, row[x], h, outer[x]);
-                                tma_load_4d(d2 + kHalfTileBytes, &map_k, full, 64, row[x], h, outer[x]);
-                                tma_load_4d(d2 + kTileBytes, &map_v, full, 0, row[x], h, outer[x]);
-                                tma_load_4d(d2 + kTileBytes + kHalfTileBytes, &map_v, full, 64, row[x], h, outer[x]);
+                    for (int x = 0; x < 4; ++x) {
+                        r[x] = __shfl_sync(0xffffffffu, row[x], s);
+                        o[x] = __shfl_sync(0xffffffffu, outer[x], s);
+                    }
+                    if (!dead && !mbar_wait(&sm.empty[st], ((n / kStages) & 1) ^ 1, p.status)) dead = true;
+                    dead = __any_sync(0xffffffffu, dead);
+                    if (elect_one()) {
+                        sm.meta[n % kArrivals] = nv;       // (the tile kArrivals back has been read: the one kStages back has, which came after it)
+                        if (dead || subs == 0) {
+                            mbar_arrive(full);
+                        } else {
+                            const int sub_bytes = p.block_size * 128;      // one half (64 channels) of one block
+                            mbar_arrive_expect_tx(full, (uint32_t)(subs * 4 * sub_bytes));
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) {
+                                if ((nv >> (8 * x)) & 0xff) {
+                                    unsigned char* d2 = dst + x * sub_bytes;
+                                    tma_load_4d(d2, &map_k, full, 0, r[x], h, o[x]);
+                                    tma_load_4d(d2 + kHalfTileBytes, &map_k, full, 64, r[x], h, o[x]);
+                                    tma_load_4d(d2 + kTileBytes, &map_v, full, 0, r[x], h, o[x]);
+                                    tma_load_4d(d2 + kTileBytes + kHalfTileBytes, &map_v, full, 64, r[x], h, o[x]);
+                                }
                             }
                         }
+                    }
+                } else if (lane == s) {
+                    if (!dead && !mbar_wait(&sm.empty[st], ((n / kStages) & 1) ^ 1, p.status)) dead = true;
+                    sm.meta[n % kArrivals] = nv_all;
+                    if (dead || n_sub == 0) {
+                        mbar_arrive(full);
                     } else {
                         mbar_arrive_expect_tx(full, kStageBytes);
                         tma_load_4d(dst, &map_k, full, 0, row[0], h, outer[0]);
@@ -1467,16 +1488,14 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     cluster_wait();
 }
 
-template <int NW, bool GATE, bool MULTI, bool SPREAD>
-cudaError_t configure() {
-    cudaError_t e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI, SPREAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(StepSmem<NW, MULTI>) + 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(step_cluster_kernel<NW, GATE, MULTI, SPREAD>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+template <int NW, bool MULTI, typename Kernel>
+cudaError_t configure(Kernel* kernel) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StepSmem<NW, MULTI>) + 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
-template <int NW, bool GATE, bool MULTI>
+template <int NW, bool MULTI>
 cudaLaunchConfig_t config_of(int S, int units, int parts, cudaStream_t stream, cudaLaunchAttribute (&attr)[2]) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, units, parts);
@@ -1494,16 +1513,21 @@ cudaLaunchConfig_t config_of(int S, int units, int parts, cudaStream_t stream, c
     return cfg;
 }
 
-template <int NW, bool GATE, bool MULTI, bool SPREAD = false>
+template <int NW, bool GATE, bool MULTI, bool SPREAD, bool SMALL>
 int resident_of(int k) {
-    if (configure<NW, GATE, MULTI, SPREAD>() != cudaSuccess) return 0;
+    const auto kernel = step_cluster_kernel<NW, GATE, MULTI, SPREAD, SMALL>;
+    if (configure<NW, MULTI>(kernel) != cudaSuccess) return 0;
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = config_of<NW, GATE, MULTI>(1 << k, 1, 1, nullptr, attr);
+    cudaLaunchConfig_t cfg = config_of<NW, MULTI>(1 << k, 1, 1, nullptr, attr);
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, step_cluster_kernel<NW, GATE, MULTI, SPREAD>, &cfg) != cudaSuccess) n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
     cudaGetLastError();                                    // (a refused size is no error of the caller's)
     return n;
+}
+template <int NW, bool GATE, bool MULTI, bool SPREAD = false>
+int resident_of(int k) {
+    return min(resident_of<NW, GATE, MULTI, SPREAD, false>(k), resident_of<NW, GATE, MULTI, SPREAD, true>(k));
 }
 
 // Clusters of 2^k CTAs that the device holds at once (`wide`: of the NW = 16 kernels), asked once per device; 0: the
@@ -1592,21 +1616,24 @@ StepPlan step_plan(int units, int rows, int q_len, long long max_tiles, long lon
 
 namespace {
 
-template <int NW, bool MULTI>
+template <int NW, bool MULTI, bool SMALL>
 cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g, const StepPlan& plan,
                       cudaStream_t stream) {
     cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = config_of<NW, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
     if (g) {
-        const cudaLaunchConfig_t cfg = config_of<NW, true, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
         if constexpr (!MULTI)
-            if (plan.spread) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, false, true>, map_k, map_v, p, GateArg<true>{*g});
-        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, MULTI>, map_k, map_v, p, GateArg<true>{*g});
+            if (plan.spread) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, false, true, SMALL>, map_k, map_v, p, GateArg<true>{*g});
+        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, MULTI, false, SMALL>, map_k, map_v, p, GateArg<true>{*g});
     }
-    if constexpr (MULTI) {
-        const cudaLaunchConfig_t cfg = config_of<NW, false, true>(plan.S, p.num_units, plan.parts, stream, attr);
-        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, false, true>, map_k, map_v, p, GateArg<false>{});
-    }
+    if constexpr (MULTI) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, false, true, false, SMALL>, map_k, map_v, p, GateArg<false>{});
     return cudaErrorInvalidValue;                          // (lists of one query token: seer_lists.cu)
+}
+template <int NW, bool MULTI>
+cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, const GateParams* g, const StepPlan& plan,
+                      cudaStream_t stream) {
+    return p.block_idx && p.blocks_per_tile > 1 ? launch_of<NW, MULTI, true>(map_k, map_v, p, g, plan, stream)
+                                                : launch_of<NW, MULTI, false>(map_k, map_v, p, g, plan, stream);
 }
 
 }  // namespace

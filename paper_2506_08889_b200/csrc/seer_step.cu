@@ -729,14 +729,17 @@ __device__ __forceinline__ void key_sums(Pieces&& pieces, const uint32_t (*parts
 // three, the selection by one CTA and its lists stored into the others, it was 2.9, 7.2, 10.6, 11.8 to 13.3, 15.3, 16.2.
 // Longer calls by memory: of a step of 64 units x 205 blocks (430 MB) the tiles take 66 us, 6.5 TB/s, from the first CTA's
 // first to the last one's last; CTAs that share a unit read neighbouring blocks at the same time.
-// SPREAD: the lists may be so long that it matters whether they are even; where they are not, the lists and the append are all
-// that is done here, and the list kernel behind this launch does the rest (else nothing).
+// What it does: a step by the token budget; or one whose lists may be so long that it matters whether they are even (where they
+// are not, the lists and the append are all that is done here, and the list kernel behind this launch does the rest); or the
+// gate alone, by either method; or attention over given lists or all blocks.
+enum Kind { STEP, SPREAD_STEP, GATE_ALONE, LISTS };
 // SMALL: lists of blocks of 16 or 32 tokens, four or two to a tile.  (Told apart at run time both kinds' look-ups and copies took
 // registers from one another, and spilled.)
-template <int NW, bool GATE, bool MULTI, bool SPREAD, bool SMALL>
+template <int NW, Kind KIND, bool MULTI, bool SMALL>
 __global__ void __launch_bounds__(Size<NW, MULTI>::kThreads, NW == 8 ? 2 : 1)
 step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                    const __grid_constant__ DecodeParams p, const __grid_constant__ GateArg<GATE> ga) {
+                    const __grid_constant__ DecodeParams p, const __grid_constant__ GateArg<KIND != LISTS> ga) {
+    constexpr bool GATE = KIND != LISTS, ALONE = KIND == GATE_ALONE;
     using Z = Size<NW, MULTI>;
     using Smem = StepSmem<NW, MULTI>;
     constexpr int kWorkers = Z::kWorkers, kStages = Z::kStages, kArrivals = Z::kArrivals, kRows = Z::kRows;
@@ -779,7 +782,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     // (another CTA's shared memory is written only after the barrier this opens: it is then known to be running, and its
     // mbarriers are initialised)
     cluster_arrive();
-    if (producer && lane == 0 && p.q) {
+    if (producer && lane == 0 && !ALONE) {
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
     }
@@ -829,7 +832,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             for (int x = tid; x < kBins; x += kWorkers) gs.hist[x] = 0;
         }
         pdl_wait();                                        // queries, lengths and compressed keys are final
-        if (!SPREAD && !p.q && p.next_early) pdl_launch_dependents();     // (the gate alone has no work for which it wants the SMs)
+        if (ALONE && p.next_early) pdl_launch_dependents();     // (the gate alone has no work for which it wants the SMs)
         L = p.seq_lens[i];
         // (what the second round of loads reads of the queries, if there is one)
         if (producer && lane < q_len && units > 4 * slices)
@@ -842,9 +845,9 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const int j_f = max(0, L - q_len) >> b_shift;
         int n_forced = min(n_i - j_f, g.max_sel);
         int n_cand = min(j_f, g.max_blocks);
-        const bool appends = g.k_nope && blockIdx.z == 0 && L >= g.block_size && (L & (g.block_size - 1)) < q_len && (L >> b_shift) <= g.max_blocks;
+        const bool appends = !ALONE && g.k_nope && blockIdx.z == 0 && L >= g.block_size && (L & (g.block_size - 1)) < q_len && (L >> b_shift) <= g.max_blocks;
         int need = 0;                                      // (threshold method: known once the scores are)
-        if (n_i > 0 && !g.threshold_mode) {
+        if (n_i > 0 && !(ALONE && g.threshold_mode)) {
             const int k = min(max(g.token_budget >> b_shift, 1), min(n_i, g.max_sel));
             // (kListed: only a sequence longer than max_seq_len, which the host's rule went by, gets that far)
             need = max(0, min(min(k - n_forced, n_cand), kListed));
@@ -859,10 +862,9 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const int t_skip = MULTI ? kMaxQLen - q_len : 0;
         uint32_t (*parts)[3][kMaxDGate / 2 + 16] = gs.parts + t_skip;
         slots.place(sm.ring, n_tiles, Place::kScratch + t_skip * (int)sizeof(gs.parts[0]), g.d_gate);
-        const bool even = !SPREAD || !step_uneven(p, S);
-        auto attends = [&]() -> bool { return SPREAD ? even : p.q != nullptr; };
+        const bool attends = KIND == SPREAD_STEP ? !step_uneven(p, S) : !ALONE;
         // who selects: every CTA that will read tiles, or (the gate alone) the first one
-        const int n_sel = attends() ? S : 1, sel_shift = attends() ? s_shift : 0;
+        const int n_sel = attends ? S : 1, sel_shift = attends ? s_shift : 0;
         const bool selects = rank < n_sel;
         if (producer) {
             // (the scores of the other CTAs' key tiles, and from every CTA their smallest and largest key)
@@ -1024,7 +1026,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     const bool ok = j < n_cand;
                     sc_all[j] = ok ? v : -INFINITY;
                     if (ok) {
-                        if (g.scores_user) g.scores_user[(size_t)u * g.max_blocks + j] = v;
+                        if (ALONE && g.scores_user) g.scores_user[(size_t)u * g.max_blocks + j] = v;
                         const uint32_t key = score_key(v);
                         kmn = min(kmn, key);
                         kmx = max(kmx, key);
@@ -1074,7 +1076,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             dead = worker_any<NW>(!wait_sent(&sm.got_scores, p.status) || dead);
             if (dead) n_cand = need = n_forced = n_blocks = 0;
             if (dead && tid == 0) sm.no_list = 1;
-            if (g.threshold_mode) {
+            if (ALONE && g.threshold_mode) {
                 // Threshold method (Sec. 3.1): softmax of the scores over the candidates; those above tau are the `above`
                 // highest-scoring ones (equal scores have equal probabilities), so only the number differs
                 auto sum_all = [&](float v) -> float {
@@ -1102,7 +1104,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             // entry e of the list is block j: its tile(s) among this CTA's, if they are
             auto take = [&](int e, int j) {
                 if (lists) dst[e] = j;
-                if (!attends()) return;
+                if (!attends) return;
                 if constexpr (!SMALL) {
                     for (int x = 0; x < p.tiles_per_block; ++x) {
                         const int t = (e << p.tpb_shift) + x;
@@ -1134,8 +1136,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 for (int e = n_blocks + tid; e < g.max_sel; e += kWorkers) dst[e] = -1;
             }
         }
-        if (!attends()) {                                  // the gate alone
-            if (SPREAD && appends) {
+        if (!attends) {                                  // the gate alone
+            if (!ALONE && appends) {
                 if (producer) append_pool(g, sm, i, h, (L >> b_shift) - 1, rank, S);
                 else if (!dead) append_project<NW>(g, sm, u, h, (L >> b_shift) - 1, rank, S);
             }
@@ -1513,9 +1515,9 @@ cudaLaunchConfig_t config_of(int S, int units, int parts, cudaStream_t stream, c
     return cfg;
 }
 
-template <int NW, bool GATE, bool MULTI, bool SPREAD, bool SMALL>
+template <int NW, Kind KIND, bool MULTI, bool SMALL>
 int resident_of(int k) {
-    const auto kernel = step_cluster_kernel<NW, GATE, MULTI, SPREAD, SMALL>;
+    const auto kernel = step_cluster_kernel<NW, KIND, MULTI, SMALL>;
     if (configure<NW, MULTI>(kernel) != cudaSuccess) return 0;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = config_of<NW, MULTI>(1 << k, 1, 1, nullptr, attr);
@@ -1525,9 +1527,9 @@ int resident_of(int k) {
     cudaGetLastError();                                    // (a refused size is no error of the caller's)
     return n;
 }
-template <int NW, bool GATE, bool MULTI, bool SPREAD = false>
+template <int NW, Kind KIND, bool MULTI>
 int resident_of(int k) {
-    return min(resident_of<NW, GATE, MULTI, SPREAD, false>(k), resident_of<NW, GATE, MULTI, SPREAD, true>(k));
+    return min(resident_of<NW, KIND, MULTI, false>(k), resident_of<NW, KIND, MULTI, true>(k));
 }
 
 // Clusters of 2^k CTAs that the device holds at once (`wide`: of the NW = 16 kernels), asked once per device; 0: the
@@ -1536,9 +1538,10 @@ int resident_clusters(bool wide, int k) {
     static int cached[kMaxDevices][2][5];                  // (value + 1; 0: not asked yet.  A race asks twice and stores the same)
     int& c = cached[current_device_slot()][wide][k];
     if (c == 0) {
-        c = wide ? min(resident_of<16, true, true>(k), resident_of<16, false, true>(k)) + 1
-                 : min(min(resident_of<8, true, false>(k), resident_of<8, true, false, true>(k)),
-                       min(resident_of<8, true, true>(k), resident_of<8, false, true>(k))) + 1;
+        c = wide ? min(resident_of<16, STEP, true>(k), resident_of<16, LISTS, true>(k)) + 1
+                 : min(min(min(resident_of<8, STEP, false>(k), resident_of<8, SPREAD_STEP, false>(k)),
+                           min(resident_of<8, STEP, true>(k), resident_of<8, LISTS, true>(k))),
+                       min(resident_of<8, GATE_ALONE, false, false>(k), resident_of<8, GATE_ALONE, true, false>(k))) + 1;
     }
     return c - 1;
 }
@@ -1622,11 +1625,13 @@ cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const 
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = config_of<NW, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
     if (g) {
+        if constexpr (NW == 8 && !SMALL)
+            if (!p.q) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<8, GATE_ALONE, MULTI, false>, map_k, map_v, p, GateArg<true>{*g});
         if constexpr (!MULTI)
-            if (plan.spread) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, false, true, SMALL>, map_k, map_v, p, GateArg<true>{*g});
-        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, true, MULTI, false, SMALL>, map_k, map_v, p, GateArg<true>{*g});
+            if (plan.spread) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, SPREAD_STEP, false, SMALL>, map_k, map_v, p, GateArg<true>{*g});
+        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, STEP, MULTI, SMALL>, map_k, map_v, p, GateArg<true>{*g});
     }
-    if constexpr (MULTI) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, false, true, false, SMALL>, map_k, map_v, p, GateArg<false>{});
+    if constexpr (MULTI) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, LISTS, true, SMALL>, map_k, map_v, p, GateArg<false>{});
     return cudaErrorInvalidValue;                          // (lists of one query token: seer_lists.cu)
 }
 template <int NW, bool MULTI>

@@ -735,7 +735,9 @@ __device__ __forceinline__ void key_sums(Pieces&& pieces, const uint32_t (*parts
 enum Kind { STEP, SPREAD_STEP, GATE_ALONE, LISTS };
 // SMALL: lists of blocks of 16 or 32 tokens, four or two to a tile.  (Told apart at run time both kinds' look-ups and copies took
 // registers from one another, and spilled.)
-template <int NW, Kind KIND, bool MULTI, bool SMALL>
+// DG: channels of the gate, 0: known at run time (where the constant did not help the registers: several query tokens 35.4 ->
+// 36.6 us, steps of 256 channels 10.6 -> 11.0)
+template <int NW, Kind KIND, bool MULTI, bool SMALL, int DG>
 __global__ void __launch_bounds__(Size<NW, MULTI>::kThreads, NW == 8 ? 2 : 1)
 step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ DecodeParams p, const __grid_constant__ GateArg<KIND != LISTS> ga) {
@@ -775,7 +777,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         mbar_fence_init();
         if (tid == 0) {
-            if constexpr (GATE) mbar_arrive_expect_tx(&sm.got_query, (uint32_t)(q_len * ga.g.d_gate * 6));
+            if constexpr (GATE) mbar_arrive_expect_tx(&sm.got_query, (uint32_t)(q_len * (DG ? DG : ga.g.d_gate) * 6));
             mbar_arrive_expect_tx(&sm.got_parts, (uint32_t)(rows * kHeadDim * 4 + S * rows * 8));
         }
     }
@@ -793,8 +795,9 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     bool dead = false;                                     // a wait ran out: go through the motions, the results are invalid
     if constexpr (GATE) {
         const GateParams& g = ga.g;
-        const int n = g.group * kHeadDim, half = g.d_gate / 2;
-        const unsigned char* kc = reinterpret_cast<const unsigned char*>(g.kcomp + (size_t)u * g.max_blocks * g.d_gate);
+        const int d_gate = DG ? DG : g.d_gate;
+        const int n = g.group * kHeadDim, half = d_gate / 2;
+        const unsigned char* kc = reinterpret_cast<const unsigned char*>(g.kcomp + (size_t)u * g.max_blocks * d_gate);
         // Gate query: a CTA makes the rotary pairs (c, c + d_gate/2) c_first .. c_first + ppc of all query tokens, by MMAs of 16
         // rows of W_q (eight pairs) by 8 tokens; the contraction, in units of 32 channels, is split over the warps that share
         // a row tile (`slices` of them), whose partial sums meet in shared memory.  A lane holds pieces of 16 bytes as they lie
@@ -811,7 +814,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         uint4 wa[4], wb[4], xx[4];
         auto load_w = [&](int m0, int u0) {
             const int pair = 8 * (m0 + (warp & ((1 << mt_shift) - 1))) + row8;
-            const uint4* w = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * g.d_gate + c_first + min(pair, ppc - 1)) * n) + (lane & 3);
+            const uint4* w = reinterpret_cast<const uint4*>(g.w_q + ((size_t)h * d_gate + c_first + min(pair, ppc - 1)) * n) + (lane & 3);
             const uint4* x = reinterpret_cast<const uint4*>(
                 g.q_nope + (((size_t)i * q_len + min(row8, q_len - 1)) * g.num_q_heads + (size_t)h * g.group) * kHeadDim) + (lane & 3);
             const size_t step = (size_t)half * n / 8;
@@ -825,7 +828,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         };
         // (W_q into L2 only, which follows later writes: the kernel before this one may be the one that makes it)
-        if (producer && lane < 2) prefetch_l2(g.w_q + ((size_t)h * g.d_gate + c_first + lane * half) * n, 2 * n * ppc);
+        if (producer && lane < 2) prefetch_l2(g.w_q + ((size_t)h * d_gate + c_first + lane * half) * n, 2 * n * ppc);
         float* sc_all = reinterpret_cast<float*>(sm.ring);
         auto& gs = *reinterpret_cast<typename Place::Scratch*>(sm.ring + Place::kScratch);
         if (!producer) {
@@ -861,7 +864,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         // (the queries' parts: those of the last q_len of kMaxQLen places, so that the keys have what is in front of them)
         const int t_skip = MULTI ? kMaxQLen - q_len : 0;
         uint32_t (*parts)[3][kMaxDGate / 2 + 16] = gs.parts + t_skip;
-        slots.place(sm.ring, n_tiles, Place::kScratch + t_skip * (int)sizeof(gs.parts[0]), g.d_gate);
+        slots.place(sm.ring, n_tiles, Place::kScratch + t_skip * (int)sizeof(gs.parts[0]), d_gate);
         const bool attends = KIND == SPREAD_STEP ? !step_uneven(p, S) : !ALONE;
         // who selects: every CTA that will read tiles, or (the gate alone) the first one
         const int n_sel = attends ? S : 1, sel_shift = attends ? s_shift : 0;
@@ -871,7 +874,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             if (selects && lane == 0) mbar_arrive_expect_tx(&sm.got_scores, (uint32_t)((n_tiles - my_tiles) * kKeyTile * 4 + S * 8));
             if (appends && lane < 3) {
                 if (lane == 0) mbar_arrive_expect_tx(&sm.got_feat, 3 * kHeadDim * 4);
-                else prefetch_l2(g.w_k + ((size_t)h * g.d_gate + c_first + (lane - 1) * half) * 3 * kHeadDim, ppc * 3 * kHeadDim * 2);
+                else prefetch_l2(g.w_k + ((size_t)h * d_gate + c_first + (lane - 1) * half) * 3 * kHeadDim, ppc * 3 * kHeadDim * 2);
             }
         }
         cluster_wait();                                    // every CTA of the cluster has started
@@ -956,7 +959,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         uint32_t kmn = 0xffffffffu, kmx = 0u;              // smallest and largest key of this warp's scores
         auto scores = [&](auto xs_c) {
             constexpr int XS = decltype(xs_c)::value;
-            const float inv = rsqrtf((float)g.d_gate);
+            const float inv = rsqrtf((float)d_gate);
             // this lane's first piece of its first key in slot 0; the second key is kOff bytes behind the first
             const int rr = lane >> 2, k_of = 8 * (rr & 1) + (rr >> 1) + 4 * (lane & 1);
             const unsigned char* at = ((rr & 1) ? slots.b : slots.a) + (rr >> 1) * (64 * XS) + 16 * (lane & 3);
@@ -1016,7 +1019,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 #pragma unroll 1
                     for (int k = 0; k < kKeyTile; ++k) {
                         if ((((k & 4) ? odds1 : odds0) >> (4 * (2 * (k & 3) + (k >> 3)))) & 15u) {
-                            const float x = score_key_plain(reinterpret_cast<const uint4*>(kc + (size_t)(j0 + k) * (64 * XS)), parts, q_len, g.d_gate, lane);
+                            const float x = score_key_plain(reinterpret_cast<const uint4*>(kc + (size_t)(j0 + k) * (64 * XS)), parts, q_len, d_gate, lane);
                             if (k == k_of) v = x;
                         }
                     }
@@ -1042,8 +1045,8 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         };
         if (!producer) {
-            if (g.d_gate == 128) scores(std::integral_constant<int, 4>());
-            else if (g.d_gate == 64) scores(std::integral_constant<int, 2>());
+            if (d_gate == 128) scores(std::integral_constant<int, 4>());
+            else if (d_gate == 64) scores(std::integral_constant<int, 2>());
             else scores(std::integral_constant<int, 8>());
             kmn = __reduce_min_sync(0xffffffffu, kmn);
             kmx = __reduce_max_sync(0xffffffffu, kmx);
@@ -1515,9 +1518,11 @@ cudaLaunchConfig_t config_of(int S, int units, int parts, cudaStream_t stream, c
     return cfg;
 }
 
-template <int NW, Kind KIND, bool MULTI, bool SMALL>
+constexpr int wide_gate(Kind kind) { return kind == GATE_ALONE ? 256 : 0; }
+
+template <int NW, Kind KIND, bool MULTI, bool SMALL, int DG>
 int resident_of(int k) {
-    const auto kernel = step_cluster_kernel<NW, KIND, MULTI, SMALL>;
+    const auto kernel = step_cluster_kernel<NW, KIND, MULTI, SMALL, DG>;
     if (configure<NW, MULTI>(kernel) != cudaSuccess) return 0;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = config_of<NW, MULTI>(1 << k, 1, 1, nullptr, attr);
@@ -1526,6 +1531,11 @@ int resident_of(int k) {
     if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
     cudaGetLastError();                                    // (a refused size is no error of the caller's)
     return n;
+}
+template <int NW, Kind KIND, bool MULTI, bool SMALL>
+int resident_of(int k) {
+    if constexpr (KIND == LISTS || MULTI) return resident_of<NW, KIND, MULTI, SMALL, 0>(k);
+    else return min(resident_of<NW, KIND, MULTI, SMALL, 64>(k), min(resident_of<NW, KIND, MULTI, SMALL, 128>(k), resident_of<NW, KIND, MULTI, SMALL, wide_gate(KIND)>(k)));
 }
 template <int NW, Kind KIND, bool MULTI>
 int resident_of(int k) {
@@ -1624,14 +1634,25 @@ cudaError_t launch_of(const CUtensorMap& map_k, const CUtensorMap& map_v, const 
                       cudaStream_t stream) {
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = config_of<NW, MULTI>(plan.S, p.num_units, plan.parts, stream, attr);
+    auto launch = [&](auto kind, auto multi, auto dg) {
+        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, decltype(kind)::value, decltype(multi)::value, SMALL, decltype(dg)::value>, map_k, map_v, p,
+                                  GateArg<true>{*g});
+    };
+    auto launch_gate = [&](auto kind, auto multi) {
+        if constexpr (MULTI) return launch(kind, multi, std::integral_constant<int, 0>());
+        else return g->d_gate == 64    ? launch(kind, multi, std::integral_constant<int, 64>())
+                    : g->d_gate == 128 ? launch(kind, multi, std::integral_constant<int, 128>())
+                                       : launch(kind, multi, std::integral_constant<int, wide_gate(decltype(kind)::value)>());
+    };
+    using Multi = std::integral_constant<bool, MULTI>;
     if (g) {
         if constexpr (NW == 8 && !SMALL)
-            if (!p.q) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<8, GATE_ALONE, MULTI, false>, map_k, map_v, p, GateArg<true>{*g});
+            if (!p.q) return launch_gate(std::integral_constant<Kind, GATE_ALONE>(), Multi());
         if constexpr (!MULTI)
-            if (plan.spread) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, SPREAD_STEP, false, SMALL>, map_k, map_v, p, GateArg<true>{*g});
-        return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, STEP, MULTI, SMALL>, map_k, map_v, p, GateArg<true>{*g});
+            if (plan.spread) return launch_gate(std::integral_constant<Kind, SPREAD_STEP>(), Multi());
+        return launch_gate(std::integral_constant<Kind, STEP>(), Multi());
     }
-    if constexpr (MULTI) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, LISTS, true, SMALL>, map_k, map_v, p, GateArg<false>{});
+    if constexpr (MULTI) return cudaLaunchKernelEx(&cfg, step_cluster_kernel<NW, LISTS, true, SMALL, 0>, map_k, map_v, p, GateArg<false>{});
     return cudaErrorInvalidValue;                          // (lists of one query token: seer_lists.cu)
 }
 template <int NW, bool MULTI>

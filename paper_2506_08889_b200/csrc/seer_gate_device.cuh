@@ -68,10 +68,10 @@ __device__ __forceinline__ float key_score(uint32_t key) {
 
 // Split cluster barrier (all threads of all CTAs of the cluster execute both halves).  The aligned forms are for a warp
 // whose lanes are together; behind a branch that only some lanes take they need not be, so they are brought together here.
-__device__ __forceinline__ void cluster_arrive() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
+#define SEER_CLUSTER_ARRIVE(sem) do { __syncwarp(); asm volatile("barrier.cluster.arrive" sem ".aligned;" ::: "memory"); } while (0)
+__device__ __forceinline__ void cluster_arrive() { SEER_CLUSTER_ARRIVE(".release"); }
+// ... where nothing that this thread has written is handed over with it: it does not wait for its stores.
+__device__ __forceinline__ void cluster_arrive_relaxed() { SEER_CLUSTER_ARRIVE(".relaxed"); }
 __device__ __forceinline__ void cluster_wait() {
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

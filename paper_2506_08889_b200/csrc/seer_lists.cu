@@ -463,7 +463,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
             ++piece;
         } while (next_piece());
         cluster_wait();                                    // (the barrier opened at the top)
-        cluster_arrive();
+        cluster_arrive_relaxed();
     } else {
         const int group = warp >> 2, w4 = warp & 3, qd = lane & 3, rw = lane >> 2;
         // Q^T B-fragments: this thread supplies row rw of the unit's queries
@@ -592,7 +592,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
                 if (lane == 0) mbar_arrive(&sm.empty[st]);
             }
             wait_sent(&sm.got_parts[turn], p.status, (piece >> 1) & 1);
-            if (!more) cluster_arrive();
+            if (!more) cluster_arrive_relaxed();           // (all that was sent to this CTA is here)
             else if (tid == 0) mbar_arrive_expect_tx(&sm.got_parts[turn], part_bytes);       // (for the piece after the next)
             // ---- this CTA's slice of the channels: the output, or the piece's part of it --------------------------------
             const int pairs = rows << (c_shift - 1);       // channel pairs of the slice, all rows

@@ -1296,7 +1296,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         }
         if (!GATE) cluster_wait();                         // (the barrier opened at the top)
-        cluster_arrive();
+        cluster_arrive_relaxed();
     } else {
         const int group = warp >> 2, my_n = MULTI ? group % tiles_n : 0, pace = MULTI ? group / tiles_n : group;
         // Q^T B-fragments: this thread supplies row 8 * my_n + rw of the unit's queries
@@ -1459,7 +1459,7 @@ step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     }
     if (!producer) {
         wait_sent(&sm.got_parts, p.status);
-        cluster_arrive();
+        cluster_arrive_relaxed();                          // (all that was sent to this CTA is here)
         const int c_shift = 7 - s_shift;
         const int pairs = rows << (c_shift - 1);           // channel pairs of this CTA's slice, all rows
 #pragma unroll 1

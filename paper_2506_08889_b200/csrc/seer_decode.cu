@@ -977,7 +977,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__
                 const int c = ct - pend_n, b = c % kTcSBufs;
                 if (__shfl_sync(0xffffffffu, lane == 0 ? (int)mbar_test_wait(&sm.v.bar_p[b], (c / kTcSBufs) & 1) : 0, 0)) {
                     __syncwarp();
-                    if (lane == 0) {
+                    if (elect_one()) {
                         tc_fence_after_sync();
                         const uint32_t v_addr = smem_u32(sm.stage[0]) + pend_stage[b] * kTileBytes;
 #pragma unroll
@@ -1023,7 +1023,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__
                                 __syncwarp();
                             }
                             const int b = ct % kTcSBufs;
-                            if (lane == 0) {
+                            if (elect_one()) {
                                 tc_fence_after_sync();
                                 const uint32_t k_addr = smem_u32(sm.stage[0]) + (kTcStages + it % kTcKStages) * kTileBytes;
 #pragma unroll

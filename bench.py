@@ -31,12 +31,11 @@ METRIC = "sparse_decode_selected_kv_GBps"
 UNIT = "GB/s"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
-# dram__bytes_read.sum + dram__bytes_write.sum of one sparse launch of decode_kernel, from an ncu capture of a
-# quarter-size case (batch 2, SEER_STEP_CLUSTERS=0): 107.7 MB read + 3.0 MB written for 107.5 MB of algorithmic
-# bytes.  Reads grow with the selected tiles, writes (partials) with the number of CTAs, so a launch on
-# `batch` sequences moves about batch/2 * 107.7 MB + 3.0 MB.
-NCU_READ_BYTES_PER_2_SEQUENCES = 107.695e6
-NCU_WRITE_BYTES_PER_LAUNCH = 2.97e6
+# dram__bytes_read.sum + dram__bytes_write.sum of one sparse launch of the list kernel, from an ncu capture of a
+# quarter-size case (batch 2): 107.6 MB read + 3.4 MB written (other kernels' dirty lines) for 107.5 MB of algorithmic
+# bytes.  Reads grow with the selected tiles, so a launch on `batch` sequences moves about batch/2 * 107.6 MB + 3.4 MB.
+NCU_READ_BYTES_PER_2_SEQUENCES = 107.576e6
+NCU_WRITE_BYTES_PER_LAUNCH = 3.44e6
 
 
 def measured_hbm_peak():
@@ -409,7 +408,7 @@ def run_ours(args):
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": round(e2e_ms, 5)},
             "gpu_launches": int(launches),
             "clocks": clocks,
-            "roofline": {"bound": "hbm", "kernel": "seer_sparse_decode on the step's lists (decode_kernel; in the step itself "
+            "roofline": {"bound": "hbm", "kernel": "seer_sparse_decode on the step's lists (dealt_decode_kernel; in the step itself "
                                                     "step_cluster_kernel does this work)" if B >= 8 else "seer_sparse_decode",
                          "achieved": round(kern_gbs, 1),
                          "peak": peak, "unit": "GB/s", "frac": round(kern_gbs / peak, 4), "peak_kind": f"of {peak_kind}",
@@ -418,7 +417,7 @@ def run_ours(args):
                          "event_samples": n_ev, "empty_launch_between_events_us": round(empty_ms * 1e3, 2),
                          "traffic": (int(NCU_READ_BYTES_PER_2_SEQUENCES * B / 2 * (1.0 - args.sparsity) / 0.1
                                          + NCU_WRITE_BYTES_PER_LAUNCH) if abs(args.sparsity - 0.9) < 1e-9 and B >= 8 else None),
-                         "traffic_note": "ncu capture of decode_kernel at batch 2, scaled by the units processed",
+                         "traffic_note": "ncu capture of the list kernel at batch 2, scaled by the units processed",
                          # the same kernel launched back to back (no event between launches, so that each
                          # launch's set-up overlaps its predecessor's tail as it does inside the step)
                          "us_per_launch_back_to_back": round(sparse_b2b_ms * 1e3, 2),

@@ -352,7 +352,7 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
  * on `stream` (where step and gate call take different forms, up to blocks whose scores agree to within
  * fp32 rounding; see seer_gate_select), with one host round trip instead of three.  (With at most 64 tiles per CTA of the lists'
  * clusters and at most 16384 compressed keys per sequence, gate, attention and append are one
- * launch.  Otherwise the launches go out as gate, attention, append: the block that has just filled is
+ * launch; up to 128, one launch and a second that does the attention where the lists are uneven.  Otherwise the launches go out as gate, attention, append: the block that has just filled is
  * the sequence's last block, which the gate takes without scoring it, so the entry the append writes is
  * first read in the next step.  When gate->max_blocks
  * blocks cover kv->max_seq_len, the attention kernel knows every list's length from the sequence

@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(kKcThreads, 4) kcomp_bulk_kernel(const KcompPa
 //   producer (1 warp)    keeps a ring of 64-row stages (16 KiB) full with tiled copies, so the bytes in
 //                        flight do not depend on what the other warps are doing;
 //   pooling (10 warps)   each takes one portion at a time out of shared memory -- a block of 64 or 128 rows
-//                        (one or two stages), or the two or four blocks of 32 or 16 rows in a stage -- and leaves
+//                        (one or two stages), or two blocks of 32 or 16 rows (a stage, or half of one) -- and leaves
 //                        each block's 3*128 features (bf16; the mean as high part + correction: 512 numbers) in one
 //                        of two feature buffers, laid out as the tensor cores read a K-major operand;
 //   MMA (1 warp)         once an item's (up to 16) blocks are pooled, one thread multiplies them in: Y (128 rows of
@@ -366,13 +366,17 @@ __global__ void __launch_bounds__(kKcThreads, 4) kcomp_bulk_kernel(const KcompPa
 //     2 x 8 heads x 128k (0.54 GB)              124 -> 92 .. 96   116 -> 89         (floor 83)
 //     6 ragged sequences of 5k .. 32k           79.9 -> 48.0      69.9 -> 46.1      (floor 36)
 //     one sequence of 8k                        19.3 -> 11.6      28.3 -> 11.7      (launch, lengths, one trip through the kernel)
-// Blocks of 32 and 16 are bound by what is done per block (shuffles, features, rotation): 0.54 GB 190 -> 116, 309 -> 168
-// (one box of 64 rows instead of a box per block: 106 and 166, but it may reach past the last complete block).
+// With the products issued by an elected lane (3600 -> 470 cycles an item) and warps that go straight to their portions the first
+// take 88.2, the second 44.4 (blocks of 128), the third 8.5; blocks of 32 and 16, 0.54 GB, 110 -> 96 and 166 -> 129: with
+// those, and two blocks pooled at a time, one per half warp.  Blocks of 16 are bound by what is done per item of 16 (barriers,
+// features, rotation), four times as often as with 64 rows; the others by memory.
 //
 // Portion number n of a CTA (counted over all its items) is pooled by warp n % kPoolWarps, its stages n * SPB + part live
 // in ring slots (..) % kStreamStages and are announced on barrier (..) % (SPB * kPoolWarps): a barrier is always waited
 // for by the same warp, which goes through its stages in order, so a wait is never more than one phase away from the
-// barrier's own, which is what a parity wait needs to be unambiguous.  (With a block-of-the-item -> warp rule a fast warp
+// barrier's own, which is what a parity wait needs to be unambiguous.  (A stage of four blocks of 16 is two portions, and two warps
+// wait for it, on one of 20 barriers: the stage 20 before it belongs to an item whose products are done, and the one 20 behind
+// it needs its slot, which both have to give back.)  (With a block-of-the-item -> warp rule a fast warp
 // could ask for a slot's next use before the slot's current use had landed for another warp, and the parity test would
 // pass on stale data.)
 constexpr int kStreamStages = 10;                      // 160 KiB in flight per SM

@@ -327,9 +327,10 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
     p.trace = reinterpret_cast<unsigned long long*>(ctx->ws + (ctx->ws_bytes - (size_t)(1 << 20)));
 #endif
     if (!gate && ctx->use_clusters && !ctx->chain_attention && !(wide && ctx->wide_variant) && ctx->list_gen == 0 && ctx->sel_from_lens == 0) {
-        const ListPlan lists = q_len == 1 ? list_plan(U, max_tiles / U) : ListPlan{0, false, false};
-        if (lists.S > 0 && (!lists.spread || w.scratch + list_part_bytes(U, lists.S) <= ctx->ws_bytes)) {
+        const ListPlan lists = q_len == 1 ? list_plan(U, max_tiles / U) : ListPlan{0, 0, false, false};
+        if (lists.S > 0 && (!lists.spread || w.scratch + list_part_bytes(U, lists.clusters, lists.S) <= ctx->ws_bytes)) {
             p.part_o = reinterpret_cast<float*>(ctx->ws + w.scratch);
+            p.clusters = lists.clusters;
             p.spread = lists.spread;
             p.next_early = lists.next_early;
             ce = launch_lists(mk_copy, *mv, p, lists.S, static_cast<cudaStream_t>(stream));
@@ -351,6 +352,7 @@ seer_status decode_common(seer_ctx* ctx, const seer_shape* shape, const seer_kv*
         ctx->launches += 1;
         if (plan.spread) {
             p.part_o = reinterpret_cast<float*>(ctx->ws + w.scratch);
+            p.clusters = U;
             p.spread = 1;
             ce = launch_lists(mk_copy, *mv, p, plan.S, static_cast<cudaStream_t>(stream));
             if (ce != cudaSuccess) return fail(ctx, SEER_ERR_CUDA, "decode launch: %s", cudaGetErrorString(ce));
@@ -831,7 +833,7 @@ static StepPlan plan_of_step(seer_ctx* ctx, const seer_shape* shape, const seer_
     StepPlan plan = step_plan(U, rows, q_len, tiles, bs < kTileTokens ? tiles * (kTileTokens / bs) : tiles, gate->max_blocks);
     if (plan.S > 0 && plan.spread) {
         if (shape->batch == 1) plan.spread = false;        // (the heads' lists are equally long)
-        else if (list_plan(U, tiles).S != plan.S || ws_layout(U, 0, 0, 0).scratch + list_part_bytes(U, plan.S) > ctx->ws_bytes) plan.S = 0;
+        else if (list_plan(U, tiles).S != plan.S || ws_layout(U, 0, 0, 0).scratch + list_part_bytes(U, U, plan.S) > ctx->ws_bytes) plan.S = 0;
     }
     return plan;
 }

@@ -74,6 +74,7 @@ struct DecodeParams {
                                     // counts follow from the lengths and the schedule can be made before the kernel
                                     // that writes the lists has finished (0: read block_cnt)
     int next_early;                     // cluster kernels: StepPlan's, ListPlan's
+    int clusters;                       // list kernel: ListPlan's
     int spread;                         // list kernel: ListPlan's (sel_from_lens > 0: behind a step that has done even lists itself)
     unsigned int* status;
     unsigned long long* tickets;    // [num_units]: tiles done << 32 | valid-slot bits; zero between launches
@@ -151,12 +152,13 @@ constexpr int kListTiles = 128;         // most tiles a CTA
 constexpr int kListUnits = 320;         // most units whose tiles it counts
 struct ListPlan {
     int S;                              // CTAs per cluster; 0: the decode kernel
+    int clusters;                       // one per unit, and more where units are few and long
     bool spread;                        // the lists may be so long that it matters whether they are even
     bool next_early;                    // the stream's next launch may start beside this one
 };
 ListPlan list_plan(int units, long long max_tiles);
 // Bytes of partial results (DecodeParams::part_o) that a launch may need.
-size_t list_part_bytes(int units, int S);
+size_t list_part_bytes(int units, int clusters, int S);
 cudaError_t launch_lists(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, int S, cudaStream_t stream);
 // The gate by itself as one launch of such clusters (at most 8192 compressed keys per unit), while they are resident all at
 // once; false: not that size, and nothing has been launched.

@@ -11,7 +11,8 @@
 //                  is dealt to the clusters whose own lists end well before it.  A cluster goes through its share piece by
 //                  piece, each a run of tiles of one unit; a unit of several pieces is put together from their partial
 //                  results, in global memory, by the CTAs that deliver the last one (rank r of the clusters has slice r of the
-//                  channels, so each slice is a matter of its own, with its own counter).
+//                  channels, so each slice is a matter of its own, with its own counter).  Where units are few and long there are
+//                  clusters without a unit of their own for it, as many as there is room for.
 // Every CTA comes to the same decision from the same numbers, so that nothing is waited for across clusters.
 //
 // What bounds it: memory, from the first tiles (2.8 us after the kernel may read its inputs) to the last; 128 ragged lists of 13 to
@@ -156,23 +157,23 @@ __device__ __forceinline__ int place_of(const int* v, int n, int x) {
     return lo;
 }
 
-// The deal, by one warp, whose lane l has the tiles of units l, l + 32, ... in n[]: the lowest line at which the helpers have
+// The deal, by one warp, whose lane l has the tiles of clusters l, l + 32, ... in n[]: the lowest line at which the helpers have
 // room below it for what is above it.  (Every cluster has the first tiles of its own unit, which are asked for before the
 // deal.  Few tiles are not worth a piece: a unit that ends a little above the line keeps what is its, a cluster with little
 // room is no helper, and where a helper's share ends a few tiles from a unit's end it ends there.)
 template <int COUNTS>
-__device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int units, int S, int cluster_id, int total, int most) {
+__device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int clusters, int S, int cluster_id, int total, int most) {
     const int lane = threadIdx.x & 31, cost = kPieceTiles * S, few = cost / 2;
     auto above = [&](int line, int t) { return t - line >= few ? t - line : 0; };
     auto below = [&](int line, int t) { return line - cost - t >= few ? line - cost - t : 0; };
-    int lo = max(total / units, kStages * S), hi = max(lo, most);      // (line `most`: nothing is above it)
+    int lo = max(total / clusters, kStages * S), hi = max(lo, most);      // (line `most`: nothing is above it)
 #pragma unroll 1
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         int free = 0;
 #pragma unroll
         for (int k = 0; k < COUNTS; ++k)
-            if (lane + 32 * k < units) free += below(mid, n[k]) - above(mid, n[k]);
+            if (lane + 32 * k < clusters) free += below(mid, n[k]) - above(mid, n[k]);
         if (__reduce_add_sync(0xffffffffu, free) >= 0) hi = mid;
         else lo = mid + 1;
     }
@@ -180,9 +181,9 @@ __device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int u
     int rest = 0, room = 0, helpers = 0;
 #pragma unroll
     for (int k = 0; k < COUNTS; ++k) {
-        if (32 * k >= units) break;
+        if (32 * k >= clusters) break;
         const int v = lane + 32 * k;
-        const int over = v < units ? above(line, n[k]) : 0, mine = v < units ? below(line, n[k]) : 0;
+        const int over = v < clusters ? above(line, n[k]) : 0, mine = v < clusters ? below(line, n[k]) : 0;
         int a = over, b = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -190,7 +191,7 @@ __device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int u
             if (lane >= o) { a += ta; b += tb; }
         }
         const unsigned has = __ballot_sync(0xffffffffu, mine > 0);
-        if (v < units) sm.rest[v] = rest + a - over;
+        if (v < clusters) sm.rest[v] = rest + a - over;
         if (mine > 0) {
             const int at = helpers + __popc(has & ((1u << lane) - 1u));
             sm.room[at] = room + b - mine;
@@ -201,7 +202,7 @@ __device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int u
         room += __shfl_sync(0xffffffffu, b, 31);
     }
     if (lane == 0) {
-        sm.rest[units] = rest;
+        sm.rest[clusters] = rest;
         sm.room[helpers] = room;
         sm.helpers = helpers;
         sm.line = line;
@@ -210,14 +211,14 @@ __device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int u
     for (int k = lane; k < helpers; k += 32) {
         const int x = sm.room[k];
         if (x >= rest) break;
-        const int u = place_of(sm.rest, units, x), r0 = sm.rest[u], r1 = sm.rest[u + 1];
+        const int u = place_of(sm.rest, clusters, x), r0 = sm.rest[u], r1 = sm.rest[u + 1];
         if (2 * (x - r0) < few) sm.room[k] = r0;
         else if (2 * (r1 - x) < few) sm.room[k] = r1;
     }
     __syncwarp();
 }
 
-// grid (S, units), cluster (S, 1, 1).  SPREAD: the lists may be so long that it matters whether they are even.
+// grid (S, clusters), cluster (S, 1, 1).  SPREAD: the lists may be so long that it matters whether they are even.
 template <bool SPREAD>
 __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p) {
     extern __shared__ unsigned char smem_raw[];
@@ -273,7 +274,8 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
     }
     // (the first entries are asked for beside the count that says how many there are, not behind it)
     int entry[4] = {-1, -1, -1, -1}, entry2[4] = {-1, -1, -1, -1};      // the list's entries of this lane's first tile, and of the second piece's
-    if (producer && !dense) {
+    const bool owner = cluster_id < p.num_units;           // (the others have no unit of their own)
+    if (producer && !dense && owner) {
         const int t = (lane << s_shift) + rank;
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
@@ -282,7 +284,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         }
     }
     Piece pc;
-    int L = p.seq_lens[sequence_of(cluster_id)], n_blocks = blocks_of(cluster_id, L);
+    int L = owner ? p.seq_lens[sequence_of(cluster_id)] : 0, n_blocks = owner ? blocks_of(cluster_id, L) : 0;
     pc.u = cluster_id;
     pc.a = 0;
     pc.b = pc.n = tiles_of(n_blocks, L);
@@ -293,13 +295,13 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         if (sm.line < 0x7fffffff && sm.rest[cluster_id + 1] > sm.rest[cluster_id]) pc.b = sm.line;
         if (sm.helper >= 0) {
             pc.x = sm.room[sm.helper];
-            pc.end = min(sm.room[sm.helper + 1], sm.rest[p.num_units]);
+            pc.end = min(sm.room[sm.helper + 1], sm.rest[p.clusters]);
         }
     };
     // on to the next piece; false: that was the last
     auto next_piece = [&]() -> bool {
         if (pc.x >= pc.end) return false;
-        pc.u = place_of(sm.rest, p.num_units, pc.x);       // (the last one that begins there: the others have nothing above the line)
+        pc.u = place_of(sm.rest, p.clusters, pc.x);        // (the last one that begins there: the others have nothing above the line)
         const int r0 = sm.rest[pc.u], r1 = sm.rest[pc.u + 1], line = sm.line;
         pc.a = line + pc.x - r0;
         pc.x = min(r1, pc.end);
@@ -323,7 +325,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
             __syncwarp();
             take_share();
             if (pc.x < pc.end) {
-                const int u = place_of(sm.rest, p.num_units, pc.x), t = sm.line + pc.x - sm.rest[u] + (lane << s_shift) + rank;
+                const int u = place_of(sm.rest, p.clusters, pc.x), t = sm.line + pc.x - sm.rest[u] + (lane << s_shift) + rank;
                 L2 = p.seq_lens[sequence_of(u)];
                 n_blocks2 = blocks_of(u, L2);
                 if (!dense) {
@@ -478,7 +480,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
                 bq[ks][1] = rw < rows ? __ldg(qrow + 8 * ks + 4 + qd) : 0u;
             }
         };
-        load_q(pc.u);
+        load_q(min(pc.u, p.num_units - 1));
         if (p.next_early) pdl_launch_dependents();
         // blocks of 16 or 32 tokens: which of the gathered blocks this warp's rows belong to, and where in it
         const int sub_w = !small ? 0 : p.block_size == 16 ? w4 : w4 >> 1;
@@ -502,7 +504,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
             }
             total = __reduce_add_sync(0xffffffffu, total);
             most = __reduce_max_sync(0xffffffffu, most);
-            if (list_uneven(total, most, p.num_units, S)) deal(sm, n, p.num_units, S, cluster_id, total, most);
+            if (list_uneven(total, most, p.clusters, S)) deal(sm, n, p.clusters, S, cluster_id, total, most);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.dealt);
         }
@@ -629,7 +631,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
                     }
                 }
                 if (whole) {
-                    write_out(r, c, M, l, a0, a1);
+                    if (!SPREAD || done.u < p.num_units) write_out(r, c, M, l, a0, a1);
                 } else {
                     float* dst = part_of(done.a == 0 ? done.u : p.num_units + sm.helper + done.u);
                     if (c == 0) *reinterpret_cast<float2*>(dst + 2 * r) = make_float2(M, l);
@@ -759,28 +761,35 @@ int resident_lists(int k) {
 //     192, dense           8 sequences           241 -> 228 / 147 -> 151
 //     256, dense           8 sequences           313 -> 305 / 193 -> 201
 // (One long sequence among short ones: as clusters without a deal 64 instead of 39 us where its lists have 102 tiles a CTA.)
+// Where half of the clusters that fit would do, and a list may have more than 32 tiles a CTA, all that fit are launched, and the long
+// units dealt to those without one (a CTA by itself is far from what the memory gives): dense, one KV head of 128k 54.9 (decode
+// kernel) -> 24.4, two of 55k and 156k 48.9 -> 29.6, lists of 615 tiles 21.5 -> 15.8; with 25 tiles a CTA or less nothing is gained.
 ListPlan list_plan(int units, long long max_tiles) {
-    ListPlan plan = {0, false, false};
+    ListPlan plan = {0, units, false, false};
     if (units > kListUnits || units * max_tiles >= (1ll << 30)) return plan;
     for (int k = 4; k >= 0; --k) {
         const int S = 1 << k;
         if (k > 0 && S > max_tiles) continue;              // a CTA would have nothing to do
         if (units > resident_lists(k)) continue;
-        if (max_tiles <= (long long)kListTiles * S) plan.S = S;
         plan.spread = max_tiles > (long long)S * (16 + 2 * S);       // (shorter lists gain nothing by a deal)
-        plan.next_early = 2 * units <= resident_lists(k);
+        if (2 * units <= resident_lists(k) && max_tiles > 32ll * S) {
+            plan.clusters = resident_lists(k);
+            plan.spread = true;
+        }
+        if (max_tiles * units <= (long long)kListTiles * S * plan.clusters) plan.S = S;
+        plan.next_early = 2 * plan.clusters <= resident_lists(k);
         break;
     }
     return plan;
 }
 
-size_t list_part_bytes(int units, int S) {
-    return (size_t)units * 3 * S * (2 * kRows + (size_t)kRows * kHeadDim / S) * sizeof(float);
+size_t list_part_bytes(int units, int clusters, int S) {
+    return (size_t)(2 * units + clusters) * S * (2 * kRows + (size_t)kRows * kHeadDim / S) * sizeof(float);
 }
 
 cudaError_t launch_lists(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, int S, cudaStream_t stream) {
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = config_of(S, p.num_units, stream, attr);
+    const cudaLaunchConfig_t cfg = config_of(S, p.clusters, stream, attr);
     return cudaLaunchKernelEx(&cfg, p.spread ? dealt_decode_kernel : list_step_cluster_kernel, map_k, map_v, p);
 }
 

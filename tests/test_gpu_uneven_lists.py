@@ -18,6 +18,8 @@ CASES = [
     (16, 8, 32, 128, [5120, 4999, 5120] + [512 - x for x in range(22)], [160, 150, 155] + [3 + x % 7 for x in range(22)]),      # 200 units, a CTA each
     (20, 4, 128, 0, [130] * 13 + [8192 - 64] + [1000] * 6, [2] * 13 + [60] + [1, 0, 7, 3, 2, 5]),                      # 80 units, the long one among them
     (8, 2, 16, 64, [9000] * 2 + [50 * x + 1 for x in range(18)], [500, 411] + [x % 9 for x in range(18)]),             # 40 units, four blocks a tile
+    (4, 1, 64, 0, [70001], None),                                                                                     # one unit, all other clusters without
+    (8, 2, 32, 64, [60000, 300], [1800, 5]),                                                                          # 4 units, two of them long
     (8, 1, 64, 0, [20000, 0, 0, 0, 19000, 63, 64, 65, 0, 128], None),                                                  # runs that begin behind empty units
 ]
 

@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kKcThreads, 4) kcomp_bulk_kernel(const KcompPa
 // One persistent CTA per SM, four kinds of warps that meet only through mbarriers:
 //   producer (1 warp)    keeps a ring of 64-row stages (16 KiB) full with tiled copies, so the bytes in
 //                        flight do not depend on what the other warps are doing;
-//   pooling (10 warps)   each takes one portion at a time out of shared memory -- a block of 64 or 128 rows
+//   pooling (8 or 10)    each takes one portion at a time out of shared memory -- a block of 64 or 128 rows
 //                        (one or two stages), or two blocks of 32 or 16 rows (a stage, or half of one) -- and leaves
 //                        each block's 3*128 features (bf16; the mean as high part + correction: 512 numbers) in one
 //                        of two feature buffers, laid out as the tensor cores read a K-major operand;
@@ -375,43 +375,50 @@ __global__ void __launch_bounds__(kKcThreads, 4) kcomp_bulk_kernel(const KcompPa
 // in ring slots (..) % kStreamStages and are announced on barrier (..) % (SPB * kPoolWarps): a barrier is always waited
 // for by the same warp, which goes through its stages in order, so a wait is never more than one phase away from the
 // barrier's own, which is what a parity wait needs to be unambiguous.  (A stage of four blocks of 16 is two portions, and two warps
-// wait for it, on one of 20 barriers: the stage 20 before it belongs to an item whose products are done, and the one 20 behind
+// wait for it, on one of 20 barriers (ten warps): the stage 20 before it belongs to an item whose products are done, and the one 20 behind
 // it needs its slot, which both have to give back.)  (With a block-of-the-item -> warp rule a fast warp
 // could ask for a slot's next use before the slot's current use had landed for another warp, and the parity test would
 // pass on stale data.)
-constexpr int kStreamStages = 10;                      // 160 KiB in flight per SM
 constexpr int kStageRows = kKcompStageRows;
 constexpr int kStageBytes = kStageRows * kHeadDim * 2;
 constexpr int kStreamDGate = 128;
 constexpr int kMaxSeqs = 4096;                         // sequences whose block counts are kept in shared memory
-constexpr int kPoolWarps = 10;                       // with 4 + 1 + 1 others: 16 warps
 constexpr int kProjWarps = 5;                        // warps 0..3 epilogue, 4 MMA
 constexpr int kEpiWarps = 4, kEpiThreads = 128;
 constexpr int kFeatBytes = 8 * kBulkBlocks * 128;      // one feature buffer
 constexpr int kKcTmemCols = 512;                       // W_k 256 columns (512 bf16 per row), Y twice 16
-constexpr int kStreamThreads = 32 * (kProjWarps + kPoolWarps + 1);
-static_assert(kStreamStages <= 32, "one producer lane per ring slot");
-static_assert(kStreamStages % kPoolWarps == 0 && 2 * kPoolWarps % kStreamStages == 0, "a barrier stands for one ring slot");
+// Pooling warps (beside 4 + 1 + 1 others), and as many stages: ten, or eight with 128 KiB in flight per SM.  Eight end closer together
+// and have less to start; ten pool faster.  us a call, ten -> eight: blocks of 128, 6 ragged sequences 44.3 -> 42.5, 0.27 GB 48.5 ->
+// 47.5; of 64, 0.54 GB 88.3 -> 89.1, one sequence of 8k 8.54 -> 8.70; of 32, 92 MB 25.0 -> 24.1, 14 short sequences 18.2 -> 16.9, 0.54
+// GB 95 -> 97; of 16, 0.54 GB 128 -> 136.
+template <int B>
+struct StreamSize {
+    static constexpr int kPool = B == 16 || B == 64 ? 10 : 8, kStages = kPool, kThreads = 32 * (kProjWarps + kPool + 1);
+    static_assert(kStages <= 32, "one producer lane per ring slot");
+    static_assert(kStages % kPool == 0 && 2 * kPool % kStages == 0, "a barrier stands for one ring slot");
+};
 
+template <int B>
 struct __align__(1024) StreamSmem {
+    using Z = StreamSize<B>;
     // a stage: channels 0..63 of its 64 rows (128 B per row, 16-byte pieces swizzled by row as the copy engine
     // lays them out), then channels 64..127
-    unsigned char ring[kStreamStages][kStageBytes];
+    unsigned char ring[Z::kStages][kStageBytes];
     // features of 16 blocks, twice: [8 slabs of 64 features][16 blocks][128 B], 16-byte pieces swizzled by
     // block (what a K-major operand with the 128-byte swizzle looks like); slabs: max 0-1, min 2-3, the mean's
     // high part 4-5, its correction 6-7
     unsigned char feat[2][kFeatBytes];
     float ybuf[kBulkBlocks][kStreamDGate];
-    uint64_t full[2 * kPoolWarps], empty[kStreamStages];
+    uint64_t full[2 * Z::kPool], empty[Z::kStages];
     uint64_t feat_full[2], feat_empty[2];
     uint64_t y_full[2], y_free[2];       // the products of an even / odd item are complete / have been read
     uint64_t w_ready;                    // a head's W_k is in tensor memory
     uint64_t tmem_done;                  // the epilogue warps have made their last tensor-memory access
     uint32_t tmem_base;
-    int scan[kStreamThreads / 32];
+    int scan[Z::kThreads / 32];
     int first[kMaxSeqs + 1];             // blocks of the sequences before (prefix sums of the complete blocks in the call's range)
 };
-static_assert(sizeof(StreamSmem) + 1024 <= 227 * 1024, "one CTA's shared memory");
+static_assert(sizeof(StreamSmem<16>) + 1024 <= 227 * 1024, "one CTA's shared memory");
 static_assert(kStageBytes % 2048 == 0, "both halves of a stage start on a swizzle-pattern boundary");
 
 // A CTA's run of blocks [x, end), item by item; every warp goes through it for itself.
@@ -429,9 +436,12 @@ struct Run {
 #endif
 
 // Barriers among parts of the CTA: the epilogue warps; the others; the others' arrival for the epilogue warps to wait for.
-__device__ __forceinline__ void rest_sync() { asm volatile("bar.sync 2, %0;" ::"n"(kStreamThreads - kEpiThreads) : "memory"); }
-__device__ __forceinline__ void lengths_arrive() { asm volatile("bar.arrive 3, %0;" ::"n"(kStreamThreads) : "memory"); }
-__device__ __forceinline__ void lengths_wait() { asm volatile("bar.sync 3, %0;" ::"n"(kStreamThreads) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void rest_sync() { asm volatile("bar.sync 2, %0;" ::"n"(THREADS - kEpiThreads) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void lengths_arrive() { asm volatile("bar.arrive 3, %0;" ::"n"(THREADS) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void lengths_wait() { asm volatile("bar.sync 3, %0;" ::"n"(THREADS) : "memory"); }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // A block's features of one lane (eight channels: piece `cchunk`) to row q of a feature buffer: 16 bytes per kind, each at its
@@ -464,15 +474,16 @@ __device__ __forceinline__ void store_features(unsigned char* feat, int q, bool 
 }
 
 template <int B>
-__global__ void __launch_bounds__(kStreamThreads, 1)
+__global__ void __launch_bounds__(StreamSize<B>::kThreads, 1)
 kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams p) {
+    constexpr int kPoolWarps = StreamSize<B>::kPool, kStreamStages = StreamSize<B>::kStages, kStreamThreads = StreamSize<B>::kThreads;
     constexpr int SPB = B > kStageRows ? B / kStageRows : 1;       // stages of a portion
     constexpr int BPS = B < kStageRows ? kStageRows / B : 1;       // blocks of a portion
     constexpr int SHARE = BPS > 2 ? BPS / 2 : 1;                   // portions of a stage: two blocks of 16 rows each
     constexpr int kArrivals = SPB * SHARE * kPoolWarps;
     extern __shared__ unsigned char smem_raw[];
     // (aligned by an offset, not by a cast through an integer: the compiler then still knows the accesses for shared ones)
-    StreamSmem& sm = *reinterpret_cast<StreamSmem*>(smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023));
+    StreamSmem<B>& sm = *reinterpret_cast<StreamSmem<B>*>(smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         for (int s = 0; s < kArrivals; ++s) mbar_init(&sm.full[s], 1);
@@ -545,7 +556,7 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
         pdl_wait();
         if (few_seqs) sum_lengths();
         load_w(h_first);
-        if (!few_seqs) lengths_wait();
+        if (!few_seqs) lengths_wait<kStreamThreads>();
     } else if (few_seqs) {
         pdl_wait();
         pdl_launch_dependents();
@@ -567,7 +578,7 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
             if (lane >= o) incl += v;
         }
         if (lane == 31) sm.scan[warp] = incl;
-        rest_sync();
+        rest_sync<kStreamThreads>();
         int acc = incl - mine;
 #pragma unroll
         for (int w = kEpiWarps; w < kStreamThreads / 32; ++w) acc += w < warp ? sm.scan[w] : 0;
@@ -576,8 +587,8 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
             acc += per == 1 ? mine : blocks_of(i);
         }
         if (hi == p.batch && lo < hi) sm.first[p.batch] = acc;
-        lengths_arrive();
-        rest_sync();
+        lengths_arrive<kStreamThreads>();
+        rest_sync<kStreamThreads>();
     }
 
     const int per_head = sm.first[p.batch];
@@ -936,14 +947,14 @@ cudaError_t launch_stream(const KcompParams& p, const CUtensorMap& map_k, cudaSt
     static bool configured[kMaxDevices] = {};
     const int slot = current_device_slot();
     if (!configured[slot]) {
-        const cudaError_t e = cudaFuncSetAttribute(kcomp_stream_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StreamSmem) + 1024);
+        const cudaError_t e = cudaFuncSetAttribute(kcomp_stream_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StreamSmem<B>) + 1024);
         if (e != cudaSuccess) return e;
         configured[slot] = true;
     }
     // a CTA less per head or so keeps every run within one head
     const int per_head = p.sm_count / p.num_kv_heads;
     const int grid = 20 * per_head * p.num_kv_heads >= 19 * p.sm_count ? per_head * p.num_kv_heads : p.sm_count;
-    return launch_pdl(kcomp_stream_kernel<B>, dim3(grid), dim3(kStreamThreads), sizeof(StreamSmem) + 1024, stream, map_k, p);
+    return launch_pdl(kcomp_stream_kernel<B>, dim3(grid), dim3(StreamSize<B>::kThreads), sizeof(StreamSmem<B>) + 1024, stream, map_k, p);
 }
 }  // namespace
 

@@ -32,7 +32,8 @@ namespace seer {
 namespace {
 
 constexpr int kNW = 8;                                     // consumer warps; with the producer warp two CTAs per SM
-constexpr int kThreads = 32 * kNW + 32;
+template <bool SPREAD>
+constexpr int kThreads = 32 * (kNW + (SPREAD ? 2 : 1));    // uneven lists are dealt by a warp of its own
 constexpr int kStages = 3, kGroups = kNW / 4, kArrivals = kStages * kGroups;
 constexpr int kRows = kMaxGroup;
 
@@ -49,7 +50,7 @@ struct __align__(1024) ListSmem {
     uint64_t full[kArrivals], empty[kStages];
     // A stage, behind a piece, to put its partials together: given[piece % kStages].  (Pieces may be without a tile for a CTA; that
     // of three before has been put together when a stage is given.)
-    uint64_t got_parts[2], dealt, given[kStages];
+    uint64_t got_parts[2], given[kStages];
     int meta[kArrivals];                                   // tokens from the tile's first row on (blocks of 16 or 32 tokens: per block, 8 bits each)
     // uneven lists: how the tiles are dealt
     int rest[kListUnits + 1];                              // tiles above the line of the units before
@@ -59,6 +60,18 @@ struct __align__(1024) ListSmem {
 static_assert(sizeof(ListSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
 
 __device__ __forceinline__ void consumers_sync() { worker_sync<kNW>(); }
+// The deal is made: the dealing warp arrives for the consumer groups (barriers 2 and 3) and the producer (4), which wait for it.
+// (Barriers of the hardware, not mbarriers: the dealing warp waits for nothing, and a wait that could run out would leave its warp
+// with another idea of its pieces than the others.)
+__device__ __forceinline__ void deal_made() {
+    __syncwarp();
+    asm volatile("bar.arrive 2, 160;\n\tbar.arrive 3, 160;\n\tbar.arrive 4, 64;" ::: "memory");
+}
+__device__ __forceinline__ void await_deal(int group) {    // (group 2: the producer)
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + group), "r"(group < kGroups ? 160 : 64) : "memory");
+}
+static_assert(kNW == 8 && kGroups == 2, "five warps at each of barriers 2 and 3");
 __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n) : "memory");
 }
@@ -239,7 +252,6 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         }
         if (tid < 2) mbar_init(&sm.got_parts[tid], 1);
         if (tid == 0) {
-            mbar_init(&sm.dealt, 1);
             sm.line = 0x7fffffff;                          // (even lists)
             sm.helper = -1;
         }
@@ -318,11 +330,10 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
     using Later = std::false_type;
     if (producer) {
         if (p.next_early) pdl_launch_dependents();
-        // the deal is made (by a consumer warp); a helper's first piece is looked up at once
+        // a helper's first piece is looked up as soon as the deal is made
         int L2 = 0, n_blocks2 = 0;
         auto see_deal = [&]() {
-            if (!mbar_wait(&sm.dealt, 0, p.status)) dead = true;
-            __syncwarp();
+            await_deal(kGroups);
             take_share();
             if (pc.x < pc.end) {
                 const int u = place_of(sm.rest, p.clusters, pc.x), t = sm.line + pc.x - sm.rest[u] + (lane << s_shift) + rank;
@@ -466,6 +477,28 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         } while (next_piece());
         cluster_wait();                                    // (the barrier opened at the top)
         cluster_arrive_relaxed();
+    } else if (SPREAD && warp > kNW) {
+        // The deal, while the first tiles travel.  The units' tiles, a few units a lane:
+        constexpr int kCounts = (kListUnits + 31) / 32;
+        int n[kCounts], len[kCounts], total = 0, most = 0;
+#pragma unroll
+        for (int k = 0; k < kCounts; ++k) {                // (all loads on their way before the first is looked at)
+            const int v = min(lane + 32 * k, p.num_units - 1);
+            len[k] = p.seq_lens[sequence_of(v)];
+            n[k] = p.block_cnt ? p.block_cnt[v] : p.max_sel;
+        }
+#pragma unroll
+        for (int k = 0; k < kCounts; ++k) {
+            n[k] = lane + 32 * k < p.num_units ? tiles_of(len[k] > 0 ? max(0, min(n[k], p.max_sel)) : 0, len[k]) : 0;
+            total += n[k];
+            most = max(most, n[k]);
+        }
+        total = __reduce_add_sync(0xffffffffu, total);
+        most = __reduce_max_sync(0xffffffffu, most);
+        if (list_uneven(total, most, p.clusters, S)) deal(sm, n, p.clusters, S, cluster_id, total, most);
+        deal_made();
+        cluster_wait();                                    // (the barrier opened at the top)
+        cluster_arrive_relaxed();
     } else {
         const int group = warp >> 2, w4 = warp & 3, qd = lane & 3, rw = lane >> 2;
         // Q^T B-fragments: this thread supplies row rw of the unit's queries
@@ -486,42 +519,23 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         const int sub_w = !small ? 0 : p.block_size == 16 ? w4 : w4 >> 1;
         const int off_w = !small ? 16 * w4 : p.block_size == 16 ? 0 : (w4 & 1) * 16;
         constexpr int back[2] = {0, 0};
-        if (SPREAD && warp == 0) {
-            // The deal, while the first tiles travel.  The units' tiles, a few units a lane:
-            constexpr int kCounts = (kListUnits + 31) / 32;
-            int n[kCounts], len[kCounts], total = 0, most = 0;
-#pragma unroll
-            for (int k = 0; k < kCounts; ++k) {            // (all loads on their way before the first is looked at)
-                const int v = min(lane + 32 * k, p.num_units - 1);
-                len[k] = p.seq_lens[sequence_of(v)];
-                n[k] = p.block_cnt ? p.block_cnt[v] : p.max_sel;
-            }
-#pragma unroll
-            for (int k = 0; k < kCounts; ++k) {
-                n[k] = lane + 32 * k < p.num_units ? tiles_of(len[k] > 0 ? max(0, min(n[k], p.max_sel)) : 0, len[k]) : 0;
-                total += n[k];
-                most = max(most, n[k]);
-            }
-            total = __reduce_add_sync(0xffffffffu, total);
-            most = __reduce_max_sync(0xffffffffu, most);
-            if (list_uneven(total, most, p.clusters, S)) deal(sm, n, p.clusters, S, cluster_id, total, most);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.dealt);
-        }
-        if (SPREAD) {
-            mbar_wait(&sm.dealt, 0, p.status);             // (before the first tile is there)
-            __syncwarp();
-            take_share();
-        }
         // false: that was the last piece
         auto consume = [&](auto first_c) -> bool {
             constexpr bool FIRST = decltype(first_c)::value;
             const int tile0 = FIRST ? 0 : tiles_before, piece = FIRST ? 0 : pieces_before;
-            const int n_end = tile0 + mine_of();
+            int n_end = tile0 + mine_of();
             float o[8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
 #pragma unroll
             for (int a = 0; a < 8; ++a) o[a][0] = o[a][1] = o[a][2] = o[a][3] = 0.f;
-            for (int n = FIRST ? group : tile0 + ((tile0 ^ group) & 1); n < n_end; n += kGroups) {
+            bool dealt = !(SPREAD && FIRST);               // (a CTA's first tiles do not depend on the deal)
+            for (int n = FIRST ? group : tile0 + ((tile0 ^ group) & 1);; n += kGroups) {
+                if (!dealt && n >= min(n_end, kStages)) {
+                    await_deal(group);
+                    take_share();
+                    n_end = mine_of();
+                    dealt = true;
+                }
+                if (n >= n_end) break;
                 const int st = (n + piece) % kStages;
                 if (!dead && !mbar_wait(&sm.full[n % kArrivals], (n / kArrivals) & 1, p.status)) dead = true;
                 const int nvw = (small ? (sm.meta[n % kArrivals] >> (8 * sub_w)) & 0xff : sm.meta[n % kArrivals]) - off_w;   // valid tokens from this warp's first row on
@@ -698,21 +712,21 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
     cluster_wait();
 }
 
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads<false>, 2)
 list_step_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                          const __grid_constant__ DecodeParams p) {
     list_body<false>(map_k, map_v, p);
 }
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads<true>, 2)
 dealt_decode_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ DecodeParams p) {
     list_body<true>(map_k, map_v, p);
 }
 
-cudaLaunchConfig_t config_of(int S, int units, cudaStream_t stream, cudaLaunchAttribute (&attr)[2]) {
+cudaLaunchConfig_t config_of(bool spread, int S, int units, cudaStream_t stream, cudaLaunchAttribute (&attr)[2]) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, units);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(spread ? kThreads<true> : kThreads<false>);
     cfg.dynamicSmemBytes = sizeof(ListSmem) + 1024;
     cfg.stream = stream;
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -727,13 +741,13 @@ cudaLaunchConfig_t config_of(int S, int units, cudaStream_t stream, cudaLaunchAt
 }
 
 template <typename Kernel>
-int resident_of(Kernel* kernel, int k) {
+int resident_of(Kernel* kernel, bool spread, int k) {
     int n = 0;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ListSmem) + 1024);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) {
         cudaLaunchAttribute attr[2];
-        cudaLaunchConfig_t cfg = config_of(1 << k, 1, nullptr, attr);
+        cudaLaunchConfig_t cfg = config_of(spread, 1 << k, 1, nullptr, attr);
         cfg.numAttrs = 1;
         if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
     }
@@ -745,7 +759,7 @@ int resident_of(Kernel* kernel, int k) {
 int resident_lists(int k) {
     static int cached[kMaxDevices][5];                     // (value + 1; 0: not asked yet.  A race asks twice and stores the same)
     int& c = cached[current_device_slot()][k];
-    if (c == 0) c = min(resident_of(list_step_cluster_kernel, k), resident_of(dealt_decode_kernel, k)) + 1;
+    if (c == 0) c = min(resident_of(list_step_cluster_kernel, false, k), resident_of(dealt_decode_kernel, true, k)) + 1;
     return c - 1;
 }
 
@@ -789,7 +803,7 @@ size_t list_part_bytes(int units, int clusters, int S) {
 
 cudaError_t launch_lists(const CUtensorMap& map_k, const CUtensorMap& map_v, const DecodeParams& p, int S, cudaStream_t stream) {
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = config_of(S, p.clusters, stream, attr);
+    const cudaLaunchConfig_t cfg = config_of(p.spread, S, p.clusters, stream, attr);
     return cudaLaunchKernelEx(&cfg, p.spread ? dealt_decode_kernel : list_step_cluster_kernel, map_k, map_v, p);
 }
 

@@ -48,3 +48,14 @@ def test_weights_are_read_after_the_wait_for_the_kernel_before():
 def test_the_one_launch_step_reads_no_compressed_key_through_the_read_only_path():
     # it appends one in the same launch, and the next step starts under its end
     assert not re.search(r"__ldg\(\s*kc\b", _kernel("step_cluster_kernel"))
+
+
+def test_nothing_is_read_behind_a_wait_that_ran_out():
+    # what it stood for need not be there: numbers made of it are no indices.  (Tensor memory is given back all the same.)
+    for name, text in _sources().items():
+        for m in re.finditer(r"[;{})]\s*mbar_wait\(&sm\.([\w.]+)", text):
+            assert m.group(1).endswith("tmem_done"), (name, m.group(0))
+    # (the deal of uneven lists: behind a barrier of the hardware, whose warps all come)
+    text = _sources()["seer_lists.cu"]
+    shares = [m.start() for m in re.finditer(r"\btake_share\(\);", text)]
+    assert len(shares) == 2 and all(re.search(r"await_deal\(\w+\);\s*$", text[:at]) for at in shares)

@@ -66,12 +66,13 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status, u
 
 // Whether the lists are dealt.  In hundredths of a microsecond: a CTA that has the memory to itself gets through a tile in 0.46
 // us (three stages, of which one or two are being read); all CTAs together through one in 0.0047 us, taken as 0.004 because
-// the last ones are alone with their tiles; a deal costs 8 us: 2 to make it, 4 for the pieces' way through global memory, and
-// the helpers' second start.
-constexpr int kTileTime = 46, kPieceTiles = 8;             // (a piece costs a helper as much as so many tiles a CTA)
+// the last ones are alone with their tiles; a deal costs 5 us: the pieces' way through global memory and the helpers' second start.
+// (24 sequences, a quarter of them with 32 tiles a CTA, the others with 4: dealt 20.3 us, not dealt, as by a line of 8 us, 24.2; 10
+// sequences, lengths spread evenly up to 48 tiles a CTA: not dealt 34.1, dealt, as by a line of 3 us, 43.2.)
+constexpr int kTileTime = 46, kPieceTiles = 6;             // (a piece costs a helper as much as so many tiles a CTA; by 8, 17 -> 18 us)
 __device__ __forceinline__ bool list_uneven(int total, int most, int units, int S) {
-    // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S)) + 800, without its divisions)
-    return 5ll * kTileTime * most * units > max(2ll * total * S * units, 5ll * kTileTime * total) + 4000ll * S * units;
+    // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S)) + 500, without its divisions)
+    return 5ll * kTileTime * most * units > max(2ll * total * S * units, 5ll * kTileTime * total) + 2500ll * S * units;
 }
 // The same of a step's lists, as the sequences' lengths give them (whole warp).
 __device__ __forceinline__ bool step_uneven(const DecodeParams& p, int S) {

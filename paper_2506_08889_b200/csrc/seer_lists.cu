@@ -13,12 +13,15 @@
 //                  results, in global memory, by the CTAs that deliver the last one (rank r of the clusters has slice r of the
 //                  channels, so each slice is a matter of its own, with its own counter).  Where units are few and long there are
 //                  clusters without a unit of their own for it, as many as there is room for.
-// Every CTA comes to the same decision from the same numbers, so that nothing is waited for across clusters.
+// Every CTA comes to the same decision from the same numbers, so that nothing is waited for across clusters.  A warp of its own
+// decides while a unit's first tiles, which are never dealt, travel and are consumed.
 //
 // What bounds it: memory, from the first tiles (2.8 us after the kernel may read its inputs) to the last; 128 ragged lists of 13 to
-// 102 tiles (247 MB) take 44.8 us, 52.6 by the decode kernel, whose CTAs make a schedule first and publish their partial
-// results with a fence and a ticket each; 64 lists of 103 tiles (216 MB) 37.9 and 47.1.  A CTA by itself is bound by its three
-// stages, of which the consumers hold one or two: 0.46 us a tile.
+// 102 tiles (247 MB) take 44.5 us, 52.7 by the decode kernel, whose CTAs make a schedule first and publish their partial
+// results with a fence and a ticket each; 64 lists of 103 tiles (216 MB) 37.0 and 47.1.  A CTA by itself is bound by its three
+// stages, of which the consumers hold one or two: 0.46 us a tile.  Short uneven lists: the chain of two pieces.  24 sequences, one of
+// 32 tiles a CTA among ones of 4, by time stamps: deal seen 4.5 us, first pieces over 5 (long ones 9.4), their output 6.8,
+// second pieces over 9.7 to 10.5, their partials written 11 to 11.8, counted 12.1, put together 14.2.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -36,6 +39,8 @@ template <bool SPREAD>
 constexpr int kThreads = 32 * (kNW + (SPREAD ? 2 : 1));    // uneven lists are dealt by a warp of its own
 constexpr int kStages = 3, kGroups = kNW / 4, kArrivals = kStages * kGroups;
 constexpr int kRows = kMaxGroup;
+// A unit's first tiles, by the CTA, that are never dealt: a helper ends a piece's cost and half of it again below the line.
+constexpr int kOwnTiles = kPieceTiles + kPieceTiles / 2;
 
 struct __align__(1024) ListSmem {
     unsigned char ring[kStages * kStageBytes];
@@ -56,6 +61,7 @@ struct __align__(1024) ListSmem {
     int rest[kListUnits + 1];                              // tiles above the line of the units before
     int room[kListUnits + 1];                              // tiles that the helpers before take (on the way there: the units' tiles)
     int line, helpers, helper, is_last;                    // helper: number of this cluster among the helpers, or -1
+    int share[2], pieces[2];                               // the helper's share of the rest; first and last helper with a piece of a unit
 };
 static_assert(sizeof(ListSmem) + 1024 <= 113 * 1024, "two CTAs per SM");
 
@@ -170,49 +176,77 @@ __device__ __forceinline__ int place_of(const int* v, int n, int x) {
     return lo;
 }
 
-// The deal, by one warp, whose lane l has the tiles of clusters l, l + 32, ... in n[]: the lowest line at which the helpers have
-// room below it for what is above it.  (Every cluster has the first tiles of its own unit, which are asked for before the
-// deal.  Few tiles are not worth a piece: a unit that ends a little above the line keeps what is its, a cluster with little
-// room is no helper, and where a helper's share ends a few tiles from a unit's end it ends there.)
+// Where helper k's share of the rest begins.  Where that is a little before or behind a unit's end it is there: a helper with parts of
+// two units pays for two pieces.  Each unit's end takes the nearest share's only, so that no share becomes empty but the last.
+__device__ __forceinline__ int share_begin(const ListSmem& sm, int clusters, int k, int cost) {
+    const int x = sm.room[k];
+    if (k == 0 || k == sm.helpers || x >= sm.rest[clusters]) return x;
+    const int prev = sm.room[k - 1], next = sm.room[k + 1], u = place_of(sm.rest, clusters, x), r0 = sm.rest[u], r1 = sm.rest[u + 1];
+    const int back = r0 > prev && x - r0 <= r0 - prev ? x - r0 : cost, ahead = r1 < next && r1 - x < next - r1 ? r1 - x : cost;
+    return min(back, ahead) >= cost ? x : back <= ahead ? r0 : r1;
+}
+
+// The deal, by one warp, from the units' tiles in sm.room: the lowest line at which the helpers have room below it for what is
+// above it.  (Few tiles are not worth a piece: a unit that ends a little above the line keeps what is its, a cluster with little
+// room is no helper.)  A lane has the tiles of `per` clusters that follow one another, so that one scan over the lanes is enough: with
+// every 32nd, and shares' ends moved for all helpers, the deal of 192 units was seen at 6.4 us instead of 4.5.
 template <int COUNTS>
-__device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int clusters, int S, int cluster_id, int total, int most) {
-    const int lane = threadIdx.x & 31, cost = kPieceTiles * S, few = cost / 2;
+__device__ __forceinline__ void deal(ListSmem& sm, int clusters, int s_shift, int cluster_id, int total, int most) {
+    const int lane = threadIdx.x & 31, per = (clusters + 31) >> 5, v0 = lane * per, cost = kPieceTiles << s_shift, few = cost / 2;
     auto above = [&](int line, int t) { return t - line >= few ? t - line : 0; };
     auto below = [&](int line, int t) { return line - cost - t >= few ? line - cost - t : 0; };
-    int lo = max(total / clusters, kStages * S), hi = max(lo, most);      // (line `most`: nothing is above it)
+    int n[COUNTS];
+#pragma unroll
+    for (int k = 0; k < COUNTS; ++k) n[k] = k < per && v0 + k < clusters ? sm.room[v0 + k] : 0;
+    __syncwarp();
+    const int S1 = (1 << s_shift) - 1;
+    int lo = max((total / clusters + S1) >> s_shift, kOwnTiles), hi = max(lo, (most + S1) >> s_shift);      // (tiles a CTA; line `hi`: nothing is above it)
 #pragma unroll 1
     while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
+        const int mid = (lo + hi) >> 1, line = mid << s_shift;
         int free = 0;
 #pragma unroll
-        for (int k = 0; k < COUNTS; ++k)
-            if (lane + 32 * k < clusters) free += below(mid, n[k]) - above(mid, n[k]);
+        for (int k = 0; k < COUNTS; ++k) {
+            if (k >= per) break;
+            if (v0 + k < clusters) free += below(line, n[k]) - above(line, n[k]);
+        }
         if (__reduce_add_sync(0xffffffffu, free) >= 0) hi = mid;
         else lo = mid + 1;
     }
-    const int line = lo;
-    int rest = 0, room = 0, helpers = 0;
+    const int line = lo << s_shift;
+    int rest = 0, room = 0, helpers = 0;                   // this lane's, then all lanes' up to it
 #pragma unroll
     for (int k = 0; k < COUNTS; ++k) {
-        if (32 * k >= clusters) break;
-        const int v = lane + 32 * k;
-        const int over = v < clusters ? above(line, n[k]) : 0, mine = v < clusters ? below(line, n[k]) : 0;
-        int a = over, b = mine;
+        if (k >= per) break;
+        if (v0 + k >= clusters) break;
+        const int mine = below(line, n[k]);
+        rest += above(line, n[k]);
+        room += mine;
+        helpers += mine > 0;
+    }
+    int a = rest, b = room, c = helpers;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int ta = __shfl_up_sync(0xffffffffu, a, o), tb = __shfl_up_sync(0xffffffffu, b, o);
-            if (lane >= o) { a += ta; b += tb; }
-        }
-        const unsigned has = __ballot_sync(0xffffffffu, mine > 0);
-        if (v < clusters) sm.rest[v] = rest + a - over;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int ta = __shfl_up_sync(0xffffffffu, a, o), tb = __shfl_up_sync(0xffffffffu, b, o), tc = __shfl_up_sync(0xffffffffu, c, o);
+        if (lane >= o) { a += ta; b += tb; c += tc; }
+    }
+    int at = a - rest, to = b - room, helper = c - helpers;
+    rest = __shfl_sync(0xffffffffu, a, 31);
+    room = __shfl_sync(0xffffffffu, b, 31);
+    helpers = __shfl_sync(0xffffffffu, c, 31);
+#pragma unroll
+    for (int k = 0; k < COUNTS; ++k) {
+        if (k >= per) break;
+        const int v = v0 + k, mine = below(line, n[k]);
+        if (v >= clusters) break;
+        sm.rest[v] = at;
+        at += above(line, n[k]);
         if (mine > 0) {
-            const int at = helpers + __popc(has & ((1u << lane) - 1u));
-            sm.room[at] = room + b - mine;
-            if (v == cluster_id) sm.helper = at;
+            sm.room[helper] = to;
+            if (v == cluster_id) sm.helper = helper;
+            to += mine;
+            ++helper;
         }
-        helpers += __popc(has);
-        rest += __shfl_sync(0xffffffffu, a, 31);
-        room += __shfl_sync(0xffffffffu, b, 31);
     }
     if (lane == 0) {
         sm.rest[clusters] = rest;
@@ -221,13 +255,8 @@ __device__ __forceinline__ void deal(ListSmem& sm, const int (&n)[COUNTS], int c
         sm.line = line;
     }
     __syncwarp();
-    for (int k = lane; k < helpers; k += 32) {
-        const int x = sm.room[k];
-        if (x >= rest) break;
-        const int u = place_of(sm.rest, clusters, x), r0 = sm.rest[u], r1 = sm.rest[u + 1];
-        if (2 * (x - r0) < few) sm.room[k] = r0;
-        else if (2 * (r1 - x) < few) sm.room[k] = r1;
-    }
+    helper = sm.helper;
+    if (helper >= 0 && lane < 2) sm.share[lane] = min(share_begin(sm, clusters, helper + lane, cost), rest);
     __syncwarp();
 }
 
@@ -269,10 +298,10 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
     const bool small = !dense && p.blocks_per_tile > 1;
     auto sequence_of = [&](int u) { return p.kvh_magic ? (int)__umulhi((unsigned)u, p.kvh_magic) : u; };
     // a unit's listed blocks, and its tiles
+    auto listed = [&](int count, int L) -> int { return L > 0 ? max(0, min(count, p.max_sel)) : 0; };
     auto blocks_of = [&](int u, int L) -> int {
         if (dense) return 0;
-        const int cnt = p.block_cnt ? p.block_cnt[u] : p.max_sel;          // (not behind a test on L: both loads in flight)
-        return L > 0 ? max(0, min(cnt, p.max_sel)) : 0;
+        return listed(p.block_cnt ? p.block_cnt[u] : p.max_sel, L);        // (not behind a test on L: both loads in flight)
     };
     auto tiles_of = [&](int n_blocks, int L) -> int {
         if (dense) return L > 0 ? min((L + kTileTokens - 1) / kTileTokens, p.max_blocks_cap) : 0;
@@ -306,8 +335,8 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
     auto take_share = [&]() {
         if (sm.line < 0x7fffffff && sm.rest[cluster_id + 1] > sm.rest[cluster_id]) pc.b = sm.line;
         if (sm.helper >= 0) {
-            pc.x = sm.room[sm.helper];
-            pc.end = min(sm.room[sm.helper + 1], sm.rest[p.clusters]);
+            pc.x = sm.share[0];
+            pc.end = sm.share[1];
         }
     };
     // on to the next piece; false: that was the last
@@ -331,14 +360,14 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
     if (producer) {
         if (p.next_early) pdl_launch_dependents();
         // a helper's first piece is looked up as soon as the deal is made
-        int L2 = 0, n_blocks2 = 0;
+        int L2 = 0, count2 = 0;
         auto see_deal = [&]() {
             await_deal(kGroups);
             take_share();
             if (pc.x < pc.end) {
                 const int u = place_of(sm.rest, p.clusters, pc.x), t = sm.line + pc.x - sm.rest[u] + (lane << s_shift) + rank;
                 L2 = p.seq_lens[sequence_of(u)];
-                n_blocks2 = blocks_of(u, L2);
+                if (!dense) count2 = p.block_cnt ? p.block_cnt[u] : p.max_sel;
                 if (!dense) {
 #pragma unroll
                     for (int x = 0; x < 4; ++x) {
@@ -353,7 +382,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
             if (SPREAD && piece > 0) {
                 const bool first = piece == 1;
                 L = first ? L2 : p.seq_lens[sequence_of(pc.u)];
-                n_blocks = first ? n_blocks2 : blocks_of(pc.u, L);
+                n_blocks = first ? listed(count2, L) : blocks_of(pc.u, L);
 #pragma unroll
                 for (int x = 0; x < 4; ++x) entry[x] = entry2[x];
             }
@@ -365,7 +394,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
             // (a CTA's first tiles do not depend on the deal)
             const bool own = SPREAD && piece == 0;
             for (int base = 0, count; base < n_local; base += count) {
-                count = !own || base > kStages ? 32 : base == 0 ? kStages : 32 - kStages;
+                count = !own || base > kOwnTiles ? 32 : base == 0 ? kOwnTiles : 32 - kOwnTiles;
                 const int it = base + lane;
                 int row[4] = {0, 0, 0, 0}, outer[4] = {0, 0, 0, 0}, nv_all = 0, n_sub = 0;
                 if (it < n_local) {
@@ -459,7 +488,7 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
                     see_deal();
                     n_local = mine_of();
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) entry[x] = __shfl_down_sync(0xffffffffu, entry[x], kStages);
+                    for (int x = 0; x < 4; ++x) entry[x] = __shfl_down_sync(0xffffffffu, entry[x], kOwnTiles);
                 }
             }
             if (!SPREAD) break;
@@ -478,24 +507,30 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         cluster_wait();                                    // (the barrier opened at the top)
         cluster_arrive_relaxed();
     } else if (SPREAD && warp > kNW) {
-        // The deal, while the first tiles travel.  The units' tiles, a few units a lane:
+        // The deal, while the first tiles travel.  The units' tiles (read by neighbouring lanes from neighbouring places: the lanes'
+        // own runs of them cost even lists 0.4 us):
         constexpr int kCounts = (kListUnits + 31) / 32;
         int n[kCounts], len[kCounts], total = 0, most = 0;
 #pragma unroll
         for (int k = 0; k < kCounts; ++k) {                // (all loads on their way before the first is looked at)
+            if (32 * k >= p.clusters) break;
             const int v = min(lane + 32 * k, p.num_units - 1);
             len[k] = p.seq_lens[sequence_of(v)];
             n[k] = p.block_cnt ? p.block_cnt[v] : p.max_sel;
         }
 #pragma unroll
         for (int k = 0; k < kCounts; ++k) {
-            n[k] = lane + 32 * k < p.num_units ? tiles_of(len[k] > 0 ? max(0, min(n[k], p.max_sel)) : 0, len[k]) : 0;
+            const int v = lane + 32 * k;
+            if (32 * k >= p.clusters) break;
+            n[k] = v < p.num_units ? tiles_of(listed(n[k], len[k]), len[k]) : 0;
             total += n[k];
             most = max(most, n[k]);
+            if (v < p.clusters) sm.room[v] = n[k];
         }
+        __syncwarp();
         total = __reduce_add_sync(0xffffffffu, total);
         most = __reduce_max_sync(0xffffffffu, most);
-        if (list_uneven(total, most, p.clusters, S)) deal(sm, n, p.clusters, S, cluster_id, total, most);
+        if (list_uneven(total, most, p.clusters, S)) deal<kCounts>(sm, p.clusters, s_shift, cluster_id, total, most);
         deal_made();
         cluster_wait();                                    // (the barrier opened at the top)
         cluster_arrive_relaxed();
@@ -524,18 +559,20 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
             constexpr bool FIRST = decltype(first_c)::value;
             const int tile0 = FIRST ? 0 : tiles_before, piece = FIRST ? 0 : pieces_before;
             int n_end = tile0 + mine_of();
-            float o[8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+float o[8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
 #pragma unroll
             for (int a = 0; a < 8; ++a) o[a][0] = o[a][1] = o[a][2] = o[a][3] = 0.f;
             bool dealt = !(SPREAD && FIRST);               // (a CTA's first tiles do not depend on the deal)
+            int stop = dealt ? n_end : min(n_end, kOwnTiles);
             for (int n = FIRST ? group : tile0 + ((tile0 ^ group) & 1);; n += kGroups) {
-                if (!dealt && n >= min(n_end, kStages)) {
+                if (n >= stop) {
+                    if (dealt) break;
                     await_deal(group);
                     take_share();
-                    n_end = mine_of();
+                    stop = n_end = mine_of();
                     dealt = true;
+                    if (n >= stop) break;
                 }
-                if (n >= n_end) break;
                 const int st = (n + piece) % kStages;
                 if (!dead && !mbar_wait(&sm.full[n % kArrivals], (n / kArrivals) & 1, p.status)) dead = true;
                 const int nvw = (small ? (sm.meta[n % kArrivals] >> (8 * sub_w)) & 0xff : sm.meta[n % kArrivals]) - off_w;   // valid tokens from this warp's first row on
@@ -653,33 +690,45 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
                 }
             }
             if (!whole) {
-                // the helpers that have a piece of the unit; whoever counts the last puts the pieces together, in order
-                const int k_lo = place_of(sm.room, sm.helpers, sm.rest[done.u]), k_hi = place_of(sm.room, sm.helpers, sm.rest[done.u + 1] - 1);
+                // whoever counts the unit's last tiles puts its pieces together, in order
                 int* count = reinterpret_cast<int*>(p.tickets) + done.u * kMaxS + rank;
-                __threadfence();
                 consumers_sync();
-                if (tid == 0) sm.is_last = atomicAdd(count, 1) == k_hi - k_lo + 1;
+                if (tid == 32) {                           // (behind the barrier: its release and acquire are all threads')
+                    int before;
+                    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;" : "=r"(before) : "l"(count), "r"(done.b - done.a) : "memory");
+                    sm.is_last = before + done.b - done.a == done.n;
+                } else if (warp == 0) {                    // the helpers that have a piece of the unit
+                    const int r0 = sm.rest[done.u], r1 = sm.rest[done.u + 1], at = place_of(sm.room, sm.helpers, lane == 0 ? r0 : r1 - 1);
+                    const int begin = share_begin(sm, p.clusters, lane == 0 ? at + 1 : at, kPieceTiles << s_shift);
+                    if (lane < 2) sm.pieces[lane] = lane == 0 ? at + (begin <= r0) : at - (begin >= r1);
+                }
                 consumers_sync();
                 if (sm.is_last) {
-                    __threadfence();
                     if (tid == 0) *count = 0;              // (as every launch finds it)
+                    const int k_lo = sm.pieces[0], count_k = sm.pieces[1] - k_lo + 1;
 #pragma unroll 1
                     for (int x = tid; x < pairs; x += 32 * kNW) {
                         const int r = x >> (c_shift - 1), c = 2 * (x & ((slice >> 1) - 1));
                         float M = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f;
+                        // piece -1: the owner's
+                        const float* const first = part_of(done.u);
+                        const float* const others = part_of(p.num_units + k_lo + done.u);
+                        const int at_ml = 2 * r, at_v = 2 * kRows + (r << c_shift) + c, step = S * part_stride;
 #pragma unroll 1
-                        for (int k0 = k_lo - 1; k0 <= k_hi; k0 += 4) {
-                            float2 ml[4], v[4];            // (four pieces' numbers on their way at a time)
+                        for (int k0 = -1; k0 < count_k; k0 += 4) {
+                            float2 ml[4], v[4];        // (so many pieces' numbers on their way at a time)
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
-                                const int k = k0 + e;
-                                const float* src = part_of(k < k_lo ? done.u : p.num_units + min(k, k_hi) + done.u);
-                                ml[e] = k <= k_hi ? __ldcg(reinterpret_cast<const float2*>(src + 2 * r)) : make_float2(-INFINITY, 0.f);
-                                v[e] = k <= k_hi ? __ldcg(reinterpret_cast<const float2*>(src + 2 * kRows + (r << c_shift) + c)) : make_float2(0.f, 0.f);
+                                const float* src = k0 + e < 0 ? first : others + min(k0 + e, count_k - 1) * step;
+                                ml[e] = __ldcg(reinterpret_cast<const float2*>(src + at_ml));
+                                v[e] = __ldcg(reinterpret_cast<const float2*>(src + at_v));
                             }
                             float m = M;
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) m = fmaxf(m, ml[e].x);
+                            for (int e = 0; e < 4; ++e) {
+                                if (k0 + e >= count_k) ml[e].x = -INFINITY;
+                                m = fmaxf(m, ml[e].x);
+                            }
                             const float mb = m == -INFINITY ? 0.f : m, f = fast_exp2(M - mb);
                             M = m;
                             l *= f;
@@ -768,13 +817,15 @@ int resident_lists(int k) {
 // As many CTAs per unit as keep every cluster resident at once and still have something to do each.  Above 128 tiles a CTA the
 // decode kernel, whose CTAs share all tiles throughout, is ahead where lists are ragged.  us a call, decode kernel -> clusters, 8
 // KV heads; all lists equally long / lengths spread evenly from an eighth on / one sequence's lists eight times the others':
-//     32 tiles a CTA      16 sequences (S = 2)  54.0 -> 43 / 40.8 -> 30.8 / 21.3 -> 20.4      24 (S = 1)  - / 39.3 -> 28.2 / 14.7 -> 19.1
-//                          8 sequences (S = 4)  47.0 -> 37.5 / 39.4 -> 31.8 / 24.8 -> 23.1    10 (S = 2)  - / 31.1 -> 24.6 / 16.5 -> 18.8
-//     48                  16 sequences          75.1 -> 64 / 50.8 -> 42.8 / 26.8 -> 26.5       8          73.8 -> 64.0 / 50.8 -> 44.4 / 32.4 -> 28.0
-//     128, dense           8 sequences           164 -> 154 / 105 -> 103
+//     32 tiles a CTA      16 sequences (S = 2)  56.2 -> 45.8 / 39.8 -> 30.9 / 18.7 -> 15.5      24 (S = 1)  51.6 -> 35.8 / 39.1 -> 27.1 / 13.8 -> 15.1
+//                          8 sequences (S = 4)  54.4 -> 45.1 / 38.8 -> 30.5 / 24.4 -> 19.1      10 (S = 2)  40.9 -> 31.3 / 30.5 -> 24.6 / 14.9 -> 13.8
+//     48                  16 sequences          74.5 -> 64.0 / 50.1 -> 43.0 / 25.9 -> 21.3       8, dense   70.8 -> 62.5 / 47.7 -> 41.7 / 31.1 -> 22.9
+//     96, dense           10 sequences (S = 2)  85.3 -> 77.1 / 55.9 -> 58.0 / 32.1 -> 26.6       4 (S = 8)  90.9 -> 83.0 / 59.1 -> 52.4 / 43.8 -> 34.8
+//     128, dense           8 sequences           164 -> 155 / 101 -> 101 / 51.5 -> 46.0
 //     192, dense           8 sequences           241 -> 228 / 147 -> 151
 //     256, dense           8 sequences           313 -> 305 / 193 -> 201
-// (One long sequence among short ones: as clusters without a deal 64 instead of 39 us where its lists have 102 tiles a CTA.)
+// One long sequence among nearly empty ones: 32 tiles a CTA 16.3 -> 14.6 (24 sequences), 15.7 -> 13.9 (16), 16.8 -> 14.4 (8); 48
+// 15.5 -> 15.9 (16); 64 15.3 -> 16.3 (24).  (A deal of 8 us, that all of a CTA's tiles but three waited for, lost up to 30 % there.)
 // Where half of the clusters that fit would do, and a list may have more than 32 tiles a CTA, all that fit are launched, and the long
 // units dealt to those without one (a CTA by itself is far from what the memory gives): dense, one KV head of 128k 54.9 (decode
 // kernel) -> 24.4, two of 55k and 156k 48.9 -> 29.6, lists of 615 tiles 21.5 -> 15.8; with 25 tiles a CTA or less nothing is gained.

@@ -1,5 +1,6 @@
-"""Given lists and dense calls whose lists are so uneven that the clusters share all tiles instead of taking a unit each:
-units cut anywhere, units without a tile, runs of many units, every cluster size, against the oracle."""
+"""Given lists and dense calls whose lists are so uneven that what long units have above a line is dealt to the clusters that end
+before it: units cut anywhere, units without a tile, shares of several units, units of many shares, every cluster size, against
+the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -20,7 +21,9 @@ CASES = [
     (8, 2, 16, 64, [9000] * 2 + [50 * x + 1 for x in range(18)], [500, 411] + [x % 9 for x in range(18)]),             # 40 units, four blocks a tile
     (4, 1, 64, 0, [70001], None),                                                                                     # one unit, all other clusters without
     (8, 2, 32, 64, [60000, 300], [1800, 5]),                                                                          # 4 units, two of them long
-    (8, 1, 64, 0, [20000, 0, 0, 0, 19000, 63, 64, 65, 0, 128], None),                                                  # runs that begin behind empty units
+    (8, 1, 64, 0, [55000, 0, 0, 0, 52000, 63, 64, 65, 0, 128], None),                                                  # shares that begin behind empty units
+    (16, 8, 64, 0, [4096 - 7 if x % 11 == 3 else 60 for x in range(24)], None),                                        # 192 units, 24 of them of many shares
+    (16, 8, 64, 0, [64 * (2 + 3 * x) if x % 7 else 6000 + 64 * x for x in range(18)], None),                           # shares that end near units' ends
 ]
 
 
@@ -62,3 +65,31 @@ def test_uneven_lists(ctx, case):
         if ctx.one_launch:                                  # the pieces are put together in a fixed order
             assert torch.equal(out, outs[0][0]) and torch.equal(lse, outs[0][1])
     assert ctx.device_status() == binding.SEER_OK
+
+
+@pytest.mark.parametrize("batch,tiles", [(24, 64), (16, 96)])
+def test_one_long_list_among_short_ones_costs_no_more_than_without_clusters(monkeypatch, batch, tiles):
+    # (dealt at 8 us a deal it took 1.3 and 1.25 times as long; host-bound runs make both alike)
+    Hq, Hkv, d, cap = 32, 8, 128, 64 * tiles
+    lens = torch.as_tensor(np.array([cap if i == batch // 2 else 64 for i in range(batch)], np.int32), device=DEV)
+    q, k, v = (torch.randn(s, device=DEV, dtype=torch.bfloat16) for s in ((batch, Hq, d), (batch, Hkv, cap, d), (batch, Hkv, cap, d)))
+    out, lse = torch.empty_like(q), torch.empty((batch, Hq), device=DEV)
+    shape, kv = binding.make_shape(batch, Hq, Hkv, d, 64, SCALE), binding.make_kv(k, v, lens)
+    ctxs = []
+    for clusters in ("1", "0"):
+        monkeypatch.setenv("SEER_STEP_CLUSTERS", clusters)
+        ctxs.append(binding.Context(0))
+    times = [[], []]
+    for _ in range(9):
+        for c, t in zip(ctxs, times):
+            a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            for i in range(60):
+                if i == 10:
+                    a.record()
+                c.seer_dense_decode(shape, kv, q, out, lse)
+            z.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(z))
+    for c in ctxs:
+        c.close()
+    assert np.median(times[0]) <= 1.17 * np.median(times[1]), times

@@ -69,10 +69,13 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status, u
 // the last ones are alone with their tiles; a deal costs 5 us: the pieces' way through global memory and the helpers' second start.
 // (24 sequences, a quarter of them with 32 tiles a CTA, the others with 4: dealt 20.3 us, not dealt, as by a line of 8 us, 24.2; 10
 // sequences, lengths spread evenly up to 48 tiles a CTA: not dealt 34.1, dealt, as by a line of 3 us, 43.2.)
-constexpr int kTileTime = 46, kPieceTiles = 6;             // (a piece costs a helper as much as so many tiles a CTA; by 8, 17 -> 18 us)
-__device__ __forceinline__ bool list_uneven(int total, int most, int units, int S) {
-    // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S)) + 500, without its divisions)
-    return 5ll * kTileTime * most * units > max(2ll * total * S * units, 5ll * kTileTime * total) + 2500ll * S * units;
+// A step's lists are dealt by a kernel behind it: 8 us (10 sequences, half of them with 72 tiles a CTA, the others with 9: not dealt
+// 62.2, dealt, as by a line of 5 us, 68.6; 8, a quarter with 80: dealt 59.3, not dealt, as by one of 11 us, 70.6).
+constexpr int kTileTime = 46, kDealTime = 500, kStepDealTime = 800;
+constexpr int kPieceTiles = 6;                             // a piece costs a helper as much as so many tiles a CTA (by 8, lists of 17 us 18)
+__device__ __forceinline__ bool list_uneven(int total, int most, int units, int S, int deal = kDealTime) {
+    // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S)) + deal, without its divisions)
+    return 5ll * kTileTime * most * units > max(2ll * total * S * units, 5ll * kTileTime * total) + 5ll * deal * S * units;
 }
 // The same of a step's lists, as the sequences' lengths give them (whole warp).
 __device__ __forceinline__ bool step_uneven(const DecodeParams& p, int S) {
@@ -83,7 +86,7 @@ __device__ __forceinline__ bool step_uneven(const DecodeParams& p, int S) {
         total += tiles;
         most = max(most, tiles);
     }
-    return list_uneven(__reduce_add_sync(0xffffffffu, total) * p.num_kv_heads, __reduce_max_sync(0xffffffffu, most), p.num_units, S);
+    return list_uneven(__reduce_add_sync(0xffffffffu, total) * p.num_kv_heads, __reduce_max_sync(0xffffffffu, most), p.num_units, S, kStepDealTime);
 }
 
 }  // namespace seer

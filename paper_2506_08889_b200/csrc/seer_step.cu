@@ -1576,13 +1576,19 @@ int resident_clusters(bool wide, int k) {
 // Given lists and dense calls of several query tokens, whose lengths follow the sequences', keep to where one long sequence
 // does not lose much: 16 + 2 S tiles a CTA (a decode call pays for its parts whatever its size, and more the longer its
 // longest unit is; lists of one query token are dealt: seer_lists.cu).  The lists of a step are all as long as the budget but for
-// sequences shorter than that: one launch up to 64 tiles a CTA, where all but the most uneven batches gain (80 units in 160
-// CTAs, twelve SMs with two of them: 48 tiles a CTA 78.6 -> 61.6, two query tokens 79.6 -> 64.7).  From there to 128 tiles
-// (line_spread: one query token) it is the sequences' lengths that decide, in the kernels: even lists are done in the one
-// launch, uneven ones by the list kernel behind it, which costs 5 us where it has nothing to do.  Chain -> two launches, all
-// lists long / lengths spread from 1/32 on / one of 410 tiles a unit among short ones:
-//     80 tiles a CTA, 8 sequences   129 -> 123 / 124 -> 111 / 79 -> 64        96, 10 sequences   114 -> 104 / 112 -> 94
-//     96, 16 sequences              150 -> 142 / 140 -> 125                   97, 10 sequences, blocks of 32   129 -> 104
+// sequences shorter than that: one launch up to 64 tiles a CTA, where all but the most uneven batches gain.  So do 80 units in
+// 160 CTAs, although twelve SMs have two of them; chain -> one launch, lists all long / spread evenly from an eighth on / half of the
+// sequences' long, the others an eighth / a quarter long / one / one among nearly empty ones:
+//     48 tiles a CTA    69.5 -> 53.8 / 62.8 -> 45.7 / 52.5 -> 42.4 / 40.4 -> 38.7 / 34.0 -> 37.4 / 27.6 -> 34.5
+//     64                81.9 -> 65.6 / 69.8 -> 54.5 / 62.1 -> 50.7 / 46.5 -> 46.6 / 39.8 -> 46.0 / 33.1 -> 43.3
+//     48, two tokens    72.8 -> 55.5 / 65.7 -> 47.7 / 54.5 -> 44.5 / 41.4 -> 40.3 / 36.2 -> 39.1 / 27.7 -> 36.0
+// (The list kernel behind them as well, from 32 tiles a CTA on: 59.9 / 51.4 / 48.8 / 40.8 / 37.1 / 29.4 for 48, 71.8 / 60.1 / 60.2 / 48.3 /
+// 43.1 / 32.7 for 64: six microseconds for all, for a gain in the last two.)  From there to 128 tiles (line_spread: one query
+// token) it is the sequences' lengths that decide, in the kernels: even lists are done in the one launch, uneven ones by the list
+// kernel behind it, which costs 5 us where it has nothing to do.  Chain -> two launches:
+//     80, 8 sequences   124 -> 115 / 99.2 -> 88.0 / 88.2 -> 77.4 / 67.3 -> 59.3 / 53.3 -> 51.6 / 47.2 -> 41.1
+//     96, 10 sequences  102 -> 96.7 / 86.4 -> 82.4 / 74.9 -> 73.2 / 54.3 -> 59.2 / 46.9 -> 49.1 / 38.2 -> 37.5
+//     96, 16 sequences  146 -> 138 / 122 -> 111 / 98.9 -> 92.1 / 75.8 -> 75.6 / 55.7 -> 55.8 / 42.3 -> 39.4
 // 149 to 296 units, a CTA each, gain like fewer: steps of 24 / 30 / 36 sequences, all long, 16 tiles a CTA 45.9 -> 33.8, 52.7 ->
 // 39.1, 59.3 -> 43.1; 64 tiles 93.5 -> 82.1, 108 -> 96, 127 -> 109.
 static StepPlan plan_of(bool wide, int units, int rows, long long max_tiles, long long max_codes, int max_keys, bool line_spread = false) {

@@ -1,5 +1,6 @@
 """Steps of more than 64 and up to 128 tiles a CTA: two launches, of which the first does even lists and the second, where they
-are uneven, the attention; batches on both sides of that line, a block that has just filled among them, against the oracle."""
+are uneven, the attention; batches on both sides of that line, a block that has just filled among them, every width of the gate,
+the one launch of a single sequence and the chain of blocks of 16 tokens, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -12,19 +13,35 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 SCALE, THETA = 0.0884, 1.0e6
 
+EVEN, UNEVEN = [5120 - 64 * (x % 5) - 7 * (x % 3) for x in range(25)], [640] * 12 + [5120] + [64 * x for x in range(12)]
 CASES = [
-    # Hq, Hkv, b, page, cached tokens, budget in blocks
-    (32, 8, 64, 0, [5120 - 64 * (x % 5) - 7 * (x % 3) for x in range(25)], 72),                 # 200 units, a CTA each, even
-    (16, 8, 64, 0, [640] * 12 + [5120] + [64 * x for x in range(12)], 72),                      # one long sequence, an empty one
-    (40, 8, 32, 64, [10432, 10048] + [128 + 32 * x for x in range(8)], 300),                    # 80 units, clusters of 2, two long
-    (8, 2, 128, 0, [16384 + 128 * x for x in range(40)], 100),                                  # 80 units, two tiles a block, even
+    # Hq, Hkv, b, page, cached tokens, budget in blocks, d_gate, launches, lists uneven (tiles a CTA by 0.46 us above what all take and 8 us)
+    (32, 8, 64, 0, EVEN, 72, 128, 2, False),                                                                       # 200 units, a CTA each
+    (16, 8, 64, 0, UNEVEN, 72, 128, 2, True),                                                                      # one long sequence, an empty one
+    (40, 8, 32, 64, [10432, 10048] + [128 + 32 * x for x in range(8)], 300, 128, 2, True),                         # 80 units, clusters of 2, two long
+    (8, 2, 128, 0, [16384 + 128 * x for x in range(40)], 100, 128, 2, False),                                      # 80 units, two tiles a block
+    (16, 8, 64, 0, EVEN, 72, 256, 2, False),
+    (16, 8, 32, 0, UNEVEN, 144, 256, 2, True),
+    (16, 8, 32, 64, EVEN, 150, 64, 2, False),
+    (8, 8, 64, 0, UNEVEN, 75, 64, 2, True),
+    (16, 8, 64, 0, [70400 - 5], 1030, 128, 1, False),                                                              # one sequence: its heads' lists are as long
+    (16, 8, 16, 0, EVEN, 280, 128, 3, False),                                                                      # more numbers than a CTA holds
 ]
+
+
+def _uneven(lens, b, budget, Hkv, S):
+    """The rule that both launches go by."""
+    tiles = [min(-(-L // b), budget) * b / 64 if b >= 64 else -(-min(-(-L // b), budget) * b // 64) for L in lens]
+    total, most, units = sum(tiles) * Hkv, max(tiles), len(lens) * Hkv
+    return 0.46 * most / S > max(0.004 * total, 0.46 * total / (units * S)) + 8
 
 
 @pytest.mark.parametrize("case", range(len(CASES)))
 def test_step_of_long_lists(ctx, case):
-    Hq, Hkv, b, page, lens, budget = CASES[case]
-    B, d, dg, seed = len(lens), 128, 128, 700 + case
+    Hq, Hkv, b, page, lens, budget, dg, want_launches, uneven = CASES[case]
+    B, d, seed = len(lens), 128, 700 + case
+    if want_launches == 2:
+        assert _uneven(lens, b, budget, Hkv, 1 if B * Hkv > 148 else 2) == uneven
     unit = max(page, b, 64)
     cap = -(-max(lens) // unit) * unit
     nb = cap // b
@@ -63,7 +80,7 @@ def test_step_of_long_lists(ctx, case):
         ctx.seer_decode_step(shape, kv, gate, q, qn, window, budget * b, idx, cnt, budget, out, lse, rows_block_local=True)
         launches = ctx.launch_count() - before
     torch.cuda.synchronize()
-    assert launches == (2 if ctx.one_launch else 3)
+    assert launches == (want_launches if ctx.one_launch else 3)
     assert np.array_equal(cnt.cpu().numpy(), want_cnt) and np.array_equal(idx.cpu().numpy(), want_idx)
     assert torch.equal(got_kc, want_kc)
     check_attention(out, lse, *ref, what=f"case {case}")

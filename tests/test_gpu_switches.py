@@ -1,8 +1,9 @@
-"""Which kernels a call takes: short calls are one launch of the cluster kernel up to its lines, and never where a switch of the
-environment is set that chooses among the other kernels.  The kernels' names come from the profiler's activity records; a
-process of its own takes them, all at once (this file run as a program)."""
+"""Which kernels a call takes: clusters up to their lines, one launch or two, and never where a switch of the environment is set
+that chooses among the other kernels.  The kernels' names come from the profiler's activity records; a process of its own takes
+them, all at once (this file run as a program)."""
 import json
 import os
+import re
 import subprocess
 import sys
 
@@ -34,12 +35,25 @@ SETTINGS = [                              # a switch, its value, the calls that 
     ("SEER_DECODE_POOL_DIV", "0", ATTENTION),
     ("SEER_DECODE_MIN_TILES", "4", ATTENTION),
 ]
-LINES = [                                 # a call, its sequences, the tiles of its one long list, whether clusters take it
-    # two hundred units of one CTA each: 18 tiles a CTA for lists and dense calls, 64 for a step
-    ("sparse", 25, 18, True), ("sparse", 25, 19, False), ("dense", 25, 18, True), ("dense", 25, 19, False),
-    ("step", 25, 64, True), ("step", 25, 65, False),
-    # sixty-four units of four CTAs: 24
-    ("sparse", 8, 96, True), ("sparse", 8, 97, False),
+EVEN, DEALT, DECODE, STEP, GATE = "list_step_cluster_kernel", "dealt_decode_kernel", "decode_kernel", "step_cluster_kernel", "gate_cluster_kernel"
+SMALL_WS = 3_600_000                      # bytes: the decode kernel's partials of 200 units, not the dealt lists'
+LINES = [                                 # a call, its sequences, the tiles of its one long list, its kernels (, block, workspace)
+    # two hundred units of one CTA each: above 18 tiles lists may be dealt, above 128 the decode kernel; a step is one launch up
+    # to 64, and from there to 128 the dealing kernel follows
+    ("sparse", 25, 18, [EVEN]), ("sparse", 25, 19, [DEALT]), ("dense", 25, 18, [EVEN]), ("dense", 25, 19, [DEALT]),
+    ("dense", 25, 128, [DEALT]), ("dense", 25, 129, [DECODE]),
+    ("step", 25, 64, [STEP]), ("step", 25, 65, [STEP, DEALT]), ("step", 25, 128, [STEP, DEALT]), ("step", 25, 129, [GATE, DECODE]),
+    # 304 units: more than there are places
+    ("sparse", 38, 4, [DECODE]), ("dense", 38, 4, [DECODE]),
+    # sixty-four units of four CTAs
+    ("sparse", 8, 96, [EVEN]), ("sparse", 8, 97, [DEALT]), ("dense", 8, 512, [DEALT]), ("dense", 8, 513, [DECODE]),
+    # eight of sixteen: up to 32 tiles a CTA a cluster per unit; the heads of one sequence have lists as long, which are not dealt
+    ("dense", 1, 512, [EVEN]), ("dense", 1, 769, [DEALT]),
+    ("step", 1, 1024, [STEP]), ("step", 1, 1025, [STEP]), ("step", 1, 2049, [GATE, DECODE]),
+    # blocks of 16 tokens: 256 numbers a CTA
+    ("step", 25, 64, [STEP], 16), ("step", 25, 65, [GATE, DECODE], 16),
+    # partial results that do not fit
+    ("sparse", 25, 18, [EVEN], 64, SMALL_WS), ("sparse", 25, 19, [DECODE], 64, SMALL_WS), ("step", 25, 65, [GATE, DECODE], 64, SMALL_WS),
 ]
 
 
@@ -67,24 +81,25 @@ def _switch_calls(c):
     }
 
 
-def _line_call(c, kind, B, tiles):
+def _line_call(c, kind, B, tiles, b=64):
     """One long sequence among short ones, every block listed: the call, and its output to be checked."""
-    Hq, Hkv, d, dg, b = 16, 8, 128, 64, 64
-    S = tiles * b
+    Hq, Hkv, d, dg = 16, 8, 128, 64
+    S = tiles * 64
+    blocks = S // b
     lens = np.array([S - 5] + [(64, 1, 200, 0)[i % 4] for i in range(B - 1)], np.int32)
     q, k, v = make_qkv(B, Hq, Hkv, S, d, 32, DEV)
     wq = synth.normal_bf16((Hkv, dg, Hq // Hkv * d), 32, "wq", DEV, std=0.02)
-    kc = synth.normal_bf16((B, Hkv, tiles, dg), 32, "kc", DEV)
+    kc = synth.normal_bf16((B, Hkv, blocks, dg), 32, "kc", DEV)
     lens_t = torch.as_tensor(lens, device=DEV)
-    shape, gate, kv = binding.make_shape(B, Hq, Hkv, d, b, 0.1), binding.make_gate(dg, 1.0e6, wq, None, kc, tiles), binding.make_kv(k, v, lens_t)
+    shape, gate, kv = binding.make_shape(B, Hq, Hkv, d, b, 0.1), binding.make_gate(dg, 1.0e6, wq, None, kc, blocks), binding.make_kv(k, v, lens_t)
     n = -(-lens // b)
-    idx = torch.as_tensor(np.where(np.arange(tiles) < n[:, None, None], np.arange(tiles), -1).astype(np.int32).repeat(Hkv, 1), device=DEV)
+    idx = torch.as_tensor(np.where(np.arange(blocks) < n[:, None, None], np.arange(blocks), -1).astype(np.int32).repeat(Hkv, 1), device=DEV)
     cnt = torch.as_tensor(n.astype(np.int32)[:, None].repeat(Hkv, 1), device=DEV)
     out = torch.full((B, Hq, d), float("nan"), dtype=torch.bfloat16, device=DEV)
     lse = torch.full((B, Hq), float("nan"), dtype=torch.float32, device=DEV)
-    call = {"sparse": lambda: c.seer_sparse_decode(shape, kv, q, idx, cnt, tiles, out, lse),
+    call = {"sparse": lambda: c.seer_sparse_decode(shape, kv, q, idx, cnt, blocks, out, lse),
             "dense": lambda: c.seer_dense_decode(shape, kv, q, out, lse),
-            "step": lambda: c.seer_decode_step(shape, kv, gate, q, q, None, tiles * b, idx, cnt, tiles, out, lse)}[kind]
+            "step": lambda: c.seer_decode_step(shape, kv, gate, q, q, None, S, idx, cnt, blocks, out, lse)}[kind]
     return call, lambda: check_attention(out, lse, *ref_dense(bits(q), bits(k), bits(v), lens, 0.1), what=kind)
 
 
@@ -100,6 +115,11 @@ def _kernels_of(call):
     return [name for _, name in found if "seer" in name and "kernel" in name]
 
 
+def _name(kernel):
+    """A kernel's own name, without its scope and parameters."""
+    return re.search(r"(\w+_kernel)\b", kernel).group(1)
+
+
 def _main():
     seen = {"switches": [], "lines": []}
     for switch, value, _ in SETTINGS:
@@ -112,9 +132,10 @@ def _main():
         c.close()
     for name in SWITCHES:
         os.environ.pop(name, None)
-    c = binding.Context(0)
-    seen["lines"] = [_kernels_of(_line_call(c, kind, B, tiles)[0]) for kind, B, tiles, _ in LINES]
-    c.close()
+    for kind, B, tiles, _, *more in LINES:
+        c = binding.Context(0, *more[1:])
+        seen["lines"].append(_kernels_of(_line_call(c, kind, B, tiles, *more[:1])[0]))
+        c.close()
     print(json.dumps(seen))
 
 
@@ -133,7 +154,8 @@ def test_calls_take_the_kernels_that_a_switch_is_about(seen, at):
     switch, value, chain = SETTINGS[at]
     for name, took in seen["switches"][at].items():
         if name not in chain:
-            want = ["step_cluster_kernel"]
+            want = [EVEN if name in ("sparse", "dense") else STEP]
+            took = [_name(t) for t in took]
         else:
             # (the part of a step that the switch is not about may be either; decode_kernel<sparse, paged, tiles of rows,
             # small blocks, tensor memory>)
@@ -144,14 +166,13 @@ def test_calls_take_the_kernels_that_a_switch_is_about(seen, at):
         assert len(took) == len(want) and all(w in t for w, t in zip(want, took)), (name, want, took)
 
 
-@pytest.mark.parametrize("at", range(len(LINES)), ids=["%s-%d-%d" % s[:3] for s in LINES])
-def test_lines_between_the_one_launch_form_and_the_decode_kernel(seen, at):
-    kind, B, tiles, clusters = LINES[at]
-    took = seen["lines"][at]
-    assert ("decode_kernel" in took[-1]) != clusters and (len(took) == 1) == (clusters or kind != "step"), took
-    c = binding.Context(0)
+@pytest.mark.parametrize("at", range(len(LINES)), ids=["-".join(str(x) for x in (*l[:3], *l[4:])) for l in LINES])
+def test_lines_between_the_forms(seen, at):
+    kind, B, tiles, kernels, *more = LINES[at]
+    assert [_name(t) for t in seen["lines"][at]] == kernels, seen["lines"][at]
+    c = binding.Context(0, *more[1:])
     try:
-        call, check = _line_call(c, kind, B, tiles)
+        call, check = _line_call(c, kind, B, tiles, *more[:1])
         call()
         torch.cuda.synchronize()
         check()

@@ -23,13 +23,22 @@ CASES = [
     (8, 2, 32, 64, [60000, 300], [1800, 5]),                                                                          # 4 units, two of them long
     (8, 1, 64, 0, [55000, 0, 0, 0, 52000, 63, 64, 65, 0, 128], None),                                                  # shares that begin behind empty units
     (16, 8, 64, 0, [4096 - 7 if x % 11 == 3 else 60 for x in range(24)], None),                                        # 192 units, 24 of them of many shares
-    (16, 8, 64, 0, [64 * (2 + 3 * x) if x % 7 else 6000 + 64 * x for x in range(18)], None),                           # shares that end near units' ends
+    (16, 8, 64, 0, [64 * (1 + x) if x % 7 else 8000 + 64 * x for x in range(18)], None),                           # shares that end near units' ends
 ]
+CLUSTERS = [(2, 128), (16, 3), (1, 200), (2, 80), (4, 40), (16, 16), (16, 16), (16, 10), (1, 192), (2, 144)]      # CTAs each, how many
+
+
+def _uneven(tiles, S, clusters):
+    """The kernel's rule: a CTA alone takes 0.46 us a tile, all together 0.004, a deal 5 us."""
+    total, most = sum(tiles), max(tiles)
+    return 0.46 * most / S > max(0.004 * total, 0.46 * total / (clusters * S)) + 5
 
 
 @pytest.mark.parametrize("case", range(len(CASES)))
 def test_uneven_lists(ctx, case):
     Hq, Hkv, b, page, lens, keep = CASES[case]
+    n = [-(-L // 64) for L in lens] if keep is None else [-(-min(k, -(-L // b)) * b // 64) for k, L in zip(keep, lens)]
+    assert _uneven([x for x in n for _ in range(Hkv)], *CLUSTERS[case]) and max(n) <= 128 * CLUSTERS[case][0]
     B, d, seed = len(lens), 128, 500 + case
     unit = max(page, b, 64)
     cap = -(-max(lens) // unit) * unit

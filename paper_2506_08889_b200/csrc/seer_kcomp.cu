@@ -822,7 +822,7 @@ kcomp_stream_kernel(const __grid_constant__ CUtensorMap map_k, const KcompParams
 #endif
         }
     } else if (warp == kEpiWarps) {
-        // ---- MMA warp: Y = W_k[h] . features^T per item, issued by lane 0 ----
+        // ---- MMA warp: Y = W_k[h] . features^T per item, issued by an elected lane (the same one always, so that a commit is of its MMAs) ----
         const uint32_t tbase = sm.tmem_base;
         constexpr uint32_t idesc = tc_idesc_bf16(128, kBulkBlocks, false);
         int h_held = -1;

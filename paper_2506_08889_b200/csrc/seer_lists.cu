@@ -83,13 +83,12 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
 }
 
 // A consumer warp's step over a staged K/V tile (as in the one-launch step, whose registers do not allow a copy of it that both
-// kernels share: 0.2 us of 14), for eight rows (query token, head) of the unit: the 16 tokens `w4` of the tile,
+// kernels share: 0.2 us of 14), for the unit's up to eight heads: the 16 tokens `w4` of the tile,
 // online softmax with running maximum m_run, sum l_run and output o of its own.  S^T = K . Q^T and O^T += V^T . P^T by mma.sync,
 // tokens (channels) on M, rows on N.
-// stage: K and V of the tile; bq: the Q^T fragments; nvw: valid tokens from this warp's first one on (at least one); back: newest
-// cached tokens that this thread's two rows may not see.
+// stage: K and V of the tile; bq: the Q^T fragments; nvw: valid tokens from this warp's first one on (at least one).
 __device__ __forceinline__ void tile_step(float (&o)[8][4], float (&m_run)[2], float (&l_run)[2], unsigned char* stage,
-                                          const uint32_t (&bq)[8][2], int nvw, const int (&back)[2], float scale_log2, int lane, int w4) {
+                                          const uint32_t (&bq)[8][2], int nvw, float scale_log2, int lane, int w4) {
     const int rw = lane >> 2;
     // lane-constant parts of the ldmatrix addresses (swizzle: 16-B chunk ^= row & 7)
     const int k_row = 16 * w4 + ((lane >> 3) & 1) * 8 + (lane & 7), k_csel = lane >> 4;
@@ -121,11 +120,8 @@ __device__ __forceinline__ void tile_step(float (&o)[8][4], float (&m_run)[2], f
     float s[4];
 #pragma unroll
     for (int x = 0; x < 4; ++x) s[x] = ((sa[0][x] + sa[1][x]) + (sa[2][x] + sa[3][x])) * scale_log2;
-    const int lim0 = nvw - back[0], lim1 = nvw - back[1];      // tokens that a row sees of this warp's 16
-    if (rw >= lim0) s[0] = -INFINITY;
-    if (rw >= lim1) s[1] = -INFINITY;
-    if (rw + 8 >= lim0) s[2] = -INFINITY;
-    if (rw + 8 >= lim1) s[3] = -INFINITY;
+    if (rw >= nvw) s[0] = s[1] = -INFINITY;
+    if (rw + 8 >= nvw) s[2] = s[3] = -INFINITY;
     // ---- online softmax over this warp's 16 tokens, per row (column of S^T) ----
     float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
 #pragma unroll
@@ -553,7 +549,6 @@ __device__ __forceinline__ void list_body(const CUtensorMap& map_k, const CUtens
         // blocks of 16 or 32 tokens: which of the gathered blocks this warp's rows belong to, and where in it
         const int sub_w = !small ? 0 : p.block_size == 16 ? w4 : w4 >> 1;
         const int off_w = !small ? 16 * w4 : p.block_size == 16 ? 0 : (w4 & 1) * 16;
-        constexpr int back[2] = {0, 0};
         // false: that was the last piece
         auto consume = [&](auto first_c) -> bool {
             constexpr bool FIRST = decltype(first_c)::value;
@@ -576,7 +571,7 @@ float o[8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
                 const int st = (n + piece) % kStages;
                 if (!dead && !mbar_wait(&sm.full[n % kArrivals], (n / kArrivals) & 1, p.status)) dead = true;
                 const int nvw = (small ? (sm.meta[n % kArrivals] >> (8 * sub_w)) & 0xff : sm.meta[n % kArrivals]) - off_w;   // valid tokens from this warp's first row on
-                if (nvw > 0 && !dead) tile_step(o, m_run, l_run, sm.ring + st * kStageBytes, bq, nvw, back, p.scale_log2, lane, w4);
+                if (nvw > 0 && !dead) tile_step(o, m_run, l_run, sm.ring + st * kStageBytes, bq, nvw, p.scale_log2, lane, w4);
                 __syncwarp();
                 if (lane == 0) mbar_arrive_n(&sm.empty[st], kNW / 4);
             }

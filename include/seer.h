@@ -350,11 +350,13 @@ seer_status seer_kcomp_append(seer_ctx* ctx, const seer_shape* shape, const seer
  * blocks (Sec. 3.3).  The results are those of the three calls
  *     seer_kcomp_append(.., first_block = -1) ; seer_gate_select(.., scores_in = NULL) ; seer_sparse_decode
  * on `stream` (where step and gate call take different forms, up to blocks whose scores agree to within
- * fp32 rounding; see seer_gate_select), with one host round trip instead of three.  (With at most 64 tiles per CTA of the lists'
- * clusters and at most 16384 compressed keys per sequence, gate, attention and append are one
- * launch; up to 128, one launch and a second that does the attention where the lists are uneven.  Otherwise the launches go out as gate, attention, append: the block that has just filled is
- * the sequence's last block, which the gate takes without scoring it, so the entry the append writes is
- * first read in the next step.  When gate->max_blocks
+ * fp32 rounding; see seer_gate_select), with one host round trip instead of three.  (With at most 64 tiles per CTA of the
+ * lists' clusters and at most 16384 compressed keys per sequence, gate, attention and append are one launch.  Up to 128
+ * tiles a batch of one, whose lists are equally long, still is; others have a second launch, which does the attention
+ * where the lists are uneven (not with blocks of 16 tokens, of which a CTA lists 256).  Otherwise, and where the
+ * partial results of the second launch do not fit the workspace, the launches go out as gate, attention, append: the block
+ * that has just filled is the sequence's last block, which the gate takes without scoring it, so the entry the append
+ * writes is first read in the next step.  When gate->max_blocks
  * blocks cover kv->max_seq_len, the attention kernel knows every list's length from the sequence
  * lengths and the budget; the gate kernel then marks each list as it finishes it and the attention
  * kernel starts on a sequence's blocks as soon as that list is marked, with a bounded wait that ends

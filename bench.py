@@ -31,11 +31,11 @@ METRIC = "sparse_decode_selected_kv_GBps"
 UNIT = "GB/s"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
-# dram__bytes_read.sum + dram__bytes_write.sum of one sparse launch of the list kernel, from an ncu capture of a
-# quarter-size case (batch 2): 107.6 MB read + 3.4 MB written (other kernels' dirty lines) for 107.5 MB of algorithmic
-# bytes.  Reads grow with the selected tiles, so a launch on `batch` sequences moves about batch/2 * 107.6 MB + 3.4 MB.
-NCU_READ_BYTES_PER_2_SEQUENCES = 107.576e6
-NCU_WRITE_BYTES_PER_LAUNCH = 3.44e6
+# dram__bytes_read.sum + dram__bytes_write.sum of one sparse launch of dealt_decode_kernel, from an ncu capture of a half-size
+# case (batch 8 at 65536 tokens): 216.2 MB read + 3.8 MB written (other kernels' dirty lines) for 216.0 MB of selected K and
+# V.  Reads grow with the selected tiles.
+NCU_READ_BYTES_PER_SELECTED_BYTE = 216.207e6 / 216.007e6
+NCU_WRITE_BYTES_PER_LAUNCH = 3.79e6
 
 
 def measured_hbm_peak():
@@ -393,6 +393,8 @@ def run_ours(args):
         peak, peak_kind = measured_hbm_peak()
         value = job_throughput_gbs(world, sel_kv_bytes, step_ms)
         kern_gbs = decode_bytes / (sparse_ms * 1e-3) / 1e9
+        # (other batches and sparsities may take another kernel: by the tiles a CTA)
+        own_config = B == 8 and L == 131072 and abs(args.sparsity - 0.9) < 1e-9
         result = {
             "metric": METRIC, "value": round(value, 1), "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
             "repeats": repeats,
@@ -409,15 +411,14 @@ def run_ours(args):
             "gpu_launches": int(launches),
             "clocks": clocks,
             "roofline": {"bound": "hbm", "kernel": "seer_sparse_decode on the step's lists (dealt_decode_kernel; in the step itself "
-                                                    "step_cluster_kernel does this work)" if B >= 8 else "seer_sparse_decode",
+                                                    "step_cluster_kernel does this work)" if own_config else "seer_sparse_decode",
                          "achieved": round(kern_gbs, 1),
                          "peak": peak, "unit": "GB/s", "frac": round(kern_gbs / peak, 4), "peak_kind": f"of {peak_kind}",
                          "frac_of_nominal_8000": round(kern_gbs / NOMINAL_HBM_GBS, 4),
                          "algorithmic_bytes_per_launch": decode_bytes, "us_per_launch": round(sparse_ms * 1e3, 2),
                          "event_samples": n_ev, "empty_launch_between_events_us": round(empty_ms * 1e3, 2),
-                         "traffic": (int(NCU_READ_BYTES_PER_2_SEQUENCES * B / 2 * (1.0 - args.sparsity) / 0.1
-                                         + NCU_WRITE_BYTES_PER_LAUNCH) if abs(args.sparsity - 0.9) < 1e-9 and B >= 8 else None),
-                         "traffic_note": "ncu capture of the list kernel at batch 2, scaled by the units processed",
+                         "traffic": int(NCU_READ_BYTES_PER_SELECTED_BYTE * sel_kv_bytes + NCU_WRITE_BYTES_PER_LAUNCH) if own_config else None,
+                         "traffic_note": "ncu capture of dealt_decode_kernel at batch 8 and 65536 tokens, scaled by the selected bytes",
                          # the same kernel launched back to back (no event between launches, so that each
                          # launch's set-up overlaps its predecessor's tail as it does inside the step)
                          "us_per_launch_back_to_back": round(sparse_b2b_ms * 1e3, 2),

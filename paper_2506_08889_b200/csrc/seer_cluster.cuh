@@ -67,6 +67,8 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status, u
 // Whether the lists are dealt.  In hundredths of a microsecond: a CTA that has the memory to itself gets through a tile in 0.46
 // us (three stages, of which one or two are being read); all CTAs together through one in 0.0047 us, taken as 0.004 because
 // the last ones are alone with their tiles; a deal costs 5 us: the pieces' way through global memory and the helpers' second start.
+// Dealt lists take as long as twelve tiles a CTA at least, nine that are never dealt and a piece's three (24 sequences, one of 20 tiles a
+// CTA, the others of 2: not dealt 13.0, dealt, without this bound, 14.0).
 // (24 sequences, a quarter of them with 32 tiles a CTA, the others with 4: dealt 20.3 us, not dealt, as by a line of 8 us, 24.2; 10
 // sequences, lengths spread evenly up to 48 tiles a CTA: not dealt 34.1, dealt, as by a line of 3 us, 43.2.)
 // A step's lists are dealt by a kernel behind it: 8 us (10 sequences, half of them with 72 tiles a CTA, the others with 9: not dealt
@@ -74,8 +76,9 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status, u
 constexpr int kTileTime = 46, kDealTime = 500, kStepDealTime = 800;
 constexpr int kPieceTiles = 6;                             // a piece costs a helper as much as so many tiles a CTA (by 8, lists of 17 us 18)
 __device__ __forceinline__ bool list_uneven(int total, int most, int units, int S, int deal = kDealTime) {
-    // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S)) + deal, without its divisions)
-    return 5ll * kTileTime * most * units > max(2ll * total * S * units, 5ll * kTileTime * total) + 5ll * deal * S * units;
+    // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S), 12 * kTileTime) + deal, without its divisions)
+    return 5ll * kTileTime * most * units >
+           max(max(2ll * total * S * units, 5ll * kTileTime * total), 5ll * kTileTime * (2 * kPieceTiles) * S * units) + 5ll * deal * S * units;
 }
 // The same of a step's lists, as the sequences' lengths give them (whole warp).
 __device__ __forceinline__ bool step_uneven(const DecodeParams& p, int S) {

@@ -29,9 +29,9 @@ CLUSTERS = [(2, 128), (16, 3), (1, 200), (2, 80), (4, 40), (16, 16), (16, 16), (
 
 
 def _uneven(tiles, S, clusters):
-    """The kernel's rule: a CTA alone takes 0.46 us a tile, all together 0.004, a deal 5 us."""
+    """The kernel's rule: a CTA alone takes 0.46 us a tile, all together 0.004, a deal 5 us and twelve tiles at least."""
     total, most = sum(tiles), max(tiles)
-    return 0.46 * most / S > max(0.004 * total, 0.46 * total / (clusters * S)) + 5
+    return 0.46 * most / S > max(0.004 * total, 0.46 * total / (clusters * S), 0.46 * 12) + 5
 
 
 @pytest.mark.parametrize("case", range(len(CASES)))

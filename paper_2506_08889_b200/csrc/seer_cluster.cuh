@@ -75,6 +75,9 @@ __device__ __forceinline__ bool wait_sent(uint64_t* bar, unsigned int* status, u
 // 62.2, dealt, as by a line of 5 us, 68.6; 8, a quarter with 80: dealt 59.3, not dealt, as by one of 11 us, 70.6).
 constexpr int kTileTime = 46, kDealTime = 500, kStepDealTime = 800;
 constexpr int kPieceTiles = 6;                             // a piece costs a helper as much as so many tiles a CTA (by 8, lists of 17 us 18)
+// Lists of so many tiles a CTA are even to list_uneven: the kernel that does not ask (24 sequences, one of 20 tiles a CTA, the others of 2,
+// 13.1 -> 11.4 us; half of them of 20 19.5 -> 18.8).
+constexpr int kUndealtTiles = 2 * kPieceTiles + kDealTime / kTileTime;
 __device__ __forceinline__ bool list_uneven(int total, int most, int units, int S, int deal = kDealTime) {
     // (most * kTileTime / S > max(0.4 * total, total * kTileTime / (units * S), 12 * kTileTime) + deal, without its divisions)
     return 5ll * kTileTime * most * units >

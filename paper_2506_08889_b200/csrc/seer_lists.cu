@@ -831,7 +831,7 @@ ListPlan list_plan(int units, long long max_tiles) {
         const int S = 1 << k;
         if (k > 0 && S > max_tiles) continue;              // a CTA would have nothing to do
         if (units > resident_lists(k)) continue;
-        plan.spread = max_tiles > (long long)S * (16 + 2 * S);       // (shorter lists gain nothing by a deal)
+        plan.spread = max_tiles > (long long)S * max(16 + 2 * S, kUndealtTiles);       // (shorter lists gain nothing by a deal)
         if (2 * units <= resident_lists(k) && max_tiles > 32ll * S) {
             plan.clusters = resident_lists(k);
             plan.spread = true;

@@ -38,9 +38,9 @@ SETTINGS = [                              # a switch, its value, the calls that 
 EVEN, DEALT, DECODE, STEP, GATE = "list_step_cluster_kernel", "dealt_decode_kernel", "decode_kernel", "step_cluster_kernel", "gate_cluster_kernel"
 SMALL_WS = 3_600_000                      # bytes: the decode kernel's partials of 200 units, not the dealt lists'
 LINES = [                                 # a call, its sequences, the tiles of its one long list, its kernels (, block, workspace)
-    # two hundred units of one CTA each: above 18 tiles lists may be dealt, above 128 the decode kernel; a step is one launch up
+    # two hundred units of one CTA each: above 22 tiles lists may be dealt, above 128 the decode kernel; a step is one launch up
     # to 64, and from there to 128 the dealing kernel follows
-    ("sparse", 25, 18, [EVEN]), ("sparse", 25, 19, [DEALT]), ("dense", 25, 18, [EVEN]), ("dense", 25, 19, [DEALT]),
+    ("sparse", 25, 22, [EVEN]), ("sparse", 25, 23, [DEALT]), ("dense", 25, 22, [EVEN]), ("dense", 25, 23, [DEALT]),
     ("dense", 25, 128, [DEALT]), ("dense", 25, 129, [DECODE]),
     ("step", 25, 64, [STEP]), ("step", 25, 65, [STEP, DEALT]), ("step", 25, 128, [STEP, DEALT]), ("step", 25, 129, [GATE, DECODE]),
     # 304 units: more than there are places
@@ -53,7 +53,7 @@ LINES = [                                 # a call, its sequences, the tiles of 
     # blocks of 16 tokens: 256 numbers a CTA
     ("step", 25, 64, [STEP], 16), ("step", 25, 65, [GATE, DECODE], 16),
     # partial results that do not fit
-    ("sparse", 25, 18, [EVEN], 64, SMALL_WS), ("sparse", 25, 19, [DECODE], 64, SMALL_WS), ("step", 25, 65, [GATE, DECODE], 64, SMALL_WS),
+    ("sparse", 25, 22, [EVEN], 64, SMALL_WS), ("sparse", 25, 23, [DECODE], 64, SMALL_WS), ("step", 25, 65, [GATE, DECODE], 64, SMALL_WS),
 ]
 
 

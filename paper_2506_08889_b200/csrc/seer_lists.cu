@@ -820,7 +820,9 @@ int resident_lists(int k) {
 //     192, dense           8 sequences           241 -> 228 / 147 -> 151
 //     256, dense           8 sequences           313 -> 305 / 193 -> 201
 // One long sequence among nearly empty ones: 32 tiles a CTA 16.3 -> 14.6 (24 sequences), 15.7 -> 13.9 (16), 16.8 -> 14.4 (8); 48
-// 15.5 -> 15.9 (16); 64 15.3 -> 16.3 (24).  (A deal of 8 us, that all of a CTA's tiles but three waited for, lost up to 30 % there.)
+// 15.5 -> 15.9 (16); 64 15.3 -> 16.3 (24).  What still loses is one long list of 32 tiles a CTA among ones of 4, a CTA each (24 sequences
+// 13.8 -> 15.1, dense 12.6 -> 14.7; 20 13.3 -> 14.2): the decode kernel has four tiles a CTA there, the clusters nine and a second piece.
+// (A deal of 8 us, that all of a CTA's tiles but three waited for, lost up to 30 %.)
 // Where half of the clusters that fit would do, and a list may have more than 32 tiles a CTA, all that fit are launched, and the long
 // units dealt to those without one (a CTA by itself is far from what the memory gives): dense, one KV head of 128k 54.9 (decode
 // kernel) -> 24.4, two of 55k and 156k 48.9 -> 29.6, lists of 615 tiles 21.5 -> 15.8; with 25 tiles a CTA or less nothing is gained.
